@@ -456,7 +456,7 @@ bool batch_slot_of(fluid_solver* s, double* U, double t_end, BatchSlot& out) {
   for (int D = 0; D < 3; ++D) {
     out.seg[D] = 1;
     out.FB[D] = nullptr;
-    if (D >= s->geo.ndim || s->mixed) continue;
+    if (D == 0 || D >= s->geo.ndim || s->mixed) continue;
     int block = 128, seg = s->face_seg_d[D], grid = 0;
     face_shape(D, s->geo, block, seg, grid);
     out.seg[D] = seg;
@@ -529,6 +529,7 @@ int create_impl(const fluid_config* cfg, fluid_solver** out, SolverAlloc al) {
   ph.cfl = c.cfl;
   ph.dt_fixed = c.dt_fixed;
   ph.dt_visc_k = 2.0 * std::fmax(4.0 / 3.0, c.gamma / c.prandtl);
+  set_ff(ph);
 
   // device scratch
   const size_t nc = (size_t)g.ncell;

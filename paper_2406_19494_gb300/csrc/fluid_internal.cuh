@@ -5,7 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/fluid.h"
-#include "fast_math.cuh"
+#include "ff_math.cuh"
 
 struct fluid_solver;
 
@@ -39,6 +39,11 @@ struct Geo {
   const float* idx32[3]; // FP32 copy of idx (mixed path only, else null)
 };
 
+// The constants that the two-float terms of the FP64 face kernels use (set_ff)
+struct PhysFF {
+  ff gamma, gm1, igm1, eps4, mu_ref, mu_TS, iT_ref, suth_S, lam_fac;   // mu_TS = mu_ref (T_ref + S)
+};
+
 struct Phys {
   double gamma, gm1, igm1, R, iR, cp, Pr, lam_fac;
   double mu_ref, T_ref, iT_ref, visc_exp, suth_S;
@@ -51,6 +56,7 @@ struct Phys {
   double f[3];
   int has_force;
   double cfl, dt_fixed, dt_visc_k;
+  PhysFF k;         // two-float copies
 };
 
 struct BC {
@@ -133,6 +139,22 @@ inline void set_power_law(Phys& ph, double e) {
   }
 }
 
+// The ff constants of Phys (after its other members are set).  The indicators' 4 epsilon is kept at
+// 2^-120 or above, so that its reciprocal stays an FP32 number: smaller values only act where every
+// difference of the stencil is below 2^-60, far under the rounding of the states the ff path takes.
+inline void set_ff(Phys& ph) {
+  ph.k.gamma = ff_of(ph.gamma);
+  ph.k.gm1 = ff_of(ph.gm1);
+  ph.k.igm1 = ff_of(ph.igm1);
+  const double e4 = 4.0 * ph.eps;
+  ph.k.eps4 = ff_of(e4 < 7.52316384526264e-37 ? 7.52316384526264e-37 : e4);
+  ph.k.mu_ref = ff_of(ph.mu_ref);
+  ph.k.mu_TS = ff_of(ph.mu_ref * (ph.T_ref + ph.suth_S));
+  ph.k.iT_ref = ff_of(ph.iT_ref);
+  ph.k.suth_S = ff_of(ph.suth_S);
+  ph.k.lam_fac = ff_of(ph.lam_fac);
+}
+
 // Configuration check shared by the entry points: NULL if valid, else a static message.
 const char* config_error(const fluid_config* c);
 
@@ -159,10 +181,14 @@ constexpr int kSeamMinSeg = 4;
 long long seam_capacity(const Geo& g);   // items for segments of kSeamMinSeg cells on every axis
 // the buffer for a launch of segments of `seg` cells along D, or null when it runs without
 double* seam_buffer(int D, const Geo& g, int seg, SeamBuf fb);
-// the first cells of the segments after each line's first, from the fluxes in FB (fused: the
-// TENO kernel's update form fma(-1/dx, F+ - F-, R), else the FP64 kernel's)
+// the first cells of the segments after each line's first, from the fluxes in FB
 cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, int accumulate,
-                             int seg, bool fused, cudaStream_t st);
+                             int seg, cudaStream_t st);
+// ---- WENO5 face kernels (face_launch.cuh, one translation unit per scheme) ----------------------
+cudaError_t launch_face_js(int D, const double* W, const double* G, double* R, const Geo& g,
+                           const Phys& ph, int accumulate, int block, int seg, SeamBuf fb, cudaStream_t st);
+cudaError_t launch_face_z(int D, const double* W, const double* G, double* R, const Geo& g,
+                          const Phys& ph, int accumulate, int block, int seg, SeamBuf fb, cudaStream_t st);
 cudaError_t launch_face(int D, const double* W, const double* G, double* R, const Geo& g,
                         const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
                         cudaStream_t st);
@@ -317,6 +343,29 @@ __device__ __forceinline__ uint3 batch_bid(const int vg[3], long long lb) {
   b.z = (unsigned)(lb / ((long long)vg[0] * vg[1]));
   return b;
 }
+#define FL_BATCH_LOOP(K)                                                        \
+  const long long total_ = t->prefix[K][t->nslots];                             \
+  for (long long vb = blockIdx.x; vb < total_; vb += gridDim.x) {                \
+    const int si_ = batch_slot(t, K, vb);                                       \
+    const BatchSlot& S = t->slot[si_];                                          \
+    const uint3 bid = batch_bid(S.vgrid[K], vb - t->prefix[K][si_]);            \
+    const uint3 gdim = make_uint3(S.vgrid[K][0], S.vgrid[K][1], S.vgrid[K][2]);
+#define FL_BATCH_END \
+    __syncthreads(); \
+  }
+// blocks of a batched launch: as many as fit the GPU at once (each walks virtual blocks)
+template <class K>
+int batch_grid(K kernel, int block, size_t smem = 0) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
+    per_sm = 1;
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return per_sm * sms;
+}
+// the batched WENO5 FP64 face kernels of one axis, per scheme
+cudaError_t launch_batch_face_js(const BatchTable* dev, int D, int step, bool visc, cudaStream_t st);
+cudaError_t launch_batch_face_z(const BatchTable* dev, int D, int step, bool visc, cudaStream_t st);
 // fluid_create with stream-ordered allocations on st (cudaMallocAsync): set-up copies are enqueued
 // on st and nothing synchronises; fluid_destroy of such a solver frees on st without waiting
 int solver_create_async(const fluid_config* cfg, cudaStream_t st, fluid_solver** out);

@@ -1,0 +1,13 @@
+// WENO5-Z face kernels of the FP64 path.
+#include "face_launch.cuh"
+
+namespace fl {
+
+cudaError_t launch_face_z(int D, const double* W, const double* G, double* R, const Geo& g,
+                          const Phys& ph, int accumulate, int block, int seg, SeamBuf fb, cudaStream_t st) {
+  if (ph.visc == FLUID_VISC_NONE)
+    return launch_scheme<FLUID_WENO_Z, false>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
+  return launch_scheme<FLUID_WENO_Z, true>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
+}
+
+}  // namespace fl

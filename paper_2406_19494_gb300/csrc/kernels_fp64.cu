@@ -7,12 +7,12 @@
 //               order (Section 3.2: halo cells take values assigned by the boundary conditions)
 //   k_grad      fourth- or sixth-order central velocity gradients at cell centres (tangential
 //               derivatives of the dissipative fluxes)
-//   k_face<D>   per axis D: WENO5 reconstruction of the primitives, HLLC convective flux, the
-//               dissipative flux at the same face, and the flux difference -(F+ - F-)/dx into R.
-//               One thread marches along a segment of a grid line so each face is computed once
-//               and reused by the two cells that share it; a segment starts with the carried
-//               terms formed by the march's own operations (march_start), so the result is the
-//               same for every segment length.
+//   k_face_x, k_face<D>   per axis (face_kernels.cuh): WENO5 reconstruction of the primitives, HLLC
+//               convective flux, the dissipative flux at the same face, and the flux difference
+//               -(F+ - F-)/dx into R.  Along y and z one thread marches along a segment of a grid
+//               line so each face is computed once and reused by the two cells that share it; a
+//               segment starts with the carried terms formed by the march's own operations
+//               (march_start), so the result is the same for every segment length.
 //   k_face_seam<D>   the first cell of every segment after a line's first, from the two fluxes
 //               the neighbouring segments hand over in the seam buffer (with the buffer no face
 //               is formed twice)
@@ -28,7 +28,7 @@
 
 #include <algorithm>
 
-#include "flux_math.cuh"
+#include "face_kernels.cuh"
 #include "fluid_internal.cuh"
 
 namespace fl {
@@ -232,159 +232,11 @@ __global__ void k_grad(const double* __restrict__ W, double* __restrict__ G, Geo
 }
 
 // ------------------------------------------------------------------------------------------------
-// face flux F^c - F^d at face a+1/2 along D; `cell` is the padded index of cell a, s its stride
+// seams of the face kernels' segments (face_kernels.cuh, kernels_teno.cu)
 // ------------------------------------------------------------------------------------------------
-template <int D, int SCHEME, int VORD>
-__device__ __forceinline__ void face_flux(const double* __restrict__ W, const double* __restrict__ G,
-                                          int cell, int s, int a, const Geo& g, const Phys& ph,
-                                          double F[5], double xl[5][3], double k0[5], double k1[5]) {
-  // Carried along the march, per primitive: xl, the scaled weights (weno_x) of the left-biased
-  // value at this face, whose indicator set (A_{a-1}, B_a, C_{a+1}) was the right-biased set of
-  // the previous face; k0, k1 = (13/3) t^2 + 4 eps of the stencils centred at a and a+1 (epsilon
-  // enters each indicator through its stencil's carried term).  The right-biased value needs
-  // C_{a+2}, B_{a+1}, A_a: one new stencil (centred at a+2) per face.
-  // The indicators are taken times 4 (13/3 t^2 + s^2) with epsilon times 4: the weights of
-  // either scheme are homogeneous in (beta + eps, tau), so the normalised weights are unchanged.
-  const int nc = g.ncell;
-  const double eps4 = 4.0 * ph.eps;
-  double q[5][6];
-#pragma unroll
-  for (int v = 0; v < 5; ++v)
-#pragma unroll
-    for (int o = 0; o < 6; ++o) q[v][o] = __ldg(W + v * nc + cell + (o - 2) * s);
-  double wl[5], wr[5];
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    // cells a-2 .. a+3 are q[v][0..5]; d_j = q[v][j+1] - q[v][j]
-    const double d0 = q[v][1] - q[v][0], d1 = q[v][2] - q[v][1], d2 = q[v][3] - q[v][2];
-    const double d3 = q[v][4] - q[v][3], d4 = q[v][5] - q[v][4];
-    const double t2 = d4 - d3;
-    const double k2 = fma((4.0 * k1312) * t2, t2, eps4);   // (13/3) t^2 + 4 eps, cells a+1 .. a+3
-    const double sA = fma(3.0, d2, -d1);                   // q_{a-1} - 4 q_a + 3 q_{a+1}
-    const double sB = d2 + d3;                             // -(q_a - q_{a+2})
-    const double sC = fma(-3.0, d3, d4);                   // 3 q_{a+1} - 4 q_{a+2} + q_{a+3}
-    const double An = fma(sA, sA, k0[v]);                  // 4 (A_a + eps)
-    const double Bn = fma(sB, sB, k1[v]);                  // 4 (B_{a+1} + eps)
-    const double Cn = fma(sC, sC, k2);                     // 4 (C_{a+2} + eps)
-    wl[v] = weno_x_value(q[v][2], d0, d1, d2, d3, xl[v]);
-    double xr[3];
-    weno_x<SCHEME>(Cn, Bn, An, xr);
-    // mirrored stencil: centre q_{a+1}, differences -d4, -d3, -d2, -d1
-    wr[v] = weno_x_value(q[v][3], -d4, -d3, -d2, -d1, xr);
-    xl[v][0] = xr[2];
-    xl[v][1] = xr[1];
-    xl[v][2] = xr[0];
-    k0[v] = k1[v];
-    k1[v] = k2;
-  }
-  hllc<D>(wl, wr, ph, F);
-  if (VORD) add_visc_face<D, VORD ? VORD : 4>(W, G, cell, s, a, g, ph, q, F);
-}
-
-// The carried terms with which the march arrives at face a+1/2, formed by the operations the
-// march itself uses at face a-1/2 from cells a-2 .. a+2 (q[0..4]): the scaled weights xl of the
-// left-biased set (A_{a-1}, B_a, C_{a+1}) and k0, k1 = (13/3) t^2 + 4 eps of the stencils centred at
-// a and a+1.  A segment start therefore continues bit for bit as if the march had come from
-// further back, and the right-hand side does not depend on the segment length.
-template <int SCHEME>
-__device__ __forceinline__ void march_start(const double q[5], double eps4, double xl[3],
-                                            double& k0, double& k1) {
-  const double d1 = q[1] - q[0], d2 = q[2] - q[1], d3 = q[3] - q[2], d4 = q[4] - q[3];
-  const double c = 4.0 * k1312;
-  const double t1 = d2 - d1, t2 = d3 - d2, t3 = d4 - d3;
-  const double km = fma(c * t1, t1, eps4);                  // centred at a-1
-  k0 = fma(c * t2, t2, eps4);                               // centred at a
-  k1 = fma(c * t3, t3, eps4);                               // centred at a+1
-  const double sA = fma(3.0, d2, -d1), sB = d2 + d3, sC = fma(-3.0, d3, d4);
-  double xr[3];
-  weno_x<SCHEME>(fma(sC, sC, k1), fma(sB, sB, k0), fma(sA, sA, km), xr);
-  xl[0] = xr[2];
-  xl[1] = xr[1];
-  xl[2] = xr[0];
-}
-
-// R_a (+)= -(F_{a+1/2} - F_{a-1/2}) / dx_a with the product rounded before the sum (no fused
-// multiply-add), so that k_face and k_face_seam give the same bits
-__device__ __forceinline__ void update_r(double* dst, double F, double Fp, double id, int accumulate) {
-  const double val = __dmul_rn(-(F - Fp), id);
-  *dst = accumulate ? *dst + val : val;
-}
-
-// With a seam buffer FB (2 x 5 doubles per segment, [side][v][item]), a segment after the first
-// starts its march at face a0+1/2 instead of a0-1/2: it leaves its first cell a0 to k_face_seam,
-// with the flux at a0+1/2 in FB side 0, and its own last flux goes to FB side 1 of the next
-// segment, which is the flux at that segment's a0-1/2.  Every face is then formed once; without FB
-// each segment forms the face before its first cell as well.  Both give the same bits.
-template <int D, int SCHEME, int VORD>
-__device__ __forceinline__ void k_face_body(const double* __restrict__ W,
-                                              const double* __restrict__ G, double* __restrict__ R,
-                                              double* __restrict__ FB, Geo g, Phys ph,
-                                              int accumulate, int seg,
-    uint3 bid, uint3 gdim) {
-  constexpr int A1 = (D == 0) ? 1 : 0;
-  constexpr int A2 = (D == 2) ? 1 : 2;
-  const int n1 = g.n[A1], n2 = g.n[A2], nd = g.n[D];
-  const int nseg = (nd + seg - 1) / seg;
-  const long long lines = (long long)n1 * n2;
-  const long long total = lines * nseg;
-  const int s = D == 0 ? 1 : (D == 1 ? g.sy : g.sz);
-  const int nc = g.ncell;
-  for (long long t = bid.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gdim.x * blockDim.x) {
-    const int i1 = (int)(t % n1);
-    const long long r = t / n1;
-    const int i2 = (int)(r % n2);
-    const int sg = (int)(r / n2);
-    int c[3];
-    c[A1] = i1 + g.h[A1];
-    c[A2] = i2 + g.h[A2];
-    const int a0 = g.h[D] + sg * seg;
-    const int a1 = min(a0 + seg, g.h[D] + nd);
-    const bool seam = FB != nullptr && sg > 0;
-    c[D] = seam ? a0 : a0 - 1;
-    int cell = c[0] + c[1] * g.sy + c[2] * g.sz;
-    double Fp[5], F[5], xl[5][3], k0[5], k1[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      // the left-biased set of the march's first face and the stencil terms it carries forward
-      const double* f = W + v * nc + cell;
-      const double qw[5] = {__ldg(f - 2 * s), __ldg(f - s), __ldg(f), __ldg(f + s), __ldg(f + 2 * s)};
-      march_start<SCHEME>(qw, 4.0 * ph.eps, xl[v], k0[v], k1[v]);
-    }
-    face_flux<D, SCHEME, VORD>(W, G, cell, s, c[D], g, ph, Fp, xl, k0, k1);
-    if (seam) {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) FB[v * total + t] = Fp[v];
-    }
-    for (int a = seam ? a0 + 1 : a0; a < a1; ++a) {
-      cell += s;
-      face_flux<D, SCHEME, VORD>(W, G, cell, s, a, g, ph, F, xl, k0, k1);
-      const double id = g.idx[D][a];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        update_r(R + v * nc + cell, F[v], Fp[v], id, accumulate);
-        Fp[v] = F[v];
-      }
-    }
-    if (FB != nullptr && sg + 1 < nseg) {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) FB[(5 + v) * total + t + lines] = Fp[v];
-    }
-  }
-}
-
-template <int D, int SCHEME, int VORD>
-__global__ void __launch_bounds__(128) k_face(const double* __restrict__ W,
-                                              const double* __restrict__ G, double* __restrict__ R,
-                                              double* __restrict__ FB, Geo g, Phys ph,
-                                              int accumulate, int seg) {
-  k_face_body<D, SCHEME, VORD>(W, G, R, FB, g, ph, accumulate, seg, blockIdx, gridDim);
-}
-
 // The first cell a0 of every segment after the first: the same update as the face kernel that
-// filled FB, from the two fluxes its neighbouring segments left there (FUSED: the TENO kernel's
-// form, R = fma(-1/dx, F+ - F-, R))
-template <int D, bool FUSED>
+// filled FB, from the two fluxes its neighbouring segments left there
+template <int D>
 __device__ __forceinline__ void k_face_seam_body(const double* __restrict__ FB, double* __restrict__ R, Geo g,
                             int accumulate, int seg,
     uint3 bid, uint3 gdim) {
@@ -410,21 +262,15 @@ __device__ __forceinline__ void k_face_seam_body(const double* __restrict__ FB, 
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const double Fv = FB[v * total + t], Fpv = FB[(5 + v) * total + t];
-      double* dst = R + v * nc + cell;
-      if (FUSED) {
-        const double dF = Fv - Fpv;
-        *dst = accumulate ? fma(-id, dF, *dst) : -id * dF;
-      } else {
-        update_r(dst, Fv, Fpv, id, accumulate);
-      }
+      update_r(R + v * nc + cell, Fv, Fpv, id, accumulate);
     }
   }
 }
 
-template <int D, bool FUSED>
+template <int D>
 __global__ void k_face_seam(const double* __restrict__ FB, double* __restrict__ R, Geo g,
                             int accumulate, int seg) {
-  k_face_seam_body<D, FUSED>(FB, R, g, accumulate, seg, blockIdx, gridDim);
+  k_face_seam_body<D>(FB, R, g, accumulate, seg, blockIdx, gridDim);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -792,54 +638,10 @@ __global__ void k_wall_velocity(const double* __restrict__ phi, double* __restri
   }
 }
 
-template <int D, int SCHEME, int VORD>
-cudaError_t launch_face_t(const double* W, const double* G, double* R, const Geo& g,
-                          const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
-                          cudaStream_t st) {
-  int grid;
-  face_shape(D, g, block, seg, grid);
-  double* FB = seam_buffer(D, g, seg, fb);
-  (k_face<D, SCHEME, VORD><<<grid, block, 0, st>>>(W, G, R, FB, g, ph, accumulate, seg), ++t_launches);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || !FB) return e;
-  return launch_face_seam(D, FB, R, g, accumulate, seg, false, st);
-}
-
-template <int SCHEME, int VORD>
-cudaError_t launch_face_sv(int D, const double* W, const double* G, double* R, const Geo& g,
-                           const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
-                           cudaStream_t st) {
-  if (D == 0) return launch_face_t<0, SCHEME, VORD>(W, G, R, g, ph, accumulate, block, seg, fb, st);
-  if (D == 1) return launch_face_t<1, SCHEME, VORD>(W, G, R, g, ph, accumulate, block, seg, fb, st);
-  return launch_face_t<2, SCHEME, VORD>(W, G, R, g, ph, accumulate, block, seg, fb, st);
-}
-
-template <int SCHEME>
-cudaError_t launch_face_s(int D, const double* W, const double* G, double* R, const Geo& g,
-                          const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
-                          cudaStream_t st) {
-  if (ph.visc == FLUID_VISC_NONE)
-    return launch_face_sv<SCHEME, 0>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-  if (ph.visc_order == 6)
-    return launch_face_sv<SCHEME, 6>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-  return launch_face_sv<SCHEME, 4>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-}
-
 // ------------------------------------------------------------------------------------------------
 // batched kernels of the serving loop (see BatchTable): each block walks virtual blocks of all the
 // bucket's solves and runs the standalone body with the solve's data, block index and grid size
 // ------------------------------------------------------------------------------------------------
-#define FL_BATCH_LOOP(K)                                                        \
-  const long long total_ = t->prefix[K][t->nslots];                             \
-  for (long long vb = blockIdx.x; vb < total_; vb += gridDim.x) {                \
-    const int si_ = batch_slot(t, K, vb);                                       \
-    const BatchSlot& S = t->slot[si_];                                          \
-    const uint3 bid = batch_bid(S.vgrid[K], vb - t->prefix[K][si_]);            \
-    const uint3 gdim = make_uint3(S.vgrid[K][0], S.vgrid[K][1], S.vgrid[K][2]);
-#define FL_BATCH_END \
-    __syncthreads(); \
-  }
-
 template <bool MIXED>
 __global__ void __launch_bounds__(128) kb_prim(const BatchTable* __restrict__ t) {
   FL_BATCH_LOOP(BK_PRIM)
@@ -865,18 +667,10 @@ __global__ void __launch_bounds__(256) kb_grad(const BatchTable* __restrict__ t,
   FL_BATCH_END
 }
 
-template <int D, int SCHEME, int VORD>
-__global__ void __launch_bounds__(128) kb_face(const BatchTable* __restrict__ t, int step) {
-  FL_BATCH_LOOP(BK_FACE0 + D)
-  if (step < S.steps)
-    k_face_body<D, SCHEME, VORD>(S.W, S.G, S.R, S.FB[D], S.g, S.ph, D > 0, S.seg[D], bid, gdim);
-  FL_BATCH_END
-}
-
 template <int D>
 __global__ void __launch_bounds__(256) kb_seam(const BatchTable* __restrict__ t, int step) {
   FL_BATCH_LOOP(BK_SEAM0 + D)
-  if (step < S.steps) k_face_seam_body<D, false>(S.FB[D], S.R, S.g, D > 0, S.seg[D], bid, gdim);
+  if (step < S.steps) k_face_seam_body<D>(S.FB[D], S.R, S.g, D > 0, S.seg[D], bid, gdim);
   FL_BATCH_END
 }
 
@@ -906,29 +700,16 @@ __global__ void __launch_bounds__(256) kb_stage(const BatchTable* __restrict__ t
   FL_BATCH_END
 }
 
-// blocks of a batched launch: as many as fit the GPU at once (each walks virtual blocks)
-template <class K>
-int batch_grid(K kernel, int block, size_t smem = 0) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
-    per_sm = 1;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return per_sm * sms;
-}
-
-template <int SCHEME, int VORD>
-cudaError_t launch_batch_faces(const BatchTable* dev, int step, cudaStream_t st) {
-  static const int g0 = batch_grid(kb_face<0, SCHEME, VORD>, 128);
-  static const int g1 = batch_grid(kb_face<1, SCHEME, VORD>, 128);
-  static const int g2 = batch_grid(kb_face<2, SCHEME, VORD>, 128);
-  static const int gs = batch_grid(kb_seam<0>, 256);
-  (kb_face<0, SCHEME, VORD><<<g0, 128, 0, st>>>(dev, step), ++t_launches);
-  (kb_seam<0><<<gs, 256, 0, st>>>(dev, step), ++t_launches);
-  (kb_face<1, SCHEME, VORD><<<g1, 128, 0, st>>>(dev, step), ++t_launches);
-  (kb_seam<1><<<gs, 256, 0, st>>>(dev, step), ++t_launches);
-  (kb_face<2, SCHEME, VORD><<<g2, 128, 0, st>>>(dev, step), ++t_launches);
-  (kb_seam<2><<<gs, 256, 0, st>>>(dev, step), ++t_launches);
+cudaError_t launch_batch_faces(const BatchTable* dev, int step, int weno, bool visc,
+                               cudaStream_t st) {
+  static const int gs = batch_grid(kb_seam<1>, 256);
+  for (int D = 0; D < 3; ++D) {
+    const cudaError_t e = weno == FLUID_WENO_JS ? launch_batch_face_js(dev, D, step, visc, st)
+                                                : launch_batch_face_z(dev, D, step, visc, st);
+    if (e != cudaSuccess) return e;
+    if (D == 1) (kb_seam<1><<<gs, 256, 0, st>>>(dev, step), ++t_launches);
+    if (D == 2) (kb_seam<2><<<gs, 256, 0, st>>>(dev, step), ++t_launches);
+  }
   return cudaGetLastError();
 }
 
@@ -967,9 +748,10 @@ void batch_plan(BatchTable& t, bool mixed) {
         else set(BK_FACE0 + D, ceil_div(g.n[0], 32), ceil_div(g.n[D], kMixedTileCells), g.n[D == 1 ? 2 : 1]);
         set(BK_SEAM0 + D, 0);
       } else {
-        const long long nseg = ceil_div(g.n[D], S.seg[D]);
-        set(BK_FACE0 + D, ceil_div(lines * nseg, 128));
-        set(BK_SEAM0 + D, S.FB[D] ? ceil_div(lines * (nseg - 1), 256) : 0);
+        if (D == 0) set(BK_FACE0, tile_cols<0>(g), tile_rows<0>(g));
+        else if (D == 1) set(BK_FACE1, tile_cols<1>(g), tile_rows<1>(g));
+        else set(BK_FACE2, tile_cols<2>(g), tile_rows<2>(g));
+        set(BK_SEAM0 + D, 0);
       }
     }
     set(BK_STAGEP, ceil_div(g.n[0], 128), std::min((g.n[1] + 1) / 2, 65535), std::min(g.n[2], 65535));
@@ -1005,11 +787,7 @@ cudaError_t launch_batch_chunk(const BatchTable* dev, int chunk, bool mixed, int
           if ((e = launch_batch_mixed_faces(dev, D, k, weno, visc, st)) != cudaSuccess) return e;
       } else {
         if (visc) (kb_grad<<<gg, 256, 0, st>>>(dev, k), ++t_launches);
-        if (weno == FLUID_WENO_JS)
-          e = visc ? launch_batch_faces<FLUID_WENO_JS, 4>(dev, k, st) : launch_batch_faces<FLUID_WENO_JS, 0>(dev, k, st);
-        else
-          e = visc ? launch_batch_faces<FLUID_WENO_Z, 4>(dev, k, st) : launch_batch_faces<FLUID_WENO_Z, 0>(dev, k, st);
-        if (e != cudaSuccess) return e;
+        if ((e = launch_batch_faces(dev, k, weno, visc, st)) != cudaSuccess) return e;
       }
       if (stage < 3 || k + 1 < chunk) {
         if (mixed) {
@@ -1034,20 +812,13 @@ double* seam_buffer(int D, const Geo& g, int seg, SeamBuf fb) {
 }
 
 cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, int accumulate,
-                             int seg, bool fused, cudaStream_t st) {
+                             int seg, cudaStream_t st) {
   const long long lines = (long long)g.n[D == 0 ? 1 : 0] * g.n[D == 2 ? 1 : 2];
   const long long items = lines * ((g.n[D] + seg - 1) / seg - 1);
   const int grid = grid_for(items, 256);
-  if (D == 0) {
-    if (fused) (k_face_seam<0, true><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-    else (k_face_seam<0, false><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-  } else if (D == 1) {
-    if (fused) (k_face_seam<1, true><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-    else (k_face_seam<1, false><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-  } else {
-    if (fused) (k_face_seam<2, true><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-    else (k_face_seam<2, false><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-  }
+  if (D == 0) (k_face_seam<0><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
+  else if (D == 1) (k_face_seam<1><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
+  else (k_face_seam<2><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
   return cudaGetLastError();
 }
 
@@ -1096,9 +867,8 @@ cudaError_t launch_face(int D, const double* W, const double* G, double* R, cons
                         cudaStream_t st) {
   if (ph.weno == FLUID_TENO6A)
     return launch_face_teno(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-  if (ph.weno == FLUID_WENO_JS)
-    return launch_face_s<FLUID_WENO_JS>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-  return launch_face_s<FLUID_WENO_Z>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
+  if (ph.weno == FLUID_WENO_JS) return launch_face_js(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
+  return launch_face_z(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
 }
 
 long long seam_capacity(const Geo& g) {

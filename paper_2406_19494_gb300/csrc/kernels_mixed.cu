@@ -767,17 +767,6 @@ __global__ void __launch_bounds__(kDtBlock) k_dt_partial32(const float* __restri
 }
 
 // ---- batched kernels of the serving loop (see BatchTable in fluid_internal.cuh) -----------------
-#define FL_BATCH_LOOP(K)                                                        \
-  const long long total_ = t->prefix[K][t->nslots];                             \
-  for (long long vb = blockIdx.x; vb < total_; vb += gridDim.x) {                \
-    const int si_ = batch_slot(t, K, vb);                                       \
-    const BatchSlot& S = t->slot[si_];                                          \
-    const uint3 bid = batch_bid(S.vgrid[K], vb - t->prefix[K][si_]);            \
-    const uint3 gdim = make_uint3(S.vgrid[K][0], S.vgrid[K][1], S.vgrid[K][2]);
-#define FL_BATCH_END \
-    __syncthreads(); \
-  }
-
 __device__ __forceinline__ MixedIn batch_in(const BatchSlot& S) {
   return MixedIn{S.W, S.W32, S.W32 + (size_t)NW * S.g.ncell, S.G32};
 }
@@ -810,21 +799,11 @@ __global__ void __launch_bounds__(kDtBlock) kbm_dtp(const BatchTable* __restrict
   FL_BATCH_END
 }
 
-template <class K>
-int batch_grid_m(K kernel, int block, size_t smem = 0) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
-    per_sm = 1;
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return per_sm * sms;
-}
-
 template <int SCHEME, bool VISC>
 cudaError_t batch_face_m(const BatchTable* dev, int D, int step, cudaStream_t st) {
   constexpr size_t smem = t_smem<kMixedTileWarps, kMixedTileFaces>();
   if (D == 0) {
-    static const int gx = batch_grid_m(kbm_face_x<SCHEME, VISC>, 32 * kXRows);
+    static const int gx = batch_grid(kbm_face_x<SCHEME, VISC>, 32 * kXRows);
     (kbm_face_x<SCHEME, VISC><<<gx, dim3(32, kXRows), 0, st>>>(dev, step), ++t_launches);
     return cudaGetLastError();
   }
@@ -835,8 +814,8 @@ cudaError_t batch_face_m(const BatchTable* dev, int D, int step, cudaStream_t st
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kbm_face_t<2, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    g1 = batch_grid_m(kbm_face_t<1, SCHEME, VISC>, 128, smem);
-    g2 = batch_grid_m(kbm_face_t<2, SCHEME, VISC>, 128, smem);
+    g1 = batch_grid(kbm_face_t<1, SCHEME, VISC>, 128, smem);
+    g2 = batch_grid(kbm_face_t<2, SCHEME, VISC>, 128, smem);
     init = true;
   }
   if (D == 1) (kbm_face_t<1, SCHEME, VISC><<<g1, dim3(32, kMixedTileWarps), smem, st>>>(dev, step), ++t_launches);
@@ -1031,8 +1010,8 @@ cudaError_t launch_bulk_probe(const float* src, float* dst, int nrows, unsigned 
 }
 
 cudaError_t launch_batch_mixed(const BatchTable* dev, int kind, int D, int step, cudaStream_t st) {
-  static const int gg = batch_grid_m(kbm_grad, 256);
-  static const int gd = batch_grid_m(kbm_dtp, kDtBlock);
+  static const int gg = batch_grid(kbm_grad, 256);
+  static const int gd = batch_grid(kbm_dtp, kDtBlock);
   if (kind == BMX_GRAD) {
     (kbm_grad<<<gg, 256, 0, st>>>(dev, step), ++t_launches);
     return cudaGetLastError();

@@ -239,6 +239,7 @@ extern "C" int fluid_rhs_noalloc(const fluid_config* cfg, const double* U_dev, d
   ph.cfl = c.cfl;
   ph.dt_fixed = c.dt_fixed;
   ph.dt_visc_k = 2.0 * std::fmax(4.0 / 3.0, c.gamma / c.prandtl);
+  fl::set_ff(ph);
 
   AxisArgs A{};
   for (int a = 0; a < 3; ++a) {
