@@ -111,10 +111,47 @@ constexpr float k24H = 0.0416666679f, k24L = (float)(1.0 / 24.0 - (double)0.0416
 constexpr float kSixthH = 0.166666672f;
 __device__ __forceinline__ ff sixth() { return ff{kSixthH, (float)(1.0 / 6.0 - (double)kSixthH)}; }
 
-// face value (9 (f1 + f2) - (f0 + f3)) / 16 of an FP64 array
+// face value of an FP64 array: (9 (f1 + f2) - (f0 + f3)) / 16, or with six cells
+// (150 (f2 + f3) - 25 (f1 + f4) + 3 (f0 + f5)) / 256
+template <int NP>
 __device__ __forceinline__ ff interp_ff(const double* __restrict__ f, int s) {
   const ff f0 = ff_of(__ldg(f - s)), f1 = ff_of(__ldg(f)), f2 = ff_of(__ldg(f + s)), f3 = ff_of(__ldg(f + 2 * s));
-  return ff_scale(mul_weak(add_weak(f1, f2), 9.0f) - add_weak(f0, f3), 0.0625f);
+  if (NP == 4) return ff_scale(mul_weak(add_weak(f1, f2), 9.0f) - add_weak(f0, f3), 0.0625f);
+  const ff e = add_weak(ff_of(__ldg(f - 2 * s)), ff_of(__ldg(f + 3 * s)));
+  return ff_scale(mul_weak(add_weak(f1, f2), 150.0f) + (mul_weak(e, 3.0f) - mul_weak(add_weak(f0, f3), 25.0f)), 1.0f / 256);
+}
+
+template <int D, int NP>
+__device__ __forceinline__ void add_visc_fp64(const double* __restrict__ W, const double* __restrict__ G, int cell,
+                                              int s, int a, const Geo& g, const Phys& ph, double F[5]) {
+  const Flux5 e = visc_flux_fp64<D, NP>(W, G, cell, s, a, &g, &ph);
+#pragma unroll
+  for (int v = 1; v < 5; ++v) F[v] += e.f[v];
+}
+
+// Subtract the dissipative flux of the face: in ff from X where it is small against the state, else in
+// FP64 from F.  dv, dt: the differences of the velocities and the temperature per cell, vf and Tf their
+// face values.  sc: scales of cell a+1.
+template <int D, int NP>
+__device__ __forceinline__ void add_visc(const double* __restrict__ W, const double* __restrict__ G, int cell,
+                                         int s, int a, const Geo& g, const Phys& ph, const Scale& sc,
+                                         const ff dv[3], const ff vf[3], ff Tf, ff dt, ff X[5], double F[5]) {
+  ff Fd[4], gd[3], gb[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    if (b == D || b >= g.ndim) continue;
+    gd[b] = interp_ff<NP>(G + (D * 3 + b) * g.ncell + cell, s);
+    gb[b] = interp_ff<NP>(G + (b * 3 + b) * g.ncell + cell, s);
+  }
+  bool ok = sc.ok && visc_ff<D>(dv, vf, Tf, dt, ff_of(g.mf[D][a]), gd, gb, g.ndim, ph, Fd);
+  const float lm = kFFVisc * sc.p;
+  ok = ok && fabsf(Fd[0].h) <= lm && fabsf(Fd[1].h) <= lm && fabsf(Fd[2].h) <= lm && fabsf(Fd[3].h) <= lm * sc.c;
+  if (ok) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) X[1 + v] = X[1 + v] - Fd[v];
+  } else {
+    add_visc_fp64<D, NP>(W, G, cell, s, a, g, ph, F);
+  }
 }
 
 // The face flux F^c - F^d at a+1/2 from the terms of its two cells: d[v] = q_{a+1} - q_a, cL and cR
@@ -177,33 +214,13 @@ __device__ __forceinline__ void face_of_terms(const double* __restrict__ W, cons
     }
   }
   if (VISC) {
-    bool vok = sc.ok && ph.visc_order == 4;
-    ff Fd[4];
-    if (vok) {
-      ff vf[3], gd[3], gb[3];
+    ff vf[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) vf[c] = m3[c] - ff_scale(tv[c], 0.0625f);
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        if (b == D || b >= g.ndim) continue;
-        gd[b] = interp_ff(G + (D * 3 + b) * g.ncell + cell, s);
-        gb[b] = interp_ff(G + (b * 3 + b) * g.ncell + cell, s);
-      }
-      const ff Tf = ff_of(tm) - ff_scale(tt, 0.0625f);
-      vok = visc_ff<D>(dv, vf, Tf, dt, ff_of(g.mf[D][a]), gd, gb, g.ndim, ph, Fd);
-      const float lm = kFFVisc * sc.p;
-      vok = vok && fabsf(Fd[0].h) <= lm && fabsf(Fd[1].h) <= lm && fabsf(Fd[2].h) <= lm &&
-            fabsf(Fd[3].h) <= lm * sc.c;
-    }
-    if (vok) {
-#pragma unroll
-      for (int v = 0; v < 4; ++v) X[1 + v] = X[1 + v] - Fd[v];
-    } else {
-      const Flux5 e = ph.visc_order == 6 ? visc_flux_fp64<D, 6>(W, G, cell, s, a, &g, &ph)
-                                         : visc_flux_fp64<D, 4>(W, G, cell, s, a, &g, &ph);
-#pragma unroll
-      for (int v = 1; v < 5; ++v) F[v] += e.f[v];
-    }
+    for (int c = 0; c < 3; ++c) vf[c] = m3[c] - ff_scale(tv[c], 0.0625f);
+    if (ph.visc_order == 4)
+      add_visc<D, 4>(W, G, cell, s, a, g, ph, sc, dv, vf, ff_of(tm) - ff_scale(tt, 0.0625f), dt, X, F);
+    else
+      add_visc_fp64<D, 6>(W, G, cell, s, a, g, ph, F);
   }
 #pragma unroll
   for (int v = 0; v < 5; ++v) F[v] = __dadd_rn(F[v], ff_to_double(X[v]));
@@ -422,34 +439,49 @@ __host__ __device__ __forceinline__ int tile_cols(const Geo& g) {
   return D == 0 ? 1 : (g.n[0] + TileShape<D>::TX - 1) / TileShape<D>::TX;
 }
 
+// this thread's cell: its padded index i along D and its cell; live: on a line of the grid, pair: the
+// line has a cell after it
+struct TileCell {
+  int i, cell;
+  bool live, pair;
+};
+template <int D>
+__device__ __forceinline__ TileCell tile_cell(const Geo& g, int col, long long tile) {
+  constexpr int TX = TileShape<D>::TX;
+  constexpr int A1 = D == 0 ? 1 : 0, A2 = D == 2 ? 1 : 2;
+  const int t = threadIdx.x, P = g.p[D];
+  const long long idx = tile * TileShape<D>::step + t / TX;
+  const long long line = idx / P;
+  TileCell r;
+  r.i = (int)(idx - line * P);
+  int c[3];
+  if (D == 0) {
+    r.live = line < (long long)g.n[1] * g.n[2];
+    c[1] = g.h[1] + (r.live ? (int)(line % g.n[1]) : 0);
+    c[2] = g.h[2] + (r.live ? (int)(line / g.n[1]) : 0);
+  } else {
+    const int x = col * TX + t % TX;
+    r.live = line < g.n[A2] && x < g.n[0];
+    c[A1] = g.h[0] + (r.live ? x : 0);
+    c[A2] = g.h[A2] + (r.live ? (int)line : 0);
+  }
+  c[D] = r.live ? r.i : 0;
+  r.cell = c[0] + c[1] * g.sy + c[2] * g.sz;
+  r.pair = r.live && r.i + 1 < P;
+  return r;
+}
+
 template <int D, int SCHEME, bool VISC>
 __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, const double* __restrict__ G,
                                                  double* __restrict__ R, const Geo& g, const Phys& ph,
                                                  int accumulate, TileShared<TileShape<D>::threads>& sh,
                                                  int col, long long tile) {
   constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD;
-  constexpr int A1 = D == 0 ? 1 : 0, A2 = D == 2 ? 1 : 2;
-  const int t = threadIdx.x, row = t / TX, nc = g.ncell, P = g.p[D];
+  const int t = threadIdx.x, row = t / TX, nc = g.ncell;
   const int s = D == 0 ? 1 : (D == 1 ? g.sy : g.sz);
-  const long long idx = tile * TileShape<D>::step + row;
-  const long long line = idx / P;
-  const int i = (int)(idx - line * P);
-  int c[3];
-  c[D] = i;
-  bool live;
-  if (D == 0) {
-    live = line < (long long)g.n[1] * g.n[2];
-    c[1] = g.h[1] + (live ? (int)(line % g.n[1]) : 0);
-    c[2] = g.h[2] + (live ? (int)(line / g.n[1]) : 0);
-  } else {
-    const int x = col * TX + t % TX;
-    live = line < g.n[A2] && x < g.n[0];
-    c[A1] = g.h[0] + (live ? x : 0);
-    c[A2] = g.h[A2] + (live ? (int)line : 0);
-  }
-  if (!live) c[D] = 0;
-  const int cell = c[0] + c[1] * g.sy + c[2] * g.sz;
-  const bool pair = live && i + 1 < P;                     // the line has a cell after this one
+  const TileCell tc = tile_cell<D>(g, col, tile);
+  const bool live = tc.live, pair = tc.pair;
+  const int i = tc.i, cell = tc.cell;
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     const double* f = W + v * nc + cell;

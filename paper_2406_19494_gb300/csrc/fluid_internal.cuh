@@ -213,8 +213,7 @@ cudaError_t launch_dt_final(const double* partial, int nparts, const Phys& ph, C
 int dt_partial_count(const Geo& g);
 // ---- TENO6-A face kernels implemented in kernels_teno.cu ----------------------------------------
 cudaError_t launch_face_teno(int D, const double* W, const double* G, double* R, const Geo& g,
-                             const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
-                             cudaStream_t st);
+                             const Phys& ph, int accumulate, cudaStream_t st);
 // ---- mixed-precision launchers implemented in kernels_mixed.cu --------------------------------
 // seg 1 on the y / z tiles stages their rows by bulk copies; a copy that does not complete within
 // its bounded wait sets FLAG_STAGING in *flags (when given) and leaves its tile undone

@@ -865,8 +865,7 @@ cudaError_t launch_grad(const double* W, double* G, const Geo& g, const Phys& ph
 cudaError_t launch_face(int D, const double* W, const double* G, double* R, const Geo& g,
                         const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
                         cudaStream_t st) {
-  if (ph.weno == FLUID_TENO6A)
-    return launch_face_teno(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
+  if (ph.weno == FLUID_TENO6A) return launch_face_teno(D, W, G, R, g, ph, accumulate, st);
   if (ph.weno == FLUID_WENO_JS) return launch_face_js(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
   return launch_face_z(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
 }

@@ -1,183 +1,241 @@
 // FP64 face kernels with the paper's channel-flow reconstruction (Sec. 3.1): TENO6-A on the
 // primitive variables with the interpolation limiter, the HLLC flux, and the dissipative flux by
-// central differences of order 4 or 6 (template VORD; 0 = inviscid).
+// central differences of order 4 or 6 (template NP; 0 = inviscid).
 //
 // Interpolation limiter (reading of the paper's "interpolation limiter", its solver's
 // positivity-preserving limiting of reconstructed states): a face state with rho <= 0 or p <= 0
 // falls back, in all five primitives, to the cell on its side of the face.
 //
-// One thread marches along a segment of a grid line, as the WENO5 kernel does; each face is
-// computed once and serves the two cells that share it (across segments through the seam buffer,
-// as in k_face).  The cut-off levels of the TENO-A scale
-// sensors depend on single cells, so three of the four a face needs carry over from the previous
-// face, as do the right state's three-cell measures (the next left state's) and their factors.  A
-// segment starts with the terms the march would have carried there, formed by the same
-// operations, so the result is the same for every segment length.
+// Split between the pipes as in face_kernels.cuh (an FP64 warp instruction costs the issue slots of 64
+// others).  The scheme's weights are decisions: they depend on the two keep masks of the face and its
+// cut-off level only, and those are taken in FP32 with an error bound, in FP64 where the bound does
+// not decide (about 2 windows in 1e5).  The face values are FP64 combinations of the second differences
+// with tabulated factors; HLLC's star correction and the dissipative flux are two-float terms where
+// they are small against the state, else FP64.  On the channel 192 x 128 x 128 with 5 % noise (where
+// HLLC stays FP64 on most faces) a launch takes 1.8 to 2.2 ms; with everything in FP64 (1,149 FP64-pipe
+// instructions per face) it took 7.8 ms.
 #include <cuda_runtime.h>
 
-#include "fluid_internal.cuh"
+#include "face_kernels.cuh"
 #include "teno_math.cuh"
 
 namespace fl {
 
 namespace {
 
-// face flux F^c - F^d at face a+1/2 along D; `cell` is the padded index of cell a, s its stride;
-// lev[v][0..2] carry the cut-off levels of cells a-1, a, a+1 and b3[v] the three-cell smoothness
-// measures of the left state (see teno::face_states); both advance by one cell
-template <int D, int VORD>
-__device__ __forceinline__ void face_flux_teno(const double* __restrict__ W, const double* __restrict__ G,
-                                               int cell, int s, int a, const Geo& g, const Phys& ph,
-                                               double F[5], int lev[5][3], double b3[5][3],
-                                               double i3[5][3], double kk[5][2],
-                                               const double (*omega)[16]) {
-  const int nc = g.ncell;
-  double q[5][6];
+struct TwoValues {
+  double l, r;
+};
+
+// the face values in FP64 (a decision that FP32 leaves open)
+__device__ __noinline__ TwoValues face_values_fp64(const double* __restrict__ f, int s, double ct,
+                                                   const double (*omega)[16]) {
+  double q[6], d[5];
 #pragma unroll
-  for (int v = 0; v < 5; ++v)
+  for (int o = 0; o < 6; ++o) q[o] = __ldg(f + (o - 2) * s);
 #pragma unroll
-    for (int o = 0; o < 6; ++o) q[v][o] = __ldg(W + v * nc + cell + (o - 2) * s);
-  double wl[5], wr[5];
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    // cells a-2 .. a+3 are q[v][0..5] and d their differences (formed again from the loaded
-    // values rather than carried: the same subtractions, so the same bits, and 20 doubles fewer
-    // live across faces); the sensor level of cell a+2 is the new one
-    const double d[5] = {q[v][1] - q[v][0], q[v][2] - q[v][1], q[v][3] - q[v][2], q[v][4] - q[v][3],
-                         q[v][5] - q[v][4]};
-    const int l3 = teno::sensor_level(d[3], d[4]);
-    const double ct = teno::cutoff_of_level(min(min(lev[v][0], lev[v][1]), min(lev[v][2], l3)));
-    teno::face_states(q[v], d, ct, b3[v], i3[v], kk[v], omega, wl[v], wr[v]);
-    lev[v][0] = lev[v][1];
-    lev[v][1] = lev[v][2];
-    lev[v][2] = l3;
-  }
-  // interpolation limiter
-  if (wl[0] <= 0.0 || wl[4] <= 0.0) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) wl[v] = q[v][2];
-  }
-  if (wr[0] <= 0.0 || wr[4] <= 0.0) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) wr[v] = q[v][3];
-  }
-  hllc<D>(wl, wr, ph, F);
-  if (VORD) add_visc_face<D, VORD ? VORD : 4>(W, G, cell, s, a, g, ph, q, F);
+  for (int o = 0; o < 5; ++o) d[o] = q[o + 1] - q[o];
+  double b3[3] = {weno_B(q[1], q[2], q[3]), weno_C(q[2], q[3], q[4]), weno_A(q[0], q[1], q[2])};
+  double i3[3] = {teno::rcp6(b3[0]), teno::rcp6(b3[1]), teno::rcp6(b3[2])};
+  const double t0 = d[2] - d[1], t1 = d[3] - d[2];
+  double kk[2] = {k1312 * t0 * t0, k1312 * t1 * t1};
+  TwoValues w;
+  teno::face_states(q, d, ct, b3, i3, kk, omega, w.l, w.r);
+  return w;
 }
 
-template <int D, int VORD>
-__global__ void __launch_bounds__(128) k_face_teno(const double* __restrict__ W,
-                                                   const double* __restrict__ G, double* __restrict__ R,
-                                                   double* __restrict__ FB, Geo g, Phys ph,
-                                                   int accumulate, int seg) {
-  constexpr int A1 = (D == 0) ? 1 : 0;
-  constexpr int A2 = (D == 2) ? 1 : 2;
-  const int n1 = g.n[A1], n2 = g.n[A2], nd = g.n[D];
-  const int nseg = (nd + seg - 1) / seg;
-  const long long lines = (long long)n1 * n2;
-  const long long total = lines * nseg;
+__device__ __noinline__ int level_fp64(double dm, double dp) { return teno::sensor_level(dm, dp); }
+
+// one tile: cells (col, row) as in k_face_tile_body; NVW: primitives with differences in shared memory
+template <int N, int NVW>
+struct TenoShared {
+  double T[NVW][N];           // second differences
+  double d[NVW][N];           // q_{j+1} - q_j
+  double F[5][N];
+  unsigned char lev[5][N];    // cut-off levels of the cells
+  double alpha[4][16], omega[4][16];
+};
+
+template <int D, int NP>
+__global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>::threads) k_face_teno(
+    const double* __restrict__ W, const double* __restrict__ G, double* __restrict__ R,
+    const __grid_constant__ Geo g, const __grid_constant__ Phys ph, int accumulate) {
+  constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD, N = TileShape<D>::threads;
+  constexpr int NVW = NP ? 6 : 5;
+  extern __shared__ __align__(16) unsigned char raw[];
+  TenoShared<N, NVW>& sh = *reinterpret_cast<TenoShared<N, NVW>*>(raw);
+  const int t = threadIdx.x, row = t / TX, nc = g.ncell;
   const int s = D == 0 ? 1 : (D == 1 ? g.sy : g.sz);
-  const int nc = g.ncell;
-  // normalised weights per keep mask, k-major: for each k the 16 masks' weights sit in distinct
-  // pairs of banks, so lanes reading different masks do not conflict
-  __shared__ double omega[4][16];
-  for (int i = threadIdx.x; i < 64; i += blockDim.x) teno::weight_entry(i, omega);
+  const int cols = tile_cols<D>(g);
+  const TileCell c = tile_cell<D>(g, blockIdx.x % cols, blockIdx.x / cols);
+  const int i = c.i, cell = c.cell;
+  if (t < 64) {
+    teno::factor_entry(t, sh.alpha);
+    teno::weight_entry(t, sh.omega);
+  }
+#pragma unroll
+  for (int v = 0; v < NVW; ++v) {
+    const double* f = W + v * nc + cell;
+    sh.d[v][t] = c.pair ? __ldg(f + s) - __ldg(f) : 0.0;
+  }
   __syncthreads();
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int i1 = (int)(t % n1);
-    const long long r = t / n1;
-    const int i2 = (int)(r % n2);
-    const int sg = (int)(r / n2);
-    int c[3];
-    c[A1] = i1 + g.h[A1];
-    c[A2] = i2 + g.h[A2];
-    const int a0 = g.h[D] + sg * seg;
-    const int a1 = min(a0 + seg, g.h[D] + nd);
-    // with the seam buffer a segment after the first starts at the face after its first cell
-    // (as in k_face)
-    const bool seam = FB != nullptr && sg > 0;
-    c[D] = seam ? a0 : a0 - 1;
-    int cell = c[0] + c[1] * g.sy + c[2] * g.sz;
-    double Fp[5], F[5], b3[5][3], i3[5][3], kk[5][2];
-    int lev[5][3];
+#pragma unroll 1
+  for (int v = 0; v < NVW; ++v) {
+    const double d0 = sh.d[v][t], dm = row > 0 ? sh.d[v][t - TX] : 0.0;
+    sh.T[v][t] = d0 - dm;
+    if (v < 5) {
+      bool clear;
+      int l = teno::sensor_level32(ff_of(dm).h, ff_of(d0).h, clear);
+      if (!clear) l = level_fp64(dm, d0);
+      sh.lev[v][t] = (unsigned char)l;
+    }
+  }
+  __syncthreads();
+  // face j + 1/2
+  const bool face = row >= 2 && row < TD - 2 && c.live && i >= g.h[D] - 1 && i < g.h[D] + g.n[D];
+  double F[5];
+  if (face) {
+    const Scale sc = scale_of(__ldg(W + cell + s), __ldg(W + 4 * nc + cell + s), ph);
+    double cL[5], cR[5], d[5];
+    bool small = sc.ok;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      const double* f = W + v * nc + cell;                   // cell a = c[D]
-      const double qm2 = __ldg(f - 2 * s), qm1 = __ldg(f - s), q0 = __ldg(f), qp1 = __ldg(f + s),
-                   qp2 = __ldg(f + 2 * s);
-      // the differences of cells a-2 .. a+2 (a = a0 - 1), and the terms the march carries into
-      // the first face formed by the march's own operations (teno::face_states at the face
-      // before), so that a segment start continues bit for bit: the sensor levels of cells a-1,
-      // a, a+1, K of the stencils centred at a-1, a, a+1, then B centred at a, A centred at a+1
-      // and C centred at a-1, with their reciprocal factors
-      const double D0 = qm1 - qm2, D1 = q0 - qm1, D2 = qp1 - q0, D3 = qp2 - qp1;
-      lev[v][0] = teno::sensor_level(D0, D1);
-      lev[v][1] = teno::sensor_level(D1, D2);
-      lev[v][2] = teno::sensor_level(D2, D3);
-      const double tm = D1 - D0, ta = D2 - D1, tb = D3 - D2;
-      const double Km = k1312 * tm * tm, Ka = k1312 * ta * ta, Kb = k1312 * tb * tb;
-      const double sB = D1 + D2, sA = fma(-3.0, D2, D3), sC = fma(3.0, D1, -D0);
-      b3[v][0] = fma(0.25 * sB, sB, Ka);
-      b3[v][1] = fma(0.25 * sA, sA, Kb);
-      b3[v][2] = fma(0.25 * sC, sC, Km);
-      kk[v][0] = Ka;
-      kk[v][1] = Kb;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) i3[v][j] = teno::rcp6(b3[v][j]);
+      d[v] = sh.d[v][t];
+      const double Tm = sh.T[v][t - TX], T0 = sh.T[v][t], T1 = sh.T[v][t + TX], Tp = sh.T[v][t + 2 * TX];
+      const int lev = min(min(sh.lev[v][t - TX], sh.lev[v][t]), min(sh.lev[v][t + TX], sh.lev[v][t + 2 * TX]));
+      const float ct = lev >= 3 ? 1e-10f : (lev == 2 ? 1e-9f : (lev == 1 ? 1e-8f : 1e-7f));
+      const ff fm = ff_of(Tm), f0 = ff_of(T0), f1 = ff_of(T1), fp = ff_of(Tp);
+      const float Vm = s_add(s_sub(f0.h, fm.h), s_sub(f0.l, fm.l)), V = s_add(s_sub(f1.h, f0.h), s_sub(f1.l, f0.l));
+      const float Vp = s_add(s_sub(fp.h, f1.h), s_sub(fp.l, f1.l)), Df = ff_of(d[v]).h;
+      bool kl, kr;
+      const int mL = teno::keep_mask32(Df, f0.h, f1.h, fm.h, Vm, V, Vp, ct, kl);
+      const int mR = teno::keep_mask32(-Df, f1.h, f0.h, fp.h, -Vp, -V, -Vm, ct, kr);
+      if (kl && kr) {
+        cL[v] = fma(sh.alpha[0][mL], Tm, fma(sh.alpha[1][mL], T0, fma(sh.alpha[2][mL], T1, sh.alpha[3][mL] * Tp)));
+        cR[v] = fma(sh.alpha[0][mR], Tp, fma(sh.alpha[1][mR], T1, fma(sh.alpha[2][mR], T0, sh.alpha[3][mR] * Tm)));
+      } else {
+        const TwoValues w = face_values_fp64(W + v * nc + cell, s, teno::cutoff_of_level(lev), sh.omega);
+        const double q0 = __ldg(W + v * nc + cell), q1 = __ldg(W + v * nc + cell + s);
+        cL[v] = fma(6.0, w.l - q0, -3.0 * d[v]);
+        cR[v] = fma(6.0, w.r - q1, 3.0 * d[v]);
+      }
+      small = small && fabsf(ff_of(cR[v] - cL[v]).h) <= 6.0f * kFFJump * scale_at(sc, v);
     }
-    face_flux_teno<D, VORD>(W, G, cell, s, c[D], g, ph, Fp, lev, b3, i3, kk, omega);
-    if (seam) {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) FB[v * total + t] = Fp[v];
-    }
-    for (int a = seam ? a0 + 1 : a0; a < a1; ++a) {
-      cell += s;
-      face_flux_teno<D, VORD>(W, G, cell, s, a, g, ph, F, lev, b3, i3, kk, omega);
-      const double id = g.idx[D][a];
+    ff X[5], m3[3];
+    if (small) {
+      ff wl[5], J[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double dF = F[v] - Fp[v];
-        double* dst = R + v * nc + cell;
-        *dst = accumulate ? fma(-id, dF, *dst) : -id * dF;
-        Fp[v] = F[v];
+        const ff m = ff_of(__ldg(W + v * nc + cell)) + ff_scale(ff_of(d[v]), 0.5f);
+        if (NP && v >= 1 && v <= 3) m3[v - 1] = m;
+        J[v] = ff_of(cR[v] - cL[v]) * sixth();
+        wl[v] = ff_fma(ff_of(cL[v]), sixth(), m);
       }
-    }
-    if (FB != nullptr && sg + 1 < nseg) {
+      // the limiter's states go to FP64
+      small = wl[0].h > 0.0f && wl[4].h > 0.0f && (wl[0] + J[0]).h > 0.0f && (wl[4] + J[4]).h > 0.0f;
+      if (small) {
+        bool left;
+        hllc_ff<D>(wl, J, ph.k, left, X);
+        double w[5];
+        const int o = left ? 0 : s;
+        const double three = left ? 3.0 : -3.0;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) FB[(5 + v) * total + t + lines] = Fp[v];
+        for (int v = 0; v < 5; ++v)
+          w[v] = fma(kSixth, fma(three, d[v], left ? cL[v] : cR[v]), __ldg(W + v * nc + cell + o));
+        euler_flux<D>(w, ph, F);
+      }
+    } else if (NP) {
+#pragma unroll
+      for (int v = 1; v <= 3; ++v)
+        m3[v - 1] = ff_of(__ldg(W + v * nc + cell)) + ff_scale(ff_of(d[v]), 0.5f);
     }
+    if (!small) {
+      Flux5 l, r;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        const double* f = W + v * nc + cell;
+        l.f[v] = fma(kSixth, fma(3.0, d[v], cL[v]), __ldg(f));
+        r.f[v] = fma(kSixth, fma(-3.0, d[v], cR[v]), __ldg(f + s));
+        X[v] = ff{0.0f, 0.0f};
+      }
+      // interpolation limiter
+      if (l.f[0] <= 0.0 || l.f[4] <= 0.0) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) l.f[v] = __ldg(W + v * nc + cell);
+      }
+      if (r.f[0] <= 0.0 || r.f[4] <= 0.0) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) r.f[v] = __ldg(W + v * nc + cell + s);
+      }
+      const Flux5 e = hllc_fp64<D>(l, r, &ph);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) F[v] = e.f[v];
+    }
+    if (NP) {
+      // face values and derivatives of the velocities and the temperature in their second differences:
+      // order 4 as in face_of_terms; order 6 value m + (3 (T_{a-1} + T_{a+2}) - 19 (T_a + T_{a+1})) / 256,
+      // derivative D + (9 (T_{a+2} - T_{a-1}) - 107 (T_{a+1} - T_a)) / 1920
+      ff dv[4], vf[4];
+#pragma unroll
+      for (int c4 = 0; c4 < 4; ++c4) {
+        const int v = c4 < 3 ? 1 + c4 : NVW - 1;
+        const ff Dv = ff_of(sh.d[v][t]);
+        const ff m = c4 < 3 ? m3[c4] : ff_of(__ldg(W + 5 * nc + cell)) + ff_scale(Dv, 0.5f);
+        const ff f0 = ff_of(sh.T[v][t]), f1 = ff_of(sh.T[v][t + TX]);
+        if (NP == 4) {
+          dv[c4] = Dv - add_weak(f1, -f0) * ff{k24H, k24L};
+          vf[c4] = m - ff_scale(add_weak(f0, f1), 0.0625f);
+        } else {
+          const ff fm = ff_of(sh.T[v][t - TX]), fp = ff_of(sh.T[v][t + 2 * TX]);
+          const ff k1920{5.20833360e-04f, (float)(1.0 / 1920.0 - (double)5.20833360e-04f)};
+          dv[c4] = Dv + (mul_weak(add_weak(fp, -fm), 9.0f) - mul_weak(add_weak(f1, -f0), 107.0f)) * k1920;
+          vf[c4] = m + ff_scale(mul_weak(add_weak(fm, fp), 3.0f) - mul_weak(add_weak(f0, f1), 19.0f), 1.0f / 256);
+        }
+      }
+      add_visc<D, NP ? NP : 4>(W, G, cell, s, i, g, ph, sc, dv, vf, vf[3], dv[3], X, F);
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      F[v] = __dadd_rn(F[v], ff_to_double(X[v]));
+      sh.F[v][t] = F[v];
+    }
+  }
+  __syncthreads();
+  if (face && row >= 3 && i >= g.h[D]) {
+    const double id = g.idx[D][i];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) update_r(R + v * nc + cell, F[v], sh.F[v][t - TX], id, accumulate);
   }
 }
 
-template <int D, int VORD>
+template <int D, int NP>
 cudaError_t launch_d(const double* W, const double* G, double* R, const Geo& g, const Phys& ph,
-                     int accumulate, int block, int seg, SeamBuf fb, cudaStream_t st) {
-  int grid;
-  face_shape(D, g, block, seg, grid);
-  double* FB = seam_buffer(D, g, seg, fb);
-  (k_face_teno<D, VORD><<<grid, block, 0, st>>>(W, G, R, FB, g, ph, accumulate, seg), ++t_launches);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || !FB) return e;
-  return launch_face_seam(D, FB, R, g, accumulate, seg, st);
+                     int accumulate, cudaStream_t st) {
+  constexpr int n = TileShape<D>::threads;
+  constexpr size_t smem = sizeof(TenoShared<n, NP ? 6 : 5>);
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_face_teno<D, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const unsigned grid = (unsigned)(tile_rows<D>(g) * tile_cols<D>(g));
+  (k_face_teno<D, NP><<<grid, n, smem, st>>>(W, G, R, g, ph, accumulate), ++t_launches);
+  return cudaGetLastError();
 }
 
-template <int VORD>
-cudaError_t launch_v(int D, const double* W, const double* G, double* R, const Geo& g,
-                     const Phys& ph, int accumulate, int block, int seg, SeamBuf fb, cudaStream_t st) {
-  if (D == 0) return launch_d<0, VORD>(W, G, R, g, ph, accumulate, block, seg, fb, st);
-  if (D == 1) return launch_d<1, VORD>(W, G, R, g, ph, accumulate, block, seg, fb, st);
-  return launch_d<2, VORD>(W, G, R, g, ph, accumulate, block, seg, fb, st);
+template <int NP>
+cudaError_t launch_v(int D, const double* W, const double* G, double* R, const Geo& g, const Phys& ph,
+                     int accumulate, cudaStream_t st) {
+  if (D == 0) return launch_d<0, NP>(W, G, R, g, ph, accumulate, st);
+  if (D == 1) return launch_d<1, NP>(W, G, R, g, ph, accumulate, st);
+  return launch_d<2, NP>(W, G, R, g, ph, accumulate, st);
 }
 
 }  // namespace
 
 cudaError_t launch_face_teno(int D, const double* W, const double* G, double* R, const Geo& g,
-                             const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
-                             cudaStream_t st) {
-  if (ph.visc == FLUID_VISC_NONE) return launch_v<0>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-  if (ph.visc_order == 6) return launch_v<6>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-  return launch_v<4>(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
+                             const Phys& ph, int accumulate, cudaStream_t st) {
+  if (ph.visc == FLUID_VISC_NONE) return launch_v<0>(D, W, G, R, g, ph, accumulate, st);
+  if (ph.visc_order == 6) return launch_v<6>(D, W, G, R, g, ph, accumulate, st);
+  return launch_v<4>(D, W, G, R, g, ph, accumulate, st);
 }
 
 }  // namespace fl

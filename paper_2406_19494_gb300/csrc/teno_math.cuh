@@ -15,6 +15,7 @@
 // same four cells for the sensor, so one cut-off serves both states of a face.
 #pragma once
 
+#include "ff_math.cuh"
 #include "flux_math.cuh"
 #include "teno_coeffs.cuh"
 
@@ -79,11 +80,11 @@ FL_HD void weight_entry(int i, double omega[4][16]) {
 // 1 / (6 (beta + eps)), the factor of tau in gamma_k
 FL_HD double rcp6(double beta) { return rcp_decide(fma(6.0, beta, 6.0 * kEps)); }
 
-FL_HD double combine(double p0, double p1, double p2, double p3, double b0, double b1, double b2,
-                     double i0, double i1, double i2, double i3, double b6, double ct,
-                     const double (*omega)[16]) {
-  // b6 is 6 beta6 (beta6_pair), so tau = 6 tau6 and gamma_k = (1 + tau / (6 (beta_k + eps)))^6;
-  // i_k = rcp6(beta_k)
+// Which stencils are kept (bit k), from the three-cell smoothness measures b_k, i_k = rcp6(b_k) of all
+// four stencils, b6 = 6 beta6 (beta6_pair) and the cut-off: tau = 6 tau6 and
+// gamma_k = (1 + tau / (6 (beta_k + eps)))^6
+FL_HD int keep_mask(double b0, double b1, double b2, double i0, double i1, double i2, double i3, double b6,
+                    double ct) {
   const double tau = fabs(b6 - fma(4.0, b0, b1 + b2));
   double g[4];
   const double ik[4] = {i0, i1, i2, i3};
@@ -94,7 +95,13 @@ FL_HD double combine(double p0, double p1, double p2, double p3, double b0, doub
     g[k] = x2 * x2 * x2;
   }
   const double thr = ct * ((g[0] + g[1]) + (g[2] + g[3]));
-  const int mask = (g[0] < thr ? 0 : 1) | (g[1] < thr ? 0 : 2) | (g[2] < thr ? 0 : 4) | (g[3] < thr ? 0 : 8);
+  return (g[0] < thr ? 0 : 1) | (g[1] < thr ? 0 : 2) | (g[2] < thr ? 0 : 4) | (g[3] < thr ? 0 : 8);
+}
+
+FL_HD double combine(double p0, double p1, double p2, double p3, double b0, double b1, double b2,
+                     double i0, double i1, double i2, double i3, double b6, double ct,
+                     const double (*omega)[16]) {
+  const int mask = keep_mask(b0, b1, b2, i0, i1, i2, i3, b6, ct);
   return fma(omega[3][mask], p3, fma(omega[2][mask], p2, fma(omega[1][mask], p1, omega[0][mask] * p0)));
 }
 
@@ -148,6 +155,90 @@ FL_HD void face_states(const double q[6], const double d[5], double ct, double b
   i3c[0] = ib0;
   i3c[1] = ib2;
   i3c[2] = ib1;
+}
+
+// ------------------------------------------------------------------------------------------------
+// The same decisions in FP32, with a bound of their error: the weights of a face are those of its two
+// keep masks and its cut-off level, so an FP32 decision that its error bound cannot turn is the FP64
+// decision.  The few that it could turn are taken in FP64.
+// ------------------------------------------------------------------------------------------------
+// sensor_level in FP32; clear: no threshold lies within the error (each of N and D is within 6 2^-24
+// of itself, the differences within 2^-23)
+FL_HD int sensor_level32(float dm, float dp, bool& clear) {
+  const float e = (float)kSensorE;
+  const float N = s_fma(2.0f, fabsf(s_mul(dp, dm)), e);
+  const float Dn = s_fma(dp, dp, s_fma(dm, dm, e));
+  const float t8 = s_fma((float)-kCutEta8, Dn, N), t9 = s_fma((float)-kCutEta9, Dn, N);
+  const float t10 = s_fma((float)-kCutEta10, Dn, N);
+  clear = fminf(fminf(fabsf(t8), fabsf(t9)), fabsf(t10)) > 4e-6f * (N + Dn);
+  return (t8 >= 0.0f ? 1 : 0) + (t9 >= 0.0f ? 1 : 0) + (t10 >= 0.0f ? 1 : 0);
+}
+
+// The left state's keep mask in FP32 from the face's difference D = q_{a+1} - q_a, the second
+// differences T0, T1 of cells a and a+1 and Tm of cell a-1, and the third differences
+// Vm = T0 - Tm, V = T1 - T0, Vp = T_{a+2} - T1; the right state's is that of the mirrored window
+// (-D, T1, T0, T_{a+2}, -Vp, -V, -Vm).  In these terms the measures are sums of few terms, without
+// the cancellation of their plain forms:
+//   beta0 = 13/12 T0^2 + (D - T0/2)^2, beta1 = 13/12 T1^2 + (D - T1/2)^2,
+//   beta2 = 13/12 Tm^2 + (d + Tm/2)^2 with d = D - T0,
+//   beta3 = D^2 - D T1 + 4/3 T1^2 + 2/3 D Vp - 5/2 T1 Vp + 547/240 Vp^2,
+//   6 tau6 = 2/5 D (F1 - F0) + V (481/120 V - 3379/5040 F0 - 16823/5040 F1) - T0 (46/15 F0 + 1/5 F1)
+//            + F0 (27211/2240 F0 - 12281/1008 F1) + 139633/20160 F1^2, F0 = V - Vm, F1 = Vp - V.
+// clear: the error of tau (E, twice the largest error found over 5e6 random windows) and of the measures
+// (2^-19 of themselves) cannot turn a decision.
+FL_HD int keep_mask32(float D, float T0, float T1, float Tm, float Vm, float V, float Vp, float ct, bool& clear) {
+  const float k = 13.0f / 12.0f, tiny = 7.5e-37f;
+  const float s0 = s_fma(-0.5f, T0, D), s1 = s_fma(-0.5f, T1, D), s2 = s_fma(0.5f, Tm, s_sub(D, T0));
+  const float b0 = s_fma(k * T0, T0, s_mul(s0, s0)), b1 = s_fma(k * T1, T1, s_mul(s1, s1));
+  const float b2 = s_fma(k * Tm, Tm, s_mul(s2, s2));
+  const float b3 = s_fma(D, s_fma(2.0f / 3.0f, Vp, s_sub(D, T1)),
+                         s_fma(T1, s_fma(4.0f / 3.0f, T1, -2.5f * Vp), (547.0f / 240.0f) * Vp * Vp));
+  const float F0 = s_sub(V, Vm), F1 = s_sub(Vp, V);
+  float t = s_mul(0.4f * D, s_sub(F1, F0));
+  t = s_fma(V, s_fma(481.0f / 120.0f, V, s_fma(-3379.0f / 5040.0f, F0, (-16823.0f / 5040.0f) * F1)), t);
+  t = s_fma(-T0, s_fma(46.0f / 15.0f, F0, 0.2f * F1), t);
+  t = s_fma(F0, s_fma(27211.0f / 2240.0f, F0, (-12281.0f / 1008.0f) * F1), t);
+  t = s_fma((139633.0f / 20160.0f) * F1, F1, t);
+  const float tau = fabsf(t);
+  const float vm = fmaxf(fmaxf(fabsf(Vm), fabsf(V)), fabsf(Vp));
+  const float E = 8e-6f * vm * (fabsf(D) + fabsf(T0) + fabsf(T1) + 10.0f * vm);
+  const float i0 = s_rcp(s_fma(6.0f, b0, tiny)), i1 = s_rcp(s_fma(6.0f, b1, tiny));
+  const float i2 = s_rcp(s_fma(6.0f, b2, tiny)), i3 = s_rcp(s_fma(6.0f, b3, tiny));
+  const float im = fmaxf(fmaxf(i0, i1), fmaxf(i2, i3));
+  // no gamma ratio below (1 / 10)^6 / 4, above every cut-off: all kept
+  clear = true;
+  if ((tau + E) * im < 9.0f) return 15;
+  const float margin = 14.0f * E * s_rcp(tau) + 6e-5f;
+  const float ix = s_rcp(s_fma(tau, im, 1.0f));
+  float g[4] = {s_fma(tau, i0, 1.0f) * ix, s_fma(tau, i1, 1.0f) * ix, s_fma(tau, i2, 1.0f) * ix, s_fma(tau, i3, 1.0f) * ix};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    g[j] = g[j] * g[j] * g[j];
+    g[j] = g[j] * g[j];
+  }
+  const float thr = ct * ((g[0] + g[1]) + (g[2] + g[3]));
+  int mask = 0;
+  clear = margin < 0.25f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    mask |= g[j] < thr ? 0 : 1 << j;
+    clear = clear && fabsf(g[j] - thr) > margin * (g[j] + thr);
+  }
+  return mask;
+}
+
+// Six times the correction of a face value, w = q + (3 D + c) / 6, as factors of (T_{a-1}, T_a, T_{a+1},
+// T_{a+2}) per keep mask: the candidates are 3 D - T_a, 3 D - T_{a+1}, 3 D - 3 T_a + 2 T_{a-1} and
+// 3 D - 3/2 T_{a+1} + 1/2 T_{a+2}.  Entry i of the 64 is written by call i.
+FL_HD void factor_entry(int i, double alpha[4][16]) {
+  const int k = i >> 4, mask = i & 15;
+  double w[4], den = 0.0;
+  for (int j = 0; j < 4; ++j) {
+    w[j] = ((mask >> j) & 1) ? lin_weight(j) : 0.0;
+    den += w[j];
+  }
+  const double f = k == 0 ? 2.0 * w[2] : (k == 1 ? -(w[0] + 3.0 * w[2]) : (k == 2 ? -(w[1] + 1.5 * w[3]) : 0.5 * w[3]));
+  alpha[k][mask] = mask ? f / den : 0.0;
 }
 
 }  // namespace teno

@@ -1,11 +1,14 @@
-// Host build of the two-float terms of the FP64 face kernels (ff_math.cuh, face_ff.cuh), for a CPU
-// check: seeded cell windows and face states through the two-float formulas and through the FP64
+// Host build of the two-float terms of the FP64 face kernels (ff_math.cuh, face_ff.cuh) and of the FP32
+// decisions of TENO6-A (teno_math.cuh), for a CPU check: seeded cell windows and face states through the two-float formulas and through the FP64
 // ones (flux_math.cuh), both against the same formulas in long double.  Prints one line per case:
-// name, root-mean-square errors of the FP64 and the two-float results.
+// name, root-mean-square errors of the FP64 and the two-float results (TENO: decisions that FP32 left
+// open and decisions that differ, as shares of all).
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 
 #include "../../paper_2406_19494_gb300/csrc/face_ff.cuh"
+#include "../../paper_2406_19494_gb300/csrc/teno_math.cuh"
 
 using namespace fl;
 typedef long double L;
@@ -129,6 +132,50 @@ static void riemann(double mach, double jump) {
   std::printf("hllc%d_%g_%g %.6e %.6e\n", D, mach, jump, std::sqrt(e64 / n), std::sqrt(eff / n));
 }
 
+static void decisions(int kind) {
+  long n = 0, open_ = 0, wrong = 0;
+  for (int it = 0; it < 50000; ++it) {
+    double q[6], amp = std::pow(10.0, -4.0 + 3.5 * std::fabs(u())), k = 0.05 + 0.5 * std::fabs(u()), p = 3.0 * u();
+    const int cut = 1 + it % 5;
+    for (int i = 0; i < 6; ++i) {
+      if (kind == 0) q[i] = 1.0 + amp * std::sin(k * i + p);
+      else if (kind == 1) q[i] = 1.0 + 0.05 * u();
+      else if (kind == 2) q[i] = 1.0 + (i >= cut ? p / 3.0 : 0.0) + 0.1 * std::sin(k * i);
+      else q[i] = 0.5 * u() * std::pow(10.0, -3.0 * std::fabs(u()));
+    }
+    double d[5], t[4];
+    for (int i = 0; i < 5; ++i) d[i] = q[i + 1] - q[i];
+    for (int i = 0; i < 4; ++i) t[i] = d[i + 1] - d[i];
+    int level = 3;
+    for (int j = 0; j < 4; ++j) {
+      const int l = teno::sensor_level(d[j], d[j + 1]);
+      bool clear;
+      const int f = teno::sensor_level32(ff_of(d[j]).h, ff_of(d[j + 1]).h, clear);
+      n += 1; open_ += !clear; wrong += clear && f != l;
+      level = std::min(level, l);
+    }
+    const double ct = teno::cutoff_of_level(level);
+    const double b[3] = {weno_B(q[1], q[2], q[3]), weno_C(q[2], q[3], q[4]), weno_A(q[0], q[1], q[2])};
+    const double r[3] = {weno_B(q[4], q[3], q[2]), weno_C(q[3], q[2], q[1]), weno_A(q[5], q[4], q[3])};
+    double b6l, b6r;
+    teno::beta6_pair_diff(d, b6l, b6r);
+    auto mask = [&](const double* e, double b4, double b6) {
+      return teno::keep_mask(e[0], e[1], e[2], teno::rcp6(e[0]), teno::rcp6(e[1]), teno::rcp6(e[2]), teno::rcp6(b4), b6, ct);
+    };
+    ff T[4];
+    for (int i = 0; i < 4; ++i) T[i] = ff_of(t[i]);
+    const float Vm = (T[1].h - T[0].h) + (T[1].l - T[0].l), V = (T[2].h - T[1].h) + (T[2].l - T[1].l);
+    const float Vp = (T[3].h - T[2].h) + (T[3].l - T[2].l), D = ff_of(d[2]).h;
+    bool cl, cr;
+    const int fl_ = teno::keep_mask32(D, T[1].h, T[2].h, T[0].h, Vm, V, Vp, (float)ct, cl);
+    const int fr = teno::keep_mask32(-D, T[2].h, T[1].h, T[3].h, -Vp, -V, -Vm, (float)ct, cr);
+    n += 2; open_ += !cl + !cr;
+    wrong += (cl && fl_ != mask(b, teno::beta4_diff(d[2], d[3], d[4]), b6l)) +
+             (cr && fr != mask(r, teno::beta4_diff(d[2], d[1], d[0]), b6r));
+  }
+  std::printf("teno%d %.6e %.6e\n", kind, (double)open_ / n, (double)wrong / n);
+}
+
 int main() {
   // conversions: |x - (h + l)| <= 2^-48 |x|, and back within 2^-52
   double w1 = 0, w2 = 0;
@@ -145,5 +192,6 @@ int main() {
   for (double amp : {1e-6, 1e-4, 1e-3}) { weno<FLUID_WENO_Z>(amp); weno<FLUID_WENO_JS>(amp); }
   for (double mach : {0.1, 1.0, 3.0})
     for (double jump : {1e-7, 1e-4, 4e-3}) { riemann<0>(mach, jump); riemann<1>(mach, jump); riemann<2>(mach, jump); }
+  for (int kind = 0; kind < 4; ++kind) decisions(kind);
   return 0;
 }

@@ -63,6 +63,7 @@ def check(n, amp, kind, **kw):
 def test_tile_edges(n):
     check(n, 0.02, "wave")
     check(n, 0.2, "noise", weno="js", visc="none")
+    check(n, 0.1, "noise", weno="teno6a", visc_order=6)
 
 
 @pytest.mark.parametrize("kind", ["wave", "noise"])
@@ -70,3 +71,4 @@ def test_tile_edges(n):
 def test_limits_of_the_two_float_path(amp, kind):
     check((33, 30, 4), amp, kind)
     check((33, 30, 4), amp, kind, weno="js", visc="sutherland", mu_ref=1e-4)
+    check((33, 30, 4), amp, kind, weno="teno6a", visc_order=6, mu_ref=1e-3)
