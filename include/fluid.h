@@ -281,22 +281,17 @@ int fluid_set_time(fluid_solver* s, double t, void* stream);
  * non-positive ghost temperature since the last check (and clear the flag), else FLUID_OK. */
 int fluid_check(fluid_solver* s, void* stream);
 
-/* Launch shape of the face kernels: threads per block (a multiple of 32 in [32, 128]; 0 = 128)
- * and cells per thread segment along the face axis (0 = automatic: the longest of 64/32/16/8/4
- * that still fills the GPU), for every axis (fluid_autotune_faces picks one per axis).  For FLUID_PREC_MIXED the y and z face kernels are shared-memory
- * tiles of 2 warps (block 64) or 4 warps (otherwise) by default; seg < 0 selects the register-window
- * marching kernels with |seg| cells per segment and `block` threads instead; seg = 1 selects the
- * 4-warp tiles whose (hi, lo) rows are staged into shared memory by bulk copies (cp.async.bulk on an
- * mbarrier; a copy that does not complete within its bounded wait makes fluid_check return
- * FLUID_ECUDA).  With the tiles,
- * fluid_step folds each RK3 stage (and the primitives of its result) into the last axis's tile
- * kernel, with the same arithmetic as the separate stage kernel.  FP64 results and those of the two
- * mixed tiles are bitwise the same for every shape; the mixed register-window kernels agree with
- * the tiles to FP32 rounding. */
+/* Launch shape of the FP64 WENO5 face kernels, for every axis (fluid_autotune_faces picks one per
+ * axis): seg = 0 (automatic) runs the tiled kernels; seg > 0 the marching kernels with that many cells
+ * per thread segment along the face axis and `block` threads per block (a multiple of 32 in
+ * [32, 128]; 0 = 128).  The channel scheme and FLUID_PREC_MIXED have one shape, whatever is set (seg < 0
+ * is accepted for FLUID_PREC_MIXED only); the mixed fluid_step folds each RK3 stage and the
+ * primitives of its result into the last axis's face kernel.  Results are bitwise the same for
+ * every shape. */
 int fluid_tune_faces(fluid_solver* s, int block, int seg);
 
-/* Time the FP64 face kernels (blocks of 128 threads with segments of 8 to 32 cells and the
- * automatic choice, then blocks of 64 and 32 threads with the fastest segment length) on the
+/* Time the FP64 face kernels (the automatic choice and segments of 8 to 32 cells with blocks of 128
+ * threads, then blocks of 64 and 32 threads with the fastest segment length) on the
  * primitives of U_dev (device, the solver's padded layout; not modified) and keep the fastest shape
  * per axis; the launch shape never changes a result, so this only changes speed.
  * Enqueued on `stream` and synchronised; uses the solver's scratch, so no other call on the solver
@@ -357,7 +352,7 @@ int fluid_check_pow(const double* x_dev, double* fast_dev, double* lib_dev, int 
 int fluid_check_widen(const float* x_dev, double* bits_dev, double* cvt_dev, int n, void* stream);
 
 
-/* Check of the bulk-copy staging the mixed y / z tiles can use (fluid_tune_faces seg = 1): one warp
+/* Check of the bulk-copy helpers (cp.async.bulk on an mbarrier with a bounded wait): one warp
  * stages nrows (1..8) rows of 36 floats from src_dev (16-byte aligned, device) into shared memory
  * with cp.async.bulk on an mbarrier expecting the rows' bytes plus extra_bytes, waits with the
  * tiles' bounded wait and writes the rows to dst_dev.  extra_bytes > 0 makes the wait run out

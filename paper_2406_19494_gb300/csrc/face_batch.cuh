@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(TileShape<D>::threads, TileShape<D>::blocks) k
   FL_BATCH_LOOP(BK_FACE0 + D)
   (void)gdim;
   if (step < S.steps)
-    k_face_tile_body<D, SCHEME, VISC>(S.W, S.G, S.R, S.g, S.ph, D > 0,
+    k_face_tile_body<D, SCHEME, VISC>(S.W, S.G, S.R, S.g, S.ph,
                                       *reinterpret_cast<TileShared<TileShape<D>::threads>*>(raw), bid.x, bid.y);
   FL_BATCH_END
 }

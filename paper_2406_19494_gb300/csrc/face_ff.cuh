@@ -194,4 +194,26 @@ FL_HD bool visc_ff(const ff dn[3], const ff vf[3], ff Tf, ff dT, ff mf, const ff
   return true;
 }
 
+// x as ff, NaN where x is not finite or |x| >= 2^127 (so that the non-finite check sees it)
+FL_HD ff ff_checked(double x) {
+  ff a = ff_of(x);
+  if ((d_hi(x) & 0x7fffffff) - ((1023 - 127) << 20) > 0x0fefffff) a = ff{s_from(0x7fc00000), s_from(0x7fc00000)};
+  return a;
+}
+
+// The mixed path's conservative -> primitive conversion (prim_from_cons) in ff
+FL_HD void prim_ff(const double U[5], const Phys& ph, ff w[6]) {
+  const ff r = ff_checked(U[0]), ir = ff_rcp(r);
+  const ff m0 = ff_checked(U[1]), m1 = ff_checked(U[2]), m2 = ff_checked(U[3]);
+  const ff u = m0 * ir, v = m1 * ir, x = m2 * ir;
+  const ff ke2 = ff_fma(m0, u, ff_fma(m1, v, m2 * x));
+  const ff p = ph.k.gm1 * (ff_checked(U[4]) - ff_scale(ke2, 0.5f));
+  w[0] = quick_sum(r.h, r.l);
+  w[1] = u;
+  w[2] = v;
+  w[3] = x;
+  w[4] = p;
+  w[5] = (p * ir) * ph.k.iR;
+}
+
 }  // namespace fl

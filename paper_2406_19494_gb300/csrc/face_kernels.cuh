@@ -226,10 +226,12 @@ __device__ __forceinline__ void face_of_terms(const double* __restrict__ W, cons
   for (int v = 0; v < 5; ++v) F[v] = __dadd_rn(F[v], ff_to_double(X[v]));
 }
 
-// R_a (+)= -(F_{a+1/2} - F_{a-1/2}) / dx_a, the same operations in every kernel
-__device__ __forceinline__ void update_r(double* dst, double F, double Fp, double id, int accumulate) {
+// R_a (+)= -(F_{a+1/2} - F_{a-1/2}) / dx_a along D, the same operations in every kernel: the first axis
+// writes R, the others add to it (a constant, as a run-time choice executes both)
+template <int D>
+__device__ __forceinline__ void update_r(double* dst, double F, double Fp, double id) {
   const double dF = __dsub_rn(F, Fp);
-  *dst = accumulate ? fma(-id, dF, *dst) : __dmul_rn(-id, dF);
+  *dst = D > 0 ? fma(-id, dF, *dst) : __dmul_rn(-id, dF);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -349,7 +351,7 @@ __device__ __forceinline__ void march_face(const double* __restrict__ W, const d
 template <int D, int SCHEME, bool VISC>
 __device__ __forceinline__ void k_face_body(const double* __restrict__ W, const double* __restrict__ G,
                                             double* __restrict__ R, double* __restrict__ FB, const Geo& g,
-                                            const Phys& ph, int accumulate, int seg, uint3 bid, uint3 gdim) {
+                                            const Phys& ph, int seg, uint3 bid, uint3 gdim) {
   constexpr int A1 = (D == 0) ? 1 : 0;
   constexpr int A2 = (D == 2) ? 1 : 2;
   const int n1 = g.n[A1], n2 = g.n[A2], nd = g.n[D];
@@ -384,7 +386,7 @@ __device__ __forceinline__ void k_face_body(const double* __restrict__ W, const 
       if (a > first) {
         const double id = g.idx[D][a];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) update_r(R + v * nc + cell, F[v], Fp[v], id, accumulate);
+        for (int v = 0; v < 5; ++v) update_r<D>(R + v * nc + cell, F[v], Fp[v], id);
       } else if (seam) {
 #pragma unroll
         for (int v = 0; v < 5; ++v) FB[v * total + t] = F[v];
@@ -429,14 +431,14 @@ struct TileShared {
 };
 
 // tiles along (x, D) that cover the interior cells
-template <int D>
+template <int D, class S = TileShape<D>>
 __host__ __device__ __forceinline__ long long tile_rows(const Geo& g) {
   const long long lines = (long long)g.n[0] * g.n[1] * g.n[2] / g.n[D] / (D == 0 ? 1 : g.n[0]);
-  return (lines * g.p[D] + TileShape<D>::step - 1) / TileShape<D>::step;
+  return (lines * g.p[D] + S::step - 1) / S::step;
 }
-template <int D>
+template <int D, class S = TileShape<D>>
 __host__ __device__ __forceinline__ int tile_cols(const Geo& g) {
-  return D == 0 ? 1 : (g.n[0] + TileShape<D>::TX - 1) / TileShape<D>::TX;
+  return D == 0 ? 1 : (g.n[0] + S::TX - 1) / S::TX;
 }
 
 // this thread's cell: its padded index i along D and its cell; live: on a line of the grid, pair: the
@@ -445,12 +447,12 @@ struct TileCell {
   int i, cell;
   bool live, pair;
 };
-template <int D>
+template <int D, class S = TileShape<D>>
 __device__ __forceinline__ TileCell tile_cell(const Geo& g, int col, long long tile) {
-  constexpr int TX = TileShape<D>::TX;
+  constexpr int TX = S::TX;
   constexpr int A1 = D == 0 ? 1 : 0, A2 = D == 2 ? 1 : 2;
   const int t = threadIdx.x, P = g.p[D];
-  const long long idx = tile * TileShape<D>::step + t / TX;
+  const long long idx = tile * S::step + t / TX;
   const long long line = idx / P;
   TileCell r;
   r.i = (int)(idx - line * P);
@@ -474,7 +476,7 @@ __device__ __forceinline__ TileCell tile_cell(const Geo& g, int col, long long t
 template <int D, int SCHEME, bool VISC>
 __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, const double* __restrict__ G,
                                                  double* __restrict__ R, const Geo& g, const Phys& ph,
-                                                 int accumulate, TileShared<TileShape<D>::threads>& sh,
+                                                 TileShared<TileShape<D>::threads>& sh,
                                                  int col, long long tile) {
   constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD;
   const int t = threadIdx.x, row = t / TX, nc = g.ncell;
@@ -567,7 +569,7 @@ __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, c
   if (face && row >= 3 && i >= g.h[D]) {
     const double id = g.idx[D][i];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) update_r(R + v * nc + cell, F[v], sh.F[v][t - TX], id, accumulate);
+    for (int v = 0; v < 5; ++v) update_r<D>(R + v * nc + cell, F[v], sh.F[v][t - TX], id);
   }
 }
 

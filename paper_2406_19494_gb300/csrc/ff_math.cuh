@@ -150,13 +150,14 @@ FL_HD ff ff_of(double x) {
 // h + l as FP64 for a normalised pair, within 2^-52 of it: h's bits widened, then l added in units
 // of the result's last place.  The bit pattern of a double grows by one per unit in the last
 // place, so the addition is an integer one; below a power of two the unit is half as large.
-// |h| < 2^-70 gives h rounded to a few bits or 0; h must be finite.
+// |h| < 2^-70 gives h rounded to a few bits or 0; an infinite h or a NaN gives NaN.
 FL_HD double ff_to_double(ff a) {
   const int u = s_bits(a.h);
   const int e = u & 0x7f800000;
   // below 2^-70 the binade of 2^-70 stands in: the value is far below any use
   const int eb = e < (57 << 23) ? (57 << 23) : e;
-  const int hi = (u & (int)0x80000000u) | (((u & 0x7fffffff) >> 3) + (e == 0 ? 0 : (1023 - 127) << 20));
+  int hi = (u & (int)0x80000000u) | (((u & 0x7fffffff) >> 3) + (e == 0 ? 0 : (1023 - 127) << 20));
+  if (e == 0x7f800000) hi = 0x7ff80000;
   const int lo = u << 29;
   float k = s_mul(a.l, s_from((306 << 23) - eb));               // l times 2^(52 - (e - 127))
   // same sign as h: away from zero

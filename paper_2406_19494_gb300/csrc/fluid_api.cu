@@ -52,9 +52,8 @@ struct fluid_solver {
   double* G = nullptr;             // velocity gradients, NG * ncell (viscous, FP64 path)
   bool mixed = false;              // FLUID_PREC_MIXED: FP32 fluxes, FP64 state
   bool exchange = false;           // some face is FLUID_BC_EXCHANGE (a block of a decomposition)
-  float* W32 = nullptr;            // FP32 (hi, lo) primitives, 2 NW * ncell (mixed)
-  double* Wb = nullptr;            // mixed: the second pair of primitive buffers (W with its H row,
-  float* W32b = nullptr;           // W32), written by a stage fused into the last face kernel
+  float* W32 = nullptr;            // primitives as pairs of floats, 2 NW * ncell (mixed)
+  float* W32b = nullptr;           // mixed: the second buffer, written by a stage fused into the last face kernel
   float* mf32 = nullptr;           // FP32 face metrics, centre metrics and inverse widths of the three axes (mixed)
   float* G32 = nullptr;            // FP32 velocity gradients (mixed, viscous)
   double* A = nullptr;             // RK stage state, NV * ncell
@@ -76,7 +75,6 @@ struct fluid_solver {
     cudaEvent_t a, b;
     long long kernels;   // kernels enqueued between the two events
   };
-  int face_block = 0, face_seg = 0;   // launch shape of the face kernels (0 = automatic)
   int face_seg_d[3] = {0, 0, 0};      // FP64 path: segment length per axis (0 = automatic)
   int face_block_d[3] = {0, 0, 0};    // FP64 path: threads per block per axis (0 = 128)
   // adjoint scratch (cfg.adjoint != 0)
@@ -313,15 +311,14 @@ int grad_faces(fluid_solver* s, double* R, cudaStream_t st) {
       FL_TIMED(s, FLUID_KERNEL_GRAD, st, fl::launch_grad32(s->W32, s->G32, g, st));
     for (int d = 0; d < g.ndim; ++d)
       FL_TIMED(s, FLUID_KERNEL_FACE_X + d, st,
-               fl::launch_face_mixed(d, s->W, s->W32, s->G32, R, g, s->ph, d > 0, s->face_block,
-                                     s->face_seg, st, &s->ctl->flags));
+               fl::launch_face_mixed(d, s->W32, s->G32, R, g, s->ph, st));
     return FLUID_OK;
   }
   if (s->ph.visc != FLUID_VISC_NONE)
     FL_TIMED(s, FLUID_KERNEL_GRAD, st, fl::launch_grad(s->W, s->G, g, s->ph, st));
   for (int d = 0; d < g.ndim; ++d)
     FL_TIMED(s, FLUID_KERNEL_FACE_X + d, st,
-             fl::launch_face(d, s->W, s->G, R, g, s->ph, d > 0, s->face_block_d[d], s->face_seg_d[d],
+             fl::launch_face(d, s->W, s->G, R, g, s->ph, s->face_block_d[d], s->face_seg_d[d],
                              fl::SeamBuf{s->FB, s->fb_cap}, st));
   return FLUID_OK;
 }
@@ -347,7 +344,7 @@ int dt_into(fluid_solver* s, double* dt_out, int clip, double t_end, cudaStream_
 int stage_into(fluid_solver* s, int stage, const double* Un, const double* Us, double* Ud,
                double t_end, cudaStream_t st) {
   FL_TIMED(s, FLUID_KERNEL_STAGE, st,
-           fl::launch_stage(stage, Un, Us, s->R, Ud, s->W, s->geo, s->ph, s->ctl, t_end, st));
+           fl::launch_stage(stage, Un, Us, s->R, Ud, s->W, s->W32, s->geo, s->ph, s->ctl, t_end, st));
   return FLUID_OK;
 }
 
@@ -360,11 +357,11 @@ int stage_prim_into(fluid_solver* s, int stage, const double* Un, const double* 
   return FLUID_OK;
 }
 
-// Mixed path, one RK3 stage from the primitives of its input (in W / W32): the face kernels of the
+// Mixed path, one RK3 stage from the primitives of its input (in W32): the face kernels of the
 // axes before the last into R, then the last axis's face kernel fused with the stage combination
-// into Ud and the primitives of Ud into the second buffer pair (prims), whose halo cells follow;
-// the pairs then swap, so W / W32 hold the primitives of Ud.  Without prims (the last stage of a
-// call) only Ud is written.
+// into Ud and the primitives of Ud into the second buffer (prims), whose halo cells follow; the
+// buffers then swap, so W32 holds the primitives of Ud.  Without prims (the last stage of a call)
+// only Ud is written.
 int stage_fused_into(fluid_solver* s, int stage, const double* Un, const double* Us, double* Ud,
                      bool prims, double t_end, cudaStream_t st) {
   const Geo& g = s->geo;
@@ -372,15 +369,12 @@ int stage_fused_into(fluid_solver* s, int stage, const double* Un, const double*
     FL_TIMED(s, FLUID_KERNEL_GRAD, st, fl::launch_grad32(s->W32, s->G32, g, st));
   for (int d = 0; d + 1 < g.ndim; ++d)
     FL_TIMED(s, FLUID_KERNEL_FACE_X + d, st,
-             fl::launch_face_mixed(d, s->W, s->W32, s->G32, s->R, g, s->ph, d > 0, s->face_block,
-                                   s->face_seg, st, &s->ctl->flags));
-  const fl::StageOut so{stage, prims ? 1 : 0, Un, Us, Ud, s->Wb, s->W32b, s->ctl, t_end};
+             fl::launch_face_mixed(d, s->W32, s->G32, s->R, g, s->ph, st));
+  const fl::StageOut so{stage, prims ? 1 : 0, Un, Us, Ud, s->W32b, s->ctl, t_end};
   FL_TIMED(s, FLUID_KERNEL_FACE_X + g.ndim - 1, st,
-           fl::launch_face_mixed_stage(s->W, s->W32, s->G32, s->R, g, s->ph, s->face_block, s->face_seg,
-                                       so, st));
+           fl::launch_face_mixed_stage(s->W32, s->G32, s->R, g, s->ph, so, st));
   if (prims) {
-    FL_TIMED(s, FLUID_KERNEL_STAGE, st, fl::launch_halo_prim(s->Wb, s->W32b, g, s->ph, s->bc, s->ctl, st));
-    std::swap(s->W, s->Wb);
+    FL_TIMED(s, FLUID_KERNEL_STAGE, st, fl::launch_halo_prim(nullptr, s->W32b, g, s->ph, s->bc, s->ctl, st));
     std::swap(s->W32, s->W32b);
   }
   return FLUID_OK;
@@ -543,14 +537,11 @@ int create_impl(const fluid_config* cfg, fluid_solver** out, SolverAlloc al) {
   };
   if ((e = al.malloc((void**)&s->metric, nmetric * sizeof(double))) != cudaSuccess) return bail(e, "cudaMalloc metric");
   s->mixed = c.precision == FLUID_PREC_MIXED;
-  // the mixed path keeps H = E + p in one more FP64 row of W
-  if ((e = al.malloc((void**)&s->W, (fl::NW + (s->mixed ? 1 : 0)) * nc * sizeof(double))) != cudaSuccess)
+  if ((e = al.malloc((void**)&s->W, fl::NW * nc * sizeof(double))) != cudaSuccess)
     return bail(e, "cudaMalloc W");
   if (s->mixed) {
-    // W32 buffers: 64 floats of slack past the end for the aligned tails of bulk-staged rows
-    if ((e = al.malloc((void**)&s->W32, (2 * fl::NW * nc + 64) * sizeof(float))) != cudaSuccess) return bail(e, "cudaMalloc W32");
-    if ((e = al.malloc((void**)&s->Wb, (fl::NW + 1) * nc * sizeof(double))) != cudaSuccess) return bail(e, "cudaMalloc Wb");
-    if ((e = al.malloc((void**)&s->W32b, (2 * fl::NW * nc + 64) * sizeof(float))) != cudaSuccess) return bail(e, "cudaMalloc W32b");
+    if ((e = al.malloc((void**)&s->W32, 2 * fl::NW * nc * sizeof(float))) != cudaSuccess) return bail(e, "cudaMalloc W32");
+    if ((e = al.malloc((void**)&s->W32b, 2 * fl::NW * nc * sizeof(float))) != cudaSuccess) return bail(e, "cudaMalloc W32b");
     if ((e = al.malloc((void**)&s->mf32, 3 * (nmetric / 5) * sizeof(float))) != cudaSuccess) return bail(e, "cudaMalloc mf32");
     if (c.visc_law != FLUID_VISC_NONE)
       if ((e = al.malloc((void**)&s->G32, fl::NG * nc * sizeof(float))) != cudaSuccess) return bail(e, "cudaMalloc G32");
@@ -715,7 +706,6 @@ void fluid_destroy(fluid_solver* s) {
   al.free(s->W);
   al.free(s->G);
   al.free(s->W32);
-  al.free(s->Wb);
   al.free(s->W32b);
   al.free(s->mf32);
   al.free(s->G32);
@@ -797,7 +787,7 @@ int fluid_rhs(fluid_solver* s, const double* U_dev, double* R_dev, void* stream)
   cudaStream_t st = as_stream(stream);
   if (int r = rhs_into(s, U_dev, R_dev, st)) return r;
   if (s->ph.has_force)
-    FL_TIMED(s, FLUID_KERNEL_SOURCE, st, fl::launch_source(R_dev, s->W, s->geo, s->ph, st));
+    FL_TIMED(s, FLUID_KERNEL_SOURCE, st, fl::launch_source(R_dev, s->W, s->W32, s->geo, s->ph, st));
   return FLUID_OK;
 }
 
@@ -821,8 +811,8 @@ int fluid_step(fluid_solver* s, double* U_dev, int nsteps, double t_end, void* s
   // and the call's last stage, whose primitives nothing reads, is the plain combination.
   if (nsteps > 0)
     FL_TIMED(s, FLUID_KERNEL_PRIM_BC, st, fl::launch_prim_bc(U_dev, s->W, s->W32, s->geo, s->ph, s->bc, s->ctl, st));
-  // the mixed path on the y / z tile kernels folds each stage into the last axis's face kernel
-  const bool fused = s->mixed && fl::mixed_stage_fusable(s->geo, s->face_seg);
+  // the mixed path folds each stage into the last axis's face kernel
+  const bool fused = s->mixed;
   for (int k = 0; k < nsteps; ++k) {
     if (fused) {
       if (int r = dt_into(s, nullptr, 1, t_end, st)) return r;
@@ -901,11 +891,11 @@ int fluid_adjoint_step(fluid_solver* s, const double* Un_dev, const double* U1_d
     s->W = s->Wn;
     s->G = s->Gn;
     if (int r = rhs_into(s, Un_dev, s->R, st)) return r;
-    FL_TIMED(s, FLUID_KERNEL_STAGE, st, fl::launch_stage(1, Un_dev, Un_dev, s->R, s->S1, s->W, g, s->ph, s->ctl, 0.0, st, dt));
+    FL_TIMED(s, FLUID_KERNEL_STAGE, st, fl::launch_stage(1, Un_dev, Un_dev, s->R, s->S1, s->W, nullptr, g, s->ph, s->ctl, 0.0, st, dt));
     s->W = s->W1;
     s->G = s->G1;
     if (int r = rhs_into(s, s->S1, s->R, st)) return r;
-    FL_TIMED(s, FLUID_KERNEL_STAGE, st, fl::launch_stage(2, Un_dev, s->S1, s->R, s->S2, s->W, g, s->ph, s->ctl, 0.0, st, dt));
+    FL_TIMED(s, FLUID_KERNEL_STAGE, st, fl::launch_stage(2, Un_dev, s->S1, s->R, s->S2, s->W, nullptr, g, s->ph, s->ctl, 0.0, st, dt));
     X1 = s->S1;
     X2 = s->S2;
   }
@@ -935,7 +925,7 @@ int fluid_wall_fluxes(fluid_solver* s, const double* U_dev, int axis, int side, 
   if (kind != FLUID_BC_WALL && kind != FLUID_BC_POROUS)
     return fail(s, FLUID_EINVAL, "wall fluxes need an isothermal or porous face");
   cudaStream_t st = as_stream(stream);
-  FL_TIMED(s, FLUID_KERNEL_PRIM_BC, st, fl::launch_prim_bc(U_dev, s->W, s->W32, s->geo, s->ph, s->bc, s->ctl, st));
+  FL_TIMED(s, FLUID_KERNEL_PRIM_BC, st, fl::launch_prim_bc(U_dev, s->W, nullptr, s->geo, s->ph, s->bc, s->ctl, st));
   FL_CUDA(s, fl::launch_wall_fluxes(s->W, qw_dev, tw_dev, s->geo, s->ph, axis, side, s->bc.Tw[axis][side], st));
   return FLUID_OK;
 }
@@ -1004,7 +994,7 @@ int fluid_rk3_stage(fluid_solver* s, int stage, const double* Un_dev, const doub
   cudaStream_t st = as_stream(stream);
   if (int r = rhs_into(s, Us_dev, s->R, st)) return r;
   FL_TIMED(s, FLUID_KERNEL_STAGE, st,
-           fl::launch_stage(stage, Un_dev, Us_dev, s->R, Ud_dev, s->W, s->geo, s->ph, s->ctl, 0.0,
+           fl::launch_stage(stage, Un_dev, Us_dev, s->R, Ud_dev, s->W, s->W32, s->geo, s->ph, s->ctl, 0.0,
                             st, dt));
   return FLUID_OK;
 }
@@ -1052,8 +1042,6 @@ int fluid_tune_faces(fluid_solver* s, int block, int seg) {
   if (block != 0 && (block < 32 || block > 128 || block % 32 != 0))
     return fail(s, FLUID_EINVAL, "block must be 0 or a multiple of 32 in [32, 128]");
   if (seg < 0 && !s->mixed) return fail(s, FLUID_EINVAL, "seg must be >= 0 for the FP64 path");
-  s->face_block = block;
-  s->face_seg = seg;
   for (int d = 0; d < 3; ++d) {
     s->face_seg_d[d] = seg;
     s->face_block_d[d] = block;
@@ -1085,7 +1073,7 @@ int fluid_autotune_faces(fluid_solver* s, const double* U_dev, void* stream) {
     bool have = false;
     auto trial = [&](int block, int seg) {
       auto launch = [&]() {
-        return fl::launch_face(d, s->W, s->G, s->R, g, s->ph, 0, block, seg, fl::SeamBuf{s->FB, s->fb_cap}, st);
+        return fl::launch_face(d, s->W, s->G, s->R, g, s->ph, block, seg, fl::SeamBuf{s->FB, s->fb_cap}, st);
       };
       if ((e = launch()) != cudaSuccess) return;                      // warm-up
       if ((e = cudaEventRecord(e0, st)) != cudaSuccess) return;

@@ -19,9 +19,6 @@ constexpr int NG = 9;   // velocity-gradient scratch, component c * 3 + b = d u_
 constexpr unsigned FLAG_NONFINITE = 1u;
 constexpr unsigned FLAG_GHOST_T = 2u;
 constexpr unsigned FLAG_STAGING = 4u;   // a shared-memory staging copy did not complete in time
-// the mixed path's y / z face tiles: 4 warps of 3 faces, 11 cells along the face axis
-constexpr int kMixedTileWarps = 4, kMixedTileFaces = 3;
-constexpr int kMixedTileCells = kMixedTileWarps * kMixedTileFaces - 1;
 
 // Grid geometry: padded sizes, strides and per-axis 1-D metric arrays (device, length p[a]).
 struct Geo {
@@ -41,7 +38,7 @@ struct Geo {
 
 // The constants that the two-float terms of the FP64 face kernels use (set_ff)
 struct PhysFF {
-  ff gamma, gm1, igm1, eps4, mu_ref, mu_TS, iT_ref, suth_S, lam_fac;   // mu_TS = mu_ref (T_ref + S)
+  ff gamma, gm1, igm1, gg, iR, eps4, mu_ref, mu_TS, iT_ref, suth_S, lam_fac;   // gg = gamma / (gamma - 1), mu_TS = mu_ref (T_ref + S)
 };
 
 struct Phys {
@@ -78,22 +75,29 @@ __device__ __forceinline__ bool finite_bits(double x) {
   return ((__double2hiint(x) >> 20) & 0x7ff) != 0x7ff;
 }
 
-// Split x = hi + lo + r with |r| <= 2^-48 |x|, using integer operations only: hi keeps the sign,
-// the exponent and the leading 23 fraction bits of x (x truncated to FP32 precision, exact), lo the
-// remaining 29 fraction bits rounded to FP32.  Below 2^-73 lo is dropped (|r| < 2^-23 |x| <
-// 1.2e-29), below 2^-126 both are zero; |x| >= 2^128 or a non-finite x gives NaN, which the
-// non-finite check then reports.
-__device__ __forceinline__ void split_hi_lo(double x, float& hi, float& lo) {
-  const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
-  const unsigned sign = hw & 0x80000000u;
-  const int e = (int)((hw >> 20) & 0x7ffu);            // biased FP64 exponent
-  if (e < 1023 - 126) { hi = __int_as_float(sign); lo = 0.0f; return; }
-  if (e > 1023 + 127) { hi = __int_as_float(0x7fc00000); lo = hi; return; }
-  hi = __int_as_float(sign | ((unsigned)(e - 1023 + 127) << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29));
-  // lo = (low 29 fraction bits) * 2^(e - 1075), with 2^(e - 1075) a normal float when e > 948
-  const int es = e - 1075 + 127;
-  const float m = (float)(lw & 0x1fffffffu);
-  lo = es > 0 ? __int_as_float(sign | __float_as_int(m * __int_as_float(es << 23))) : 0.0f;
+// Primitives of the mixed path: W32 = [2 NW][ncell] floats, rows v and NW + v the two floats of
+// primitive v.
+__device__ __forceinline__ ff load_pair(const float* __restrict__ W32, int nc, int v, int cell) {
+  return ff{W32[v * nc + cell], W32[(NW + v) * nc + cell]};
+}
+__device__ __forceinline__ void store_pair(float* __restrict__ W32, int nc, int v, int cell, ff w) {
+  W32[v * nc + cell] = w.h;
+  W32[(NW + v) * nc + cell] = w.l;
+}
+
+// One RK3 stage: stage 1 Un + dt r; stage 2 3/4 Un + 1/4 (Us + dt r); stage 3 1/3 Un + 2/3 (Us + dt r).
+// The last two share their operations with the factors chosen first (a choice between the formulas
+// executes both).
+__device__ __forceinline__ void stage_combine(int stage, double dt, const double un[5], const double us[5],
+                                              const double r[5], double out[5]) {
+  if (stage == 1) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) out[v] = fma(dt, r[v], un[v]);
+  } else {
+    const double c0 = stage == 2 ? 0.75 : 1.0 / 3.0, c1 = stage == 2 ? 0.25 : 2.0 / 3.0;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) out[v] = fma(c0, un[v], __dmul_rn(c1, fma(dt, r[v], us[v])));
+  }
 }
 
 __host__ __device__ __forceinline__ double viscosity(double T, const Phys& ph) {
@@ -146,6 +150,8 @@ inline void set_ff(Phys& ph) {
   ph.k.gamma = ff_of(ph.gamma);
   ph.k.gm1 = ff_of(ph.gm1);
   ph.k.igm1 = ff_of(ph.igm1);
+  ph.k.gg = ff_of(ph.gamma * ph.igm1);
+  ph.k.iR = ff_of(ph.iR);
   const double e4 = 4.0 * ph.eps;
   ph.k.eps4 = ff_of(e4 < 7.52316384526264e-37 ? 7.52316384526264e-37 : e4);
   ph.k.mu_ref = ff_of(ph.mu_ref);
@@ -163,8 +169,7 @@ const char* config_error(const fluid_config* c);
 inline thread_local long long t_launches = 0;
 
 // ---- launchers implemented in kernels_fp64.cu --------------------------------------------------
-// W32 (mixed path only, else null): exact FP32 (hi, lo) split of the primitives, [2 NW][ncell];
-// with it W must hold NW + 1 rows, the last receiving H = E + p
+// W32 (mixed path only, else null): the primitives go there as pairs (load_pair) instead of to W
 cudaError_t launch_prim_bc(const double* U, double* W, float* W32, const Geo& g, const Phys& ph,
                            const BC& bc, Ctl* ctl, cudaStream_t st);
 cudaError_t launch_grad(const double* W, double* G, const Geo& g, const Phys& ph, cudaStream_t st);
@@ -182,28 +187,27 @@ long long seam_capacity(const Geo& g);   // items for segments of kSeamMinSeg ce
 // the buffer for a launch of segments of `seg` cells along D, or null when it runs without
 double* seam_buffer(int D, const Geo& g, int seg, SeamBuf fb);
 // the first cells of the segments after each line's first, from the fluxes in FB
-cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, int accumulate,
-                             int seg, cudaStream_t st);
+cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, int seg, cudaStream_t st);
 // ---- WENO5 face kernels (face_launch.cuh, one translation unit per scheme) ----------------------
 cudaError_t launch_face_js(int D, const double* W, const double* G, double* R, const Geo& g,
-                           const Phys& ph, int accumulate, int block, int seg, SeamBuf fb, cudaStream_t st);
+                           const Phys& ph, int block, int seg, SeamBuf fb, cudaStream_t st);
 cudaError_t launch_face_z(int D, const double* W, const double* G, double* R, const Geo& g,
-                          const Phys& ph, int accumulate, int block, int seg, SeamBuf fb, cudaStream_t st);
+                          const Phys& ph, int block, int seg, SeamBuf fb, cudaStream_t st);
 cudaError_t launch_face(int D, const double* W, const double* G, double* R, const Geo& g,
-                        const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
-                        cudaStream_t st);
-cudaError_t launch_source(double* R, const double* W, const Geo& g, const Phys& ph, cudaStream_t st);
+                        const Phys& ph, int block, int seg, SeamBuf fb, cudaStream_t st);
+// the velocities of the body force's work come from W32 when given, else from W (also below)
+cudaError_t launch_source(double* R, const double* W, const float* W32, const Geo& g, const Phys& ph,
+                          cudaStream_t st);
 // dt_arg > 0 replaces the solver's dt (used by the adjoint's stage recomputation)
 cudaError_t launch_stage(int stage, const double* Un, const double* Us, const double* R, double* Ud,
-                         const double* W, const Geo& g, const Phys& ph, Ctl* ctl, double t_end,
-                         cudaStream_t st, double dt_arg = 0.0);
-// stage `stage` of RK3 into Ud with the solver's dt, then the primitives of Ud into W (and W32 / H
-// when W32 is given) for every padded cell, equal to launch_prim_bc(Ud, ...) on the result
+                         const double* W, const float* W32, const Geo& g, const Phys& ph, Ctl* ctl,
+                         double t_end, cudaStream_t st, double dt_arg = 0.0);
+// stage `stage` of RK3 into Ud with the solver's dt, then the primitives of Ud into W (into W32 when
+// that is given) for every padded cell, equal to launch_prim_bc(Ud, ...) on the result
 cudaError_t launch_stage_prim(int stage, const double* Un, const double* Us, const double* R,
                               double* Ud, double* W, float* W32, const Geo& g, const Phys& ph,
                               const BC& bc, Ctl* ctl, double t_end, cudaStream_t st);
-// the halo cells of W (and W32 / H when W32 is given) from its interior, as launch_stage_prim's
-// second pass
+// the halo cells of W (of W32 when that is given) from its interior, as launch_stage_prim's second pass
 cudaError_t launch_halo_prim(double* W, float* W32, const Geo& g, const Phys& ph, const BC& bc, Ctl* ctl,
                              cudaStream_t st);
 cudaError_t launch_dt_partial(const double* W, const Geo& g, const Phys& ph, double* partial,
@@ -213,36 +217,29 @@ cudaError_t launch_dt_final(const double* partial, int nparts, const Phys& ph, C
 int dt_partial_count(const Geo& g);
 // ---- TENO6-A face kernels implemented in kernels_teno.cu ----------------------------------------
 cudaError_t launch_face_teno(int D, const double* W, const double* G, double* R, const Geo& g,
-                             const Phys& ph, int accumulate, cudaStream_t st);
+                             const Phys& ph, cudaStream_t st);
 // ---- mixed-precision launchers implemented in kernels_mixed.cu --------------------------------
-// seg 1 on the y / z tiles stages their rows by bulk copies; a copy that does not complete within
-// its bounded wait sets FLAG_STAGING in *flags (when given) and leaves its tile undone
-cudaError_t launch_face_mixed(int D, const double* W, const float* W32, const float* G32, double* R,
-                              const Geo& g, const Phys& ph, int accumulate, int block, int seg,
-                              cudaStream_t st, unsigned* flags = nullptr);
+cudaError_t launch_face_mixed(int D, const float* W32, const float* G32, double* R, const Geo& g,
+                              const Phys& ph, cudaStream_t st);
 // Stage output of the last axis's face kernel when the stage is fused into it: Ud = stage `stage`
-// of RK3 from Un, Us and the completed right-hand side, and the primitives of Ud (W: NW rows and
-// the H row; W32: the split) written to a second buffer pair, since the kernel still reads the
-// current one.  prims = false (the last stage of a call) writes Ud only.
+// of RK3 from Un, Us and the completed right-hand side, and the primitives of Ud written to a second
+// W32, since the kernel still reads the current one.  prims = false (the last stage of a call)
+// writes Ud only.
 struct StageOut {
   int stage;
   int prims;
   const double* Un;
   const double* Us;
   double* Ud;
-  double* W;
   float* W32;
   Ctl* ctl;
   double t_end;
 };
-// whether launch_face_mixed_stage can take the last axis of this grid (the y / z tile kernels)
-bool mixed_stage_fusable(const Geo& g, int seg);
 // the face kernel of the last axis (ndim - 1) accumulating into R's values of the other axes,
 // fused with the stage combination and the primitives of its result (interior cells; the halo
-// cells of the new buffer follow with launch_halo_prim)
-cudaError_t launch_face_mixed_stage(const double* W, const float* W32, const float* G32,
-                                    const double* R, const Geo& g, const Phys& ph, int block, int seg,
-                                    const StageOut& so, cudaStream_t st);
+// cells of the new W32 follow with launch_halo_prim)
+cudaError_t launch_face_mixed_stage(const float* W32, const float* G32, const double* R, const Geo& g,
+                                    const Phys& ph, const StageOut& so, cudaStream_t st);
 cudaError_t launch_grad32(const float* W32, float* G32, const Geo& g, cudaStream_t st);
 // check of the bulk-staging helpers (fluid_check_bulk_staging)
 cudaError_t launch_bulk_probe(const float* src, float* dst, int nrows, unsigned extra_tx,
@@ -306,9 +303,9 @@ struct BatchSlot {
   double* U;          // state (advanced in place)
   double* A;          // stage state
   double* R;          // right-hand side
-  double* W;          // primitives (mixed: plus the H row)
+  double* W;          // primitives (FP64)
   double* G;          // FP64 gradients (FP64 viscous)
-  float* W32;         // FP32 split (mixed)
+  float* W32;         // primitives (mixed)
   float* G32;         // FP32 gradients (mixed viscous)
   double* FB[3];      // seam buffer per axis (null: none)
   double* partial;    // CFL partial maxima

@@ -73,15 +73,6 @@ __device__ __forceinline__ void inflow_at(const double* __restrict__ prof, int a
   w[5] = w[4] / (w[0] * ph.R);
 }
 
-// primitives of padded cell own[] (interior: from U; halo: composed boundary maps); E receives the
-// total energy per volume of interior cells (halo cells leave it unset).
-//
-// The halo passes x -> y -> z compose: the pass of axis a sees own indices on the axes before it
-// and source indices on the axes after it, so a halo cell starts from the cell at the source index
-// on every axis and then takes the maps of its halo axes in order (an inflow axis replaces the
-// state by its profile).  Every cell therefore converts exactly one cell's U -- its own or its
-// source -- and only wall halos run map arithmetic, so warps that straddle the x halo do not run
-// the conversion twice.
 // Source cell of padded cell own[]: ghost[a] / side[a] / src[a] per axis; returns whether any axis
 // is a halo axis (then src[] is the interior cell the halo maps start from).
 // The halo layers of an exchange face (a sub-domain boundary of a block decomposition) hold the
@@ -123,9 +114,30 @@ __device__ __forceinline__ bool halo_maps(const int own[3], const bool ghost[3],
   return valued;
 }
 
-// primitives of padded cell own[] (interior: from U; halo: composed boundary maps); E receives the
-// total energy per volume of the source cell (the cell itself when interior) unless a wall or
-// inflow map changed the values, which the return value says (then E is left unset).
+// whether a halo axis of the cell changes values (a wall or inflow map) rather than only indices
+__device__ __forceinline__ bool halo_valued(const bool ghost[3], const int side[3], const BC& bc) {
+  bool valued = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int kind = bc.kind[a][side[a]];
+    valued |= ghost[a] && kind != FLUID_BC_PERIODIC && kind != FLUID_BC_ZERO_GRADIENT;
+  }
+  return valued;
+}
+
+// halo_maps on the mixed path's pairs: the value maps run in FP64
+__device__ __forceinline__ void halo_maps_ff(const int own[3], const bool ghost[3], const int side[3],
+                                             const int src[3], const Geo& g, const Phys& ph, const BC& bc,
+                                             Ctl* ctl, ff w[NW]) {
+  if (!halo_valued(ghost, side, bc)) return;
+  double d[NW];
+  for (int v = 0; v < NW; ++v) d[v] = ff_to_double(w[v]);
+  halo_maps(own, ghost, side, src, g, ph, bc, ctl, d);
+  for (int v = 0; v < NW; ++v) w[v] = ff_of(d[v]);
+}
+
+// One thread per padded cell: x from the thread index, y and z from the block index; interior cells
+// from U, halo cells by the composed boundary maps.
 //
 // The halo passes x -> y -> z compose: the pass of axis a sees own indices on the axes before it
 // and source indices on the axes after it, so a halo cell starts from the cell at the source index
@@ -133,25 +145,10 @@ __device__ __forceinline__ bool halo_maps(const int own[3], const bool ghost[3],
 // state by its profile).  Every cell therefore converts exactly one cell's U -- its own or its
 // source -- and only wall halos run map arithmetic, so warps that straddle the x halo do not run
 // the conversion twice.
-__device__ __forceinline__ bool prim_cell(const double* __restrict__ U, const int own[3], int cell,
-                                          const Geo& g, const Phys& ph, const BC& bc, Ctl* ctl,
-                                          double w[NW], double& E) {
-  bool ghost[3];
-  int side[3], src[3];
-  const bool any = halo_source(own, g, bc, ghost, side, src);
-  const int scell = any ? src[0] + src[1] * g.sy + src[2] * g.sz : cell;
-  prim_of(U, scell, g.ncell, ph, w);
-  E = U[4 * g.ncell + scell];
-  if (!any) return false;
-  return halo_maps(own, ghost, side, src, g, ph, bc, ctl, w);
-}
-
-// One thread per padded cell: x from the thread index, y and z from the block index.
-// MIXED: the primitives also go to W32 = [2 NW][ncell] floats as the split (hi, lo) above, and
-// H = E + p to the FP64 row W[NW]; the FP32 face kernels form their cell differences from the pairs.
+// MIXED: the primitives are pairs of floats and go to W32 instead of W.
 template <bool MIXED>
 __device__ __forceinline__ void k_prim_bc_body(const double* __restrict__ U, double* __restrict__ W,
-                          float* __restrict__ W32, Geo g, Phys ph, BC bc, Ctl* ctl,
+                          float* __restrict__ W32, const Geo& g, const Phys& ph, const BC& bc, Ctl* ctl,
     uint3 bid, uint3 gdim) {
   const int i = bid.x * blockDim.x + threadIdx.x;
   if (i >= g.p[0]) return;
@@ -159,18 +156,22 @@ __device__ __forceinline__ void k_prim_bc_body(const double* __restrict__ U, dou
     for (int j = bid.y; j < g.p[1]; j += gdim.y) {
       const int own[3] = {i, j, k};
       const int cell = i + j * g.sy + k * g.sz;
-      double w[NW];
-      double E = 0.0;
-      // H = E + p of a halo cell: the source cell's own value when only indices map (periodic,
-      // zero gradient, exchange), so that it equals the source's H bitwise; recomputed from the
-      // mapped primitives after a wall or inflow map
-      const bool valued = prim_cell(U, own, cell, g, ph, bc, ctl, w, E);
-      for (int v = 0; v < NW; ++v) W[v * g.ncell + cell] = w[v];
+      bool ghost[3];
+      int side[3], src[3];
+      const bool any = halo_source(own, g, bc, ghost, side, src);
+      const int scell = any ? src[0] + src[1] * g.sy + src[2] * g.sz : cell;
       if (MIXED) {
-        for (int v = 0; v < NW; ++v)
-          split_hi_lo(w[v], W32[v * g.ncell + cell], W32[(NW + v) * g.ncell + cell]);
-        if (valued) E = w[4] * ph.igm1 + 0.5 * w[0] * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
-        W[NW * g.ncell + cell] = E + w[4];
+        double u[5];
+        for (int v = 0; v < 5; ++v) u[v] = U[v * g.ncell + scell];
+        ff w[NW];
+        prim_ff(u, ph, w);
+        if (any) halo_maps_ff(own, ghost, side, src, g, ph, bc, ctl, w);
+        for (int v = 0; v < NW; ++v) store_pair(W32, g.ncell, v, cell, w[v]);
+      } else {
+        double w[NW];
+        prim_of(U, scell, g.ncell, ph, w);
+        if (any) halo_maps(own, ghost, side, src, g, ph, bc, ctl, w);
+        for (int v = 0; v < NW; ++v) W[v * g.ncell + cell] = w[v];
       }
     }
 }
@@ -238,7 +239,7 @@ __global__ void k_grad(const double* __restrict__ W, double* __restrict__ G, Geo
 // filled FB, from the two fluxes its neighbouring segments left there
 template <int D>
 __device__ __forceinline__ void k_face_seam_body(const double* __restrict__ FB, double* __restrict__ R, Geo g,
-                            int accumulate, int seg,
+                            int seg,
     uint3 bid, uint3 gdim) {
   constexpr int A1 = (D == 0) ? 1 : 0;
   constexpr int A2 = (D == 2) ? 1 : 2;
@@ -262,15 +263,14 @@ __device__ __forceinline__ void k_face_seam_body(const double* __restrict__ FB, 
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const double Fv = FB[v * total + t], Fpv = FB[(5 + v) * total + t];
-      update_r(R + v * nc + cell, Fv, Fpv, id, accumulate);
+      update_r<D>(R + v * nc + cell, Fv, Fpv, id);
     }
   }
 }
 
 template <int D>
-__global__ void k_face_seam(const double* __restrict__ FB, double* __restrict__ R, Geo g,
-                            int accumulate, int seg) {
-  k_face_seam_body<D>(FB, R, g, accumulate, seg, blockIdx, gridDim);
+__global__ void k_face_seam(const double* __restrict__ FB, double* __restrict__ R, Geo g, int seg) {
+  k_face_seam_body<D>(FB, R, g, seg, blockIdx, gridDim);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -284,12 +284,19 @@ __device__ __forceinline__ int interior_cell(int t, const Geo& g) {
   return (i + g.h[0]) + (j + g.h[1]) * g.sy + (k + g.h[2]) * g.sz;
 }
 
-__global__ void k_source(double* __restrict__ R, const double* __restrict__ W, Geo g, Phys ph) {
+// velocity component b of a cell: from the mixed path's pairs when given, else from W
+__device__ __forceinline__ double velocity(const double* __restrict__ W, const float* __restrict__ W32, int nc, int b,
+                                           int c) {
+  return W32 ? ff_to_double(load_pair(W32, nc, 1 + b, c)) : W[(1 + b) * nc + c];
+}
+
+__global__ void k_source(double* __restrict__ R, const double* __restrict__ W, const float* __restrict__ W32, Geo g,
+                         Phys ph) {
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
     const int c = interior_cell(t, g);
-    const double u = W[nc + c], v = W[2 * nc + c], w = W[3 * nc + c];
+    const double u = velocity(W, W32, nc, 0, c), v = velocity(W, W32, nc, 1, c), w = velocity(W, W32, nc, 2, c);
     R[nc + c] += ph.f[0];
     R[2 * nc + c] += ph.f[1];
     R[3 * nc + c] += ph.f[2];
@@ -299,8 +306,8 @@ __global__ void k_source(double* __restrict__ R, const double* __restrict__ W, G
 
 // stage 1: Ud = Un + dt r; stage 2: Ud = 3/4 Un + 1/4 (Us + dt r); stage 3: Ud = 1/3 Un + 2/3 (Us + dt r)
 __device__ __forceinline__ void k_stage_body(int stage, const double* Un, const double* Us, const double* __restrict__ R,
-                        double* Ud, const double* __restrict__ W, Geo g, Phys ph, Ctl* ctl,
-                        double t_end, double dt_arg,
+                        double* Ud, const double* __restrict__ W, const float* __restrict__ W32, const Geo& g,
+                        const Phys& ph, Ctl* ctl, double t_end, double dt_arg,
     uint3 bid, uint3 gdim) {
   const double dt = dt_arg > 0.0 ? dt_arg : ctl->dt;
   if (stage == 3 && dt_arg <= 0.0 && bid.x == 0 && threadIdx.x == 0 && dt > 0.0) {
@@ -317,39 +324,38 @@ __device__ __forceinline__ void k_stage_body(int stage, const double* Un, const 
 #pragma unroll
     for (int v = 0; v < 5; ++v) r[v] = R[v * nc + c];
     if (ph.has_force) {
-      const double u = W[nc + c], v = W[2 * nc + c], w = W[3 * nc + c];
+      const double u = velocity(W, W32, nc, 0, c), v = velocity(W, W32, nc, 1, c), w = velocity(W, W32, nc, 2, c);
       r[1] += ph.f[0];
       r[2] += ph.f[1];
       r[3] += ph.f[2];
       r[4] += fma(ph.f[0], u, fma(ph.f[1], v, ph.f[2] * w));
     }
+    double un[5], us[5], out[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) un[v] = Un[v * nc + c];
+    if (stage != 1) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) us[v] = Us[v * nc + c];
+    }
+    stage_combine(stage, dt, un, us, r, out);
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      const double un = Un[v * nc + c];
-      double out;
-      if (stage == 1) {
-        out = fma(dt, r[v], un);
-      } else {
-        const double us = Us[v * nc + c];
-        out = stage == 2 ? fma(0.75, un, 0.25 * fma(dt, r[v], us))
-                         : fma(1.0 / 3.0, un, (2.0 / 3.0) * fma(dt, r[v], us));
-      }
-      bad |= !finite_bits(out);
-      Ud[v * nc + c] = out;
+      bad |= !finite_bits(out[v]);
+      Ud[v * nc + c] = out[v];
     }
   }
   if (bad) atomicOr(&ctl->flags, FLAG_NONFINITE);
 }
 
 __global__ void k_stage(int stage, const double* Un, const double* Us, const double* __restrict__ R,
-                        double* Ud, const double* __restrict__ W, Geo g, Phys ph, Ctl* ctl,
-                        double t_end, double dt_arg) {
-  k_stage_body(stage, Un, Us, R, Ud, W, g, ph, ctl, t_end, dt_arg, blockIdx, gridDim);
+                        double* Ud, const double* __restrict__ W, const float* __restrict__ W32, Geo g, Phys ph,
+                        Ctl* ctl, double t_end, double dt_arg) {
+  k_stage_body(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, dt_arg, blockIdx, gridDim);
 }
 
 // One RK3 stage fused with the primitives of its result (the next right-hand side's first pass):
-// interior cell c gets Ud = the stage combination of k_stage, and W (and for MIXED the W32 split and
-// H) from Ud by the same conversion k_prim_bc applies, so the halo cells (k_halo_prim, next) and
+// interior cell c gets Ud = the stage combination of k_stage, and W (for MIXED: W32) from Ud by the same
+// conversion k_prim_bc applies, so the halo cells (k_halo_prim, next) and
 // the following kernels see exactly what k_prim_bc would have produced.  W is read (body-force
 // velocities of the stage's input state) and rewritten only at the thread's own cell.  A third
 // stage with dt <= 0 leaves Un unwritten and converts it as it is.
@@ -391,7 +397,7 @@ __device__ __forceinline__ void k_stage_prim_body(int stage, const double* Un, c
           }
           if (ph.has_force) {
 #pragma unroll
-            for (int b = 0; b < 3; ++b) vel[q][b] = W[(1 + b) * nc + c[q]];
+            for (int b = 0; b < 3; ++b) vel[q][b] = velocity(W, MIXED ? W32 : nullptr, nc, b, c[q]);
           }
         }
       }
@@ -410,28 +416,23 @@ __device__ __forceinline__ void k_stage_prim_body(int stage, const double* Un, c
             r[3] += ph.f[2];
             r[4] += fma(ph.f[0], vel[q][0], fma(ph.f[1], vel[q][1], ph.f[2] * vel[q][2]));
           }
+          stage_combine(stage, dt, un[q], us[q], r, u);
 #pragma unroll
           for (int v = 0; v < 5; ++v) {
-            double out;
-            if (stage == 1) {
-              out = fma(dt, r[v], un[q][v]);
-            } else {
-              out = stage == 2 ? fma(0.75, un[q][v], 0.25 * fma(dt, r[v], us[q][v]))
-                               : fma(1.0 / 3.0, un[q][v], (2.0 / 3.0) * fma(dt, r[v], us[q][v]));
-            }
-            bad |= !finite_bits(out);
-            Ud[v * nc + c[q]] = out;
-            u[v] = out;
+            bad |= !finite_bits(u[v]);
+            Ud[v * nc + c[q]] = u[v];
           }
         }
-        double w[NW];
-        prim_from_cons(u, ph, w);
-#pragma unroll
-        for (int v = 0; v < NW; ++v) W[v * nc + c[q]] = w[v];
         if (MIXED) {
+          ff w[NW];
+          prim_ff(u, ph, w);
 #pragma unroll
-          for (int v = 0; v < NW; ++v) split_hi_lo(w[v], W32[v * nc + c[q]], W32[(NW + v) * nc + c[q]]);
-          W[NW * nc + c[q]] = u[4] + w[4];
+          for (int v = 0; v < NW; ++v) store_pair(W32, nc, v, c[q], w[v]);
+        } else {
+          double w[NW];
+          prim_from_cons(u, ph, w);
+#pragma unroll
+          for (int v = 0; v < NW; ++v) W[v * nc + c[q]] = w[v];
         }
       }
     }
@@ -483,22 +484,20 @@ __device__ __forceinline__ void k_halo_prim_body(double* __restrict__ W, float* 
     halo_source(own, g, bc, ghost, side, src);
     const int scell = src[0] + src[1] * g.sy + src[2] * g.sz;
     const int cell = own[0] + own[1] * g.sy + own[2] * g.sz;
-    double w[NW];
-#pragma unroll
-    for (int v = 0; v < NW; ++v) w[v] = W[v * nc + scell];
-    const bool valued = halo_maps(own, ghost, side, src, g, ph, bc, ctl, w);
-#pragma unroll
-    for (int v = 0; v < NW; ++v) W[v * nc + cell] = w[v];
     if (MIXED) {
+      ff w[NW];
 #pragma unroll
-      for (int v = 0; v < NW; ++v) split_hi_lo(w[v], W32[v * nc + cell], W32[(NW + v) * nc + cell]);
-      // as k_prim_bc: index-only maps keep the source's H, value maps recompute it
-      if (valued) {
-        const double E = w[4] * ph.igm1 + 0.5 * w[0] * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
-        W[NW * nc + cell] = E + w[4];
-      } else {
-        W[NW * nc + cell] = W[NW * nc + scell];
-      }
+      for (int v = 0; v < NW; ++v) w[v] = load_pair(W32, nc, v, scell);
+      halo_maps_ff(own, ghost, side, src, g, ph, bc, ctl, w);
+#pragma unroll
+      for (int v = 0; v < NW; ++v) store_pair(W32, nc, v, cell, w[v]);
+    } else {
+      double w[NW];
+#pragma unroll
+      for (int v = 0; v < NW; ++v) w[v] = W[v * nc + scell];
+      halo_maps(own, ghost, side, src, g, ph, bc, ctl, w);
+#pragma unroll
+      for (int v = 0; v < NW; ++v) W[v * nc + cell] = w[v];
     }
   }
 }
@@ -670,7 +669,7 @@ __global__ void __launch_bounds__(256) kb_grad(const BatchTable* __restrict__ t,
 template <int D>
 __global__ void __launch_bounds__(256) kb_seam(const BatchTable* __restrict__ t, int step) {
   FL_BATCH_LOOP(BK_SEAM0 + D)
-  if (step < S.steps) k_face_seam_body<D>(S.FB[D], S.R, S.g, D > 0, S.seg[D], bid, gdim);
+  if (step < S.steps) k_face_seam_body<D>(S.FB[D], S.R, S.g, S.seg[D], bid, gdim);
   FL_BATCH_END
 }
 
@@ -696,7 +695,7 @@ __global__ void __launch_bounds__(256) kb_halo(const BatchTable* __restrict__ t,
 
 __global__ void __launch_bounds__(256) kb_stage(const BatchTable* __restrict__ t, int step) {
   FL_BATCH_LOOP(BK_STAGE)
-  if (step < S.steps) k_stage_body(3, S.U, S.A, S.R, S.U, S.W, S.g, S.ph, S.ctl, S.t_end, 0.0, bid, gdim);
+  if (step < S.steps) k_stage_body(3, S.U, S.A, S.R, S.U, S.W, S.W32, S.g, S.ph, S.ctl, S.t_end, 0.0, bid, gdim);
   FL_BATCH_END
 }
 
@@ -743,16 +742,10 @@ void batch_plan(BatchTable& t, bool mixed) {
         set(BK_SEAM0 + D, 0);
         continue;
       }
-      if (mixed) {
-        if (D == 0) set(BK_FACE0, ceil_div(g.n[0], 31), ceil_div(lines, 4));
-        else set(BK_FACE0 + D, ceil_div(g.n[0], 32), ceil_div(g.n[D], kMixedTileCells), g.n[D == 1 ? 2 : 1]);
-        set(BK_SEAM0 + D, 0);
-      } else {
-        if (D == 0) set(BK_FACE0, tile_cols<0>(g), tile_rows<0>(g));
-        else if (D == 1) set(BK_FACE1, tile_cols<1>(g), tile_rows<1>(g));
-        else set(BK_FACE2, tile_cols<2>(g), tile_rows<2>(g));
-        set(BK_SEAM0 + D, 0);
-      }
+      if (D == 0) set(BK_FACE0, tile_cols<0>(g), tile_rows<0>(g));
+      else if (D == 1) set(BK_FACE1, tile_cols<1>(g), tile_rows<1>(g));
+      else set(BK_FACE2, tile_cols<2>(g), tile_rows<2>(g));
+      set(BK_SEAM0 + D, 0);
     }
     set(BK_STAGEP, ceil_div(g.n[0], 128), std::min((g.n[1] + 1) / 2, 65535), std::min(g.n[2], 65535));
     set(BK_HALO, ceil_div(npad - nint, 256));
@@ -811,14 +804,13 @@ double* seam_buffer(int D, const Geo& g, int seg, SeamBuf fb) {
   return (fb.p != nullptr && nseg > 1 && lines * nseg <= fb.cap) ? fb.p : nullptr;
 }
 
-cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, int accumulate,
-                             int seg, cudaStream_t st) {
+cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, int seg, cudaStream_t st) {
   const long long lines = (long long)g.n[D == 0 ? 1 : 0] * g.n[D == 2 ? 1 : 2];
   const long long items = lines * ((g.n[D] + seg - 1) / seg - 1);
   const int grid = grid_for(items, 256);
-  if (D == 0) (k_face_seam<0><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-  else if (D == 1) (k_face_seam<1><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
-  else (k_face_seam<2><<<grid, 256, 0, st>>>(FB, R, g, accumulate, seg), ++t_launches);
+  if (D == 0) (k_face_seam<0><<<grid, 256, 0, st>>>(FB, R, g, seg), ++t_launches);
+  else if (D == 1) (k_face_seam<1><<<grid, 256, 0, st>>>(FB, R, g, seg), ++t_launches);
+  else (k_face_seam<2><<<grid, 256, 0, st>>>(FB, R, g, seg), ++t_launches);
   return cudaGetLastError();
 }
 
@@ -863,11 +855,10 @@ cudaError_t launch_grad(const double* W, double* G, const Geo& g, const Phys& ph
 }
 
 cudaError_t launch_face(int D, const double* W, const double* G, double* R, const Geo& g,
-                        const Phys& ph, int accumulate, int block, int seg, SeamBuf fb,
-                        cudaStream_t st) {
-  if (ph.weno == FLUID_TENO6A) return launch_face_teno(D, W, G, R, g, ph, accumulate, st);
-  if (ph.weno == FLUID_WENO_JS) return launch_face_js(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
-  return launch_face_z(D, W, G, R, g, ph, accumulate, block, seg, fb, st);
+                        const Phys& ph, int block, int seg, SeamBuf fb, cudaStream_t st) {
+  if (ph.weno == FLUID_TENO6A) return launch_face_teno(D, W, G, R, g, ph, st);
+  if (ph.weno == FLUID_WENO_JS) return launch_face_js(D, W, G, R, g, ph, block, seg, fb, st);
+  return launch_face_z(D, W, G, R, g, ph, block, seg, fb, st);
 }
 
 long long seam_capacity(const Geo& g) {
@@ -880,17 +871,18 @@ long long seam_capacity(const Geo& g) {
   return cap;
 }
 
-cudaError_t launch_source(double* R, const double* W, const Geo& g, const Phys& ph, cudaStream_t st) {
+cudaError_t launch_source(double* R, const double* W, const float* W32, const Geo& g, const Phys& ph,
+                          cudaStream_t st) {
   const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  (k_source<<<grid_for(total, 256), 256, 0, st>>>(R, W, g, ph), ++t_launches);
+  (k_source<<<grid_for(total, 256), 256, 0, st>>>(R, W, W32, g, ph), ++t_launches);
   return cudaGetLastError();
 }
 
 cudaError_t launch_stage(int stage, const double* Un, const double* Us, const double* R, double* Ud,
-                         const double* W, const Geo& g, const Phys& ph, Ctl* ctl, double t_end,
-                         cudaStream_t st, double dt_arg) {
+                         const double* W, const float* W32, const Geo& g, const Phys& ph, Ctl* ctl,
+                         double t_end, cudaStream_t st, double dt_arg) {
   const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  (k_stage<<<grid_for(total, 256), 256, 0, st>>>(stage, Un, Us, R, Ud, W, g, ph, ctl, t_end, dt_arg), ++t_launches);
+  (k_stage<<<grid_for(total, 256), 256, 0, st>>>(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, dt_arg), ++t_launches);
   return cudaGetLastError();
 }
 

@@ -1,36 +1,35 @@
 // Mixed-precision face kernels: WENO5 weights and reconstruction, HLLC wave speeds and star
-// correction, and the dissipative stencils in FP32; the state, the cell-centre convective flux,
-// the face-flux assembly and the flux-difference accumulation in FP64.
+// correction, and the dissipative stencils in FP32; the state and the flux-difference accumulation
+// in FP64; the primitives and the cell-centre convective flux as two-float numbers (ff_math.cuh,
+// about 47 bits).
 //
 // Why a delta form.  At low Mach number the pressure (and total enthalpy) is large and nearly
 // uniform, so fluxes are large and their differences across a cell small: a flux rounded to FP32
 // carries an absolute error ~6e-8 |F| that the divergence divides by dx.  Here every FP32 quantity
 // is either a coefficient (used only as a factor) or a small increment that FP32 represents to
 // ~6e-8 of its own size:
-//   * cell differences D_j = q_{j+1} - q_j of the primitives come from the exact FP32 split
-//     q = hi + lo written by the primitive kernel: (hi_{j+1} - hi_j) + (lo_{j+1} - lo_j), each
-//     FP32 subtraction rounding relative to its own result, so D_j is within ~1 ulp (FP32) of the
-//     FP64 difference, up to 2^-48 |q| from the split;
-//   * WENO5 works on offsets delta_k = q_{a+k} - q_a built from the D's (the smoothness
-//     indicators and the weights do not depend on the offset, the candidates are affine);
-//   * the face flux is F_{a+1/2} = F(q_a) [FP64, from the primitives and H = E + p] + X [FP32],
-//     where X is the change of the Euler
-//     flux from the cell state q_a to the upwind face state, written as a polynomial in the
-//     offsets, plus the HLLC star correction S_K (U*_K - U_K), written through the jumps of the
-//     reconstructed states (S* - u_K from the pressure and velocity jumps), minus the
-//     dissipative flux;
+//   * cell differences D_j = q_{j+1} - q_j of the primitives come from their pairs q = hi + lo:
+//     (hi_{j+1} - hi_j) + (lo_{j+1} - lo_j), each FP32 subtraction rounding relative to its own
+//     result, so D_j is within ~1 ulp (FP32) of the difference, up to 2^-47 |q| from the pairs;
+//   * WENO5 works on D and the second differences T_j = D_j - D_{j-1}: the indicators of a cell serve
+//     the values at both of its faces, w^L_{j+1/2} = q_j + (3 D_j + cL_j) / 6 and w^R_{j-1/2} =
+//     q_j + (cR_j - 3 D_{j-1}) / 6 (cell_terms, cell_values in face_ff.cuh have the same in ff);
+//   * the face flux is F_{a+1/2} = F(q_a) [ff] + X [FP32], where X is the change of the Euler flux from
+//     the cell state q_a to the upwind face state, written as a polynomial in the offsets, plus the
+//     HLLC star correction S_K (U*_K - U_K), written through the jumps of the reconstructed states
+//     (S* - u_K from the pressure and velocity jumps), minus the dissipative flux; the sum is
+//     rounded to FP64;
 //   * R += -(F_{a+1/2} - F_{a-1/2}) / dx in FP64, so the face fluxes telescope exactly as in the
 //     FP64 path (each face value is computed once and shared by its two cells).
 #include <cuda_runtime.h>
 
-#include "flux_math.cuh"
+#include "face_kernels.cuh"
 #include "fluid_internal.cuh"
 
 namespace fl {
 
 namespace {
 
-constexpr float k1312f = 13.0f / 12.0f;
 constexpr float kZepsF = 1e-20f;      // WENO5-Z epsilon in FP32 (a normal float)
 constexpr float kZclampF = 1e18f;     // bound of tau5 / (beta + eps): keeps its square finite
 
@@ -92,7 +91,7 @@ int grid_for(long long work, int block) {
 struct PhysF {
   float gamma, gm1, igm1, gg;            // gg = gamma / (gamma - 1)
   float mu_ref, iT_ref, visc_exp, TS, S; // TS = T_ref + S (Sutherland)
-  float lam_fac, eps, dt_visc_k;
+  float lam_fac, eps4, dt_visc_k;        // eps4 = 4 epsilon (WENO5-Z: of kZepsF)
   int visc;
 };
 
@@ -102,90 +101,85 @@ __host__ __device__ inline PhysF phys_f(const Phys& ph) {
   f.gg = (float)(ph.gamma * ph.igm1);
   f.mu_ref = (float)ph.mu_ref; f.iT_ref = (float)ph.iT_ref; f.visc_exp = (float)ph.visc_exp;
   f.TS = (float)(ph.T_ref + ph.suth_S); f.S = (float)ph.suth_S;
-  f.lam_fac = (float)ph.lam_fac; f.eps = (float)ph.eps; f.dt_visc_k = (float)ph.dt_visc_k;
+  f.lam_fac = (float)ph.lam_fac; f.eps4 = 4.0f * (ph.weno == FLUID_WENO_JS ? (float)ph.eps : kZepsF); f.dt_visc_k = (float)ph.dt_visc_k;
   f.visc = ph.visc;
   return f;
 }
 
-// inputs of the face kernels: FP64 primitives with the H = E + p row, their FP32 split, gradients
-struct MixedIn {
-  const double* W;     // [NW + 1][ncell]
-  const float* hi;     // [NW][ncell]
-  const float* lo;     // [NW][ncell]
-  const float* G32;    // [NG][ncell] (viscous only)
-};
+// Indicator terms of cell j in FP32: 4 (beta + eps) of its three-cell stencil as the left (A), centre
+// (B) and right (C) candidate (cell_terms)
+__device__ __forceinline__ void cell_terms32(float D, float T, float eps4, float& A, float& B, float& C) {
+  const float K = s_fma(s_mul(13.0f / 3.0f, T), T, eps4);
+  const float sB = s_fma(2.0f, D, -T), sA = s_fma(2.0f, T, sB), sC = s_fma(2.0f, T, -sB);
+  A = s_fma(sA, sA, K);
+  B = s_fma(sB, sB, K);
+  C = s_fma(sC, sC, K);
+}
 
-// WENO5 value at i+1/2 relative to an arbitrary offset, from offsets of q_{i-2..i+2}
+// Six times the corrections of cell j's two face values (cell_values): cL, cR from the indicator set
+// A_{j-1}, B_j, C_{j+1}, T_j and the third differences V0 = T_j - T_{j-1}, V1 = T_{j+1} - T_j
 template <int SCHEME>
-__device__ __forceinline__ float weno5f(float qm2, float qm1, float q0, float qp1, float qp2, float eps) {
-  const float p0 = 2.0f * qm2 - 7.0f * qm1 + 11.0f * q0;
-  const float p1 = -qm1 + 5.0f * q0 + 2.0f * qp1;
-  const float p2 = 2.0f * q0 + 5.0f * qp1 - qp2;
-  float t = qm2 - 2.0f * qm1 + q0, s = qm2 - 4.0f * qm1 + 3.0f * q0;
-  const float b0 = k1312f * t * t + 0.25f * s * s;
-  t = qm1 - 2.0f * q0 + qp1; s = qm1 - qp1;
-  const float b1 = k1312f * t * t + 0.25f * s * s;
-  t = q0 - 2.0f * qp1 + qp2; s = 3.0f * q0 - 4.0f * qp1 + qp2;
-  const float b2 = k1312f * t * t + 0.25f * s * s;
-  float a0, a1, a2;
+__device__ __forceinline__ void cell_corr32(float e0, float e1, float e2, float T, float V0, float V1, float& cL,
+                                            float& cR) {
+  const float r0 = rcpf(e0), r1 = rcpf(e1), r2 = rcpf(e2);
+  float W0, W1, W2;
   if (SCHEME == FLUID_WENO_JS) {
-    const float r0 = rcpf(eps + b0), r1 = rcpf(eps + b1), r2 = rcpf(eps + b2);
-    a0 = 0.1f * r0 * r0; a1 = 0.6f * r1 * r1; a2 = 0.3f * r2 * r2;
+    const float em = fminf(fminf(e0, e1), e2);           // a common factor keeps the squares in range
+    W0 = s_mul(em, r0); W1 = s_mul(em, r1); W2 = s_mul(em, r2);
+    W0 = s_mul(W0, W0); W1 = s_mul(W1, W1); W2 = s_mul(W2, W2);
   } else {
-    const float tau = fabsf(b0 - b2);
-    const float r0 = fminf(tau * rcpf(b0 + kZepsF), kZclampF);
-    const float r1 = fminf(tau * rcpf(b1 + kZepsF), kZclampF);
-    const float r2 = fminf(tau * rcpf(b2 + kZepsF), kZclampF);
-    a0 = 0.1f * (1.0f + r0 * r0); a1 = 0.6f * (1.0f + r1 * r1); a2 = 0.3f * (1.0f + r2 * r2);
+    const float tau = fabsf(s_sub(e0, e2));
+    W0 = fminf(s_mul(tau, r0), kZclampF);
+    W1 = fminf(s_mul(tau, r1), kZclampF);
+    W2 = fminf(s_mul(tau, r2), kZclampF);
+    W0 = s_fma(W0, W0, 1.0f); W1 = s_fma(W1, W1, 1.0f); W2 = s_fma(W2, W2, 1.0f);
   }
-  return (a0 * p0 + a1 * p1 + a2 * p2) * rcpf(6.0f * (a0 + a1 + a2));
+  const float P0 = s_mul(W0, V0), P2 = s_mul(W2, V1), S = s_add(P0, P2);
+  const float base = s_fma(6.0f, W1, s_add(W0, W2));
+  cL = s_fma(-s_fma(2.0f, S, P2), rcpf(s_fma(2.0f, W2, base)), -T);
+  cR = s_fma(s_fma(2.0f, S, P0), rcpf(s_fma(2.0f, W0, base)), -T);
 }
 
 __device__ __forceinline__ float viscosity_f(float T, const PhysF& pf) {
   if (pf.visc == FLUID_VISC_CONSTANT) return pf.mu_ref;
-  const float r = T * pf.iT_ref;
-  if (pf.visc == FLUID_VISC_POWER) return pf.mu_ref * __powf(r, pf.visc_exp);
-  return pf.mu_ref * (r * sqrtf_a(r)) * pf.TS * rcpf(T + pf.S);
+  const float r = s_mul(T, pf.iT_ref);
+  if (pf.visc == FLUID_VISC_POWER) return s_mul(pf.mu_ref, __powf(r, pf.visc_exp));
+  return s_mul(s_mul(s_mul(pf.mu_ref, s_mul(r, sqrtf_a(r))), pf.TS), rcpf(s_add(T, pf.S)));
 }
 
-// X: change of the face flux relative to F(q_a), in FP32 (see the file comment).
+// X: change of the face flux relative to F(q_a), in FP32 (see the file comment).  Every operation is
+// explicit, so that all kernels inlining it (and the functions below) give the same bits.
 //   b        FP32 cell state q_a (rho, u, v, w, p)
-//   dL, dR   offsets of the reconstructed left and right face states from q_a
+//   dL, J    offset of the reconstructed left face state from q_a, and the jump to the right one
 template <int D>
-__device__ __forceinline__ void hllc_delta(const float b[5], const float dL[5], const float dR[5],
+__device__ __forceinline__ void hllc_delta(const float b[5], const float dL[5], const float J[5],
                                            const PhysF& pf, float X[5]) {
   const float g = pf.gamma, gm1 = pf.gm1, igm1 = pf.igm1;
-  float wl[5], wr[5], J[5];
+  float wl[5], wr[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    wl[v] = b[v] + dL[v];
-    wr[v] = b[v] + dR[v];
-    J[v] = dR[v] - dL[v];                         // jumps, accurate to FP32 relative to themselves
+    wl[v] = s_add(b[v], dL[v]);
+    wr[v] = s_add(wl[v], J[v]);
   }
   const float rL = wl[0], pL = wl[4], rR = wr[0], pR = wr[4];
-  const float unL = wl[1 + D], unR = wr[1 + D];
-  const float q2L = wl[1] * wl[1] + wl[2] * wl[2] + wl[3] * wl[3];
-  const float q2R = wr[1] * wr[1] + wr[2] * wr[2] + wr[3] * wr[3];
-  const float EL = pL * igm1 + 0.5f * rL * q2L, ER = pR * igm1 + 0.5f * rR * q2R;
-  const float isL = rsqrtf_a(rL), isR = rsqrtf_a(rR);        // 1/sqrt(rho)
-  const float irL = isL * isL, irR = isR * isR;               // 1/rho
-  const float cL = sqrtf_a(g * pL * irL), cR = sqrtf_a(g * pR * irR);
-  const float sL = rL * isL, sR = rR * isR;                   // sqrt(rho)
-  const float is = rcpf(sL + sR);
-  const float ut0 = (sL * wl[1] + sR * wr[1]) * is;
-  const float ut1 = (sL * wl[2] + sR * wr[2]) * is;
-  const float ut2 = (sL * wl[3] + sR * wr[3]) * is;
-  const float Ht = ((EL + pL) * isL + (ER + pR) * isR) * is;   // sqrt(rho) (E+p)/rho
-  const float ct = sqrtf_a(gm1 * (Ht - 0.5f * (ut0 * ut0 + ut1 * ut1 + ut2 * ut2)));
-  const float utn = D == 0 ? ut0 : (D == 1 ? ut1 : ut2);
-  const float SL = fminf(unL - cL, utn - ct);
-  const float SR = fmaxf(unR + cR, utn + ct);
-  const float mL = rL * (SL - unL), mR = rR * (SR - unR);
-  const float iden = rcpf(mL - mR);
-  // S* - u_L and S* - u_R from the jumps: (dp - m_{R|L} du_n) / (m_L - m_R)
-  const float sigL = (J[4] - mR * J[1 + D]) * iden;
-  const float sigR = (J[4] - mL * J[1 + D]) * iden;
-  const float Ss = unL + sigL;
+  const float unL = wl[1 + D], unR = wr[1 + D], Jn = J[1 + D];
+  const float isL = rsqrtf_a(rL), isR = rsqrtf_a(rR);          // 1/sqrt(rho)
+  const float cL2 = s_mul(s_mul(g, pL), s_mul(isL, isL)), cR2 = s_mul(s_mul(g, pR), s_mul(isR, isR));
+  const float cL = sqrtf_a(cL2), cR = sqrtf_a(cR2);
+  // Roe averages as in hllc_ff: u~ = u_L + a_R J_u,
+  // c~^2 = a_L c_L^2 + a_R c_R^2 + (gamma - 1)/2 a_L a_R |J_u|^2
+  const float sL = s_mul(rL, isL), sR = s_mul(rR, isR);
+  const float aR = s_mul(sR, rcpf(s_add(sL, sR))), aL = s_sub(1.0f, aR);
+  const float q2J = s_fma(J[1], J[1], s_fma(J[2], J[2], s_mul(J[3], J[3])));
+  const float ct = sqrtf_a(s_fma(aR, s_fma(s_mul(s_mul(0.5f, gm1), aL), q2J, s_sub(cR2, cL2)), cL2));
+  const float ut = s_mul(aR, Jn);                              // u~ - u_L
+  const float sl = fminf(-cL, s_sub(ut, ct));                  // S_L - u_L
+  const float sr = fmaxf(cR, s_add(s_sub(ut, Jn), ct));        // S_R - u_R
+  const float SL = s_add(unL, sl), SR = s_add(unR, sr);
+  const float mL = s_mul(rL, sl), mR = s_mul(rR, sr);
+  // S* - u_L from the jumps: (dp - m_R du_n) / (m_L - m_R)
+  const float sigL = s_mul(s_fma(-mR, Jn, J[4]), rcpf(s_sub(mL, mR)));
+  const float Ss = s_add(unL, sigL);
 
   const bool left = (SL >= 0.0f) || (Ss >= 0.0f);
   const bool star = left ? !(SL >= 0.0f) : (SR > 0.0f);
@@ -193,144 +187,117 @@ __device__ __forceinline__ void hllc_delta(const float b[5], const float dL[5], 
   // in registers
   float d[5], w[5];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) { d[v] = left ? dL[v] : dR[v]; w[v] = left ? wl[v] : wr[v]; }
+  for (int v = 0; v < 5; ++v) { d[v] = left ? dL[v] : s_add(dL[v], J[v]); w[v] = left ? wl[v] : wr[v]; }
 
   // Euler-flux change from q_a to the face state K = b + d
   const float un = b[1 + D], unK = w[1 + D];
-  const float mn = b[0] * un;
-  const float dm = b[0] * d[1 + D] + d[0] * unK;          // rho' u_n' - rho u_n
+  const float mn = s_mul(b[0], un);
+  const float dm = s_fma(b[0], d[1 + D], s_mul(d[0], unK));    // rho' u_n' - rho u_n
   X[0] = dm;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) X[1 + c] = dm * w[1 + c] + mn * d[1 + c];
-  X[1 + D] += d[4];
-  const float q2b = b[1] * b[1] + b[2] * b[2] + b[3] * b[3];
-  const float dq2 = d[1] * (2.0f * b[1] + d[1]) + d[2] * (2.0f * b[2] + d[2]) + d[3] * (2.0f * b[3] + d[3]);
-  const float gg = pf.gg;
-  const float Hv = gg * b[4] + 0.5f * b[0] * q2b;         // E + p of q_a
-  const float dHv = gg * d[4] + 0.5f * (d[0] * (q2b + dq2) + b[0] * dq2);
-  X[4] = d[1 + D] * (Hv + dHv) + un * dHv;
+  for (int c = 0; c < 3; ++c) X[1 + c] = s_fma(dm, w[1 + c], s_mul(mn, d[1 + c]));
+  X[1 + D] = s_add(X[1 + D], d[4]);
+  const float q2b = s_fma(b[1], b[1], s_fma(b[2], b[2], s_mul(b[3], b[3])));
+  const float dq2 = s_fma(d[1], s_fma(2.0f, b[1], d[1]),
+                          s_fma(d[2], s_fma(2.0f, b[2], d[2]), s_mul(d[3], s_fma(2.0f, b[3], d[3]))));
+  const float gg = pf.gg, hr = s_mul(0.5f, b[0]);
+  const float Hv = s_fma(gg, b[4], s_mul(hr, q2b));            // E + p of q_a
+  const float q2K = s_add(q2b, dq2);
+  const float dHv = s_fma(gg, d[4], s_fma(s_mul(0.5f, d[0]), q2K, s_mul(hr, dq2)));
+  X[4] = s_fma(d[1 + D], s_add(Hv, dHv), s_mul(un, dHv));
 
   if (star) {
     // S_K (U*_K - U_K) with theta = (S* - u_K)/(S_K - S*), chi = 1 + theta
-    const float S = left ? SL : SR;
-    const float sig = left ? sigL : sigR;
+    const float S = left ? SL : SR, sK = left ? sl : sr;
+    const float sig = left ? sigL : s_sub(sigL, Jn);
     const float rK = w[0], pK = w[4];
-    const float EK = left ? EL : ER;
-    const float theta = sig * rcpf(S - Ss);
-    const float chi = 1.0f + theta;
-    float dU[5];
-    dU[0] = rK * theta;
+    const float EK = s_fma(pK, igm1, s_mul(s_mul(0.5f, rK), q2K));
+    const float theta = s_mul(sig, rcpf(s_sub(sK, sig)));
+    const float cs = s_fma(theta, sig, sig);                   // chi sigma
+    const float f0 = s_mul(S, s_mul(rK, theta));
+    X[0] = s_add(X[0], f0);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) dU[1 + c] = rK * theta * w[1 + c];
-    dU[1 + D] = rK * (theta * unK + chi * sig);
-    dU[4] = theta * EK + chi * sig * (rK * Ss + pK * rcpf(S - unK));
-#pragma unroll
-    for (int v = 0; v < 5; ++v) X[v] += S * dU[v];
+    for (int c = 0; c < 3; ++c) X[1 + c] = s_fma(f0, w[1 + c], X[1 + c]);
+    X[1 + D] = s_fma(S, s_mul(rK, cs), X[1 + D]);
+    X[4] = s_fma(S, s_fma(theta, EK, s_mul(cs, s_fma(rK, Ss, s_mul(pK, rcpf(sK))))), X[4]);
   }
 }
 
-// D-window entry: difference of one primitive between consecutive cells from its (hi, lo) split
-__device__ __forceinline__ float diff32(const float* __restrict__ hi, const float* __restrict__ lo,
-                                        int cell, int s) {
-  return (__ldg(hi + cell + s) - __ldg(hi + cell)) + (__ldg(lo + cell + s) - __ldg(lo + cell));
+__device__ __forceinline__ float interp32(const float* __restrict__ f, int s) {
+  return s_mul(s_fma(9.0f, s_add(__ldg(f), __ldg(f + s)), -s_add(__ldg(f - s), __ldg(f + 2 * s))), 0.0625f);
 }
 
-// Face flux F_{a+1/2} (FP64) along D.  `cell` is cell a; Dw[v][k] holds D_{a-2+k}, k = 0..4.
-template <int D, int SCHEME, bool VISC>
-__device__ __forceinline__ void face_flux_mixed(const MixedIn& in, int cell, int s, int a,
-                                                const float Dw[6][5], const Geo& g, const PhysF& pf,
-                                                double F[5]) {
+// The Euler flux of a cell's pairs along D plus the increment X, as FP64
+template <int D>
+__device__ __forceinline__ void assemble_flux(const ff q[5], const Phys& ph, const float X[5], double F[5]) {
+  const ff un = q[1 + D], mn = q[0] * un;
+  const ff q2 = fma_weak(q[1], q[1], fma_weak(q[2], q[2], sqr_weak(q[3])));
+  const ff gg = ph.k.gg;
+  ff f[5];
+  f[0] = mn;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) f[1 + c] = c == D ? ff_fma(mn, q[1 + c], q[4]) : mn * q[1 + c];
+  f[4] = ff_fma(mul_weak(un, gg), q[4], mul_weak(ff_scale(mn, 0.5f), q2));
+#pragma unroll
+  for (int v = 0; v < 5; ++v) F[v] = ff_to_double(f[v] + X[v]);
+}
+
+// The face flux at i+1/2 (cell i: `cell`) from its cell's pairs q, the corrections cL, cR, D = q_{i+1} -
+// q_i, and for the dissipative flux Ts = T_i + T_{i+1}, Td = T_{i+1} - T_i of the velocities and, last, the
+// temperature, whose D is Dt
+template <int D, bool VISC>
+__device__ __forceinline__ void mixed_face(const float* __restrict__ W32, const float* __restrict__ G32, int cell,
+                                           int s, int i, const Geo& g, const Phys& ph, const PhysF& pf, const ff q[5],
+                                           const float cL[5], const float cR[5], const float Dv[5], const float Ts[4],
+                                           const float Td[4], float Dt, double F[5]) {
   const int nc = g.ncell;
-  const float eps = pf.eps;
-  float b[5], dL[5], dR[5];
+  float b[5], dL[5], J[5], X[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    b[v] = __ldg(in.hi + v * nc + cell);
-    // offsets from q_a of cells a-2 .. a+3
-    const float om1 = -Dw[v][1], om2 = -(Dw[v][0] + Dw[v][1]);
-    const float op1 = Dw[v][2], op2 = Dw[v][2] + Dw[v][3], op3 = op2 + Dw[v][4];
-    dL[v] = weno5f<SCHEME>(om2, om1, 0.0f, op1, op2, eps);
-    dR[v] = weno5f<SCHEME>(op3, op2, op1, 0.0f, om1, eps);
+    b[v] = q[v].h;
+    dL[v] = s_mul(1.0f / 6.0f, s_fma(3.0f, Dv[v], cL[v]));
+    J[v] = s_mul(1.0f / 6.0f, s_sub(cR[v], cL[v]));
   }
-  float X[5];
-  hllc_delta<D>(b, dL, dR, pf, X);
-
+  hllc_delta<D>(b, dL, J, pf, X);
   if (VISC) {
-    // u, v, w, T at cells a-1..a+2 through the D window (entries 1, 2, 3 = D_{a-1}, D_a, D_{a+1})
-    const float mfa = __ldg(g.mf32[D] + a);
-    float vf[3], Gf[3][3];
+    // value f_a + D/2 - (T_a + T_{a+1}) / 16 and derivative D - (T_{a+1} - T_a) / 24 of the 4-cell stencils
+    const float mfa = __ldg(g.mf32[D] + i);
+    float vf[3], dn[3], gd[3], gb[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float d0 = Dw[1 + c][1], d1 = Dw[1 + c][2], d2 = Dw[1 + c][3];
-      vf[c] = b[1 + c] + (8.0f * d1 + d0 - d2) * (1.0f / 16.0f);
-      Gf[c][D] = (26.0f * d1 - d0 - d2) * (1.0f / 24.0f) * mfa;
+      vf[c] = s_add(b[1 + c], s_fma(-0.0625f, Ts[c], s_mul(0.5f, Dv[1 + c])));
+      dn[c] = s_mul(s_fma(-1.0f / 24.0f, Td[c], Dv[1 + c]), mfa);
     }
-    const float Tb = __ldg(in.hi + 5 * nc + cell);
-    const float Tf = Tb + (8.0f * Dw[5][2] + Dw[5][1] - Dw[5][3]) * (1.0f / 16.0f);
-    const float dT = (26.0f * Dw[5][2] - Dw[5][1] - Dw[5][3]) * (1.0f / 24.0f) * mfa;
-    auto interp = [](float fm1, float f0, float f1, float f2) {
-      return (9.0f * (f0 + f1) - (fm1 + f2)) * (1.0f / 16.0f);
-    };
+    const float Tf = s_add(__ldg(W32 + 5 * nc + cell), s_fma(-0.0625f, Ts[3], s_mul(0.5f, Dt)));
+    const float dT = s_mul(s_fma(-1.0f / 24.0f, Td[3], Dt), mfa);
+    float tr = 0.0f;
 #pragma unroll
-    for (int bb = 0; bb < 3; ++bb) {
-      if (bb == D) continue;
-      if (bb < g.ndim) {
-        const float* gd = in.G32 + (D * 3 + bb) * nc + cell;
-        const float* gb = in.G32 + (bb * 3 + bb) * nc + cell;
-        Gf[D][bb] = interp(__ldg(gd - s), __ldg(gd), __ldg(gd + s), __ldg(gd + 2 * s));
-        Gf[bb][bb] = interp(__ldg(gb - s), __ldg(gb), __ldg(gb + s), __ldg(gb + 2 * s));
-      } else {
-        Gf[D][bb] = 0.0f;
-        Gf[bb][bb] = 0.0f;
-      }
+    for (int c = 0; c < 3; ++c) {
+      if (c == D || c >= g.ndim) continue;
+      gd[c] = interp32(G32 + (D * 3 + c) * nc + cell, s);
+      gb[c] = interp32(G32 + (c * 3 + c) * nc + cell, s);
+      tr = s_add(tr, gb[c]);
     }
-    const float div = Gf[0][0] + Gf[1][1] + Gf[2][2];
     const float mu = viscosity_f(Tf, pf);
-    const float lam = mu * pf.lam_fac;
     float tau[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      if (c == D) tau[c] = mu * (Gf[D][D] + Gf[D][D]) - (2.0f / 3.0f) * mu * div;
-      else tau[c] = mu * (Gf[c][D] + Gf[D][c]);
+      if (c == D) tau[c] = s_mul(mu, s_mul(2.0f / 3.0f, s_fma(2.0f, dn[D], -tr)));
+      else tau[c] = s_mul(mu, c < g.ndim ? s_add(dn[c], gd[c]) : dn[c]);
+      X[1 + c] = s_sub(X[1 + c], tau[c]);
     }
-    X[1] -= tau[0];
-    X[2] -= tau[1];
-    X[3] -= tau[2];
-    X[4] -= vf[0] * tau[0] + vf[1] * tau[1] + vf[2] * tau[2] + lam * dT;
+    X[4] = s_sub(X[4], s_fma(vf[0], tau[0], s_fma(vf[1], tau[1], s_fma(vf[2], tau[2], s_mul(s_mul(mu, pf.lam_fac), dT)))));
   }
-
-  // FP64 cell-centre Euler flux of q_a plus the FP32 change (widened on the integer pipe)
-  const double* W = in.W;
-  const double r = W[cell], u0 = W[nc + cell], u1 = W[2 * nc + cell], u2 = W[3 * nc + cell];
-  const double p = W[4 * nc + cell], H = W[NW * nc + cell];
-  const double un = D == 0 ? u0 : (D == 1 ? u1 : u2);
-  const double mn = r * un;
-  F[0] = mn + fl_widen(X[0]);
-  F[1] = fma(mn, u0, fl_widen(X[1]));
-  F[2] = fma(mn, u1, fl_widen(X[2]));
-  F[3] = fma(mn, u2, fl_widen(X[3]));
-  F[1 + D] += p;
-  F[4] = fma(un, H, fl_widen(X[4]));
-}
-
-// R_v (+)= -(F_v - Fp_v) / dx in FP64
-__device__ __forceinline__ void divergence(double* __restrict__ R, int nc, int cell, double id,
-                                           const double F[5], const double Fp[5], int accumulate) {
-#pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    const double dF = F[v] - Fp[v];
-    double* dst = R + v * nc + cell;
-    *dst = accumulate ? fma(-id, dF, *dst) : -id * dF;
-  }
+  assemble_flux<D>(q, ph, X, F);
 }
 
 // The stage of one interior cell once its right-hand side is complete: R_v = its value from the
-// other axes' kernels minus this axis's flux difference (the FP64 accumulation of divergence()),
-// then the arithmetic of k_stage_prim -- body force, the RK3 combination into Ud, the primitives of
-// Ud, their split and H = E + p -- into the second buffer pair.  Wold: the current primitives (the
-// body-force velocities of the stage's input state).
+// other axes' kernels (null: none) minus this axis's flux difference (the FP64 accumulation of
+// update_r), then the arithmetic of k_stage_prim -- body force, the RK3 combination into Ud, the
+// primitives of Ud -- into the second buffer.  W32: the current primitives (the body-force
+// velocities of the stage's input state).
 __device__ __forceinline__ void stage_cell(const StageOut& so, const double* __restrict__ R,
-                                           const double* __restrict__ Wold, int nc, int cell, double id,
+                                           const float* __restrict__ W32, int nc, int cell, double id,
                                            const double F[5], const double Fp[5], double dt, bool hold,
                                            const Phys& ph, bool& bad) {
   double u[5];
@@ -340,349 +307,197 @@ __device__ __forceinline__ void stage_cell(const StageOut& so, const double* __r
   } else {
     double r[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) r[v] = fma(-id, F[v] - Fp[v], R[v * nc + cell]);
+    for (int v = 0; v < 5; ++v) {
+      const double dF = __dsub_rn(F[v], Fp[v]);
+      r[v] = R ? fma(-id, dF, R[v * nc + cell]) : __dmul_rn(-id, dF);
+    }
     if (ph.has_force) {
-      const double vx = Wold[nc + cell], vy = Wold[2 * nc + cell], vz = Wold[3 * nc + cell];
+      const double vx = ff_to_double(load_pair(W32, nc, 1, cell)), vy = ff_to_double(load_pair(W32, nc, 2, cell)),
+                   vz = ff_to_double(load_pair(W32, nc, 3, cell));
       r[1] += ph.f[0];
       r[2] += ph.f[1];
       r[3] += ph.f[2];
       r[4] += fma(ph.f[0], vx, fma(ph.f[1], vy, ph.f[2] * vz));
     }
+    double un[5], us[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) un[v] = so.Un[v * nc + cell];
+    if (so.stage != 1) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) us[v] = so.Us[v * nc + cell];
+    }
+    stage_combine(so.stage, dt, un, us, r, u);
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      const double un = so.Un[v * nc + cell];
-      double out;
-      if (so.stage == 1) {
-        out = fma(dt, r[v], un);
-      } else {
-        const double us = so.Us[v * nc + cell];
-        out = so.stage == 2 ? fma(0.75, un, 0.25 * fma(dt, r[v], us))
-                            : fma(1.0 / 3.0, un, (2.0 / 3.0) * fma(dt, r[v], us));
-      }
-      bad |= !finite_bits(out);
-      so.Ud[v * nc + cell] = out;
-      u[v] = out;
+      bad |= !finite_bits(u[v]);
+      so.Ud[v * nc + cell] = u[v];
     }
   }
   if (!so.prims) return;
-  double w[NW];
-  prim_from_cons(u, ph, w);
+  ff w[NW];
+  prim_ff(u, ph, w);
 #pragma unroll
-  for (int v = 0; v < NW; ++v) {
-    so.W[v * nc + cell] = w[v];
-    split_hi_lo(w[v], so.W32[v * nc + cell], so.W32[(NW + v) * nc + cell]);
-  }
-  so.W[NW * nc + cell] = u[4] + w[4];
+  for (int v = 0; v < NW; ++v) store_pair(so.W32, nc, v, cell, w[v]);
 }
 
-template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(128) k_face_mixed(MixedIn in, double* __restrict__ R, Geo g,
-                                                    PhysF pf, int accumulate, int seg) {
-  constexpr int A1 = (D == 0) ? 1 : 0;
-  constexpr int A2 = (D == 2) ? 1 : 2;
-  constexpr int NVW = VISC ? 6 : 5;          // windowed primitives (T only for the heat flux)
-  const int n1 = g.n[A1], n2 = g.n[A2], nd = g.n[D];
-  const int nseg = (nd + seg - 1) / seg;
-  const long long total = (long long)n1 * n2 * nseg;
+// Tiles as in k_face_tile_body: one thread per cell of a run along D, the terms of neighbouring cells
+// through shared memory.  Waiting for memory binds (the y launch on TGV 128^3 issued in 42 % of the
+// cycles at 24 warps per SM), so the tiles take 64 registers for 32 warps and ask L2 early for the lines
+// that a thread reads last.  TGV 128^3, one launch (x, y, z with the stage): 0.095, 0.14 and 0.195 ms,
+// 0.135, 0.17 and 0.285 ms before with WENO5 formed for each side of a face and the FP64 cell flux.
+// Along y and z 8 x 32 was faster than 16 x 32, 32 x 32 and 4 x 64 (z by up to a fifth), and than a march
+// with the terms in registers (128 registers, 13 warps per SM: y 0.20, z 0.38 ms).
+template <int D>
+struct MixedShape {
+  // the FP64 tiles' shape, so that batches lay out both alike (batch_plan)
+  static constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD;
+  static constexpr int threads = TX * TD, step = TD - 5, blocks = 32 * 32 / threads;
+};
+
+__device__ __forceinline__ void prefetch_line(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+template <int N>
+struct MixedShared {
+  float D[6][N], T[5][N], A[5][N], C[5][N], cR[5][N];
+  double F[5][N];
+};
+
+template <int D, int SCHEME, bool VISC, bool STAGE>
+__device__ __forceinline__ void k_face_mixed_body(const float* __restrict__ W32, const float* __restrict__ G32,
+                                                  double* __restrict__ R, const Geo& g, const Phys& ph, const PhysF& pf,
+                                                  MixedShared<MixedShape<D>::threads>& sh, int col,
+                                                  long long tile, const StageOut* so) {
+  constexpr int TX = MixedShape<D>::TX, TD = MixedShape<D>::TD;
+  constexpr int NVW = VISC ? 6 : 5;
+  const int t = threadIdx.x, row = t / TX, nc = g.ncell;
   const int s = D == 0 ? 1 : (D == 1 ? g.sy : g.sz);
-  const int nc = g.ncell;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int i1 = (int)(t % n1);
-    const long long r = t / n1;
-    const int i2 = (int)(r % n2);
-    const int sg = (int)(r / n2);
-    int c[3];
-    c[A1] = i1 + g.h[A1];
-    c[A2] = i2 + g.h[A2];
-    const int a0 = g.h[D] + sg * seg;
-    const int a1 = min(a0 + seg, g.h[D] + nd);
-    c[D] = a0 - 1;
-    int cell = c[0] + c[1] * g.sy + c[2] * g.sz;   // cell a = a0 - 1
-    // window D_{a-2 .. a+2} for the first face a0 - 1/2
-    float Dw[6][5];
-#pragma unroll
-    for (int v = 0; v < NVW; ++v)
-#pragma unroll
-      for (int k = 0; k < 5; ++k) Dw[v][k] = diff32(in.hi + v * nc, in.lo + v * nc, cell + (k - 2) * s, s);
-    double Fp[5], F[5];
-    face_flux_mixed<D, SCHEME, VISC>(in, cell, s, a0 - 1, Dw, g, pf, Fp);
-    for (int a = a0; a < a1; ++a) {
-      cell += s;
-#pragma unroll
-      for (int v = 0; v < NVW; ++v) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) Dw[v][k] = Dw[v][k + 1];
-        Dw[v][4] = diff32(in.hi + v * nc, in.lo + v * nc, cell + 2 * s, s);
-      }
-      face_flux_mixed<D, SCHEME, VISC>(in, cell, s, a, Dw, g, pf, F);
-      divergence(R, nc, cell, g.idx[D][a], F, Fp, accumulate);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) Fp[v] = F[v];
-    }
-  }
-}
-
-// x-direction variant: lanes map to consecutive faces of one grid row so that every global load is
-// coalesced.  A warp covers 31 cells (32 faces) of a row; the cell differences D_j of the tile
-// (36 per primitive) are formed once in shared memory, each lane builds its face from that window,
-// and the flux difference takes the neighbouring face's flux from shared memory.
-constexpr int kXCells = 31;
-constexpr int kXRows = 4;
-
-template <int SCHEME, bool VISC>
-__device__ __forceinline__ void k_face_mixed_x_body(MixedIn in, double* __restrict__ R,
-                                                              Geo g, PhysF pf, int accumulate,
-    uint3 bid, uint3 gdim) {
-  constexpr int NVW = VISC ? 6 : 5;
-  constexpr int ND = kXCells + 5;               // D_j for j in [x0-3, x0+kXCells+1]
-  __shared__ float sD[kXRows][6][ND];
-  __shared__ double sF[kXRows][5][kXCells + 1];
-  const int lane = threadIdx.x, row = threadIdx.y;
-  const int n0 = g.n[0], h0 = g.h[0];
-  const int line = bid.y * kXRows + row;
-  const bool live = line < g.n[1] * g.n[2];
-  const int j1 = live ? line % g.n[1] : 0, j2 = live ? line / g.n[1] : 0;
-  const int x0 = h0 + bid.x * kXCells;      // first interior cell of the tile (padded index)
-  const int nc = g.ncell;
-  const int rowbase = (j1 + g.h[1]) * g.sy + (j2 + g.h[2]) * g.sz;
-  const int xend = h0 + n0;                      // one past the last interior cell
-  if (live) {
-    for (int k = lane; k < ND; k += 32) {
-      const int j = x0 - 3 + k;
-      const bool ok = j + 1 <= xend + 2;         // W index j + 1 stays inside the padded row
-#pragma unroll
-      for (int v = 0; v < NVW; ++v)
-        sD[row][v][k] = ok ? diff32(in.hi + v * nc, in.lo + v * nc, rowbase + j, 1) : 0.0f;
-    }
-  }
-  // each warp reads only the shared rows it wrote: a warp barrier suffices
-  __syncwarp();
-  const int a = x0 - 1 + lane;                   // this lane's face is a + 1/2
-  if (live && a < xend) {
-    float Dw[6][5];
-#pragma unroll
-    for (int v = 0; v < NVW; ++v)
-#pragma unroll
-      for (int k = 0; k < 5; ++k) Dw[v][k] = sD[row][v][lane + k];
-    double F[5];
-    face_flux_mixed<0, SCHEME, VISC>(in, rowbase + a, 1, a, Dw, g, pf, F);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) sF[row][v][lane] = F[v];
-  }
-  __syncwarp();
-  const int cx = x0 + lane;                      // cell of the divergence
-  if (live && lane < kXCells && cx < xend) {
-    double F[5], Fp[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) { F[v] = sF[row][v][lane + 1]; Fp[v] = sF[row][v][lane]; }
-    divergence(R, nc, rowbase + cx, g.idx[0][cx], F, Fp, accumulate);
-  }
-}
-
-template <int SCHEME, bool VISC>
-__global__ void __launch_bounds__(32 * kXRows) k_face_mixed_x(MixedIn in, double* __restrict__ R,
-                                                              Geo g, PhysF pf, int accumulate) {
-  k_face_mixed_x_body<SCHEME, VISC>(in, R, g, pf, accumulate, blockIdx, gridDim);
-}
-
-// y / z variant: lanes map to 32 consecutive x columns (coalesced loads); a block of NWARP warps
-// covers FPW NWARP - 1 cells along the face axis D (FPW NWARP faces) of those columns at one index
-// of the remaining axis.  The cell differences along D are staged in shared memory; warp w computes
-// the FPW consecutive faces FPW w .. FPW w + FPW - 1, keeps the previous face flux in registers for
-// the divergence of the cells between them and takes the flux of face FPW (w + 1) from the next
-// warp through shared memory.  Registers are capped at 64 so that 32 / NWARP blocks (32 warps)
-// fit an SM.
-template <int NWARP, int FPW>
-constexpr size_t t_smem() {
-  return sizeof(float) * 6 * (FPW * NWARP + 4) * 32 + sizeof(double) * NWARP * 5 * 32;
-}
-
-// Bulk-staged tiles: the (hi, lo) rows a tile's cell differences need, staged into shared memory
-// by cp.async.bulk.  Per row 36 floats: the 32 columns of the tile from the 16-byte boundary at or
-// below the first, so that both addresses of the copy are aligned (the rows' own alignment varies
-// with the row); the W32 buffers carry 64 floats of slack past their end for the last rows' tails.
-constexpr int kBulkRow = 36;
-
-template <int NWARP, int FPW, int NVW>
-constexpr size_t t_smem_bulk() {
-  return sizeof(float) * 2 * NVW * (FPW * NWARP + 5) * kBulkRow + t_smem<NWARP, FPW>();
-}
-
-template <int D, int SCHEME, bool VISC, int NWARP, int FPW, bool STAGE = false, bool BULK = false>
-__device__ __forceinline__ void k_face_mixed_t_body(MixedIn in, double* __restrict__ R,
-                                                                       Geo g, PhysF pf, int accumulate,
-    uint3 bid, uint3 gdim, const StageOut* sop = nullptr, const Phys* php = nullptr,
-    unsigned* flags = nullptr) {
-  static_assert(D == 1 || D == 2, "tiles along y or z");
-  constexpr int kTFaces = FPW;
-  constexpr int kTCells = kTFaces * NWARP - 1;
-  constexpr int kTWarps = NWARP;
-  constexpr int NVW = VISC ? 6 : 5;
-  constexpr int ND = kTCells + 5;
-  constexpr int OTHER = D == 1 ? 2 : 1;                     // the axis that is neither x nor D
-  constexpr int NA = 2 * NVW;                               // staged arrays: hi and lo of each primitive
-  constexpr int NR = ND + 1;                                // staged rows: cells d0 - 3 .. d0 + kTCells + 2
-  constexpr size_t kRawBytes = BULK ? sizeof(float) * NA * NR * kBulkRow : 0;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* raw = reinterpret_cast<float*>(smem_raw);                                      // [NA][NR][36]
-  float (*sD)[ND][32] = reinterpret_cast<float (*)[ND][32]>(smem_raw + kRawBytes);      // [6][ND][32]
-  double (*sF)[5][32] =
-      reinterpret_cast<double (*)[5][32]>(smem_raw + kRawBytes + sizeof(float) * 6 * ND * 32);  // [NWARP][5][32]
-  const int lane = threadIdx.x, warp = threadIdx.y;
-  const int x = g.h[0] + bid.x * 32 + lane;
-  const bool xok = x < g.h[0] + g.n[0];
-  const int d0 = g.h[D] + bid.y * kTCells;             // first cell of the tile along D
-  const int dend = g.h[D] + g.n[D];
-  const int o = g.h[OTHER] + bid.z;
-  const int s = D == 1 ? g.sy : g.sz;
-  const int so = OTHER == 1 ? g.sy : g.sz;
-  const int nc = g.ncell;
-  const int colbase = x + o * so;                           // cell index with D coordinate 0
+  const TileCell tc = tile_cell<D, MixedShape<D>>(g, col, tile);
+  const int i = tc.i, cell = tc.cell;
   // fused stage: dt of the step, the third stage's hold (dt <= 0) and its clock update
   double dt = 0.0;
   bool hold = false, bad = false;
   if (STAGE) {
-    dt = sop->ctl->dt;
-    hold = sop->stage == 3 && !(dt > 0.0);
-    if (sop->stage == 3 && !hold && bid.x == 0 && bid.y == 0 && bid.z == 0 && lane == 0 && warp == 0) {
-      const double tn = sop->ctl->t + dt;
-      sop->ctl->t = (sop->t_end > 0.0 && !(tn < sop->t_end)) ? sop->t_end : tn;
+    dt = so->ctl->dt;
+    hold = so->stage == 3 && !(dt > 0.0);
+    if (so->stage == 3 && !hold && col == 0 && tile == 0 && t == 0) {
+      const double tn = so->ctl->t + dt;
+      so->ctl->t = (so->t_end > 0.0 && !(tn < so->t_end)) ? so->t_end : tn;
     }
   }
-  if (BULK) {
-    // stage the rows: warp 0 issues one bulk copy per (array, row) inside the padded grid, all
-    // counted on one mbarrier; every thread then waits for the phase (bounded)
-    __shared__ __align__(8) unsigned long long s_bar;
-    const unsigned bar = smem_u32(&s_bar);
-    const int nvalid = min(NR, g.p[D] - (d0 - 3));
-    const int colbase0 = g.h[0] + bid.x * 32 + o * so;      // column of lane 0
-    if (lane == 0 && warp == 0) mbar_init(bar, 1);
-    __syncthreads();
-    if (warp == 0) {
-      if (lane == 0) mbar_arrive_expect(bar, (unsigned)(NA * nvalid * kBulkRow * sizeof(float)));
-      __syncwarp();
-      for (int q = lane; q < NA * nvalid; q += 32) {
-        const int ar = q / nvalid, k = q - ar * nvalid;
-        const float* src = (ar < NVW ? in.hi + (size_t)ar * nc : in.lo + (size_t)(ar - NVW) * nc) +
-                           colbase0 + (d0 - 3 + k) * s;
-        const uintptr_t a16 = reinterpret_cast<uintptr_t>(src) & ~uintptr_t(15);
-        bulk_to_smem(smem_u32(raw + (ar * NR + k) * kBulkRow), reinterpret_cast<const void*>(a16),
-                     kBulkRow * sizeof(float), bar);
-      }
-    }
-    const bool late = !mbar_wait_bounded(bar, 0);
-    if (__syncthreads_or(late)) {
-      // the copies did not complete in time: report it, give copies still in flight into this
-      // block's shared memory one more bounded wait, and leave the tile undone
-      if (lane == 0 && warp == 0 && flags) atomicOr(flags, FLAG_STAGING);
-      if (late) mbar_wait_bounded(bar, 0);
-      return;
-    }
-    // cell differences from the staged rows, in the order diff32 forms them
-    auto at = [&](int ar, int k) {
-      const float* src = (ar < NVW ? in.hi + (size_t)ar * nc : in.lo + (size_t)(ar - NVW) * nc) +
-                         colbase0 + (d0 - 3 + k) * s;
-      const int sh = (int)((reinterpret_cast<uintptr_t>(src) >> 2) & 3);
-      return raw[(ar * NR + k) * kBulkRow + sh + lane];
-    };
-    for (int k = warp; k < ND; k += kTWarps) {
-      const int j = d0 - 3 + k;
-      const bool ok = xok && j + 1 <= dend + 2;
+  // what the thread reads after its terms are formed (with the stage, whose own reads already fill
+  // the memory system, this costs time: z 0.195 -> 0.21 ms)
+  if (!STAGE && tc.live && i >= g.h[D] && i < g.h[D] + g.n[D]) {
+    if (D > 0) {
 #pragma unroll
-      for (int v = 0; v < NVW; ++v)
-        sD[v][k][lane] = ok ? (at(v, k + 1) - at(v, k)) + (at(NVW + v, k + 1) - at(NVW + v, k)) : 0.0f;
+      for (int v = 0; v < 5; ++v) prefetch_line(R + v * nc + cell);
     }
-  } else {
-    // each warp takes a run of consecutive rows and keeps the previous row's (hi, lo) in
-    // registers, so every value is loaded once (the differences are those diff32 forms; the
-    // rows' second loads missed L1, which holds about 11 KB per tile beside the shared memory:
-    // on TGV 128^3 the y tile 4.5 % faster, the z tile with the stage 1.3 %)
-    constexpr int KPW = (ND + kTWarps - 1) / kTWarps;
-    const int k0 = warp * KPW, k1 = min(ND, k0 + KPW);
-    const int jmax = dend + 2;                              // last padded index along D
+    if (VISC) {
 #pragma unroll
-    for (int v = 0; v < NVW; ++v) {
-      const float* hp = in.hi + v * nc + colbase;
-      const float* lp = in.lo + v * nc + colbase;
-      float h0 = 0.0f, l0 = 0.0f;
-      if (xok && k0 < k1 && d0 - 3 + k0 <= jmax) {
-        h0 = __ldg(hp + (d0 - 3 + k0) * s);
-        l0 = __ldg(lp + (d0 - 3 + k0) * s);
-      }
-      for (int k = k0; k < k1; ++k) {
-        const int j = d0 - 3 + k;
-        const bool ok = xok && j + 1 <= jmax;
-        float h1 = 0.0f, l1 = 0.0f;
-        if (ok) {
-          h1 = __ldg(hp + (j + 1) * s);
-          l1 = __ldg(lp + (j + 1) * s);
+      for (int b = 0; b < 3; ++b)
+        if (b != D && b < g.ndim) {
+          prefetch_line(G32 + (D * 3 + b) * nc + cell);
+          prefetch_line(G32 + (b * 3 + b) * nc + cell);
         }
-        sD[v][k][lane] = ok ? (h1 - h0) + (l1 - l0) : 0.0f;
-        h0 = h1;
-        l0 = l1;
-      }
+    }
+  }
+  float D0[NVW];
+  ff q[5];
+#pragma unroll
+  for (int v = 0; v < NVW; ++v) {
+    const float* hp = W32 + v * nc + cell;
+    const float* lp = W32 + (NW + v) * nc + cell;
+    const ff q0{__ldg(hp), __ldg(lp)};
+    D0[v] = tc.pair ? s_add(s_sub(__ldg(hp + s), q0.h), s_sub(__ldg(lp + s), q0.l)) : 0.0f;
+    if (v < 5) q[v] = q0;
+    sh.D[v][t] = D0[v];
+  }
+  __syncthreads();
+  const bool up = row > 0;
+  float T0[5], B0[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    T0[v] = s_sub(D0[v], up ? sh.D[v][t - TX] : 0.0f);
+    float A, C;
+    cell_terms32(D0[v], T0[v], pf.eps4, A, B0[v], C);
+    sh.T[v][t] = T0[v];
+    sh.A[v][t] = A;
+    sh.C[v][t] = C;
+  }
+  __syncthreads();
+  const bool inner = row >= 2 && row < TD - 1;
+  float cL[5], Tn[3] = {0.0f, 0.0f, 0.0f};
+  if (inner) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const float T1 = sh.T[v][t + TX];
+      if (v >= 1 && v <= 3) Tn[v - 1] = T1;
+      float cR;
+      cell_corr32<SCHEME>(sh.A[v][t - TX], B0[v], sh.C[v][t + TX], T0[v], s_sub(T0[v], sh.T[v][t - TX]),
+                          s_sub(T1, T0[v]), cL[v], cR);
+      sh.cR[v][t] = cR;
     }
   }
   __syncthreads();
-  const int f0 = warp * kTFaces;                            // face a + 1/2, a = d0 - 1 + f
-  double Fp[5];
-  for (int f = f0; f < f0 + kTFaces; ++f) {
-    const int a = d0 - 1 + f;
-    if (!xok || a >= dend) break;
-    float Dw[6][5];
+  const bool face = row >= 2 && row < TD - 2 && tc.live && i >= g.h[D] - 1 && i < g.h[D] + g.n[D];
+  double F[5];
+  if (face) {
+    float cR[5], Ts[4], Td[4];
 #pragma unroll
-    for (int v = 0; v < NVW; ++v)
+    for (int v = 0; v < 5; ++v) cR[v] = sh.cR[v][t + TX];
 #pragma unroll
-      for (int kk = 0; kk < 5; ++kk) Dw[v][kk] = sD[v][f + kk][lane];
-    double F[5];
-    face_flux_mixed<D, SCHEME, VISC>(in, colbase + a * s, s, a, Dw, g, pf, F);
-    if (f == f0) {
+    for (int c = 0; c < 3; ++c) {
+      Ts[c] = s_add(T0[1 + c], Tn[c]);
+      Td[c] = s_sub(Tn[c], T0[1 + c]);
+    }
+    if (VISC) {
+      const float Ta = s_sub(D0[NVW - 1], sh.D[NVW - 1][t - TX]), Tj = s_sub(sh.D[NVW - 1][t + TX], D0[NVW - 1]);
+      Ts[3] = s_add(Ta, Tj);
+      Td[3] = s_sub(Tj, Ta);
+    }
+    mixed_face<D, VISC>(W32, G32, cell, s, i, g, ph, pf, q, cL, cR, D0, Ts, Td, D0[NVW - 1], F);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sF[warp][v][lane] = F[v];
-    } else if (STAGE) {
-      stage_cell(*sop, R, in.W, nc, colbase + a * s, g.idx[D][a], F, Fp, dt, hold, *php, bad);
+    for (int v = 0; v < 5; ++v) sh.F[v][t] = F[v];
+  }
+  __syncthreads();
+  if (face && row >= 3 && i >= g.h[D]) {
+    const double id = g.idx[D][i];
+    double Fp[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) Fp[v] = sh.F[v][t - TX];
+    if (STAGE) {
+      stage_cell(*so, R, W32, nc, cell, id, F, Fp, dt, hold, ph, bad);
     } else {
-      divergence(R, nc, colbase + a * s, g.idx[D][a], F, Fp, accumulate);   // cell a, faces a -+ 1/2
+#pragma unroll
+      for (int v = 0; v < 5; ++v) update_r<D>(R + v * nc + cell, F[v], Fp[v], id);
     }
-#pragma unroll
-    for (int v = 0; v < 5; ++v) Fp[v] = F[v];
   }
-  __syncthreads();
-  // the last cell of this warp's run, d0 - 1 + f0 + kTFaces: right face from the next warp
-  const int a = d0 + f0 + kTFaces - 1;
-  if (warp + 1 < kTWarps && xok && a < dend) {
-    double F[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) F[v] = sF[warp + 1][v][lane];
-    if (STAGE) stage_cell(*sop, R, in.W, nc, colbase + a * s, g.idx[D][a], F, Fp, dt, hold, *php, bad);
-    else divergence(R, nc, colbase + a * s, g.idx[D][a], F, Fp, accumulate);
-  }
-  if (STAGE && bad) atomicOr(&sop->ctl->flags, FLAG_NONFINITE);
+  if (STAGE && bad) atomicOr(&so->ctl->flags, FLAG_NONFINITE);
 }
 
-template <int D, int SCHEME, bool VISC, int NWARP, int FPW>
-__global__ void __launch_bounds__(32 * NWARP, 32 / NWARP) k_face_mixed_t(MixedIn in, double* __restrict__ R,
-                                                                       Geo g, PhysF pf, int accumulate) {
-  k_face_mixed_t_body<D, SCHEME, VISC, NWARP, FPW>(in, R, g, pf, accumulate, blockIdx, gridDim);
-}
-
-// bulk-staged tile (4 warps x 4 faces): the y / z face kernel with its rows staged by cp.async.bulk
 template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(128, 4) k_face_mixed_tb(MixedIn in, double* __restrict__ R, Geo g,
-                                                          PhysF pf, int accumulate, unsigned* flags) {
-  k_face_mixed_t_body<D, SCHEME, VISC, 4, 4, false, true>(in, R, g, pf, accumulate, blockIdx, gridDim,
-                                                          nullptr, nullptr, flags);
+__global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed(
+    const float* __restrict__ W32, const float* __restrict__ G32, double* __restrict__ R,
+    const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  const int cols = tile_cols<D, MixedShape<D>>(g);
+  k_face_mixed_body<D, SCHEME, VISC, false>(W32, G32, R, g, ph, pf,
+                                            *reinterpret_cast<MixedShared<MixedShape<D>::threads>*>(raw),
+                                            blockIdx.x % cols, blockIdx.x / cols, nullptr);
 }
 
-// the last axis's tile kernel with the stage fused (StageOut): R is read, not written
-template <int D, int SCHEME, bool VISC, int NWARP, int FPW, int MINB, bool BULK = false>
-__global__ void __launch_bounds__(32 * NWARP, MINB) k_face_mixed_ts(MixedIn in, const double* __restrict__ R,
-                                                                    Geo g, PhysF pf, StageOut so, Phys ph) {
-  k_face_mixed_t_body<D, SCHEME, VISC, NWARP, FPW, true, BULK>(in, const_cast<double*>(R), g, pf, 1, blockIdx,
-                                                               gridDim, &so, &ph, &so.ctl->flags);
+// the last axis's kernel with the stage fused (StageOut): R is read, not written
+template <int D, int SCHEME, bool VISC>
+__global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed_stage(
+    const float* __restrict__ W32, const float* __restrict__ G32, const double* __restrict__ R,
+    const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf, const __grid_constant__ StageOut so) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  const int cols = tile_cols<D, MixedShape<D>>(g);
+  k_face_mixed_body<D, SCHEME, VISC, true>(W32, G32, const_cast<double*>(R), g, ph, pf,
+                                           *reinterpret_cast<MixedShared<MixedShape<D>::threads>*>(raw),
+                                           blockIdx.x % cols, blockIdx.x / cols, &so);
 }
-
 
 // centre velocity gradients in FP32 from the FP32 primitives (fourth-order central)
 __device__ __forceinline__ void k_grad32_body(const float* __restrict__ W32, float* __restrict__ G32, Geo g,
@@ -767,23 +582,16 @@ __global__ void __launch_bounds__(kDtBlock) k_dt_partial32(const float* __restri
 }
 
 // ---- batched kernels of the serving loop (see BatchTable in fluid_internal.cuh) -----------------
-__device__ __forceinline__ MixedIn batch_in(const BatchSlot& S) {
-  return MixedIn{S.W, S.W32, S.W32 + (size_t)NW * S.g.ncell, S.G32};
-}
-
-template <int SCHEME, bool VISC>
-__global__ void __launch_bounds__(32 * kXRows) kbm_face_x(const BatchTable* __restrict__ t, int step) {
-  FL_BATCH_LOOP(BK_FACE0)
-  if (step < S.steps) k_face_mixed_x_body<SCHEME, VISC>(batch_in(S), S.R, S.g, phys_f(S.ph), 0, bid, gdim);
-  FL_BATCH_END
-}
-
 template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(128, 8) kbm_face_t(const BatchTable* __restrict__ t, int step) {
+__global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) kbm_face(
+    const BatchTable* __restrict__ t, int step) {
+  extern __shared__ __align__(16) unsigned char raw[];
   FL_BATCH_LOOP(BK_FACE0 + D)
+  (void)gdim;
   if (step < S.steps)
-    k_face_mixed_t_body<D, SCHEME, VISC, kMixedTileWarps, kMixedTileFaces>(batch_in(S), S.R, S.g, phys_f(S.ph), 1,
-                                                                          bid, gdim);
+    k_face_mixed_body<D, SCHEME, VISC, false>(S.W32, S.G32, S.R, S.g, S.ph, phys_f(S.ph),
+                                              *reinterpret_cast<MixedShared<MixedShape<D>::threads>*>(raw), bid.x, bid.y,
+                                              nullptr);
   FL_BATCH_END
 }
 
@@ -799,178 +607,78 @@ __global__ void __launch_bounds__(kDtBlock) kbm_dtp(const BatchTable* __restrict
   FL_BATCH_END
 }
 
+template <int D, int SCHEME, bool VISC>
+cudaError_t batch_face_d(const BatchTable* dev, int step, cudaStream_t st) {
+  constexpr int n = MixedShape<D>::threads;
+  constexpr size_t smem = sizeof(MixedShared<n>);
+  const cudaError_t e =
+      cudaFuncSetAttribute(kbm_face<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  static const int grid = batch_grid(kbm_face<D, SCHEME, VISC>, n, smem);
+  (kbm_face<D, SCHEME, VISC><<<grid, n, smem, st>>>(dev, step), ++t_launches);
+  return cudaGetLastError();
+}
+
 template <int SCHEME, bool VISC>
 cudaError_t batch_face_m(const BatchTable* dev, int D, int step, cudaStream_t st) {
-  constexpr size_t smem = t_smem<kMixedTileWarps, kMixedTileFaces>();
-  if (D == 0) {
-    static const int gx = batch_grid(kbm_face_x<SCHEME, VISC>, 32 * kXRows);
-    (kbm_face_x<SCHEME, VISC><<<gx, dim3(32, kXRows), 0, st>>>(dev, step), ++t_launches);
-    return cudaGetLastError();
-  }
-  static bool init = false;
-  static int g1 = 0, g2 = 0;
-  if (!init) {
-    cudaError_t e = cudaFuncSetAttribute(kbm_face_t<1, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kbm_face_t<2, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    g1 = batch_grid(kbm_face_t<1, SCHEME, VISC>, 128, smem);
-    g2 = batch_grid(kbm_face_t<2, SCHEME, VISC>, 128, smem);
-    init = true;
-  }
-  if (D == 1) (kbm_face_t<1, SCHEME, VISC><<<g1, dim3(32, kMixedTileWarps), smem, st>>>(dev, step), ++t_launches);
-  else (kbm_face_t<2, SCHEME, VISC><<<g2, dim3(32, kMixedTileWarps), smem, st>>>(dev, step), ++t_launches);
-  return cudaGetLastError();
+  if (D == 0) return batch_face_d<0, SCHEME, VISC>(dev, step, st);
+  if (D == 1) return batch_face_d<1, SCHEME, VISC>(dev, step, st);
+  return batch_face_d<2, SCHEME, VISC>(dev, step, st);
 }
 
 template <int D, int SCHEME, bool VISC>
-cudaError_t launch_t(const MixedIn& in, double* R, const Geo& g, const PhysF& pf, int accumulate,
-                     int block, int seg, cudaStream_t st) {
-  constexpr int A1 = (D == 0) ? 1 : 0;
-  constexpr int A2 = (D == 2) ? 1 : 2;
-  const long long lines = (long long)g.n[A1] * g.n[A2];
-  if (block <= 0) block = 128;
-  if (seg <= 0) {
-    seg = 64;
-    while (seg > 8 && lines * ((g.n[D] + seg - 1) / seg) < 152LL * 4 * 128) seg >>= 1;
-  }
-  const long long total = lines * ((g.n[D] + seg - 1) / seg);
-  (k_face_mixed<D, SCHEME, VISC><<<grid_for(total, block), block, 0, st>>>(in, R, g, pf, accumulate, seg), ++t_launches);
-  return cudaGetLastError();
-}
-
-template <int SCHEME, bool VISC, int NWARP, int FPW>
-cudaError_t launch_tile(int D, const MixedIn& in, double* R, const Geo& g, const PhysF& pf,
-                        int accumulate, cudaStream_t st) {
-  constexpr int cells = FPW * NWARP - 1;
-  constexpr size_t smem = t_smem<NWARP, FPW>();
-  const int other = D == 1 ? 2 : 1;
-  const dim3 grid((g.n[0] + 31) / 32, (g.n[D] + cells - 1) / cells, g.n[other]);
-  // a tile may need more than the default 48 KB of dynamic shared memory (attribute is per device)
-  if (D == 1) {
-    cudaError_t e = cudaFuncSetAttribute(k_face_mixed_t<1, SCHEME, VISC, NWARP, FPW>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t launch_t(const float* W32, const float* G32, double* R, const Geo& g, const Phys& ph, const StageOut* so,
+                     cudaStream_t st) {
+  const PhysF pf = phys_f(ph);
+  constexpr int n = MixedShape<D>::threads;
+  constexpr size_t smem = sizeof(MixedShared<n>);
+  const unsigned grid = (unsigned)(tile_rows<D, MixedShape<D>>(g) * tile_cols<D, MixedShape<D>>(g));
+  // a tile may need more than the default 48 KB of dynamic shared memory (the attribute is per device)
+  cudaError_t e;
+  if (so) {
+    e = cudaFuncSetAttribute(k_face_mixed_stage<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    (k_face_mixed_t<1, SCHEME, VISC, NWARP, FPW><<<grid, dim3(32, NWARP), smem, st>>>(in, R, g, pf, accumulate), ++t_launches);
+    (k_face_mixed_stage<D, SCHEME, VISC><<<grid, n, smem, st>>>(W32, G32, R, g, ph, pf, *so), ++t_launches);
   } else {
-    cudaError_t e = cudaFuncSetAttribute(k_face_mixed_t<2, SCHEME, VISC, NWARP, FPW>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_face_mixed<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    (k_face_mixed_t<2, SCHEME, VISC, NWARP, FPW><<<grid, dim3(32, NWARP), smem, st>>>(in, R, g, pf, accumulate), ++t_launches);
+    (k_face_mixed<D, SCHEME, VISC><<<grid, n, smem, st>>>(W32, G32, R, g, ph, pf), ++t_launches);
   }
   return cudaGetLastError();
 }
 
 template <int SCHEME, bool VISC>
-cudaError_t launch_tile_bulk(int D, const MixedIn& in, double* R, const Geo& g, const PhysF& pf,
-                             int accumulate, unsigned* flags, cudaStream_t st) {
-  constexpr size_t smem = t_smem_bulk<4, 4, VISC ? 6 : 5>();
-  const int other = D == 1 ? 2 : 1;
-  const dim3 grid((g.n[0] + 31) / 32, (g.n[D] + 14) / 15, g.n[other]);
-  if (D == 1) {
-    cudaError_t e = cudaFuncSetAttribute(k_face_mixed_tb<1, SCHEME, VISC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    (k_face_mixed_tb<1, SCHEME, VISC><<<grid, dim3(32, 4), smem, st>>>(in, R, g, pf, accumulate, flags), ++t_launches);
-  } else {
-    cudaError_t e = cudaFuncSetAttribute(k_face_mixed_tb<2, SCHEME, VISC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    (k_face_mixed_tb<2, SCHEME, VISC><<<grid, dim3(32, 4), smem, st>>>(in, R, g, pf, accumulate, flags), ++t_launches);
-  }
-  return cudaGetLastError();
+cudaError_t launch_sv(int D, const float* W32, const float* G32, double* R, const Geo& g, const Phys& ph,
+                      const StageOut* so, cudaStream_t st) {
+  if (D == 0) return launch_t<0, SCHEME, VISC>(W32, G32, R, g, ph, so, st);
+  if (D == 1) return launch_t<1, SCHEME, VISC>(W32, G32, R, g, ph, so, st);
+  return launch_t<2, SCHEME, VISC>(W32, G32, R, g, ph, so, st);
 }
 
-template <int SCHEME, bool VISC>
-cudaError_t launch_sv(int D, const MixedIn& in, double* R, const Geo& g, const PhysF& pf,
-                      int accumulate, int block, int seg, unsigned* flags, cudaStream_t st) {
-  if (D == 0) {
-    const long long lines = (long long)g.n[1] * g.n[2];
-    const dim3 grid((g.n[0] + kXCells - 1) / kXCells, (unsigned)((lines + kXRows - 1) / kXRows));
-    (k_face_mixed_x<SCHEME, VISC><<<grid, dim3(32, kXRows), 0, st>>>(in, R, g, pf, accumulate), ++t_launches);
-    return cudaGetLastError();
-  }
-  const int other = D == 1 ? 2 : 1;
-  if (seg < 0 || g.n[other] > 65535) {   // register-window marching kernels
-    const int sg = seg < 0 ? -seg : 0;
-    if (D == 1) return launch_t<1, SCHEME, VISC>(in, R, g, pf, accumulate, block, sg, st);
-    return launch_t<2, SCHEME, VISC>(in, R, g, pf, accumulate, block, sg, st);
-  }
-  // seg 1: the 4 x 4 tile with its rows staged by bulk copies
-  if (seg == 1) return launch_tile_bulk<SCHEME, VISC>(D, in, R, g, pf, accumulate, flags, st);
-  // tile shape (warps x faces per warp): block 64 -> 2 x 4, otherwise 4 x 3 (on TGV 128^3 the
-  // 4 x 4 tile was the fastest of 16 x 1, 8 x 2, 4 x 4 and 2 x 4, and 4 x 3 beat 4 x 4, 4 x 5 and
-  // 4 x 2 by 2.5 % or more over the step)
-  if (block == 64) return launch_tile<SCHEME, VISC, 2, 4>(D, in, R, g, pf, accumulate, st);
-  return launch_tile<SCHEME, VISC, kMixedTileWarps, kMixedTileFaces>(D, in, R, g, pf, accumulate, st);
-}
-
-template <int SCHEME, bool VISC, int NWARP, int FPW, int MINB, bool BULK = false>
-cudaError_t launch_tile_stage(int D, const MixedIn& in, const double* R, const Geo& g, const PhysF& pf,
-                              const Phys& ph, const StageOut& so, cudaStream_t st) {
-  constexpr int cells = FPW * NWARP - 1;
-  constexpr size_t smem = BULK ? t_smem_bulk<NWARP, FPW, VISC ? 6 : 5>() : t_smem<NWARP, FPW>();
-  const int other = D == 1 ? 2 : 1;
-  const dim3 grid((g.n[0] + 31) / 32, (g.n[D] + cells - 1) / cells, g.n[other]);
-  if (D == 1) {
-    cudaError_t e = cudaFuncSetAttribute(k_face_mixed_ts<1, SCHEME, VISC, NWARP, FPW, MINB, BULK>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    (k_face_mixed_ts<1, SCHEME, VISC, NWARP, FPW, MINB, BULK><<<grid, dim3(32, NWARP), smem, st>>>(in, R, g, pf, so, ph), ++t_launches);
-  } else {
-    cudaError_t e = cudaFuncSetAttribute(k_face_mixed_ts<2, SCHEME, VISC, NWARP, FPW, MINB, BULK>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    (k_face_mixed_ts<2, SCHEME, VISC, NWARP, FPW, MINB, BULK><<<grid, dim3(32, NWARP), smem, st>>>(in, R, g, pf, so, ph), ++t_launches);
-  }
-  return cudaGetLastError();
-}
-
-template <int SCHEME, bool VISC>
-cudaError_t launch_stage_sv(const MixedIn& in, const double* R, const Geo& g, const PhysF& pf, const Phys& ph,
-                            int block, int seg, const StageOut& so, cudaStream_t st) {
-  const int D = g.ndim - 1;
-  if (seg == 1) return launch_tile_stage<SCHEME, VISC, 4, 4, 4, true>(D, in, R, g, pf, ph, so, st);
-  if (block == 64) return launch_tile_stage<SCHEME, VISC, 2, 4, 12>(D, in, R, g, pf, ph, so, st);
-  // 4 warps x 3 faces, as the unfused tile; 64 registers (a few bytes spilled) so that 8 tiles
-  // fit an SM: on TGV 128^3 6 % faster than 72 registers without spills (7 tiles) and 11 % faster
-  // than 80 (6 tiles)
-  return launch_tile_stage<SCHEME, VISC, kMixedTileWarps, kMixedTileFaces, 8>(D, in, R, g, pf, ph, so, st);
+cudaError_t launch_any(int D, const float* W32, const float* G32, double* R, const Geo& g, const Phys& ph,
+                       const StageOut* so, cudaStream_t st) {
+  const bool visc = ph.visc != FLUID_VISC_NONE;
+  if (ph.weno == FLUID_WENO_JS)
+    return visc ? launch_sv<FLUID_WENO_JS, true>(D, W32, G32, R, g, ph, so, st)
+                : launch_sv<FLUID_WENO_JS, false>(D, W32, G32, R, g, ph, so, st);
+  return visc ? launch_sv<FLUID_WENO_Z, true>(D, W32, G32, R, g, ph, so, st)
+              : launch_sv<FLUID_WENO_Z, false>(D, W32, G32, R, g, ph, so, st);
 }
 
 }  // namespace
 
-bool mixed_stage_fusable(const Geo& g, int seg) {
-  if (g.ndim < 2 || seg < 0) return false;
-  const int other = g.ndim - 1 == 1 ? 2 : 1;
-  return g.n[other] <= 65535;
+cudaError_t launch_face_mixed_stage(const float* W32, const float* G32, const double* R, const Geo& g,
+                                    const Phys& ph, const StageOut& so, cudaStream_t st) {
+  // one-dimensional: no other axis has written R
+  return launch_any(g.ndim - 1, W32, G32, g.ndim > 1 ? const_cast<double*>(R) : nullptr, g, ph, &so, st);
 }
 
-cudaError_t launch_face_mixed_stage(const double* W, const float* W32, const float* G32,
-                                    const double* R, const Geo& g, const Phys& ph, int block, int seg,
-                                    const StageOut& so, cudaStream_t st) {
-  const bool visc = ph.visc != FLUID_VISC_NONE;
-  const MixedIn in{W, W32, W32 + (size_t)NW * g.ncell, G32};
-  const PhysF pf = phys_f(ph);
-  if (ph.weno == FLUID_WENO_JS)
-    return visc ? launch_stage_sv<FLUID_WENO_JS, true>(in, R, g, pf, ph, block, seg, so, st)
-                : launch_stage_sv<FLUID_WENO_JS, false>(in, R, g, pf, ph, block, seg, so, st);
-  return visc ? launch_stage_sv<FLUID_WENO_Z, true>(in, R, g, pf, ph, block, seg, so, st)
-              : launch_stage_sv<FLUID_WENO_Z, false>(in, R, g, pf, ph, block, seg, so, st);
+cudaError_t launch_face_mixed(int D, const float* W32, const float* G32, double* R, const Geo& g, const Phys& ph,
+                              cudaStream_t st) {
+  return launch_any(D, W32, G32, R, g, ph, nullptr, st);
 }
 
-cudaError_t launch_face_mixed(int D, const double* W, const float* W32, const float* G32, double* R,
-                              const Geo& g, const Phys& ph, int accumulate, int block, int seg,
-                              cudaStream_t st, unsigned* flags) {
-  const bool visc = ph.visc != FLUID_VISC_NONE;
-  const MixedIn in{W, W32, W32 + (size_t)NW * g.ncell, G32};
-  const PhysF pf = phys_f(ph);
-  if (ph.weno == FLUID_WENO_JS)
-    return visc ? launch_sv<FLUID_WENO_JS, true>(D, in, R, g, pf, accumulate, block, seg, flags, st)
-                : launch_sv<FLUID_WENO_JS, false>(D, in, R, g, pf, accumulate, block, seg, flags, st);
-  return visc ? launch_sv<FLUID_WENO_Z, true>(D, in, R, g, pf, accumulate, block, seg, flags, st)
-              : launch_sv<FLUID_WENO_Z, false>(D, in, R, g, pf, accumulate, block, seg, flags, st);
-}
+constexpr int kBulkRow = 36;    // floats per row of the probe
 
 namespace {
 // Check of the bulk-staging helpers: one warp stages nrows rows of 36 floats (16-byte aligned) from

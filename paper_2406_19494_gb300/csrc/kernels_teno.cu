@@ -59,7 +59,7 @@ struct TenoShared {
 template <int D, int NP>
 __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>::threads) k_face_teno(
     const double* __restrict__ W, const double* __restrict__ G, double* __restrict__ R,
-    const __grid_constant__ Geo g, const __grid_constant__ Phys ph, int accumulate) {
+    const __grid_constant__ Geo g, const __grid_constant__ Phys ph) {
   constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD, N = TileShape<D>::threads;
   constexpr int NVW = NP ? 6 : 5;
   extern __shared__ __align__(16) unsigned char raw[];
@@ -204,38 +204,38 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
   if (face && row >= 3 && i >= g.h[D]) {
     const double id = g.idx[D][i];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) update_r(R + v * nc + cell, F[v], sh.F[v][t - TX], id, accumulate);
+    for (int v = 0; v < 5; ++v) update_r<D>(R + v * nc + cell, F[v], sh.F[v][t - TX], id);
   }
 }
 
 template <int D, int NP>
 cudaError_t launch_d(const double* W, const double* G, double* R, const Geo& g, const Phys& ph,
-                     int accumulate, cudaStream_t st) {
+                     cudaStream_t st) {
   constexpr int n = TileShape<D>::threads;
   constexpr size_t smem = sizeof(TenoShared<n, NP ? 6 : 5>);
   const cudaError_t e =
       cudaFuncSetAttribute(k_face_teno<D, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)(tile_rows<D>(g) * tile_cols<D>(g));
-  (k_face_teno<D, NP><<<grid, n, smem, st>>>(W, G, R, g, ph, accumulate), ++t_launches);
+  (k_face_teno<D, NP><<<grid, n, smem, st>>>(W, G, R, g, ph), ++t_launches);
   return cudaGetLastError();
 }
 
 template <int NP>
 cudaError_t launch_v(int D, const double* W, const double* G, double* R, const Geo& g, const Phys& ph,
-                     int accumulate, cudaStream_t st) {
-  if (D == 0) return launch_d<0, NP>(W, G, R, g, ph, accumulate, st);
-  if (D == 1) return launch_d<1, NP>(W, G, R, g, ph, accumulate, st);
-  return launch_d<2, NP>(W, G, R, g, ph, accumulate, st);
+                     cudaStream_t st) {
+  if (D == 0) return launch_d<0, NP>(W, G, R, g, ph, st);
+  if (D == 1) return launch_d<1, NP>(W, G, R, g, ph, st);
+  return launch_d<2, NP>(W, G, R, g, ph, st);
 }
 
 }  // namespace
 
 cudaError_t launch_face_teno(int D, const double* W, const double* G, double* R, const Geo& g,
-                             const Phys& ph, int accumulate, cudaStream_t st) {
-  if (ph.visc == FLUID_VISC_NONE) return launch_v<0>(D, W, G, R, g, ph, accumulate, st);
-  if (ph.visc_order == 6) return launch_v<6>(D, W, G, R, g, ph, accumulate, st);
-  return launch_v<4>(D, W, G, R, g, ph, accumulate, st);
+                             const Phys& ph, cudaStream_t st) {
+  if (ph.visc == FLUID_VISC_NONE) return launch_v<0>(D, W, G, R, g, ph, st);
+  if (ph.visc_order == 6) return launch_v<6>(D, W, G, R, g, ph, st);
+  return launch_v<4>(D, W, G, R, g, ph, st);
 }
 
 }  // namespace fl

@@ -107,12 +107,9 @@ size_t footprint(const fluid_config& c) {
   }
   const bool visc = c.visc_law != FLUID_VISC_NONE;
   size_t b = 8 * (nc * (fl::NW + 3 * fl::NV) + metric + 4096);   // W, A, R, the state U, metrics
-  // mixed: the H row of W, the (hi, lo) FP32 primitives, FP32 gradients, the FP32 metric copies, and the
-  // second pair of primitive buffers (W with its H row, W32)
+  // mixed: two buffers of FP32 pairs of the primitives, FP32 gradients, the FP32 metric copies
   if (c.precision == FLUID_PREC_MIXED) {
-    b += 8 * nc + 4 * (nc * (2 * fl::NW + (visc ? fl::NG : 0)) + 3 * (metric / 5));
-    b += 8 * nc * (fl::NW + 1) + 4 * nc * 2 * fl::NW;
-    b += 2 * 64 * 4;                                    // the W32 buffers' slack for staged rows
+    b += 4 * (nc * (2 * 2 * fl::NW + (visc ? fl::NG : 0)) + 3 * (metric / 5));
   } else {
     if (visc) b += 8 * nc * fl::NG;
     // seam buffer of the face kernels: 10 doubles per segment of kSeamMinSeg cells, on the axis
@@ -355,10 +352,9 @@ struct fluid_server {
     auto it = tuned.find(key);
     if (it == tuned.end()) {
       std::vector<std::pair<int, int>> cand = {{0, 0}, {32, 64}, {64, 16}, {128, 32}};
-      // only shapes whose results are bitwise those of the default shape: every FP64 segment
-      // length, and the mixed path's two tile sizes (its register-window kernels are compiled
-      // separately and agree only to FP32 rounding)
-      if (c.precision == FLUID_PREC_MIXED) cand = {{0, 0}, {64, 0}};
+      // every FP64 segment length gives bitwise the default shape's results; the mixed path has
+      // one shape
+      if (c.precision == FLUID_PREC_MIXED) cand = {{0, 0}};
       double* tmp = nullptr;
       float best = 1e30f;
       std::pair<int, int> pick{0, 0};
