@@ -22,18 +22,16 @@ FL_HD void cell_terms(ff D, ff T, ff eps4, ff& A, ff& B, ff& C) {
 // 6 times the nonlinear parts of cell j's two face values from the indicator set e0 = A_{j-1},
 // e1 = B_j, e2 = C_{j+1} and the third differences V0 = T_j - T_{j-1}, V1 = T_{j+1} - T_j:
 // w^L_{j+1/2} = q_j + (2 D_j + D_{j-1} + dL) / 6, w^R_{j-1/2} = q_j - (2 D_{j-1} + D_j - dR) / 6.
-// False when a ratio leaves the FP32 range.
+// False when the indicators leave the FP32 range.
 template <int SCHEME>
 FL_HD bool cell_values(ff e0, ff e1, ff e2, ff V0, ff V1, ff& dL, ff& dR) {
   ff W0, W1, W2;
-  bool ok;
   const ff r0 = ff_rcp(e0), r1 = ff_rcp(e1), r2 = ff_rcp(e2);
+  const float em = fminf(fminf(e0.h, e1.h), e2.h);
   if (SCHEME == FLUID_WENO_JS) {
-    const float em = fminf(fminf(e0.h, e1.h), e2.h);
     W0 = sqr_weak(mul_weak(r0, em));
     W1 = sqr_weak(mul_weak(r1, em));
     W2 = sqr_weak(mul_weak(r2, em));
-    ok = em < 1e30f;
   } else {
     const ff tau = e0 - e2;
     const ff Z0 = mul_weak(tau, r0), Z1 = mul_weak(tau, r1), Z2 = mul_weak(tau, r2);
@@ -41,7 +39,13 @@ FL_HD bool cell_values(ff e0, ff e1, ff e2, ff V0, ff V1, ff& dL, ff& dR) {
     W0 = fma_weak(Z0, Z0, one);
     W1 = fma_weak(Z1, Z1, one);
     W2 = fma_weak(Z2, Z2, one);
-    ok = fmaxf(fmaxf(W0.h, W1.h), W2.h) < 1e18f;
+    // tau above 2^30 of an indicator (next to exactly uniform cells): Z^2 drowns the 1 and may leave
+    // the FP32 range, so the weights are taken relative to the smallest indicator, as for JS
+    if (!(fmaxf(fmaxf(W0.h, W1.h), W2.h) < 1e18f)) {
+      W0 = sqr_weak(mul_weak(r0, em));
+      W1 = sqr_weak(mul_weak(r1, em));
+      W2 = sqr_weak(mul_weak(r2, em));
+    }
   }
   const ff P0 = mul_weak(W0, V0), P2 = mul_weak(W2, V1);
   const ff base = add_weak(add_weak(W0, W2), mul_weak(W1, 6.0f));
@@ -50,7 +54,7 @@ FL_HD bool cell_values(ff e0, ff e1, ff e2, ff V0, ff V1, ff& dL, ff& dR) {
   const ff S2 = ff_twice(add_weak(P0, P2));           // numL = S2 + P2, numR = S2 + P0
   dL = mul_weak(-P2 - S2, ff_rcp(denL));
   dR = mul_weak(P0 + S2, ff_rcp(denR));
-  return ok;
+  return em < 1e30f;
 }
 
 // HLLC star correction of a face in ff, from the left state wl and the jumps J = wr - wl:
