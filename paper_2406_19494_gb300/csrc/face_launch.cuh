@@ -13,6 +13,7 @@ __global__ void __launch_bounds__(128) k_face(const double* __restrict__ W, cons
                                               double* __restrict__ R, double* __restrict__ FB,
                                               const __grid_constant__ Geo g, const __grid_constant__ Phys ph,
                                               int seg) {
+  step_wait();
   k_face_body<D, SCHEME, VISC>(W, G, R, FB, g, ph, seg, blockIdx, gridDim);
 }
 
@@ -20,6 +21,7 @@ template <int D, int SCHEME, bool VISC>
 __global__ void __launch_bounds__(TileShape<D>::threads, TileShape<D>::blocks) k_face_tile(
     const double* __restrict__ W, const double* __restrict__ G, double* __restrict__ R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph) {
+  step_wait();
   extern __shared__ __align__(16) unsigned char raw[];
   const int cols = tile_cols<D>(g);                        // neighbouring blocks: neighbouring columns
   k_face_tile_body<D, SCHEME, VISC>(W, G, R, g, ph,
@@ -36,7 +38,7 @@ cudaError_t launch_tile(const double* W, const double* G, double* R, const Geo& 
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)(tile_rows<D>(g) * tile_cols<D>(g));
-  (k_face_tile<D, SCHEME, VISC><<<grid, n, smem, st>>>(W, G, R, g, ph), ++t_launches);
+  launch_step(k_face_tile<D, SCHEME, VISC>, grid, n, smem, st, W, G, R, g, ph);
   return cudaGetLastError();
 }
 
@@ -51,9 +53,9 @@ cudaError_t launch_scheme(int D, const double* W, const double* G, double* R, co
   int grid;
   face_shape(D, g, block, seg, grid);
   double* FB = seam_buffer(D, g, seg, fb);
-  if (D == 0) (k_face<0, SCHEME, VISC><<<grid, block, 0, st>>>(W, G, R, FB, g, ph, seg), ++t_launches);
-  else if (D == 1) (k_face<1, SCHEME, VISC><<<grid, block, 0, st>>>(W, G, R, FB, g, ph, seg), ++t_launches);
-  else (k_face<2, SCHEME, VISC><<<grid, block, 0, st>>>(W, G, R, FB, g, ph, seg), ++t_launches);
+  if (D == 0) launch_step(k_face<0, SCHEME, VISC>, grid, block, 0, st, W, G, R, FB, g, ph, seg);
+  else if (D == 1) launch_step(k_face<1, SCHEME, VISC>, grid, block, 0, st, W, G, R, FB, g, ph, seg);
+  else launch_step(k_face<2, SCHEME, VISC>, grid, block, 0, st, W, G, R, FB, g, ph, seg);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !FB) return e;
   return launch_face_seam(D, FB, R, g, seg, st);

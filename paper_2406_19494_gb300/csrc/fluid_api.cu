@@ -330,14 +330,9 @@ int rhs_into(fluid_solver* s, const double* U, double* R, cudaStream_t st) {
 }
 
 int dt_into(fluid_solver* s, double* dt_out, int clip, double t_end, cudaStream_t st) {
-  if (s->ph.dt_fixed <= 0.0) {
-    if (s->mixed)
-      FL_TIMED(s, FLUID_KERNEL_DT, st, fl::launch_dt_partial32(s->W32, s->geo, s->ph, s->partial, s->nparts, st));
-    else
-      FL_TIMED(s, FLUID_KERNEL_DT, st, fl::launch_dt_partial(s->W, s->geo, s->ph, s->partial, s->nparts, st));
-  }
   FL_TIMED(s, FLUID_KERNEL_DT, st,
-           fl::launch_dt_final(s->partial, s->nparts, s->ph, s->ctl, dt_out, clip, t_end, st));
+           s->mixed ? fl::launch_dt32(s->W32, s->geo, s->ph, s->partial, s->nparts, s->ctl, dt_out, clip, t_end, st)
+                    : fl::launch_dt(s->W, s->geo, s->ph, s->partial, s->nparts, s->ctl, dt_out, clip, t_end, st));
   return FLUID_OK;
 }
 

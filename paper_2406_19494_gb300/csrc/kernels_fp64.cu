@@ -20,7 +20,7 @@
 //   k_stage_prim / k_halo_prim   the stage combination fused with the primitives of its result
 //               (interior cells), then the halo cells from those; fluid_step uses this pair in
 //               place of k_stage followed by the next right-hand side's k_prim_bc
-//   k_dt_*      CFL time step: per-block minimum, then one block reduces (deterministic)
+//   k_dt        CFL time step: per-block maxima of the rate, the last block reduces (deterministic)
 //
 // The state is FP64 structure-of-arrays U[v][z][y][x]; primitives and gradients live in solver
 // scratch with the same padded layout.
@@ -179,6 +179,7 @@ __device__ __forceinline__ void k_prim_bc_body(const double* __restrict__ U, dou
 template <bool MIXED>
 __global__ void k_prim_bc(const double* __restrict__ U, double* __restrict__ W,
                           float* __restrict__ W32, Geo g, Phys ph, BC bc, Ctl* ctl) {
+  step_wait();
   k_prim_bc_body<MIXED>(U, W, W32, g, ph, bc, ctl, blockIdx, gridDim);
 }
 
@@ -229,6 +230,7 @@ __device__ __forceinline__ void k_grad_body(const double* __restrict__ W, double
 
 template <int ORDER>
 __global__ void k_grad(const double* __restrict__ W, double* __restrict__ G, Geo g) {
+  step_wait();
   k_grad_body<ORDER>(W, G, g, blockIdx, gridDim);
 }
 
@@ -270,6 +272,7 @@ __device__ __forceinline__ void k_face_seam_body(const double* __restrict__ FB, 
 
 template <int D>
 __global__ void k_face_seam(const double* __restrict__ FB, double* __restrict__ R, Geo g, int seg) {
+  step_wait();
   k_face_seam_body<D>(FB, R, g, seg, blockIdx, gridDim);
 }
 
@@ -292,6 +295,7 @@ __device__ __forceinline__ double velocity(const double* __restrict__ W, const f
 
 __global__ void k_source(double* __restrict__ R, const double* __restrict__ W, const float* __restrict__ W32, Geo g,
                          Phys ph) {
+  step_wait();
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
@@ -350,6 +354,7 @@ __device__ __forceinline__ void k_stage_body(int stage, const double* Un, const 
 __global__ void k_stage(int stage, const double* Un, const double* Us, const double* __restrict__ R,
                         double* Ud, const double* __restrict__ W, const float* __restrict__ W32, Geo g, Phys ph,
                         Ctl* ctl, double t_end, double dt_arg) {
+  step_wait();
   k_stage_body(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, dt_arg, blockIdx, gridDim);
 }
 
@@ -443,6 +448,7 @@ template <bool MIXED>
 __global__ void k_stage_prim(int stage, const double* Un, const double* Us, const double* __restrict__ R,
                              double* Ud, double* W, float* __restrict__ W32, Geo g, Phys ph, Ctl* ctl,
                              double t_end) {
+  step_wait();
   k_stage_prim_body<MIXED>(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, blockIdx, gridDim);
 }
 
@@ -505,85 +511,107 @@ __device__ __forceinline__ void k_halo_prim_body(double* __restrict__ W, float* 
 template <bool MIXED>
 __global__ void k_halo_prim(double* __restrict__ W, float* __restrict__ W32, Geo g, Phys ph, BC bc,
                             Ctl* ctl, long long total) {
+  step_wait();
   k_halo_prim_body<MIXED>(W, W32, g, ph, bc, ctl, total, blockIdx, gridDim);
 }
 
-constexpr int kDtBlock = 256;
 
 // CFL: dt = cfl * min over cells and axes of dx / (|u| + c) and dx^2 / (k nu), taken as
 // cfl / max of the rates (|u| + c) / dx and k nu / dx^2 so that a cell costs no division.
-// Per-block maxima of the rate go to `partial`.
-__device__ __forceinline__ void k_dt_partial_body(const double* __restrict__ W, Geo g, Phys ph,
-                                                         double* __restrict__ partial,
-    uint3 bid, uint3 gdim) {
-  const int total = g.n[0] * g.n[1] * g.n[2];
-  const int nc = g.ncell;
-  double best = 0.0;
-  for (int t = bid.x * blockDim.x + threadIdx.x; t < total; t += gdim.x * blockDim.x) {
-    const int i = t % g.n[0];
-    const int r = t / g.n[0];
-    const int j = r % g.n[1];
-    const int k = r / g.n[1];
-    const int ci[3] = {i + g.h[0], j + g.h[1], k + g.h[2]};
-    const int c = ci[0] + ci[1] * g.sy + ci[2] * g.sz;
-    const double rho = W[c], p = W[4 * nc + c];
-    const double irho = fl_rcp(rho);
-    const double cs = fl_sqrt(ph.gamma * p * irho);
-    double knu = 0.0;
-    if (ph.visc != FLUID_VISC_NONE) knu = ph.dt_visc_k * viscosity(W[5 * nc + c], ph) * irho;
-    for (int d = 0; d < g.ndim; ++d) {
-      const double id = g.idx[d][ci[d]];
-      best = fmax(best, (fabs(W[(1 + d) * nc + c]) + cs) * id);
-      if (ph.visc != FLUID_VISC_NONE) best = fmax(best, knu * id * id);
-    }
+__device__ __forceinline__ double cell_rate(const double* __restrict__ W, const Geo& g, const Phys& ph, int t) {
+  const int i = t % g.n[0];
+  const int r = t / g.n[0];
+  const int j = r % g.n[1];
+  const int k = r / g.n[1];
+  const int ci[3] = {i + g.h[0], j + g.h[1], k + g.h[2]};
+  const int c = ci[0] + ci[1] * g.sy + ci[2] * g.sz, nc = g.ncell;
+  const double rho = W[c], p = W[4 * nc + c];
+  const double irho = fl_rcp(rho);
+  const double cs = fl_sqrt(ph.gamma * p * irho);
+  double knu = 0.0, best = 0.0;
+  if (ph.visc != FLUID_VISC_NONE) knu = ph.dt_visc_k * viscosity(W[5 * nc + c], ph) * irho;
+  for (int d = 0; d < g.ndim; ++d) {
+    const double id = g.idx[d][ci[d]];
+    best = fmax(best, (fabs(W[(1 + d) * nc + c]) + cs) * id);
+    if (ph.visc != FLUID_VISC_NONE) best = fmax(best, knu * id * id);
   }
+  return best;
+}
+
+// The same in FP32, within 1e-4 of it (the power law's estimate is its least exact part); infinite
+// where a value leaves [1e-30, 1e30]
+__device__ __forceinline__ float cell_rate32(const double* __restrict__ W, const Geo& g, const Phys& ph, int t) {
+  const int i = t % g.n[0];
+  const int r = t / g.n[0];
+  const int j = r % g.n[1];
+  const int k = r / g.n[1];
+  const int ci[3] = {i + g.h[0], j + g.h[1], k + g.h[2]};
+  const int c = ci[0] + ci[1] * g.sy + ci[2] * g.sz, nc = g.ncell;
+  const float rho = ff_of(W[c]).h, p = ff_of(W[4 * nc + c]).h;
+  bool ok = rho >= 1e-30f && rho <= 1e30f && p >= 1e-30f && p <= 1e30f;
+  const float irho = s_rcp(rho), c2 = ph.k.gamma.h * (p * irho);
+  const float cs = c2 * s_rsqrt(c2);
+  float knu = 0.0f, best = 0.0f;
+  if (ph.visc != FLUID_VISC_NONE) {
+    const float T = ff_of(W[5 * nc + c]).h, x = T * ph.k.iT_ref.h;
+    ok = ok && x >= 1e-30f && x <= 1e30f;
+    float mu = ph.k.mu_ref.h;
+    if (ph.visc == FLUID_VISC_POWER) mu *= __powf(x, ph.visc_e32);
+    else if (ph.visc == FLUID_VISC_SUTHERLAND) mu = ph.k.mu_TS.h * (x * x) * s_rsqrt(x) * s_rcp(T + ph.k.suth_S.h);
+    knu = ph.k.dt_visc.h * mu * irho;
+  }
+  for (int d = 0; d < g.ndim; ++d) {
+    const float id = ff_of(g.idx[d][ci[d]]).h, u = fabsf(ff_of(W[(1 + d) * nc + c]).h);
+    ok = ok && u <= 1e30f;
+    best = fmaxf(best, fmaxf((u + cs) * id, knu * id * id));
+  }
+  return ok && best <= 1e36f ? best : __int_as_float(0x7f800000);
+}
+
+// Per-block maxima of the rate go to `partial`; the last block to finish reduces them and stores dt (no
+// second launch).  nparts 0: a fixed dt, one block.  Block 0 counts nothing it did not write: the
+// ticket wraps to 0 for the next call.
+// The FP64 rates bind (about 60 FP64-pipe instructions per cell), so a block first finds its largest
+// FP32 rate and forms in FP64 only the cells within 1e-3 of it: the maximum is among them, bit
+// for bit (TGV 128^3: 228 us with every cell in FP64 and the second launch).
+__device__ __forceinline__ void k_dt_body(const double* __restrict__ W, const Geo& g, const Phys& ph, double* partial,
+                                          int nparts, Ctl* ctl, double* dt_out, int clip, double t_end, uint3 bid,
+                                          uint3 gdim) {
   __shared__ double sm[kDtBlock / 32];
-  for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_down_sync(0xffffffffu, best, o));
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = best;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    best = threadIdx.x < kDtBlock / 32 ? sm[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_down_sync(0xffffffffu, best, o));
-    if (threadIdx.x == 0) partial[bid.x] = best;
-  }
-}
-
-__global__ void __launch_bounds__(kDtBlock) k_dt_partial(const double* __restrict__ W, Geo g, Phys ph,
-                                                         double* __restrict__ partial) {
-  k_dt_partial_body(W, g, ph, partial, blockIdx, gridDim);
-}
-
-// dt = cfl / max(partial rates) (or dt_fixed); clip_to_ctl: clip so that t does not pass t_end and
-// store in ctl->dt; otherwise write *dt_out.
-__device__ __forceinline__ void k_dt_final_body(const double* __restrict__ partial, int nparts,
-                                                       Phys ph, Ctl* ctl, double* dt_out, int clip,
-                                                       double t_end,
-    uint3 bid, uint3 gdim) {
+  __shared__ unsigned last;
   double best = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) best = fmax(best, partial[i]);
-  __shared__ double sm[kDtBlock / 32];
-  for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_down_sync(0xffffffffu, best, o));
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = best;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < kDtBlock / 32; ++i) best = fmax(best, sm[i]);
-    double dt = ph.dt_fixed > 0.0 ? ph.dt_fixed : ph.cfl / best;
-    if (!clip) {
-      *dt_out = dt;
-      return;
+  if (nparts > 0) {
+    const int total = g.n[0] * g.n[1] * g.n[2];
+    const int t0 = bid.x * blockDim.x + threadIdx.x, stride = gdim.x * blockDim.x;
+    float mine = 0.0f;
+    for (int t = t0; t < total; t += stride) mine = fmaxf(mine, cell_rate32(W, g, ph, t));
+    const float limit = block_max(mine, reinterpret_cast<float*>(sm)) * 0.999f;
+    // an infinite limit: some value is outside the FP32 range, so every cell is formed in FP64
+    const bool all = !(limit <= 1e36f);
+    if (all || mine >= limit)
+      for (int t = t0; t < total; t += stride)
+        if (all || cell_rate32(W, g, ph, t) >= limit) best = fmax(best, cell_rate(W, g, ph, t));
+    best = block_max(best, sm);
+    if (threadIdx.x == 0) {
+      __stcg(partial + bid.x, best);
+      __threadfence();
+      last = atomicInc(&ctl->ticket, nparts - 1) == (unsigned)(nparts - 1);
     }
-    if (t_end > 0.0) {
-      if (ctl->t >= t_end) dt = 0.0;
-      else if (ctl->t + dt > t_end) dt = t_end - ctl->t;
-    }
-    ctl->dt = dt;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    best = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += blockDim.x) best = fmax(best, __ldcg(partial + i));
+    best = block_max(best, sm);
   }
+  if (threadIdx.x == 0) dt_store(best, ph, ctl, dt_out, clip, t_end);
 }
 
-__global__ void __launch_bounds__(kDtBlock) k_dt_final(const double* __restrict__ partial, int nparts,
-                                                       Phys ph, Ctl* ctl, double* dt_out, int clip,
-                                                       double t_end) {
-  k_dt_final_body(partial, nparts, ph, ctl, dt_out, clip, t_end, blockIdx, gridDim);
+__global__ void __launch_bounds__(kDtBlock) k_dt(const double* __restrict__ W, const __grid_constant__ Geo g,
+                                                 const __grid_constant__ Phys ph, double* partial, int nparts,
+                                                 Ctl* ctl, double* dt_out, int clip, double t_end) {
+  step_wait();
+  k_dt_body(W, g, ph, partial, nparts, ctl, dt_out, clip, t_end, blockIdx, gridDim);
 }
 
 // Halo exchange of a block decomposition: element t of the buffer [5][3][e2][e1] (t1 < t2 the axes
@@ -648,15 +676,10 @@ __global__ void __launch_bounds__(128) kb_prim(const BatchTable* __restrict__ t)
   FL_BATCH_END
 }
 
-__global__ void __launch_bounds__(kDtBlock) kb_dtp(const BatchTable* __restrict__ t, int step) {
-  FL_BATCH_LOOP(BK_DTP)
-  if (step < S.steps) k_dt_partial_body(S.W, S.g, S.ph, S.partial, bid, gdim);
-  FL_BATCH_END
-}
-
-__global__ void __launch_bounds__(kDtBlock) kb_dtf(const BatchTable* __restrict__ t, int step) {
-  FL_BATCH_LOOP(BK_DTF)
-  if (step < S.steps) k_dt_final_body(S.partial, S.nparts, S.ph, S.ctl, nullptr, 1, S.t_end, bid, gdim);
+__global__ void __launch_bounds__(kDtBlock) kb_dt(const BatchTable* __restrict__ t, int step) {
+  FL_BATCH_LOOP(BK_DT)
+  if (step < S.steps)
+    k_dt_body(S.W, S.g, S.ph, S.partial, S.nparts, S.ctl, nullptr, 1, S.t_end, bid, gdim);
   FL_BATCH_END
 }
 
@@ -729,8 +752,7 @@ void batch_plan(BatchTable& t, bool mixed) {
     const long long nint = (long long)g.n[0] * g.n[1] * g.n[2];
     const long long npad = (long long)g.p[0] * g.p[1] * g.p[2];
     set(BK_PRIM, ceil_div(g.p[0], 128), std::min(g.p[1], 65535), std::min(g.p[2], 65535));
-    set(BK_DTP, S.nparts > 0 ? S.nparts : 0);
-    set(BK_DTF, 1);
+    set(BK_DT, S.nparts > 0 ? S.nparts : 1);
     const bool visc = S.ph.visc != FLUID_VISC_NONE;
     long long gt = 1;
     for (int a = 0; a < 3; ++a) gt *= g.n[a] + (a < g.ndim ? 4 : 0);   // order-4 stencils, both paths
@@ -758,7 +780,7 @@ void batch_plan(BatchTable& t, bool mixed) {
 cudaError_t launch_batch_chunk(const BatchTable* dev, int chunk, bool mixed, int weno, bool visc,
                                cudaStream_t st) {
   static const int gp = batch_grid(kb_prim<false>, 128), gpm = batch_grid(kb_prim<true>, 128);
-  static const int gd = batch_grid(kb_dtp, kDtBlock), gf = batch_grid(kb_dtf, kDtBlock);
+  static const int gd = batch_grid(kb_dt, kDtBlock);
   static const int gg = batch_grid(kb_grad, 256);
   static const int gsp = batch_grid(kb_stage_prim<false>, 128), gspm = batch_grid(kb_stage_prim<true>, 128);
   static const int gh = batch_grid(kb_halo<false>, 256), ghm = batch_grid(kb_halo<true>, 256);
@@ -768,14 +790,13 @@ cudaError_t launch_batch_chunk(const BatchTable* dev, int chunk, bool mixed, int
   else (kb_prim<false><<<gp, 128, 0, st>>>(dev), ++t_launches);
   for (int k = 0; k < chunk; ++k) {
     if (mixed) {
-      if ((e = launch_batch_mixed(dev, BMX_DTP, 0, k, st)) != cudaSuccess) return e;
+      if ((e = launch_batch_mixed(dev, BMX_DT, k, st)) != cudaSuccess) return e;
     } else {
-      (kb_dtp<<<gd, kDtBlock, 0, st>>>(dev, k), ++t_launches);
+      (kb_dt<<<gd, kDtBlock, 0, st>>>(dev, k), ++t_launches);
     }
-    (kb_dtf<<<gf, kDtBlock, 0, st>>>(dev, k), ++t_launches);
     for (int stage = 1; stage <= 3; ++stage) {
       if (mixed) {
-        if (visc && (e = launch_batch_mixed(dev, BMX_GRAD, 0, k, st)) != cudaSuccess) return e;
+        if (visc && (e = launch_batch_mixed(dev, BMX_GRAD, k, st)) != cudaSuccess) return e;
         for (int D = 0; D < 3; ++D)
           if ((e = launch_batch_mixed_faces(dev, D, k, weno, visc, st)) != cudaSuccess) return e;
       } else {
@@ -808,9 +829,9 @@ cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, i
   const long long lines = (long long)g.n[D == 0 ? 1 : 0] * g.n[D == 2 ? 1 : 2];
   const long long items = lines * ((g.n[D] + seg - 1) / seg - 1);
   const int grid = grid_for(items, 256);
-  if (D == 0) (k_face_seam<0><<<grid, 256, 0, st>>>(FB, R, g, seg), ++t_launches);
-  else if (D == 1) (k_face_seam<1><<<grid, 256, 0, st>>>(FB, R, g, seg), ++t_launches);
-  else (k_face_seam<2><<<grid, 256, 0, st>>>(FB, R, g, seg), ++t_launches);
+  if (D == 0) launch_step(k_face_seam<0>, grid, 256, 0, st, FB, R, g, seg);
+  else if (D == 1) launch_step(k_face_seam<1>, grid, 256, 0, st, FB, R, g, seg);
+  else launch_step(k_face_seam<2>, grid, 256, 0, st, FB, R, g, seg);
   return cudaGetLastError();
 }
 
@@ -840,8 +861,8 @@ cudaError_t launch_prim_bc(const double* U, double* W, float* W32, const Geo& g,
   const int block = ((g.p[0] + nb - 1) / nb + 31) / 32 * 32;
   const dim3 grid((g.p[0] + block - 1) / block, g.p[1] < 65535 ? g.p[1] : 65535,
                   g.p[2] < 65535 ? g.p[2] : 65535);
-  if (W32) (k_prim_bc<true><<<grid, block, 0, st>>>(U, W, W32, g, ph, bc, ctl), ++t_launches);
-  else (k_prim_bc<false><<<grid, block, 0, st>>>(U, W, W32, g, ph, bc, ctl), ++t_launches);
+  if (W32) launch_step(k_prim_bc<true>, grid, block, 0, st, U, W, W32, g, ph, bc, ctl);
+  else launch_step(k_prim_bc<false>, grid, block, 0, st, U, W, W32, g, ph, bc, ctl);
   return cudaGetLastError();
 }
 
@@ -849,8 +870,8 @@ cudaError_t launch_grad(const double* W, double* G, const Geo& g, const Phys& ph
   const int m = ph.visc_order == 6 ? 3 : 2;
   long long total = 1;
   for (int a = 0; a < 3; ++a) total *= g.n[a] + (a < g.ndim ? 2 * m : 0);
-  if (m == 3) (k_grad<6><<<grid_for(total, 256), 256, 0, st>>>(W, G, g), ++t_launches);
-  else (k_grad<4><<<grid_for(total, 256), 256, 0, st>>>(W, G, g), ++t_launches);
+  if (m == 3) launch_step(k_grad<6>, grid_for(total, 256), 256, 0, st, W, G, g);
+  else launch_step(k_grad<4>, grid_for(total, 256), 256, 0, st, W, G, g);
   return cudaGetLastError();
 }
 
@@ -874,7 +895,7 @@ long long seam_capacity(const Geo& g) {
 cudaError_t launch_source(double* R, const double* W, const float* W32, const Geo& g, const Phys& ph,
                           cudaStream_t st) {
   const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  (k_source<<<grid_for(total, 256), 256, 0, st>>>(R, W, W32, g, ph), ++t_launches);
+  launch_step(k_source, grid_for(total, 256), 256, 0, st, R, W, W32, g, ph);
   return cudaGetLastError();
 }
 
@@ -882,7 +903,7 @@ cudaError_t launch_stage(int stage, const double* Un, const double* Us, const do
                          const double* W, const float* W32, const Geo& g, const Phys& ph, Ctl* ctl,
                          double t_end, cudaStream_t st, double dt_arg) {
   const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  (k_stage<<<grid_for(total, 256), 256, 0, st>>>(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, dt_arg), ++t_launches);
+  launch_step(k_stage, grid_for(total, 256), 256, 0, st, stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, dt_arg);
   return cudaGetLastError();
 }
 
@@ -894,8 +915,8 @@ cudaError_t launch_stage_prim(int stage, const double* Un, const double* Us, con
   const int block = ((g.n[0] + nb - 1) / nb + 31) / 32 * 32;
   const int j2 = (g.n[1] + 1) / 2;                                     // row pairs
   const dim3 grid((g.n[0] + block - 1) / block, j2 < 65535 ? j2 : 65535, g.n[2] < 65535 ? g.n[2] : 65535);
-  if (W32) (k_stage_prim<true><<<grid, block, 0, st>>>(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end), ++t_launches);
-  else (k_stage_prim<false><<<grid, block, 0, st>>>(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end), ++t_launches);
+  if (W32) launch_step(k_stage_prim<true>, grid, block, 0, st, stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end);
+  else launch_step(k_stage_prim<false>, grid, block, 0, st, stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_halo_prim(W, W32, g, ph, bc, ctl, st);
@@ -905,8 +926,8 @@ cudaError_t launch_halo_prim(double* W, float* W32, const Geo& g, const Phys& ph
                              cudaStream_t st) {
   const long long total = (long long)g.p[0] * g.p[1] * g.p[2] - (long long)g.n[0] * g.n[1] * g.n[2];
   if (total <= 0) return cudaSuccess;
-  if (W32) (k_halo_prim<true><<<grid_for(total, 256), 256, 0, st>>>(W, W32, g, ph, bc, ctl, total), ++t_launches);
-  else (k_halo_prim<false><<<grid_for(total, 256), 256, 0, st>>>(W, W32, g, ph, bc, ctl, total), ++t_launches);
+  if (W32) launch_step(k_halo_prim<true>, grid_for(total, 256), 256, 0, st, W, W32, g, ph, bc, ctl, total);
+  else launch_step(k_halo_prim<false>, grid_for(total, 256), 256, 0, st, W, W32, g, ph, bc, ctl, total);
   return cudaGetLastError();
 }
 
@@ -932,16 +953,10 @@ int dt_partial_count(const Geo& g) {
   return (int)(b < 1 ? 1 : b);
 }
 
-cudaError_t launch_dt_partial(const double* W, const Geo& g, const Phys& ph, double* partial,
-                              int nparts, cudaStream_t st) {
-  (k_dt_partial<<<nparts, kDtBlock, 0, st>>>(W, g, ph, partial), ++t_launches);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_dt_final(const double* partial, int nparts, const Phys& ph, Ctl* ctl,
-                            double* dt_out, int clip_to_ctl, double t_end, cudaStream_t st) {
-  (k_dt_final<<<1, kDtBlock, 0, st>>>(partial, ph.dt_fixed > 0.0 ? 0 : nparts, ph, ctl, dt_out,
-                                     clip_to_ctl, t_end), ++t_launches);
+cudaError_t launch_dt(const double* W, const Geo& g, const Phys& ph, double* partial, int nparts, Ctl* ctl,
+                      double* dt_out, int clip_to_ctl, double t_end, cudaStream_t st) {
+  const int n = ph.dt_fixed > 0.0 ? 0 : nparts;
+  launch_step(k_dt, n > 0 ? n : 1, kDtBlock, 0, st, W, g, ph, partial, n, ctl, dt_out, clip_to_ctl, t_end);
   return cudaGetLastError();
 }
 

@@ -480,6 +480,7 @@ template <int D, int SCHEME, bool VISC>
 __global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed(
     const float* __restrict__ W32, const float* __restrict__ G32, double* __restrict__ R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf) {
+  step_wait();
   extern __shared__ __align__(16) unsigned char raw[];
   const int cols = tile_cols<D, MixedShape<D>>(g);
   k_face_mixed_body<D, SCHEME, VISC, false>(W32, G32, R, g, ph, pf,
@@ -492,6 +493,7 @@ template <int D, int SCHEME, bool VISC>
 __global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed_stage(
     const float* __restrict__ W32, const float* __restrict__ G32, const double* __restrict__ R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf, const __grid_constant__ StageOut so) {
+  step_wait();
   extern __shared__ __align__(16) unsigned char raw[];
   const int cols = tile_cols<D, MixedShape<D>>(g);
   k_face_mixed_body<D, SCHEME, VISC, true>(W32, G32, const_cast<double*>(R), g, ph, pf,
@@ -533,16 +535,20 @@ __device__ __forceinline__ void k_grad32_body(const float* __restrict__ W32, flo
 }
 
 __global__ void k_grad32(const float* __restrict__ W32, float* __restrict__ G32, Geo g) {
+  step_wait();
   k_grad32_body(W32, G32, g, blockIdx, gridDim);
 }
 
-constexpr int kDtBlock = 256;
 
 // CFL partial maxima of the rates (|u| + c) / dx and k nu / dx^2 (the inverse time steps, as in
 // the FP64 kernel) from the FP32 primitives: the time step needs no more than FP32 accuracy
-__device__ __forceinline__ void k_dt_partial32_body(const float* __restrict__ W32, Geo g, PhysF pf,
-                                                           double* __restrict__ partial,
-    uint3 bid, uint3 gdim) {
+__device__ __forceinline__ void k_dt32_body(const float* __restrict__ W32, const Geo& g, const Phys& ph,
+                                            const PhysF& pf, double* partial, int nparts, Ctl* ctl, double* dt_out,
+                                            int clip, double t_end, uint3 bid, uint3 gdim) {
+  if (nparts == 0) {                          // a fixed dt
+    if (threadIdx.x == 0) dt_store(0.0, ph, ctl, dt_out, clip, t_end);
+    return;
+  }
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
   float best = 0.0f;
@@ -565,20 +571,29 @@ __device__ __forceinline__ void k_dt_partial32_body(const float* __restrict__ W3
       if (pf.visc != FLUID_VISC_NONE) best = fmaxf(best, knu * id * id);
     }
   }
-  __shared__ float sm[kDtBlock / 32];
-  for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_down_sync(0xffffffffu, best, o));
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = best;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    best = threadIdx.x < kDtBlock / 32 ? sm[threadIdx.x] : 0.0f;
-    for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_down_sync(0xffffffffu, best, o));
-    if (threadIdx.x == 0) partial[bid.x] = (double)best;
+  __shared__ double sm[kDtBlock / 32];
+  __shared__ unsigned last;
+  best = block_max(best, reinterpret_cast<float*>(sm));
+  if (threadIdx.x == 0) {
+    __stcg(partial + bid.x, (double)best);
+    __threadfence();
+    last = atomicInc(&ctl->ticket, nparts - 1) == (unsigned)(nparts - 1);
   }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double top = 0.0;
+  for (int i = threadIdx.x; i < nparts; i += blockDim.x) top = fmax(top, __ldcg(partial + i));
+  top = block_max(top, sm);
+  if (threadIdx.x == 0) dt_store(top, ph, ctl, dt_out, clip, t_end);
 }
 
-__global__ void __launch_bounds__(kDtBlock) k_dt_partial32(const float* __restrict__ W32, Geo g, PhysF pf,
-                                                           double* __restrict__ partial) {
-  k_dt_partial32_body(W32, g, pf, partial, blockIdx, gridDim);
+__global__ void __launch_bounds__(kDtBlock) k_dt32(const float* __restrict__ W32, const __grid_constant__ Geo g,
+                                                   const __grid_constant__ Phys ph, const __grid_constant__ PhysF pf,
+                                                   double* partial, int nparts, Ctl* ctl, double* dt_out, int clip,
+                                                   double t_end) {
+  step_wait();
+  k_dt32_body(W32, g, ph, pf, partial, nparts, ctl, dt_out, clip, t_end, blockIdx, gridDim);
 }
 
 // ---- batched kernels of the serving loop (see BatchTable in fluid_internal.cuh) -----------------
@@ -601,9 +616,10 @@ __global__ void __launch_bounds__(256) kbm_grad(const BatchTable* __restrict__ t
   FL_BATCH_END
 }
 
-__global__ void __launch_bounds__(kDtBlock) kbm_dtp(const BatchTable* __restrict__ t, int step) {
-  FL_BATCH_LOOP(BK_DTP)
-  if (step < S.steps) k_dt_partial32_body(S.W32, S.g, phys_f(S.ph), S.partial, bid, gdim);
+__global__ void __launch_bounds__(kDtBlock) kbm_dt(const BatchTable* __restrict__ t, int step) {
+  FL_BATCH_LOOP(BK_DT)
+  if (step < S.steps)
+    k_dt32_body(S.W32, S.g, S.ph, phys_f(S.ph), S.partial, S.nparts, S.ctl, nullptr, 1, S.t_end, bid, gdim);
   FL_BATCH_END
 }
 
@@ -638,11 +654,11 @@ cudaError_t launch_t(const float* W32, const float* G32, double* R, const Geo& g
   if (so) {
     e = cudaFuncSetAttribute(k_face_mixed_stage<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    (k_face_mixed_stage<D, SCHEME, VISC><<<grid, n, smem, st>>>(W32, G32, R, g, ph, pf, *so), ++t_launches);
+    launch_step(k_face_mixed_stage<D, SCHEME, VISC>, grid, n, smem, st, W32, G32, R, g, ph, pf, *so);
   } else {
     e = cudaFuncSetAttribute(k_face_mixed<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    (k_face_mixed<D, SCHEME, VISC><<<grid, n, smem, st>>>(W32, G32, R, g, ph, pf), ++t_launches);
+    launch_step(k_face_mixed<D, SCHEME, VISC>, grid, n, smem, st, W32, G32, R, g, ph, pf);
   }
   return cudaGetLastError();
 }
@@ -717,19 +733,12 @@ cudaError_t launch_bulk_probe(const float* src, float* dst, int nrows, unsigned 
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_mixed(const BatchTable* dev, int kind, int D, int step, cudaStream_t st) {
+cudaError_t launch_batch_mixed(const BatchTable* dev, int kind, int step, cudaStream_t st) {
   static const int gg = batch_grid(kbm_grad, 256);
-  static const int gd = batch_grid(kbm_dtp, kDtBlock);
-  if (kind == BMX_GRAD) {
-    (kbm_grad<<<gg, 256, 0, st>>>(dev, step), ++t_launches);
-    return cudaGetLastError();
-  }
-  if (kind == BMX_DTP) {
-    (kbm_dtp<<<gd, kDtBlock, 0, st>>>(dev, step), ++t_launches);
-    return cudaGetLastError();
-  }
-  // the bucket key fixes the scheme and the viscosity, read from the first solve on the host side
-  return cudaErrorInvalidValue;
+  static const int gd = batch_grid(kbm_dt, kDtBlock);
+  if (kind == BMX_GRAD) (kbm_grad<<<gg, 256, 0, st>>>(dev, step), ++t_launches);
+  else (kbm_dt<<<gd, kDtBlock, 0, st>>>(dev, step), ++t_launches);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_batch_mixed_faces(const BatchTable* dev, int D, int step, int weno, bool visc,
@@ -742,13 +751,15 @@ cudaError_t launch_batch_mixed_faces(const BatchTable* dev, int D, int step, int
 cudaError_t launch_grad32(const float* W32, float* G32, const Geo& g, cudaStream_t st) {
   long long total = 1;
   for (int a = 0; a < 3; ++a) total *= g.n[a] + (a < g.ndim ? 4 : 0);
-  (k_grad32<<<grid_for(total, 256), 256, 0, st>>>(W32, G32, g), ++t_launches);
+  launch_step(k_grad32, grid_for(total, 256), 256, 0, st, W32, G32, g);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dt_partial32(const float* W32, const Geo& g, const Phys& ph, double* partial,
-                                int nparts, cudaStream_t st) {
-  (k_dt_partial32<<<nparts, kDtBlock, 0, st>>>(W32, g, phys_f(ph), partial), ++t_launches);
+cudaError_t launch_dt32(const float* W32, const Geo& g, const Phys& ph, double* partial, int nparts, Ctl* ctl,
+                        double* dt_out, int clip_to_ctl, double t_end, cudaStream_t st) {
+  const int n = ph.dt_fixed > 0.0 ? 0 : nparts;
+  launch_step(k_dt32, n > 0 ? n : 1, kDtBlock, 0, st, W32, g, ph, phys_f(ph), partial, n, ctl, dt_out, clip_to_ctl,
+              t_end);
   return cudaGetLastError();
 }
 

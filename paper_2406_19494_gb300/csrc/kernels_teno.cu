@@ -60,6 +60,7 @@ template <int D, int NP>
 __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>::threads) k_face_teno(
     const double* __restrict__ W, const double* __restrict__ G, double* __restrict__ R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph) {
+  step_wait();
   constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD, N = TileShape<D>::threads;
   constexpr int NVW = NP ? 6 : 5;
   extern __shared__ __align__(16) unsigned char raw[];
@@ -217,7 +218,7 @@ cudaError_t launch_d(const double* W, const double* G, double* R, const Geo& g, 
       cudaFuncSetAttribute(k_face_teno<D, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)(tile_rows<D>(g) * tile_cols<D>(g));
-  (k_face_teno<D, NP><<<grid, n, smem, st>>>(W, G, R, g, ph), ++t_launches);
+  launch_step(k_face_teno<D, NP>, grid, n, smem, st, W, G, R, g, ph);
   return cudaGetLastError();
 }
 
