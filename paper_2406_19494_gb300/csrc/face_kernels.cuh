@@ -32,32 +32,34 @@ struct Flux5 {
   double f[5];
 };
 
+// The two values of one primitive at a face in FP64 from its six cells (f: the primitive's cell a)
+template <int SCHEME>
+__device__ __forceinline__ void values_fp64(const double* __restrict__ f, int s, double eps4, double& wl, double& wr) {
+  double q[6];
+#pragma unroll
+  for (int o = 0; o < 6; ++o) q[o] = __ldg(f + (o - 2) * s);
+  const double d0 = q[1] - q[0], d1 = q[2] - q[1], d2 = q[3] - q[2], d3 = q[4] - q[3], d4 = q[5] - q[4];
+  const double c = 4.0 * k1312;
+  const double tm = d1 - d0, t0 = d2 - d1, t1 = d3 - d2, t2 = d4 - d3;
+  const double km = fma(c * tm, tm, eps4), k0 = fma(c * t0, t0, eps4);
+  const double k1 = fma(c * t1, t1, eps4), k2 = fma(c * t2, t2, eps4);
+  const double aA = fma(3.0, d1, -d0), aB = d1 + d2, aC = fma(-3.0, d2, d3);
+  const double bA = fma(3.0, d2, -d1), bB = d2 + d3, bC = fma(-3.0, d3, d4);
+  double X[3];
+  weno_x<SCHEME>(fma(aA, aA, km), fma(aB, aB, k0), fma(aC, aC, k1), X);
+  wl = weno_x_value(q[2], d0, d1, d2, d3, X);
+  weno_x<SCHEME>(fma(bC, bC, k2), fma(bB, bB, k1), fma(bA, bA, k0), X);
+  wr = weno_x_value(q[3], -d4, -d3, -d2, -d1, X);
+}
+
 // The convective flux of a face in FP64 from its six cells
 template <int D, int SCHEME>
 __device__ __noinline__ Flux5 face_flux_fp64(const double* __restrict__ W, int nc, int cell, int s,
                                              const Phys* __restrict__ php) {
   const Phys& ph = *php;
-  const double eps4 = 4.0 * ph.eps;
   double wl[5], wr[5];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) {
-    const double* f = W + v * nc + cell;
-    double q[6];
-#pragma unroll
-    for (int o = 0; o < 6; ++o) q[o] = __ldg(f + (o - 2) * s);
-    const double d0 = q[1] - q[0], d1 = q[2] - q[1], d2 = q[3] - q[2], d3 = q[4] - q[3], d4 = q[5] - q[4];
-    const double c = 4.0 * k1312;
-    const double tm = d1 - d0, t0 = d2 - d1, t1 = d3 - d2, t2 = d4 - d3;
-    const double km = fma(c * tm, tm, eps4), k0 = fma(c * t0, t0, eps4);
-    const double k1 = fma(c * t1, t1, eps4), k2 = fma(c * t2, t2, eps4);
-    const double aA = fma(3.0, d1, -d0), aB = d1 + d2, aC = fma(-3.0, d2, d3);
-    const double bA = fma(3.0, d2, -d1), bB = d2 + d3, bC = fma(-3.0, d3, d4);
-    double X[3];
-    weno_x<SCHEME>(fma(aA, aA, km), fma(aB, aB, k0), fma(aC, aC, k1), X);
-    wl[v] = weno_x_value(q[2], d0, d1, d2, d3, X);
-    weno_x<SCHEME>(fma(bC, bC, k2), fma(bB, bB, k1), fma(bA, bA, k0), X);
-    wr[v] = weno_x_value(q[3], -d4, -d3, -d2, -d1, X);
-  }
+  for (int v = 0; v < 5; ++v) values_fp64<SCHEME>(W + v * nc + cell, s, 4.0 * ph.eps, wl[v], wr[v]);
   Flux5 F;
   hllc<D>(wl, wr, ph, F.f);
   return F;
@@ -159,9 +161,10 @@ __device__ __forceinline__ void add_visc(const double* __restrict__ W, const dou
 // w_R = q_{a+1} + (cR - 3 d) / 6: one rounding of the state's size), and for the dissipative flux
 // vv = V_a = T_{a+1} - T_a and tv = T_a + T_{a+1} of the velocities and dt, tt, tm of the temperature
 // (D_a - V_a / 24, T_a + T_{a+1} + 8 D_a, and the value of cell a+1).  ok: the cells' own limits.  sc:
-// scales of cell a+1.
-template <int D, int SCHEME, bool VISC>
-__device__ __forceinline__ void face_of_terms(const double* __restrict__ W, const double* __restrict__ G,
+// scales of cell a+1.  DEFER: where the cells' limits fail, the convective flux is left to the caller
+// (true is returned and F holds the dissipative part).
+template <int D, int SCHEME, bool VISC, bool DEFER>
+__device__ __forceinline__ bool face_of_terms(const double* __restrict__ W, const double* __restrict__ G,
                                               int cell, int s, int a, const Geo& g, const Phys& ph,
                                               bool ok, const Scale& sc, const double d[5], const ff cL[5],
                                               const ff cR[5], const ff vv[3], const ff tv[3], ff dt, ff tt,
@@ -195,7 +198,10 @@ __device__ __forceinline__ void face_of_terms(const double* __restrict__ W, cons
     euler_flux<D>(w, ph, F);
   } else {
     Flux5 e;
-    if (ok) {
+    if (DEFER && !ok) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) e.f[v] = 0.0;
+    } else if (ok) {
       Flux5 l, r;
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
@@ -224,6 +230,7 @@ __device__ __forceinline__ void face_of_terms(const double* __restrict__ W, cons
   }
 #pragma unroll
   for (int v = 0; v < 5; ++v) F[v] = __dadd_rn(F[v], ff_to_double(X[v]));
+  return DEFER && !ok;
 }
 
 // R_a (+)= -(F_{a+1/2} - F_{a-1/2}) / dx_a along D, the same operations in every kernel: the first axis
@@ -337,7 +344,7 @@ __device__ __forceinline__ void march_face(const double* __restrict__ W, const d
     M.Dm = M.D0;
     M.D0 = Dp;
   }
-  face_of_terms<D, SCHEME, VISC>(W, G, cell, s, a, g, ph, M.ok && okj, sc, d, M.cL, cR, vv, tv, dt, tt, tm, F);
+  face_of_terms<D, SCHEME, VISC, false>(W, G, cell, s, a, g, ph, M.ok && okj, sc, d, M.cL, cR, vv, tv, dt, tt, tm, F);
 #pragma unroll
   for (int v = 0; v < 5; ++v) M.cL[v] = cLn[v];
   M.ok = okj;
@@ -428,6 +435,7 @@ struct TileShared {
   ff Dt[N];
   Scale sc[N];
   double F[5][N];          // cR (as two floats), then the face flux
+  int deferred[N], ndef;   // threads whose face takes the FP64 convective flux
 };
 
 // tiles along (x, D) that cover the interior cells
@@ -500,6 +508,7 @@ __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, c
   }
   Scale sc{1.0f, 1.0f, 1.0f, false};
   if (live) sc = scale_of(__ldg(W + cell), __ldg(W + 4 * nc + cell), ph);
+  if (t == 0) sh.ndef = 0;
   __syncthreads();
 #pragma unroll 1
   for (int v = 0; v < 5; ++v) {
@@ -534,6 +543,7 @@ __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, c
   // face j + 1/2
   const bool face = row >= 2 && row < TD - 2 && live && i >= g.h[D] - 1 && i < g.h[D] + g.n[D];
   double F[5];
+  bool mine = false;
   if (face) {
     Scale sn = sh.sc[t + TX];
     double d[5];
@@ -558,9 +568,44 @@ __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, c
     const bool both = ok && sn.ok;
     // the dissipative flux only needs the scales in range
     sn.ok = in_range(sn);
-    face_of_terms<D, SCHEME, VISC>(W, G, cell, s, i, g, ph, both, sn, d, cL, cR, vv, tv, dt, tt, tq, F);
+    mine = face_of_terms<D, SCHEME, VISC, true>(W, G, cell, s, i, g, ph, both, sn, d, cL, cR, vv, tv, dt, tt, tq, F);
+    if (mine) sh.deferred[atomicAdd(&sh.ndef, 1)] = t;
   }
   __syncthreads();
+  // Faces beyond the limits: their FP64 formulas cost ten times a face's FP64 work, so the block's few
+  // are gathered and spread over its threads, one primitive of one face each, then HLLC, one face
+  // each.  (Left to their own lanes they held up every warp that had one: shock tube 26 us a launch.)
+  const int ndef = sh.ndef;
+  if (ndef > 0) {
+    constexpr int N = TileShape<D>::threads;
+    sh.sc[t].r = __int_as_float(cell);                     // the scales are done with
+    __syncthreads();
+    double* wl = &sh.d[0][0];                              // values of (primitive, face), left then right
+    double* wr = reinterpret_cast<double*>(&sh.T[0][0]);
+    static_assert(sizeof(sh.T) == sizeof(sh.d), "one double per pair");
+    for (int k = t; k < 5 * ndef; k += N) {
+      const int v = k / ndef, o = sh.deferred[k - v * ndef];
+      values_fp64<SCHEME>(W + v * nc + __float_as_int(sh.sc[o].r), s, 4.0 * ph.eps, wl[v * N + o], wr[v * N + o]);
+    }
+    __syncthreads();
+    for (int k = t; k < ndef; k += N) {
+      const int o = sh.deferred[k];
+      double l[5], r[5], f[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        l[v] = wl[v * N + o];
+        r[v] = wr[v * N + o];
+      }
+      hllc<D>(l, r, ph, f);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sh.F[v][o] = f[v];
+    }
+    __syncthreads();
+    if (mine) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) F[v] = __dadd_rn(sh.F[v][t], F[v]);
+    }
+  }
   if (face) {
 #pragma unroll
     for (int v = 0; v < 5; ++v) sh.F[v][t] = F[v];
