@@ -38,7 +38,7 @@ struct Geo {
 
 // The constants that the two-float terms of the FP64 face kernels use (set_ff)
 struct PhysFF {
-  ff gamma, gm1, igm1, gg, iR, eps4, mu_ref, mu_TS, iT_ref, suth_S, lam_fac, dt_visc;   // gg = gamma / (gamma - 1), mu_TS = mu_ref (T_ref + S)
+  ff gamma, gm1, igm1, gg, iR, eps4, mu_ref, mu_TS, iT_ref, suth_S, lam_fac, dt_visc, visc_exp, re;   // gg = gamma / (gamma - 1), mu_TS = mu_ref (T_ref + S), re = 2 sqrt(eps)
 };
 
 struct Phys {
@@ -191,6 +191,8 @@ inline void set_ff(Phys& ph) {
   ph.k.suth_S = ff_of(ph.suth_S);
   ph.k.lam_fac = ff_of(ph.lam_fac);
   ph.k.dt_visc = ff_of(ph.dt_visc_k);
+  ph.k.visc_exp = ff_of(ph.visc_exp);
+  ph.k.re = ff_of(2.0 * sqrt(ph.eps));
 }
 
 // Configuration check shared by the entry points: NULL if valid, else a static message.

@@ -2,13 +2,13 @@
 // loss.  Given a state X and a cotangent mu of R(X) on the interior cells, the kernels below form
 // (dR/dX)^T mu and (dR/dphi)^T mu (phi: porous-wall parameters) in gather form -- every value is
 // summed in a fixed order, so the result does not depend on scheduling:
-//   k_adj_face<D>     one thread per segment of faces along a grid line: per face the face-flux
-//                     cotangent from the two adjacent cells, then the reverse of HLLC, of the ten
-//                     WENO5 reconstructions (weights included; the two values reconstructed in one
-//                     cell share its indicator set) and of the dissipative flux; the contributions
-//                     to the primitives of the six stencil cells (and to the four tangential-
-//                     gradient cells: the four cotangents of the face's interpolated tangential
-//                     gradients) go to per-face slots
+//   k_adj_face<D>     one thread per face, in tiles: per face the face-flux cotangent from the two adjacent
+//                     cells, then the reverse of HLLC, of the ten WENO5 reconstructions (weights
+//                     included; the two values reconstructed in one cell share its indicator set) and
+//                     of the dissipative flux, in two-float arithmetic; the contributions to the
+//                     primitives of the six stencil cells (and to the four tangential-gradient cells:
+//                     the four cotangents of the face's interpolated tangential gradients) go to
+//                     per-face slots
 //   k_adj_gather<D>   one thread per cell: sum of the slots of the faces whose stencil contains it
 //                     (the tangential-gradient cotangents times the cell's interpolation weight)
 //   k_adj_grad        reverse of the centre velocity gradients
@@ -18,7 +18,7 @@
 //   k_adj_phi         porous-wall parameters: d v_w / d phi_i = (A / phi0) sin(2 pi kappa x_i)
 #include <cuda_runtime.h>
 
-#include "adjoint_math.cuh"
+#include "adjoint_ff.cuh"
 #include "fluid_internal.cuh"
 
 namespace fl {
@@ -38,154 +38,257 @@ constexpr int kGComp = 4;     // tangential gradient components read by one face
 
 __device__ __forceinline__ int stride_of(const Geo& g, int d) { return d == 0 ? 1 : (d == 1 ? g.sy : g.sz); }
 
-// threads per block of k_adj_face (its WENO gradients sit in shared memory): one warp, so that a
-// launch of a few blocks per SM spreads evenly (the registers allow eight warps per SM)
-constexpr int kAdjBlock = 32;
-constexpr int kAdjWarpsPerSM = 8;
+// Tile of k_adj_face: kAdjX x kAdjY target cells, the faces after all but the last of them along D (the
+// tile's x for D = x, otherwise its y; the other of the two runs over the first tangential axis).
+constexpr int kAdjX = 32, kAdjY = 8, kAdjThreads = kAdjX * kAdjY;
+// two-float entries in shared memory: 25 + 25 gradients and the five right-biased values of each cell
+constexpr size_t kAdjShared = 55 * kAdjThreads * sizeof(ff);
 
-// One thread marches a segment of faces a+1/2 (a = cfirst .. clast) of one grid line along D; the
-// step to target cell x (x = cfirst .. clast + 1) forms both WENO5 values of x with their gradients
-// from one indicator set (weno5_vjp_cell): the right-biased value at x-1/2, which completes face
-// x-1/2, and the left-biased value at x+1/2, which waits for the next step.  The segment's first
-// cell forms only its left-biased value and the cell after its last face only its right-biased one,
-// so every value is computed once per segment and the result does not depend on the segment length
-// except through these two ends.  Face x-1/2 then takes the reverse HLLC and dissipative flux and
-// writes its contributions to the six stencil cells (and four tangential-gradient cells) to its
-// per-face slots.
+template <int D>
+struct AdjTile {
+  static constexpr int faces = (D == 0 ? kAdjX : kAdjY) - 1;      // along D
+  static constexpr int lines = D == 0 ? kAdjY : kAdjX;            // along A1
+};
+
+// Face a + 1/2 with all terms in FP64
 template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(kAdjBlock) k_adj_face(const double* __restrict__ W,
-                                                  const double* __restrict__ G,
-                                                  const double* __restrict__ mu,
-                                                  double* __restrict__ CW, double* __restrict__ CG,
-                                                  Geo g, Phys ph, int seg) {
+__device__ __forceinline__ void adj_face_fp64(const double* __restrict__ W, const double* __restrict__ G,
+                                              double* __restrict__ CW, double* __restrict__ CG, const Geo& g,
+                                              const Phys& ph, int a, int fcell, const double gF[5]) {
   constexpr int A1 = (D == 0) ? 1 : 0;
   constexpr int A2 = (D == 2) ? 1 : 2;
-  const int n1 = g.n[A1], n2 = g.n[A2], nd = g.n[D];
-  const int nf = nd + 1;                         // faces a + 1/2, a = h - 1 .. h + nd - 1
-  const int nseg = (nf + seg - 1) / seg;
-  const long long total = (long long)n1 * n2 * nseg;
   const int s = stride_of(g, D);
   const int nc = g.ncell;
   const double eps4 = 4.0 * ph.eps;
-  // gradients of the reconstructions: [x & 1] the left-biased value of target cell x (read at the
-  // next step), [2] the right-biased value of the current step
-  __shared__ double sJ[3][25][kAdjBlock];
-  const int tid = threadIdx.x;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    // consecutive threads take consecutive lines (consecutive x for D = y, z)
-    const int i1 = (int)(t % n1);
-    const long long rr = t / n1;
-    const int i2 = (int)(rr % n2);
-    const int sg = (int)(rr / n2);
-    const int cfirst = g.h[D] - 1 + sg * seg;
-    const int clast = g.h[D] - 1 + min((sg + 1) * seg, nf) - 1;
+  double wl[5], wr[5], Jl[5][5], Jr[5][5], q[5][6], un[5], none;
+#pragma unroll 1
+  for (int v = 0; v < 5; ++v) {
+#pragma unroll
+    for (int o = 0; o < 6; ++o) q[v][o] = __ldg(W + v * nc + fcell + (o - 2) * s);
+    weno5_vjp_cell<SCHEME>(q[v], eps4, true, false, wl[v], Jl[v], none, un);
+    weno5_vjp_cell<SCHEME>(q[v] + 1, eps4, false, true, none, un, wr[v], Jr[v]);
+  }
+  double gwl[5], gwr[5];
+  hllc_vjp<D>(wl, wr, ph, gF, gwl, gwr);
+  // slots k = 0 .. 5 are cells a-2 .. a+3; the left value's stencil is a-2 .. a+2, the right value's a-1 .. a+3
+  double gcell[6][kSlots];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    gcell[v][0] = gwl[v] * Jl[v][0];
+#pragma unroll
+    for (int k = 1; k < 5; ++k) gcell[v][k] = fma(gwl[v], Jl[v][k], gwr[v] * Jr[v][k - 1]);
+    gcell[v][5] = gwr[v] * Jr[v][4];
+  }
+#pragma unroll
+  for (int k = 0; k < kSlots; ++k) gcell[5][k] = 0.0;
+  if (VISC) {
+    double vel[3][4], T[4], gd[3][4], gb[3][4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      vel[0][o] = q[1][o + 1];
+      vel[1][o] = q[2][o + 1];
+      vel[2][o] = q[3][o + 1];
+      T[o] = __ldg(W + 5 * nc + fcell + (o - 1) * s);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        gd[b][o] = b == D || b >= g.ndim ? 0.0 : __ldg(G + (D * 3 + b) * nc + fcell + (o - 1) * s);
+        gb[b][o] = b == D || b >= g.ndim ? 0.0 : __ldg(G + (b * 3 + b) * nc + fcell + (o - 1) * s);
+      }
+    }
+    const double gFd[4] = {-gF[1], -gF[2], -gF[3], -gF[4]};
+    double gvel[3][4], gT[4], gGD[3], gGB[3];
+    visc_face_vjp<D>(vel, T, gd, gb, g.ndim, g.mf[D][a], ph, gFd, gvel, gT, gGD, gGB);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      gcell[1][1 + o] += gvel[0][o];
+      gcell[2][1 + o] += gvel[1][o];
+      gcell[3][1 + o] += gvel[2][o];
+      gcell[5][1 + o] += gT[o];
+    }
+    CG[0 * nc + fcell] = gGD[A1];
+    CG[1 * nc + fcell] = gGB[A1];
+    CG[2 * nc + fcell] = gGD[A2];
+    CG[3 * nc + fcell] = gGB[A2];
+  }
+#pragma unroll
+  for (int k = 0; k < kSlots; ++k)
+#pragma unroll
+    for (int v = 0; v < 6; ++v) CW[(k * 6 + v) * nc + fcell] = gcell[v][k];
+}
+
+// The value and the derivative per cell of a 4-cell stencil f[0], f[s], .. (visc_ff's forms)
+__device__ __forceinline__ void adj_stencil(const double* __restrict__ f, int s, ff& val, ff& der) {
+  const double f0 = __ldg(f - s), f1 = __ldg(f), f2 = __ldg(f + s), f3 = __ldg(f + 2 * s);
+  const ff dl = ff_of(f1 - f0), dc = ff_of(f2 - f1), dr = ff_of(f3 - f2);
+  const ff k24 = ff_const(1.0 / 24.0);
+  val = ff_of(f1) + wa(ff_scale(dc, 0.5f), ff_scale(dl - dr, 0.0625f));
+  der = dc - wm(k24, (dr - dc) - (dc - dl));
+}
+
+// The value of a 4-cell stencil f[-s] .. f[2 s]
+__device__ __forceinline__ ff adj_mean(const double* __restrict__ f, int s) {
+  const ff a = ff_of(__ldg(f - s)), b = ff_of(__ldg(f)), c = ff_of(__ldg(f + s)), d = ff_of(__ldg(f + 2 * s));
+  return ff_scale(wm(9.0f, b + c) - (a + d), 0.0625f);
+}
+
+// The share of stencil cell k = 1 .. 4 in the cotangents a of a face value and 24 b of its derivative
+__device__ __forceinline__ ff adj_spread(int k, ff a, ff b) {
+  return wa(wm(k == 1 || k == 4 ? -0.0625f : 0.5625f, a), wm(k == 1 ? 1.0f : k == 2 ? -27.0f : k == 3 ? 27.0f : -1.0f, b));
+}
+
+// A thread forms both WENO5 values of its cell with their gradients from one indicator set
+// (weno5_cell_ff) and leaves them in shared memory; after the barrier it takes the face between its
+// cell and the next along D: the face-flux cotangent, the reverse HLLC and dissipative flux, and the
+// contributions to the six stencil cells (and four tangential-gradient cells), which go to the face's
+// slots.  The face cotangents are scaled to one by a power of two and the slots scaled back, so that
+// no cotangent leaves the FP32 range.  Faces and cells outside the limits of the two-float forms take
+// adj_face_fp64.
+//
+// What bounds it: FP32 issue (58 % of the slots; FP64 pipe 13 %).  On a 512 x 128 layer a launch takes
+// 41 us on either axis; with all terms in FP64 it was bound by the FP64 pipe (82 % busy) at 184 to 187 us.
+// Of the tile the shared memory (110 KB, two blocks an SM) is the limit.  The loops over the five
+// primitives are not unrolled: unrolled, the code overflows the instruction caches (67 us a launch).
+template <int D, int SCHEME, bool VISC>
+__global__ void __launch_bounds__(kAdjThreads, 2)
+k_adj_face(const double* __restrict__ W, const double* __restrict__ G, const double* __restrict__ mu,
+           double* __restrict__ CW, double* __restrict__ CG, Geo g, Phys ph, int tiles_d, int tiles_1, long long tiles) {
+  constexpr int A1 = (D == 0) ? 1 : 0;
+  constexpr int A2 = (D == 2) ? 1 : 2;
+  constexpr int FD = AdjTile<D>::faces, L1 = AdjTile<D>::lines;
+  extern __shared__ ff sh[];
+  ff* const sJu = sh;                             // [25][kAdjThreads]
+  ff* const sJd = sh + 25 * kAdjThreads;
+  ff* const sWr = sh + 50 * kAdjThreads;          // right-biased values less the cell's; a NaN marks a cell that needs FP64
+  const int s = stride_of(g, D);
+  const int nc = g.ncell, nd = g.n[D];
+  const int tid = threadIdx.x, tx = tid % kAdjX, ty = tid / kAdjX;
+  const int along = D == 0 ? tx : ty, line = D == 0 ? ty : tx;
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const long long rr = t / tiles_1;
+    const int i1 = (int)(t % tiles_1) * L1 + line;
+    const int i2 = (int)(rr / tiles_d);
+    const int a = g.h[D] - 1 + (int)(rr % tiles_d) * FD + along;  // the thread's cell and face a + 1/2
+    const bool in = i1 < g.n[A1] && a <= g.h[D] + nd;
     int c[3];
     c[A1] = i1 + g.h[A1];
     c[A2] = i2 + g.h[A2];
-    c[D] = cfirst;
-    int cell = c[0] + c[1] * g.sy + c[2] * g.sz;
-    double wl[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int x = cfirst; x <= clast + 1; ++x, cell += s) {
-      const bool up = x <= clast, dn = x > cfirst;
-      double q[5][5];                            // cells x-2 .. x+2
+    c[D] = a;
+    const int cell = c[0] + c[1] * g.sy + c[2] * g.sz;
+    ff wu[5];                                     // left-biased values less the cell's
+    bool ok = true;
+    if (in) {
+#pragma unroll 1
+      for (int v = 0; v < 5; ++v) {
+        const double* q = W + v * nc + cell;
+        const double q2 = __ldg(q);
+        const ff d0 = ff_of(__ldg(q - 2 * s) - q2), d1 = ff_of(__ldg(q - s) - q2);
+        const ff d3 = ff_of(__ldg(q + s) - q2), d4 = ff_of(__ldg(q + 2 * s) - q2);
+        ff up, dn, Ju[5], Jd[5];
+        ok = weno5_cell_ff<SCHEME>(d0, d1, d3, d4, ph.k.re, up, Ju, dn, Jd) && ok;
+        wu[v] = up;
+        sWr[v * kAdjThreads + tid] = dn;
 #pragma unroll
-      for (int v = 0; v < 5; ++v)
-#pragma unroll
-        for (int o = 0; o < 5; ++o) q[v][o] = __ldg(W + v * nc + cell + (o - 2) * s);
-      double wn[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, wr[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int k = 0; k < 5; ++k) {
+          sJu[(v * 5 + k) * kAdjThreads + tid] = Ju[k];
+          sJd[(v * 5 + k) * kAdjThreads + tid] = Jd[k];
+        }
+      }
+      if (!ok) sWr[tid] = ff{s_from(0x7fc00000), 0.0f};
+    }
+    __syncthreads();
+    if (in && along < FD && a < g.h[D] + nd) {
+      // face-flux cotangent: R_a = -(F_{a+1/2} - F_{a-1/2}) / dx_a
+      double gF[5];
+      const bool inL = a >= g.h[D], inR = a + 1 < g.h[D] + nd;
+      const double iL = inL ? g.idx[D][a] : 0.0, iR = inR ? g.idx[D][a + 1] : 0.0;
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        double Ju[5], Jd[5];
-        weno5_vjp_cell<SCHEME>(q[v], eps4, up, dn, wn[v], Ju, wr[v], Jd);
-        if (up) {
-#pragma unroll
-          for (int k = 0; k < 5; ++k) sJ[x & 1][v * 5 + k][tid] = Ju[k];
-        }
-        if (dn) {
-#pragma unroll
-          for (int k = 0; k < 5; ++k) sJ[2][v * 5 + k][tid] = Jd[k];
-        }
+        const double mL = inL ? mu[v * nc + cell] : 0.0;
+        const double mR = inR ? mu[v * nc + cell + s] : 0.0;
+        gF[v] = mR * iR - mL * iL;
       }
-      if (dn) {
-        // face a + 1/2 between cells a = x - 1 and x
-        const int a = x - 1;
-        const int fcell = cell - s;
-        const int af = a - (g.h[D] - 1);
-        // face-flux cotangent: R_a = -(F_{a+1/2} - F_{a-1/2}) / dx_a
-        double gF[5];
-        const bool inL = af > 0, inR = af < nd;
-        const double iL = inL ? g.idx[D][a] : 0.0, iR = inR ? g.idx[D][a + 1] : 0.0;
+      const int ex = cot_exponent(gF);
+      ok = ok && ex < 900;
+      ff gf[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          const double mL = inL ? mu[v * nc + fcell] : 0.0;
-          const double mR = inR ? mu[v * nc + cell] : 0.0;
-          gF[v] = mR * iR - mL * iL;
+      for (int v = 0; v < 5; ++v) gf[v] = ff_of_shifted(gF[v], ex);
+      float bad = 0.0f;
+      ff va[4], vb[4];
+      ff gGD[3], gGB[3];
+      if (VISC) {
+        ff vf[3], dn[3], Tf, dT, fd[3], fb[3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) adj_stencil(W + (1 + b) * nc + cell, s, vf[b], dn[b]);
+        adj_stencil(W + 5 * nc + cell, s, Tf, dT);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          fd[b] = fb[b] = ff{0.0f, 0.0f};
+          if (b == D || b >= g.ndim) continue;
+          fd[b] = adj_mean(G + (D * 3 + b) * nc + cell, s);
+          fb[b] = adj_mean(G + (b * 3 + b) * nc + cell, s);
         }
-        double gwl[5], gwr[5];
-        hllc_vjp<D>(wl, wr, ph, gF, gwl, gwr);
-        // slots k = 0 .. 5 are cells a-2 .. a+3; the left value's stencil is a-2 .. a+2, the
-        // right value's a-1 .. a+3
-        const int pl = (x - 1) & 1;
-        double gcell[6][kSlots];
+        const ff gFd[4] = {-gf[1], -gf[2], -gf[3], -gf[4]};
+        ok = visc_vjp_ff<D>(dn, vf, Tf, dT, ff_of(g.mf[D][a]), fd, fb, g.ndim, ph, gFd, va, vb, gGD, gGB) && ok;
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          gcell[v][0] = gwl[v] * sJ[pl][v * 5][tid];
+        for (int v = 0; v < 4; ++v) bad = s_fma(va[v].h, 0.0f, s_fma(vb[v].h, 0.0f, bad));
+        bad = s_fma(gGD[A1].h, 0.0f, s_fma(gGB[A1].h, 0.0f, s_fma(gGD[A2].h, 0.0f, s_fma(gGB[A2].h, 0.0f, bad))));
+      }
+      const int nb = tid + (D == 0 ? 1 : kAdjX);
+      ff wl[5], J[5], gwl[5], gwr[5];
+      float usig = 0.0f;
 #pragma unroll
-          for (int k = 1; k < 5; ++k)
-            gcell[v][k] = fma(gwl[v], sJ[pl][v * 5 + k][tid], gwr[v] * sJ[2][v * 5 + k - 1][tid]);
-          gcell[v][5] = gwr[v] * sJ[2][v * 5 + 4][tid];
-        }
+      for (int v = 0; v < 5; ++v) {
+        const double qL = __ldg(W + v * nc + cell), qR = __ldg(W + v * nc + cell + s);
+        const ff up = wu[v], dq = sWr[v * kAdjThreads + nb] - up, qc = ff_of(qL);
+        wl[v] = qc + up;
+        J[v] = ff_of(qR - qL) + dq;
+        // rounding of S*: of the normal velocity, and of the pressure jump over rho c
+        if (v == 1 + D) usig = s_add(usig, s_add(fabsf(qc.h), s_add(fabsf(up.h), fabsf(J[v].h))));
+        if (v == 4) usig = s_add(usig, s_mul(s_add(fabsf(up.h), fabsf(J[v].h)), s_rsqrt(s_mul(wl[0].h, wl[4].h))));
+      }
+      ok = hllc_vjp_ff<D>(wl, J, s_mul(usig, 2.3e-13f), ph.k, gf, gwl, gwr) && ok;
 #pragma unroll
-        for (int k = 0; k < kSlots; ++k) gcell[5][k] = 0.0;
+      for (int v = 0; v < 5; ++v) bad = s_fma(gwl[v].h, 0.0f, s_fma(gwr[v].h, 0.0f, bad));
+      if (ok && bad == 0.0f) {
+        const auto put = [&](int k, int v, ff x) { CW[(k * 6 + v) * nc + cell] = shifted(ff_to_double(ff_norm(x)), ex); };
         if (VISC) {
-          double vel[3][4], T[4], gd[3][4], gb[3][4];
+          CG[0 * nc + cell] = shifted(ff_to_double(ff_norm(gGD[A1])), ex);
+          CG[1 * nc + cell] = shifted(ff_to_double(ff_norm(gGB[A1])), ex);
+          CG[2 * nc + cell] = shifted(ff_to_double(ff_norm(gGD[A2])), ex);
+          CG[3 * nc + cell] = shifted(ff_to_double(ff_norm(gGB[A2])), ex);
+        }
+        // slots k = 0 .. 5 are cells a-2 .. a+3; the left value's stencil is a-2 .. a+2, the right
+        // value's a-1 .. a+3; the dissipative flux has a-1 .. a+2
+#pragma unroll 1
+        for (int v = 0; v < 5; ++v) {
+          const ff gl = gwl[v], gr = gwr[v];
+          const ff* ju = sJu + v * 5 * kAdjThreads + tid;
+          const ff* jd = sJd + v * 5 * kAdjThreads + nb;
+          const bool vel = VISC && v > 0 && v < 4;
+          const ff k24 = ff_const(1.0 / 24.0), zero{0.0f, 0.0f};
+          const ff ya = vel ? va[v - 1] : zero, yb = vel ? wm(k24, vb[v - 1]) : zero;
 #pragma unroll
-          for (int o = 0; o < 4; ++o) {
-            vel[0][o] = q[1][o];
-            vel[1][o] = q[2][o];
-            vel[2][o] = q[3][o];
-            T[o] = __ldg(W + 5 * nc + fcell + (o - 1) * s);
+          for (int k = 0; k < kSlots; ++k) {
+            ff x{0.0f, 0.0f};
+            if (k < 5) x = wm(gl, ju[k * kAdjThreads]);
+            if (k > 0) x = wf(gr, jd[(k - 1) * kAdjThreads], x);
+            if (VISC && k > 0 && k < 5) x = wa(x, adj_spread(k, ya, yb));
+            put(k, v, x);
           }
-#pragma unroll
-          for (int b = 0; b < 3; ++b) {
-#pragma unroll
-            for (int o = 0; o < 4; ++o) {
-              gd[b][o] = 0.0;
-              gb[b][o] = 0.0;
-            }
-            if (b == D || b >= g.ndim) continue;
-            const double* pd = G + (D * 3 + b) * nc + fcell;
-            const double* pb = G + (b * 3 + b) * nc + fcell;
-#pragma unroll
-            for (int o = 0; o < 4; ++o) {
-              gd[b][o] = __ldg(pd + (o - 1) * s);
-              gb[b][o] = __ldg(pb + (o - 1) * s);
-            }
-          }
-          const double gFd[4] = {-gF[1], -gF[2], -gF[3], -gF[4]};
-          double gvel[3][4], gT[4], gGD[3], gGB[3];
-          visc_face_vjp<D>(vel, T, gd, gb, g.ndim, g.mf[D][a], ph, gFd, gvel, gT, gGD, gGB);
-#pragma unroll
-          for (int o = 0; o < 4; ++o) {
-            gcell[1][1 + o] += gvel[0][o];
-            gcell[2][1 + o] += gvel[1][o];
-            gcell[3][1 + o] += gvel[2][o];
-            gcell[5][1 + o] += gT[o];
-          }
-          CG[0 * nc + fcell] = gGD[A1];
-          CG[1 * nc + fcell] = gGB[A1];
-          CG[2 * nc + fcell] = gGD[A2];
-          CG[3 * nc + fcell] = gGB[A2];
         }
 #pragma unroll
-        for (int k = 0; k < kSlots; ++k)
-#pragma unroll
-          for (int v = 0; v < 6; ++v) CW[(k * 6 + v) * nc + fcell] = gcell[v][k];
+        for (int k = 0; k < kSlots; ++k) {
+          if (VISC && k > 0 && k < 5) put(k, 5, adj_spread(k, va[3], wm(ff_const(1.0 / 24.0), vb[3])));
+          else CW[(k * 6 + 5) * nc + cell] = 0.0;
+        }
+      } else {
+        adj_face_fp64<D, SCHEME, VISC>(W, G, CW, CG, g, ph, a, cell, gF);
       }
-#pragma unroll
-      for (int v = 0; v < 5; ++v) wl[v] = wn[v];
     }
+    __syncthreads();
   }
 }
 
@@ -533,39 +636,19 @@ __global__ void k_lincomb(double* out, double c0, const double* x0, double c1, c
   }
 }
 
-// Segment length of k_adj_face for lines of nf faces: the one that minimises the modelled time,
-// (waves of resident threads) x (faces per thread) x (FP64 work per face).  A segment of L faces
-// forms 2 + 2 (L - 1) reconstructions' worth of WENO5 work as L + 1 cells (its two ends one value
-// each, the cells between two values from one indicator set, about 1.65 times one value), against
-// 2 L for faces taken one by one; the rest of a face (reverse HLLC, dissipative flux, slots) is
-// about 0.64 of two values.  Resident threads: 8 warps per SM (the kernel's registers).
-int adj_segment(long long lines, int nf) {
-  const long long resident = 152LL * kAdjWarpsPerSM * 32;
-  int best = 1;
-  double best_t = 0.0;
-  for (int L = 1; L <= 16; L *= 2) {
-    const long long threads = lines * ((nf + L - 1) / L);
-    const long long waves = (threads + resident - 1) / resident;
-    const double per_face = 1.28 + (2.0 + 1.65 * (L - 1)) / L;
-    const double t = (double)waves * L * per_face;
-    if (L == 1 || t < best_t) {
-      best = L;
-      best_t = t;
-    }
-  }
-  return best;
-}
-
 template <int D, int SCHEME, bool VISC>
 cudaError_t adj_face_t(const double* W, const double* G, const double* mu, double* CW, double* CG,
                        const Geo& g, const Phys& ph, cudaStream_t st) {
   constexpr int A1 = (D == 0) ? 1 : 0;
   constexpr int A2 = (D == 2) ? 1 : 2;
-  const long long lines = (long long)g.n[A1] * g.n[A2];
-  const int nf = g.n[D] + 1;
-  const int seg = adj_segment(lines, nf);
-  const long long total = lines * ((nf + seg - 1) / seg);
-  (k_adj_face<D, SCHEME, VISC><<<grid_for(total, kAdjBlock), kAdjBlock, 0, st>>>(W, G, mu, CW, CG, g, ph, seg), ++t_launches);
+  const int td = (g.n[D] + 1 + AdjTile<D>::faces - 1) / AdjTile<D>::faces;
+  const int t1 = (g.n[A1] + AdjTile<D>::lines - 1) / AdjTile<D>::lines;
+  const long long tiles = (long long)td * t1 * g.n[A2];
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_adj_face<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjShared);
+  if (e != cudaSuccess) return e;
+  (k_adj_face<D, SCHEME, VISC><<<grid_for(tiles, 1), kAdjThreads, kAdjShared, st>>>(W, G, mu, CW, CG, g, ph, td, t1, tiles),
+   ++t_launches);
   return cudaGetLastError();
 }
 
