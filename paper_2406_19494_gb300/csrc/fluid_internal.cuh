@@ -207,7 +207,8 @@ inline thread_local long long t_launches = 0;
 // next kernel is set up while the last blocks of this one run, and waits (step_wait, the first
 // statement of every kernel launched this way) until this one has finished and its writes are
 // visible.  A launch that follows or precedes anything else on the stream is ordered as usual.  Shock
-// tube of 200 cells, 20 steps of 13 launches: 2.28 -> 1.91 ms (with the CFL reduction as one kernel).
+// tube of 200 cells, 20 steps of 13 launches: 2.28 -> 1.91 ms (with the CFL reduction as one kernel);
+// step adjoint of 96 x 48 and 512 x 128 cells: 427 -> 374 and 600 -> 533 us.
 // The batches' kernels, which fill the GPU, are launched plainly: eight served solves took 8.3 ms so,
 // 9.9 ms with the overlap.
 template <class... P, class... A>

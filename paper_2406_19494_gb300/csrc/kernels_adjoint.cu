@@ -296,6 +296,7 @@ k_adj_face(const double* __restrict__ W, const double* __restrict__ G, const dou
 template <int D, bool VISC>
 __global__ void k_adj_gather(const double* __restrict__ CW, const double* __restrict__ CG,
                              double* __restrict__ gW, double* __restrict__ gG, Geo g) {
+  step_wait();
   constexpr int A1 = (D == 0) ? 1 : 0;
   constexpr int A2 = (D == 2) ? 1 : 2;
   const int n1 = g.n[A1], n2 = g.n[A2], pd = g.p[D];
@@ -361,6 +362,7 @@ __global__ void k_adj_gather(const double* __restrict__ CW, const double* __rest
 
 // reverse of G[c*3+b](y) = ((u_c(y-2b) - u_c(y+2b)) + 8 (u_c(y+b) - u_c(y-b))) / 12 * mc_b(y)
 __global__ void k_adj_grad(const double* __restrict__ gG, double* __restrict__ gW, Geo g) {
+  step_wait();
   const int total = g.ncell;
   for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < total; cell += gridDim.x * blockDim.x) {
     int x[3];
@@ -388,6 +390,7 @@ __global__ void k_adj_grad(const double* __restrict__ gG, double* __restrict__ g
 }
 
 __global__ void k_adj_source(const double* __restrict__ mu, double* __restrict__ gW, Geo g, Phys ph) {
+  step_wait();
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
@@ -414,6 +417,7 @@ __device__ __forceinline__ int bc_src(int kind, int side, int a, int n, int h) {
 template <int A>
 __global__ void k_adj_bc(const double* __restrict__ W, double* __restrict__ gW,
                          double* __restrict__ gvw_col, Geo g, Phys ph, BC bc) {
+  step_wait();
   constexpr int H = FLUID_HALO;
   int lo[3], ext[3];
   for (int b = 0; b < 3; ++b) {
@@ -488,6 +492,7 @@ __global__ void k_adj_bc(const double* __restrict__ W, double* __restrict__ gW,
 
 __global__ void k_adj_prim(const double* __restrict__ U, const double* __restrict__ gW,
                            double* __restrict__ gU, Geo g, Phys ph) {
+  step_wait();
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
@@ -506,6 +511,7 @@ __global__ void k_adj_prim(const double* __restrict__ U, const double* __restric
 __global__ void k_adj_phi(const double* __restrict__ gvw_col, const double* __restrict__ xc,
                           double* __restrict__ gphi, int p_t1, int h_t1, int ext_t2, int begin,
                           int count, double amp, double two_pi_kappa) {
+  step_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
     const int a = h_t1 + begin + i;
     double s = 0.0;
@@ -619,6 +625,7 @@ __global__ void k_wall_loss_grad(const double* __restrict__ U, const double* __r
 // out = c0 x0 + c1 x1 + c2 x2 + c3 x3 on interior cells (x_k may be null when c_k == 0)
 __global__ void k_lincomb(double* out, double c0, const double* x0, double c1, const double* x1,
                           double c2, const double* x2, double c3, const double* x3, Geo g) {
+  step_wait();
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
@@ -647,6 +654,8 @@ cudaError_t adj_face_t(const double* W, const double* G, const double* mu, doubl
   const cudaError_t e =
       cudaFuncSetAttribute(k_adj_face<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjShared);
   if (e != cudaSuccess) return e;
+  // launched plainly: with the others' overlap its blocks gather on the SMs that come free first (653 against
+  // 600 us a step adjoint of 512 x 128)
   (k_adj_face<D, SCHEME, VISC><<<grid_for(tiles, 1), kAdjThreads, kAdjShared, st>>>(W, G, mu, CW, CG, g, ph, td, t1, tiles),
    ++t_launches);
   return cudaGetLastError();
@@ -662,13 +671,13 @@ cudaError_t adj_dir(int D, const double* W, const double* G, const double* mu, d
   const long long tg = ncol * g.p[D];
   if (D == 0) {
     if ((e = adj_face_t<0, SCHEME, VISC>(W, G, mu, CW, CG, g, ph, st)) != cudaSuccess) return e;
-    (k_adj_gather<0, VISC><<<grid_for(tg, 256), 256, 0, st>>>(CW, CG, gW, gG, g), ++t_launches);
+    launch_step(k_adj_gather<0, VISC>, grid_for(tg, 256), 256, 0, st, CW, CG, gW, gG, g);
   } else if (D == 1) {
     if ((e = adj_face_t<1, SCHEME, VISC>(W, G, mu, CW, CG, g, ph, st)) != cudaSuccess) return e;
-    (k_adj_gather<1, VISC><<<grid_for(tg, 256), 256, 0, st>>>(CW, CG, gW, gG, g), ++t_launches);
+    launch_step(k_adj_gather<1, VISC>, grid_for(tg, 256), 256, 0, st, CW, CG, gW, gG, g);
   } else {
     if ((e = adj_face_t<2, SCHEME, VISC>(W, G, mu, CW, CG, g, ph, st)) != cudaSuccess) return e;
-    (k_adj_gather<2, VISC><<<grid_for(tg, 256), 256, 0, st>>>(CW, CG, gW, gG, g), ++t_launches);
+    launch_step(k_adj_gather<2, VISC>, grid_for(tg, 256), 256, 0, st, CW, CG, gW, gG, g);
   }
   return cudaGetLastError();
 }
@@ -690,7 +699,7 @@ cudaError_t launch_adj_faces(const double* W, const double* G, const double* mu,
     if (e != cudaSuccess) return e;
   }
   if (visc) {
-    (k_adj_grad<<<grid_for(g.ncell, 256), 256, 0, st>>>(gG, gW, g), ++t_launches);
+    launch_step(k_adj_grad, grid_for(g.ncell, 256), 256, 0, st, gG, gW, g);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -699,7 +708,7 @@ cudaError_t launch_adj_faces(const double* W, const double* G, const double* mu,
 
 cudaError_t launch_adj_source(const double* mu, double* gW, const Geo& g, const Phys& ph, cudaStream_t st) {
   const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  (k_adj_source<<<grid_for(total, 256), 256, 0, st>>>(mu, gW, g, ph), ++t_launches);
+  launch_step(k_adj_source, grid_for(total, 256), 256, 0, st, mu, gW, g, ph);
   return cudaGetLastError();
 }
 
@@ -710,9 +719,9 @@ cudaError_t launch_adj_bc(const double* W, double* gW, double* gvw_col, const Ge
     for (int b = 0; b < 3; ++b)
       if (b != A) cols *= b < A ? g.p[b] : g.n[b];
     const int grid = grid_for(cols, 128);
-    if (A == 0) (k_adj_bc<0><<<grid, 128, 0, st>>>(W, gW, gvw_col, g, ph, bc), ++t_launches);
-    else if (A == 1) (k_adj_bc<1><<<grid, 128, 0, st>>>(W, gW, gvw_col, g, ph, bc), ++t_launches);
-    else (k_adj_bc<2><<<grid, 128, 0, st>>>(W, gW, gvw_col, g, ph, bc), ++t_launches);
+    if (A == 0) launch_step(k_adj_bc<0>, grid, 128, 0, st, W, gW, gvw_col, g, ph, bc);
+    else if (A == 1) launch_step(k_adj_bc<1>, grid, 128, 0, st, W, gW, gvw_col, g, ph, bc);
+    else launch_step(k_adj_bc<2>, grid, 128, 0, st, W, gW, gvw_col, g, ph, bc);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -722,15 +731,15 @@ cudaError_t launch_adj_bc(const double* W, double* gW, double* gvw_col, const Ge
 cudaError_t launch_adj_prim(const double* U, const double* gW, double* gU, const Geo& g,
                             const Phys& ph, cudaStream_t st) {
   const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  (k_adj_prim<<<grid_for(total, 256), 256, 0, st>>>(U, gW, gU, g, ph), ++t_launches);
+  launch_step(k_adj_prim, grid_for(total, 256), 256, 0, st, U, gW, gU, g, ph);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_phi(const double* gvw_col, const double* xc, double* gphi, int p_t1,
                            int h_t1, int ext_t2, int begin, int count, double amp,
                            double two_pi_kappa, cudaStream_t st) {
-  (k_adj_phi<<<grid_for(count, 128), 128, 0, st>>>(gvw_col, xc, gphi, p_t1, h_t1, ext_t2, begin,
-                                                   count, amp, two_pi_kappa), ++t_launches);
+  launch_step(k_adj_phi, grid_for(count, 128), 128, 0, st, gvw_col, xc, gphi, p_t1, h_t1, ext_t2, begin,
+                                                   count, amp, two_pi_kappa);
   return cudaGetLastError();
 }
 
@@ -775,7 +784,7 @@ cudaError_t launch_lincomb(double* out, double c0, const double* x0, double c1, 
                            double c2, const double* x2, double c3, const double* x3, const Geo& g,
                            cudaStream_t st) {
   const long long total = (long long)g.n[0] * g.n[1] * g.n[2];
-  (k_lincomb<<<grid_for(total, 256), 256, 0, st>>>(out, c0, x0, c1, x1, c2, x2, c3, x3, g), ++t_launches);
+  launch_step(k_lincomb, grid_for(total, 256), 256, 0, st, out, c0, x0, c1, x1, c2, x2, c3, x3, g);
   return cudaGetLastError();
 }
 
