@@ -8,12 +8,10 @@ sqrt and pow count one each), stored per workload and phase in profiles/oracle_o
 (3-D WENO5-JS / WENO5-Z with power-law or Sutherland viscosity or none, and TENO6-A with sixth-order
 dissipative fluxes) and fall back to the hand count of this module's table otherwise.
 
-The executed work of the kernels (FP64 instructions counted by ncu on the 64^3 Taylor-Green and
-96 x 64 x 64 channel workloads: flops = 2 DFMA + DADD + DMUL) is kept beside it in EXECUTED.  The
-kernels share WENO5 indicator sets between neighbouring faces, so they execute fewer flops than
-the definition needs; TENO6-A's definition as the oracle writes it evaluates its smoothness
-measures as full quadratic forms (each symmetric pair twice), which no implementation does, so for
-that kernel the executed count is the meaningful one.
+The executed FP64 work of the kernels (FP64 instructions counted by ncu on the 128^3 Taylor-Green and
+96 x 64 x 64 channel workloads: flops = 2 DFMA + DADD + DMUL) is kept beside it in EXECUTED.  The kernels
+form the terms that are small against the state in two-float FP32 arithmetic, so they execute far
+fewer FP64 flops than the definition counts, and the remaining ones are not the definition's.
 
 Hand counts (the fallback):
 
@@ -36,7 +34,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 COUNTS = os.path.join(ROOT, "profiles", "oracle_op_counts.json")
 
 # executed FP64 flops per cell and axis (ncu op counters, 2 DFMA + DADD + DMUL) of the face kernels
-EXECUTED = {"k_face": 741, "k_face_teno": 1561}
+EXECUTED = {"k_face": 69, "k_face_teno": 205}
 
 WENO = {"z": 73, "js": 69}
 TENO = 165
@@ -126,14 +124,12 @@ def cell_update_bytes(nvar=5, word=8):
 
 
 # ---- mixed FP32-flux / FP64-state face kernel (FLUID_PREC_MIXED) ------------------------------
-# FP64 per cell and axis: the cell-centre Euler flux from the primitives and the stored
-# H = E + p (rho u_n 1, adding the increment to the mass flux 1, three momentum FMAs 6, the
-# pressure 1, the energy FMA 2) and the flux difference with its scaling and accumulation (15).
-# The cell differences come from the exact FP32 split of the primitives and cost no FP64 work.
+# FP64 per cell and axis: the flux difference with its scaling and accumulation (15); the cell's Euler flux
+# is assembled from the primitives' FP32 pairs and widened, without FP64 arithmetic.
 # FP32: the WENO5 reconstructions, the HLLC increment in jump form (about 150) and the
 # dissipative flux (90).
 def mixed_cell_axis_flops64():
-    return 1 + 1 + 6 + 1 + 2 + 15
+    return 15
 
 
 def mixed_cell_axis_flops32(weno="z", visc="power"):
@@ -141,7 +137,6 @@ def mixed_cell_axis_flops32(weno="z", visc="power"):
 
 
 def mixed_face_bytes():
-    """Compulsory bytes of one face-kernel launch per cell: FP64 primitives and H 6 x 8 read, the
-    FP32 (hi, lo) split of 6 primitives 12 x 4 read, FP32 tangential gradients 4 x 4 read, R read
-    and written 2 x 40."""
-    return 48 + 48 + 16 + 80
+    """Compulsory bytes of one face-kernel launch per cell: the FP32 (hi, lo) pairs of 6 primitives
+    12 x 4 read, FP32 tangential gradients 4 x 4 read, R read and written 2 x 40."""
+    return 48 + 16 + 80

@@ -476,8 +476,21 @@ __device__ __forceinline__ void k_face_mixed_body(const float* __restrict__ W32,
   if (STAGE && bad) atomicOr(&so->ctl->flags, FLAG_NONFINITE);
 }
 
+template <int SCHEME, bool VISC>
+__global__ void __launch_bounds__(MixedShape<0>::threads, MixedShape<0>::blocks) k_face_mixed_x(
+    const float* __restrict__ W32, const float* __restrict__ G32, double* __restrict__ R,
+    const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf) {
+  step_wait();
+  extern __shared__ __align__(16) unsigned char raw[];
+  const int cols = tile_cols<0, MixedShape<0>>(g);
+  k_face_mixed_body<0, SCHEME, VISC, false>(W32, G32, R, g, ph, pf,
+                                            *reinterpret_cast<MixedShared<MixedShape<0>::threads>*>(raw),
+                                            blockIdx.x % cols, blockIdx.x / cols, nullptr);
+}
+
+// the tangential axes
 template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed(
+__global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed_t(
     const float* __restrict__ W32, const float* __restrict__ G32, double* __restrict__ R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf) {
   step_wait();
@@ -490,7 +503,7 @@ __global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks)
 
 // the last axis's kernel with the stage fused (StageOut): R is read, not written
 template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed_stage(
+__global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed_ts(
     const float* __restrict__ W32, const float* __restrict__ G32, const double* __restrict__ R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf, const __grid_constant__ StageOut so) {
   step_wait();
@@ -652,13 +665,17 @@ cudaError_t launch_t(const float* W32, const float* G32, double* R, const Geo& g
   // a tile may need more than the default 48 KB of dynamic shared memory (the attribute is per device)
   cudaError_t e;
   if (so) {
-    e = cudaFuncSetAttribute(k_face_mixed_stage<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_face_mixed_ts<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    launch_step(k_face_mixed_stage<D, SCHEME, VISC>, grid, n, smem, st, W32, G32, R, g, ph, pf, *so);
+    launch_step(k_face_mixed_ts<D, SCHEME, VISC>, grid, n, smem, st, W32, G32, R, g, ph, pf, *so);
   } else {
-    e = cudaFuncSetAttribute(k_face_mixed<D, SCHEME, VISC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr auto kernel = [] {
+      if constexpr (D == 0) return &k_face_mixed_x<SCHEME, VISC>;
+      else return &k_face_mixed_t<D, SCHEME, VISC>;
+    }();
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    launch_step(k_face_mixed<D, SCHEME, VISC>, grid, n, smem, st, W32, G32, R, g, ph, pf);
+    launch_step(kernel, grid, n, smem, st, W32, G32, R, g, ph, pf);
   }
   return cudaGetLastError();
 }
