@@ -169,7 +169,14 @@ FL_HD bool hllc_vjp_ff(const ff wl[5], const ff J[5], float usig, const PhysFF& 
   const ff Ss = unL + sig;
   bool ok = fminf(fminf(rL.h, rR.h), fminf(pL.h, pR.h)) > 1e-9f && fmaxf(fmaxf(rL.h, rR.h), fmaxf(pL.h, pR.h)) < 1e12f &&
             fmaxf(q2L.h, q2R.h) < 1e24f;
-  ok = ok && !(fabsf(ff_float(Ss)) < usig);
+  // at S* = 0 the two star fluxes agree, and their derivatives differ by rho*_K, the tangential velocities
+  // and the energy that follows from them
+  if (fabsf(ff_float(Ss)) < usig) {
+    const ff xL = mL * SR, xR = mR * SL;
+    const float ut = s_mul(ct.h, 2.3e-13f);
+    ok = ok && fabsf(ff_float(xL - xR)) <= s_mul(fabsf(xL.h), 2.3e-13f) && (D == 0 || fabsf(J[1].h) <= ut) &&
+         (D == 1 || fabsf(J[2].h) <= ut) && (D == 2 || fabsf(J[3].h) <= ut);
+  }
   if (fminf(fabsf(ff_float(SL)), fabsf(ff_float(SR))) < s_mul(ct.h, 2.3e-13f))
     ok = ok && fabsf(J[0].h) <= s_mul(rL.h, 1e-13f) && fmaxf(fmaxf(fabsf(J[1].h), fabsf(J[2].h)), fabsf(J[3].h)) <= s_mul(ct.h, 1e-13f) &&
          fabsf(J[4].h) <= s_mul(pL.h, 1e-13f);
