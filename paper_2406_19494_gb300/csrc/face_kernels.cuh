@@ -433,6 +433,14 @@ struct TileShape {
   static constexpr int blocks = 24 * 32 / threads;
 };
 
+// Tiles of a quarter of the threads along y and z, for grids that leave SMs without a tile of the shape above
+// (a tile's FP64 instructions pass through one SM's pipe): vortex 64 x 64, three steps 1.02 -> 0.96 ms;
+// right-hand side of a box of 24 x 30 x 20 cells in FP64 throughout 0.31 -> 0.28 ms.  Along x, 32
+// threads took longer than 128 (shock tube 1.35 -> 1.59 ms: fewer threads share the FP64 faces).
+struct SmallTile {
+  static constexpr int TX = 2, TD = 32, threads = TX * TD, step = TD - 5, blocks = 24 * 32 / threads;
+};
+
 template <int N>
 struct TileShared {
   double d[5][N];          // q_{j+1} - q_j
@@ -486,15 +494,15 @@ __device__ __forceinline__ TileCell tile_cell(const Geo& g, int col, long long t
   return r;
 }
 
-template <int D, int SCHEME, bool VISC>
+template <int D, int SCHEME, bool VISC, class S = TileShape<D>>
 __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, const double* __restrict__ G,
                                                  double* __restrict__ R, const Geo& g, const Phys& ph,
-                                                 TileShared<TileShape<D>::threads>& sh,
+                                                 TileShared<S::threads>& sh,
                                                  int col, long long tile) {
-  constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD;
+  constexpr int TX = S::TX, TD = S::TD;
   const int t = threadIdx.x, row = t / TX, nc = g.ncell;
   const int s = D == 0 ? 1 : (D == 1 ? g.sy : g.sz);
-  const TileCell tc = tile_cell<D>(g, col, tile);
+  const TileCell tc = tile_cell<D, S>(g, col, tile);
   const bool live = tc.live, pair = tc.pair;
   const int i = tc.i, cell = tc.cell;
 #pragma unroll
@@ -582,7 +590,7 @@ __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, c
   // each.  (Left to their own lanes they held up every warp that had one: shock tube 26 us a launch.)
   const int ndef = sh.ndef;
   if (ndef > 0) {
-    constexpr int N = TileShape<D>::threads;
+    constexpr int N = S::threads;
     sh.sc[t].r = __int_as_float(cell);                     // the scales are done with
     __syncthreads();
     double* wl = &sh.d[0][0];                              // values of (primitive, face), left then right

@@ -8,6 +8,9 @@ namespace fl {
 
 namespace {
 
+// grids of at most this many tiles (one per SM) take the small ones along y and z
+constexpr long long kSmallTiles = 152;
+
 template <int D, int SCHEME, bool VISC>
 __global__ void __launch_bounds__(128) k_face(const double* __restrict__ W, const double* __restrict__ G,
                                               double* __restrict__ R, double* __restrict__ FB,
@@ -17,28 +20,29 @@ __global__ void __launch_bounds__(128) k_face(const double* __restrict__ W, cons
   k_face_body<D, SCHEME, VISC>(W, G, R, FB, g, ph, seg, blockIdx, gridDim);
 }
 
-template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(TileShape<D>::threads, TileShape<D>::blocks) k_face_tile(
+template <int D, int SCHEME, bool VISC, class S = TileShape<D>>
+__global__ void __launch_bounds__(S::threads, S::blocks) k_face_tile(
     const double* __restrict__ W, const double* __restrict__ G, double* __restrict__ R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph) {
   step_wait();
   extern __shared__ __align__(16) unsigned char raw[];
-  const int cols = tile_cols<D>(g);                        // neighbouring blocks: neighbouring columns
-  k_face_tile_body<D, SCHEME, VISC>(W, G, R, g, ph,
-                                    *reinterpret_cast<TileShared<TileShape<D>::threads>*>(raw),
-                                    blockIdx.x % cols, blockIdx.x / cols);
+  const int cols = tile_cols<D, S>(g);                     // neighbouring blocks: neighbouring columns
+  k_face_tile_body<D, SCHEME, VISC, S>(W, G, R, g, ph, *reinterpret_cast<TileShared<S::threads>*>(raw),
+                                       blockIdx.x % cols, blockIdx.x / cols);
 }
 
-template <int D, int SCHEME, bool VISC>
+template <int D, int SCHEME, bool VISC, class S = TileShape<D>>
 cudaError_t launch_tile(const double* W, const double* G, double* R, const Geo& g, const Phys& ph,
                         cudaStream_t st) {
-  constexpr int n = TileShape<D>::threads;
+  constexpr int n = S::threads;
   constexpr size_t smem = sizeof(TileShared<n>);
-  const cudaError_t e = cudaFuncSetAttribute(k_face_tile<D, SCHEME, VISC>,
+  const long long tiles = tile_rows<D, S>(g) * tile_cols<D, S>(g);
+  if constexpr (D > 0 && n == TileShape<D>::threads)
+    if (tiles <= kSmallTiles) return launch_tile<D, SCHEME, VISC, SmallTile>(W, G, R, g, ph, st);
+  const cudaError_t e = cudaFuncSetAttribute(k_face_tile<D, SCHEME, VISC, S>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)(tile_rows<D>(g) * tile_cols<D>(g));
-  launch_step(k_face_tile<D, SCHEME, VISC>, grid, n, smem, st, W, G, R, g, ph);
+  launch_step(k_face_tile<D, SCHEME, VISC, S>, (unsigned)tiles, n, smem, st, W, G, R, g, ph);
   return cudaGetLastError();
 }
 
