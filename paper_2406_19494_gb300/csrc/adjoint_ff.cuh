@@ -362,19 +362,25 @@ FL_HD bool visc_vjp_ff(const ff dn[3], const ff vf[3], ff Tf, ff dTc, ff mf, con
   return true;
 }
 
-// x 2^-k and x 2^k for face cotangents: the exponent moved by integer operations (k from cot_exponent)
+// x 2^-k and x 2^k for face cotangents: the exponent moved by integer operations, k = cot_exponent of the
+// face's five, 0 where all of them are zero.  A zero or subnormal x gives a zero pair: its exponent field is
+// not the exponent of a leading one, and moved it would read as 2^(-k-1023) (for k = -1023 as 1).
 FL_HD int cot_exponent(const double x[5]) {
-  int e = 0;
+  int e = 0, any = 0;
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     const int t = d_hi(x[v]) & 0x7fffffff;
     e = t > e ? t : e;
+    any |= t | d_lo(x[v]);
   }
-  return (e >> 20) - 1023;
+  return any ? (e >> 20) - 1023 : 0;
 }
+// Cotangents that the scaling serves: above 2^-912 a subnormal component is below 2^-110 of the largest,
+// and below 2^880 no two-float slot (under 2^128) passes the largest FP64 exponent on its way back
+FL_HD bool cot_in_range(int k) { return k > -912 && k < 880; }
 FL_HD ff ff_of_shifted(double x, int k) {
   const int hi = d_hi(x), e = (hi & 0x7ff00000) - (k << 20);
-  return e > 0x39000000 ? ff_of(d_from(hi - (k << 20), d_lo(x))) : ff{0.0f, 0.0f};
+  return (hi & 0x7ff00000) && e > 0x39000000 ? ff_of(d_from(hi - (k << 20), d_lo(x))) : ff{0.0f, 0.0f};
 }
 FL_HD double shifted(double x, int k) {
   const int hi = d_hi(x), e = (hi & 0x7ff00000) + (k << 20);

@@ -211,7 +211,7 @@ k_adj_face(const double* __restrict__ W, const double* __restrict__ G, const dou
         gF[v] = mR * iR - mL * iL;
       }
       const int ex = cot_exponent(gF);
-      ok = ok && ex < 900;
+      ok = ok && cot_in_range(ex);
       ff gf[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) gf[v] = ff_of_shifted(gF[v], ex);
