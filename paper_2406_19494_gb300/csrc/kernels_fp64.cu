@@ -539,7 +539,8 @@ __device__ __forceinline__ double cell_rate(const double* __restrict__ W, const 
 }
 
 // The same in FP32, within 1e-4 of it (the power law's estimate is its least exact part); infinite
-// where a value leaves [1e-30, 1e30]
+// where a value leaves [1e-30, 1e30] or the square of the sound speed [1e-37, 1e37] (an infinity or a
+// zero there would become a NaN, which fmaxf drops)
 __device__ __forceinline__ float cell_rate32(const double* __restrict__ W, const Geo& g, const Phys& ph, int t) {
   const int i = t % g.n[0];
   const int r = t / g.n[0];
@@ -550,6 +551,7 @@ __device__ __forceinline__ float cell_rate32(const double* __restrict__ W, const
   const float rho = ff_of(W[c]).h, p = ff_of(W[4 * nc + c]).h;
   bool ok = rho >= 1e-30f && rho <= 1e30f && p >= 1e-30f && p <= 1e30f;
   const float irho = s_rcp(rho), c2 = ph.k.gamma.h * (p * irho);
+  ok = ok && c2 >= 1e-37f && c2 <= 1e37f;
   const float cs = c2 * s_rsqrt(c2);
   float knu = 0.0f, best = 0.0f;
   if (ph.visc != FLUID_VISC_NONE) {
