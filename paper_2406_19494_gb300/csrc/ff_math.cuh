@@ -136,10 +136,11 @@ FL_HD ff ff_sqrt(ff a) {
 
 // x = h + l (1 + 2^-48): the leading 24 bits exact, the other 29 rounded to FP32.  |x| < 2^-126
 // gives 0 or a subnormal number; |x| >= 2^127 or a non-finite x a number near 2^127, which no limit of
-// the ff path admits.
+// the ff path admits.  P: the same of x 2^P, at no more operations.
+template <int P = 0>
 FL_HD ff ff_of(double x) {
   const int hw = d_hi(x), lw = d_lo(x);
-  int t = (hw & 0x7fffffff) - ((1023 - 127) << 20);             // exponent rebiased to FP32
+  int t = (hw & 0x7fffffff) - ((1023 - 127 - P) << 20);             // exponent rebiased to FP32
   t = t < 0 ? 0 : (t > 0x0fefffff ? 0x0fefffff : t);
   const int h = (hw & (int)0x80000000u) | (t << 3) | (int)((unsigned)lw >> 29);
   // the low 29 fraction bits in units of 2^-52 of h's binade

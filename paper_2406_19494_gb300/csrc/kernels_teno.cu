@@ -105,12 +105,13 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
       const double Tm = sh.T[v][t - TX], T0 = sh.T[v][t], T1 = sh.T[v][t + TX], Tp = sh.T[v][t + 2 * TX];
       const int lev = min(min(sh.lev[v][t - TX], sh.lev[v][t]), min(sh.lev[v][t + TX], sh.lev[v][t + 2 * TX]));
       const float ct = lev >= 3 ? 1e-10f : (lev == 2 ? 1e-9f : (lev == 1 ? 1e-8f : 1e-7f));
-      const ff fm = ff_of(Tm), f0 = ff_of(T0), f1 = ff_of(T1), fp = ff_of(Tp);
+      constexpr int P = teno::kMaskScale;
+      const ff fm = ff_of<P>(Tm), f0 = ff_of<P>(T0), f1 = ff_of<P>(T1), fp = ff_of<P>(Tp);
       const float Vm = s_add(s_sub(f0.h, fm.h), s_sub(f0.l, fm.l)), V = s_add(s_sub(f1.h, f0.h), s_sub(f1.l, f0.l));
-      const float Vp = s_add(s_sub(fp.h, f1.h), s_sub(fp.l, f1.l)), Df = ff_of(d[v]).h;
+      const float Vp = s_add(s_sub(fp.h, f1.h), s_sub(fp.l, f1.l)), Df = ff_of<P>(d[v]).h;
       bool kl, kr;
-      const int mL = teno::keep_mask32(Df, f0.h, f1.h, fm.h, Vm, V, Vp, ct, kl);
-      const int mR = teno::keep_mask32(-Df, f1.h, f0.h, fp.h, -Vp, -V, -Vm, ct, kr);
+      const int mL = teno::keep_mask32_scaled(Df, f0.h, f1.h, fm.h, Vm, V, Vp, ct, kl);
+      const int mR = teno::keep_mask32_scaled(-Df, f1.h, f0.h, fp.h, -Vp, -V, -Vm, ct, kr);
       if (kl && kr) {
         cL[v] = fma(sh.alpha[0][mL], Tm, fma(sh.alpha[1][mL], T0, fma(sh.alpha[2][mL], T1, sh.alpha[3][mL] * Tp)));
         cR[v] = fma(sh.alpha[0][mR], Tp, fma(sh.alpha[1][mR], T1, fma(sh.alpha[2][mR], T0, sh.alpha[3][mR] * Tm)));

@@ -184,10 +184,22 @@ FL_HD int sensor_level32(float dm, float dp, bool& clear) {
 //   beta3 = D^2 - D T1 + 4/3 T1^2 + 2/3 D Vp - 5/2 T1 Vp + 547/240 Vp^2,
 //   6 tau6 = 2/5 D (F1 - F0) + V (481/120 V - 3379/5040 F0 - 16823/5040 F1) - T0 (46/15 F0 + 1/5 F1)
 //            + F0 (27211/2240 F0 - 12281/1008 F1) + 139633/20160 F1^2, F0 = V - Vm, F1 = Vp - V.
-// clear: the error of tau (E, twice the largest error found over 5e6 random windows) and of the measures
-// (2^-19 of themselves) cannot turn a decision.
-FL_HD int keep_mask32(float D, float T0, float T1, float Tm, float Vm, float V, float Vp, float ct, bool& clear) {
-  const float k = 13.0f / 12.0f, tiny = 7.5e-37f;
+// clear: no rounding of this function can turn a decision.  The bounds, with u = 2^-24, vm the largest of
+// |Vm|, |V|, |Vp|, and inputs within 2 u of themselves (D, T: cut to 24 bits) or of vm (V), summed over the
+// operations as written:
+//   tau      (21 |D| + 68 |T0| + 1470 vm) vm u, below E (168 u for each and 1680 for vm)
+//   measures 17 u of beta0 and beta1 and 73 u of beta3 (positive definite forms, the sum of whose terms is
+//            at most 7.8 times their value); beta2, whose d cancels next to a steeper cell,
+//            15 u + 4 u (|D| + |T0|) / sqrt(beta2)
+//   gamma    6.4 times the relative errors of tau and of its measure, and 50 u: below the margin's half
+//            of 14 E / tau, and its 6e-5 (1000 u) and its beta2 term
+// Where the third differences are below 1e-5 of |D| + |T0| + |T1|, their own rounding counts, but then
+// no tau / beta exceeds 1e-3.  The window comes times 2^16, so that epsilon (times 2^32) and the squares
+// beside it stay normal numbers; a quotient tau / beta beyond the FP32 range ends as a NaN, which is not
+// clear.
+constexpr int kMaskScale = 16;   // log2 of the window's factor
+FL_HD int keep_mask32_scaled(float D, float T0, float T1, float Tm, float Vm, float V, float Vp, float ct, bool& clear) {
+  const float k = 13.0f / 12.0f, eps6 = (float)(6.0 * kEps * (double)(1ull << 2 * kMaskScale));
   const float s0 = s_fma(-0.5f, T0, D), s1 = s_fma(-0.5f, T1, D), s2 = s_fma(0.5f, Tm, s_sub(D, T0));
   const float b0 = s_fma(k * T0, T0, s_mul(s0, s0)), b1 = s_fma(k * T1, T1, s_mul(s1, s1));
   const float b2 = s_fma(k * Tm, Tm, s_mul(s2, s2));
@@ -201,14 +213,14 @@ FL_HD int keep_mask32(float D, float T0, float T1, float Tm, float Vm, float V, 
   t = s_fma((139633.0f / 20160.0f) * F1, F1, t);
   const float tau = fabsf(t);
   const float vm = fmaxf(fmaxf(fabsf(Vm), fabsf(V)), fabsf(Vp));
-  const float E = 8e-6f * vm * (fabsf(D) + fabsf(T0) + fabsf(T1) + 10.0f * vm);
-  const float i0 = s_rcp(s_fma(6.0f, b0, tiny)), i1 = s_rcp(s_fma(6.0f, b1, tiny));
-  const float i2 = s_rcp(s_fma(6.0f, b2, tiny)), i3 = s_rcp(s_fma(6.0f, b3, tiny));
+  const float E = 1e-5f * vm * (fabsf(D) + fabsf(T0) + fabsf(T1) + 10.0f * vm);
+  const float i0 = s_rcp(s_fma(6.0f, b0, eps6)), i1 = s_rcp(s_fma(6.0f, b1, eps6));
+  const float i2 = s_rcp(s_fma(6.0f, b2, eps6)), i3 = s_rcp(s_fma(6.0f, b3, eps6));
   const float im = fmaxf(fmaxf(i0, i1), fmaxf(i2, i3));
   // no gamma ratio below (1 / 10)^6 / 4, above every cut-off: all kept
   clear = true;
   if ((tau + E) * im < 9.0f) return 15;
-  const float margin = 14.0f * E * s_rcp(tau) + 6e-5f;
+  const float margin = 14.0f * E * s_rcp(tau) + 6e-5f + 1.6e-6f * (fabsf(D) + fabsf(T0)) * s_rsqrt(b2 + eps6);
   const float ix = s_rcp(s_fma(tau, im, 1.0f));
   float g[4] = {s_fma(tau, i0, 1.0f) * ix, s_fma(tau, i1, 1.0f) * ix, s_fma(tau, i2, 1.0f) * ix, s_fma(tau, i3, 1.0f) * ix};
 #pragma unroll
@@ -225,6 +237,13 @@ FL_HD int keep_mask32(float D, float T0, float T1, float Tm, float Vm, float V, 
     clear = clear && fabsf(g[j] - thr) > margin * (g[j] + thr);
   }
   return mask;
+}
+
+// the same from the window as it is
+FL_HD int keep_mask32(float D, float T0, float T1, float Tm, float Vm, float V, float Vp, float ct, bool& clear) {
+  const float f = (float)(1 << kMaskScale);
+  return keep_mask32_scaled(s_mul(D, f), s_mul(T0, f), s_mul(T1, f), s_mul(Tm, f), s_mul(Vm, f), s_mul(V, f), s_mul(Vp, f),
+                            ct, clear);
 }
 
 // Six times the correction of a face value, w = q + (3 D + c) / 6, as factors of (T_{a-1}, T_a, T_{a+1},
