@@ -7,12 +7,14 @@
 namespace fl {
 
 // Indicator terms of cell j from D = q_{j+1} - q_j and T = q_{j+1} - 2 q_j + q_{j-1}:
-// 4 (beta + eps) of its three-cell stencil as the left (A), centre (B) and right (C) candidate.
+// 4 (beta + eps) of its three-cell stencil as the left (A), centre (B) and right (C) candidate, all times
+// kIndScale^2 (set_ff has eps4 so), a common factor that the weights do not see.
 FL_HD void cell_terms(ff D, ff T, ff eps4, ff& A, ff& B, ff& C) {
   const ff k133{4.33333349f, (float)(13.0 / 3.0 - (double)4.33333349f)};
-  const ff K = fma_weak(sqr_weak(T), k133, eps4);
-  const ff T2 = ff_twice(T);
-  const ff sB = add_weak(ff_twice(D), -T);
+  const ff Ts = ff_scale(T, kIndScale);
+  const ff K = fma_weak(sqr_weak(Ts), k133, eps4);
+  const ff T2 = ff_twice(Ts);
+  const ff sB = add_weak(ff_scale(D, 2.0f * kIndScale), -Ts);
   const ff sA = add_weak(T2, sB), sC = add_weak(T2, -sB);
   A = fma_weak(sA, sA, K);
   B = fma_weak(sB, sB, K);

@@ -174,16 +174,22 @@ inline void set_power_law(Phys& ph, double e) {
   }
 }
 
+// The factor of the cell differences in the forward faces' indicators: with 2^16 the default epsilon of 1e-40
+// and the squares beside it keep all bits of a pair (4 epsilon becomes 2^-99), and differences up to 2^33
+// stay below the limit of the indicators (cell_values).
+constexpr float kIndScale = 65536.0f;
+
 // The ff constants of Phys (after its other members are set).  The indicators' 4 epsilon is kept at
-// 2^-120 or above, so that its reciprocal stays an FP32 number: smaller values only act where every
-// difference of the stencil is below 2^-60, far under the rounding of the states the ff path takes.
+// 2^-152 or above, so that its reciprocal stays an FP32 number: smaller values only act where every
+// difference of the stencil is below 2^-76, under the rounding of the smallest states the ff path takes
+// (2^-72 at 1.9e-6).
 inline void set_ff(Phys& ph) {
   ph.k.gamma = ff_of(ph.gamma);
   ph.k.gm1 = ff_of(ph.gm1);
   ph.k.igm1 = ff_of(ph.igm1);
   ph.k.gg = ff_of(ph.gamma * ph.igm1);
   ph.k.iR = ff_of(ph.iR);
-  const double e4 = 4.0 * ph.eps;
+  const double e4 = 4.0 * ph.eps * ((double)kIndScale * kIndScale);
   ph.k.eps4 = ff_of(e4 < 7.52316384526264e-37 ? 7.52316384526264e-37 : e4);
   ph.k.mu_ref = ff_of(ph.mu_ref);
   ph.k.mu_TS = ff_of(ph.mu_ref * (ph.T_ref + ph.suth_S));
