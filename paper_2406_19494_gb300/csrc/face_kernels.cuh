@@ -37,7 +37,7 @@ template <int SCHEME>
 __device__ __forceinline__ void values_fp64(const double* __restrict__ f, int s, double eps4, double& wl, double& wr) {
   double q[6];
 #pragma unroll
-  for (int o = 0; o < 6; ++o) q[o] = __ldg(f + (o - 2) * s);
+  for (int o = 0; o < 6; ++o) q[o] = ld(f + (o - 2) * s);
   const double d0 = q[1] - q[0], d1 = q[2] - q[1], d2 = q[3] - q[2], d3 = q[4] - q[3], d4 = q[5] - q[4];
   const double c = 4.0 * k1312;
   const double tm = d1 - d0, t0 = d2 - d1, t1 = d3 - d2, t2 = d4 - d3;
@@ -87,7 +87,7 @@ __device__ __noinline__ Flux5 visc_flux_fp64(const double* __restrict__ W, const
 #pragma unroll
   for (int v = 1; v < 4; ++v)
 #pragma unroll
-    for (int o = 0; o < 6; ++o) q[v][o] = __ldg(W + v * gp->ncell + cell + (o - 2) * s);
+    for (int o = 0; o < 6; ++o) q[v][o] = ld(W + v * gp->ncell + cell + (o - 2) * s);
   Flux5 F;
 #pragma unroll
   for (int v = 0; v < 5; ++v) F.f[v] = 0.0;
@@ -122,9 +122,9 @@ __device__ __forceinline__ ff sixth() { return ff{kSixthH, (float)(1.0 / 6.0 - (
 // (150 (f2 + f3) - 25 (f1 + f4) + 3 (f0 + f5)) / 256
 template <int NP>
 __device__ __forceinline__ ff interp_ff(const double* __restrict__ f, int s) {
-  const ff f0 = ff_of(__ldg(f - s)), f1 = ff_of(__ldg(f)), f2 = ff_of(__ldg(f + s)), f3 = ff_of(__ldg(f + 2 * s));
+  const ff f0 = ff_of(ld(f - s)), f1 = ff_of(ld(f)), f2 = ff_of(ld(f + s)), f3 = ff_of(ld(f + 2 * s));
   if (NP == 4) return ff_scale(mul_weak(add_weak(f1, f2), 9.0f) - add_weak(f0, f3), 0.0625f);
-  const ff e = add_weak(ff_of(__ldg(f - 2 * s)), ff_of(__ldg(f + 3 * s)));
+  const ff e = add_weak(ff_of(ld(f - 2 * s)), ff_of(ld(f + 3 * s)));
   return ff_scale(mul_weak(add_weak(f1, f2), 150.0f) + (mul_weak(e, 3.0f) - mul_weak(add_weak(f0, f3), 25.0f)), 1.0f / 256);
 }
 
@@ -184,7 +184,7 @@ __device__ __forceinline__ bool face_of_terms(const double* __restrict__ W, cons
     small = small && fabsf(J[v].h) <= kFFJump * lim;
     // the mean of the two cells
     const ff Dv = ff_of(d[v]);
-    const ff m = ff_of(__ldg(W + v * g.ncell + cell)) + ff_scale(Dv, 0.5f);
+    const ff m = ff_of(ld(W + v * g.ncell + cell)) + ff_scale(Dv, 0.5f);
     if (VISC && v >= 1 && v <= 3) {
       m3[v - 1] = m;
       dv[v - 1] = Dv - vv[v - 1] * ff{k24H, k24L};
@@ -199,7 +199,7 @@ __device__ __forceinline__ bool face_of_terms(const double* __restrict__ W, cons
     const double three = left ? 3.0 : -3.0;
 #pragma unroll
     for (int v = 0; v < 5; ++v)
-      w[v] = fma(kSixth, fma(three, d[v], ff_to_double(left ? cL[v] : cR[v])), __ldg(W + v * g.ncell + cell + o));
+      w[v] = fma(kSixth, fma(three, d[v], ff_to_double(left ? cL[v] : cR[v])), ld(W + v * g.ncell + cell + o));
     euler_flux<D>(w, ph, F);
   } else {
     Flux5 e;
@@ -211,8 +211,8 @@ __device__ __forceinline__ bool face_of_terms(const double* __restrict__ W, cons
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         const double* f = W + v * g.ncell + cell;
-        l.f[v] = fma(kSixth, fma(3.0, d[v], ff_to_double(cL[v])), __ldg(f));
-        r.f[v] = fma(kSixth, fma(-3.0, d[v], ff_to_double(cR[v])), __ldg(f + s));
+        l.f[v] = fma(kSixth, fma(3.0, d[v], ff_to_double(cL[v])), ld(f));
+        r.f[v] = fma(kSixth, fma(-3.0, d[v], ff_to_double(cR[v])), ld(f + s));
       }
       e = hllc_fp64<D>(l, r, &ph);
     } else {
@@ -273,12 +273,12 @@ __device__ __forceinline__ bool cell_corr(ff e0, ff e1, ff e2, ff T0, ff V0, ff 
 template <int D, int SCHEME, bool VISC>
 __device__ __forceinline__ void march_start(const double* __restrict__ W, int nc, int cell, int s,
                                             const Phys& ph, March& M) {
-  const Scale sc = scale_of(__ldg(W + cell), __ldg(W + 4 * nc + cell), ph);
+  const Scale sc = scale_of(ld(W + cell), ld(W + 4 * nc + cell), ph);
   M.ok = sc.ok;
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     const double* f = W + v * nc + cell;                   // cell a
-    const double q0 = __ldg(f - 2 * s), q1 = __ldg(f - s), q2 = __ldg(f), q3 = __ldg(f + s), q4 = __ldg(f + 2 * s);
+    const double q0 = ld(f - 2 * s), q1 = ld(f - s), q2 = ld(f), q3 = ld(f + s), q4 = ld(f + 2 * s);
     const double d0 = q1 - q0, d1 = q2 - q1, d2 = q3 - q2, d3 = q4 - q3;
     const ff T1 = ff_of(d1 - d0), T2 = ff_of(d2 - d1), T3 = ff_of(d3 - d2);
     ff A1, A2, A3, B2, B3, C3, x, y, cR;
@@ -297,7 +297,7 @@ __device__ __forceinline__ void march_start(const double* __restrict__ W, int nc
   }
   if (VISC) {
     const double* f = W + 5 * nc + cell;
-    const double t0 = __ldg(f - s), t1 = __ldg(f), t2 = __ldg(f + s);
+    const double t0 = ld(f - s), t1 = ld(f), t2 = ld(f + s);
     M.Dm = ff_of(t1 - t0);
     M.D0 = ff_of(t2 - t1);
   }
@@ -309,7 +309,7 @@ __device__ __forceinline__ void march_face(const double* __restrict__ W, const d
                                            int cell, int s, int a, const Geo& g, const Phys& ph, March& M,
                                            double F[5]) {
   const int nc = g.ncell;
-  const Scale sc = scale_of(__ldg(W + cell + s), __ldg(W + 4 * nc + cell + s), ph);
+  const Scale sc = scale_of(ld(W + cell + s), ld(W + 4 * nc + cell + s), ph);
   bool okj = sc.ok;
   double d[5];
   ff cLn[5], cR[5], vv[3], tv[3], dt{0.0f, 0.0f}, tt{0.0f, 0.0f};
@@ -317,7 +317,7 @@ __device__ __forceinline__ void march_face(const double* __restrict__ W, const d
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     const double* f = W + v * nc + cell;
-    const double dp = __ldg(f + 3 * s) - __ldg(f + 2 * s);
+    const double dp = ld(f + 3 * s) - ld(f + 2 * s);
     const ff Tp = ff_of(dp - M.d0[v]);
     ff Ap, Bp, Cp;
     cell_terms(ff_of(dp), Tp, ph.k.eps4, Ap, Bp, Cp);
@@ -339,7 +339,7 @@ __device__ __forceinline__ void march_face(const double* __restrict__ W, const d
   }
   if (VISC) {
     const double* f = W + 5 * nc + cell;
-    const double t1 = __ldg(f + s), t2 = __ldg(f + 2 * s);
+    const double t1 = ld(f + s), t2 = ld(f + 2 * s);
     const ff Dp = ff_of(t2 - t1);
     const ff Ta = M.D0 - M.Dm, Tj = Dp - M.D0;
     dt = M.D0 - (Tj - Ta) * ff{k24H, k24L};
@@ -508,19 +508,19 @@ __device__ __forceinline__ void k_face_tile_body(const double* __restrict__ W, c
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     const double* f = W + v * nc + cell;
-    sh.d[v][t] = pair ? __ldg(f + s) - __ldg(f) : 0.0;
+    sh.d[v][t] = pair ? ld(f + s) - ld(f) : 0.0;
   }
   ff Dt{0.0f, 0.0f};
   double tq = 0.0;
   if (VISC) {
     if (pair) {
-      tq = __ldg(W + 5 * nc + cell + s);
-      Dt = ff_of(tq - __ldg(W + 5 * nc + cell));
+      tq = ld(W + 5 * nc + cell + s);
+      Dt = ff_of(tq - ld(W + 5 * nc + cell));
     }
     sh.Dt[t] = Dt;
   }
   Scale sc{1.0f, 1.0f, 1.0f, false};
-  if (live) sc = scale_of(__ldg(W + cell), __ldg(W + 4 * nc + cell), ph);
+  if (live) sc = scale_of(ld(W + cell), ld(W + 4 * nc + cell), ph);
   if (t == 0) sh.ndef = 0;
   __syncthreads();
 #pragma unroll 1

@@ -12,8 +12,8 @@ namespace {
 constexpr long long kSmallTiles = 152;
 
 template <int D, int SCHEME, bool VISC>
-__global__ void __launch_bounds__(128) k_face(const double* __restrict__ W, const double* __restrict__ G,
-                                              double* __restrict__ R, double* __restrict__ FB,
+__global__ void __launch_bounds__(128) k_face(const double* W, const double* G,
+                                              double* R, double* FB,
                                               const __grid_constant__ Geo g, const __grid_constant__ Phys ph,
                                               int seg) {
   step_wait();
@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(128) k_face(const double* __restrict__ W, cons
 
 template <int D, int SCHEME, bool VISC, class S = TileShape<D>>
 __global__ void __launch_bounds__(S::threads, S::blocks) k_face_tile(
-    const double* __restrict__ W, const double* __restrict__ G, double* __restrict__ R,
+    const double* W, const double* G, double* R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph) {
   step_wait();
   extern __shared__ __align__(16) unsigned char raw[];

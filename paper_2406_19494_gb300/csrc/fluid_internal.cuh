@@ -71,6 +71,12 @@ struct Ctl {
   unsigned ticket;     // blocks of the current CFL reduction that have finished
 };
 
+// a plain load, also in kernels that begin before the writer of *p has ended (launch_step)
+template <class T>
+__device__ __forceinline__ T ld(const T* p) {
+  return *p;
+}
+
 __device__ __forceinline__ bool finite_bits(double x) {
   return ((__double2hiint(x) >> 20) & 0x7ff) != 0x7ff;
 }
@@ -215,6 +221,11 @@ inline thread_local long long t_launches = 0;
 // visible.  A launch that follows or precedes anything else on the stream is ordered as usual.  Shock
 // tube of 200 cells, 20 steps of 13 launches: 2.28 -> 1.91 ms (with the CFL reduction as one kernel);
 // step adjoint of 96 x 48 and 512 x 128 cells: 427 -> 374 and 600 -> 533 us.
+// Such a kernel begins before the kernel that writes its input has ended.  The read-only load path (__ldg, or
+// what the compiler makes of a const __restrict__ kernel parameter) is defined only for data that no one
+// writes during the kernel's lifetime, and the compiler may move loads through a __restrict__ parameter ahead of
+// the wait.  So the pointer parameters of these kernels are not __restrict__, and what another kernel
+// wrote is read by plain loads (ld); only what the set-up wrote once (metrics) may take __ldg.
 // The batches' kernels, which fill the GPU, are launched plainly: eight served solves took 8.3 ms so,
 // 9.9 ms with the overlap.
 template <class... P, class... A>

@@ -288,7 +288,7 @@ __device__ __forceinline__ void add_visc_face(const double* __restrict__ W, cons
     vel[0][o] = q[1][o0 + o];
     vel[1][o] = q[2][o0 + o];
     vel[2][o] = q[3][o0 + o];
-    T[o] = __ldg(W + 5 * nc + cell + (o + o0 - 2) * s);
+    T[o] = ld(W + 5 * nc + cell + (o + o0 - 2) * s);
   }
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
@@ -297,8 +297,8 @@ __device__ __forceinline__ void add_visc_face(const double* __restrict__ W, cons
     const double* pb = G + (b * 3 + b) * nc + cell;   // d u_b / d x_b
 #pragma unroll
     for (int o = 0; o < NP; ++o) {
-      gd[b][o] = __ldg(pd + (o + o0 - 2) * s);
-      gb[b][o] = __ldg(pb + (o + o0 - 2) * s);
+      gd[b][o] = ld(pd + (o + o0 - 2) * s);
+      gb[b][o] = ld(pb + (o + o0 - 2) * s);
     }
   }
   double Fd[4];

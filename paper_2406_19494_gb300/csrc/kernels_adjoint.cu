@@ -294,8 +294,8 @@ k_adj_face(const double* __restrict__ W, const double* __restrict__ G, const dou
 
 // gW (and gG) += contributions of the faces along D whose stencils contain the cell
 template <int D, bool VISC>
-__global__ void k_adj_gather(const double* __restrict__ CW, const double* __restrict__ CG,
-                             double* __restrict__ gW, double* __restrict__ gG, Geo g) {
+__global__ void k_adj_gather(const double* CW, const double* CG,
+                             double* gW, double* gG, Geo g) {
   step_wait();
   constexpr int A1 = (D == 0) ? 1 : 0;
   constexpr int A2 = (D == 2) ? 1 : 2;
@@ -361,7 +361,7 @@ __global__ void k_adj_gather(const double* __restrict__ CW, const double* __rest
 }
 
 // reverse of G[c*3+b](y) = ((u_c(y-2b) - u_c(y+2b)) + 8 (u_c(y+b) - u_c(y-b))) / 12 * mc_b(y)
-__global__ void k_adj_grad(const double* __restrict__ gG, double* __restrict__ gW, Geo g) {
+__global__ void k_adj_grad(const double* gG, double* gW, Geo g) {
   step_wait();
   const int total = g.ncell;
   for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < total; cell += gridDim.x * blockDim.x) {
@@ -389,7 +389,7 @@ __global__ void k_adj_grad(const double* __restrict__ gG, double* __restrict__ g
   }
 }
 
-__global__ void k_adj_source(const double* __restrict__ mu, double* __restrict__ gW, Geo g, Phys ph) {
+__global__ void k_adj_source(const double* mu, double* gW, Geo g, Phys ph) {
   step_wait();
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
@@ -415,8 +415,8 @@ __device__ __forceinline__ int bc_src(int kind, int side, int a, int n, int h) {
 // cotangents), then the layers' contributions are added in layer order, as the halo pass wrote
 // them (a zero-gradient side adds all layers to one source cell, in the same order).
 template <int A>
-__global__ void k_adj_bc(const double* __restrict__ W, double* __restrict__ gW,
-                         double* __restrict__ gvw_col, Geo g, Phys ph, BC bc) {
+__global__ void k_adj_bc(const double* W, double* gW,
+                         double* gvw_col, Geo g, Phys ph, BC bc) {
   step_wait();
   constexpr int H = FLUID_HALO;
   int lo[3], ext[3];
@@ -490,8 +490,8 @@ __global__ void k_adj_bc(const double* __restrict__ W, double* __restrict__ gW,
   }
 }
 
-__global__ void k_adj_prim(const double* __restrict__ U, const double* __restrict__ gW,
-                           double* __restrict__ gU, Geo g, Phys ph) {
+__global__ void k_adj_prim(const double* U, const double* gW,
+                           double* gU, Geo g, Phys ph) {
   step_wait();
   const int total = g.n[0] * g.n[1] * g.n[2];
   const int nc = g.ncell;
@@ -508,8 +508,8 @@ __global__ void k_adj_prim(const double* __restrict__ U, const double* __restric
 }
 
 // gphi_i += sum over the t2 index of gvw_col(t1 = h + begin + i) * (A/phi0) sin(2 pi kappa x_i)
-__global__ void k_adj_phi(const double* __restrict__ gvw_col, const double* __restrict__ xc,
-                          double* __restrict__ gphi, int p_t1, int h_t1, int ext_t2, int begin,
+__global__ void k_adj_phi(const double* gvw_col, const double* xc,
+                          double* gphi, int p_t1, int h_t1, int ext_t2, int begin,
                           int count, double amp, double two_pi_kappa) {
   step_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {

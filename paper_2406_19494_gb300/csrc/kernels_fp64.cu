@@ -177,8 +177,8 @@ __device__ __forceinline__ void k_prim_bc_body(const double* __restrict__ U, dou
 }
 
 template <bool MIXED>
-__global__ void k_prim_bc(const double* __restrict__ U, double* __restrict__ W,
-                          float* __restrict__ W32, Geo g, Phys ph, BC bc, Ctl* ctl) {
+__global__ void k_prim_bc(const double* U, double* W,
+                          float* W32, Geo g, Phys ph, BC bc, Ctl* ctl) {
   step_wait();
   k_prim_bc_body<MIXED>(U, W, W32, g, ph, bc, ctl, blockIdx, gridDim);
 }
@@ -229,7 +229,7 @@ __device__ __forceinline__ void k_grad_body(const double* __restrict__ W, double
 }
 
 template <int ORDER>
-__global__ void k_grad(const double* __restrict__ W, double* __restrict__ G, Geo g) {
+__global__ void k_grad(const double* W, double* G, Geo g) {
   step_wait();
   k_grad_body<ORDER>(W, G, g, blockIdx, gridDim);
 }
@@ -271,7 +271,7 @@ __device__ __forceinline__ void k_face_seam_body(const double* __restrict__ FB, 
 }
 
 template <int D>
-__global__ void k_face_seam(const double* __restrict__ FB, double* __restrict__ R, Geo g, int seg) {
+__global__ void k_face_seam(const double* FB, double* R, Geo g, int seg) {
   step_wait();
   k_face_seam_body<D>(FB, R, g, seg, blockIdx, gridDim);
 }
@@ -293,7 +293,7 @@ __device__ __forceinline__ double velocity(const double* __restrict__ W, const f
   return W32 ? ff_to_double(load_pair(W32, nc, 1 + b, c)) : W[(1 + b) * nc + c];
 }
 
-__global__ void k_source(double* __restrict__ R, const double* __restrict__ W, const float* __restrict__ W32, Geo g,
+__global__ void k_source(double* R, const double* W, const float* W32, Geo g,
                          Phys ph) {
   step_wait();
   const int total = g.n[0] * g.n[1] * g.n[2];
@@ -351,8 +351,8 @@ __device__ __forceinline__ void k_stage_body(int stage, const double* Un, const 
   if (bad) atomicOr(&ctl->flags, FLAG_NONFINITE);
 }
 
-__global__ void k_stage(int stage, const double* Un, const double* Us, const double* __restrict__ R,
-                        double* Ud, const double* __restrict__ W, const float* __restrict__ W32, Geo g, Phys ph,
+__global__ void k_stage(int stage, const double* Un, const double* Us, const double* R,
+                        double* Ud, const double* W, const float* W32, Geo g, Phys ph,
                         Ctl* ctl, double t_end, double dt_arg) {
   step_wait();
   k_stage_body(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, dt_arg, blockIdx, gridDim);
@@ -445,8 +445,8 @@ __device__ __forceinline__ void k_stage_prim_body(int stage, const double* Un, c
 }
 
 template <bool MIXED>
-__global__ void k_stage_prim(int stage, const double* Un, const double* Us, const double* __restrict__ R,
-                             double* Ud, double* W, float* __restrict__ W32, Geo g, Phys ph, Ctl* ctl,
+__global__ void k_stage_prim(int stage, const double* Un, const double* Us, const double* R,
+                             double* Ud, double* W, float* W32, Geo g, Phys ph, Ctl* ctl,
                              double t_end) {
   step_wait();
   k_stage_prim_body<MIXED>(stage, Un, Us, R, Ud, W, W32, g, ph, ctl, t_end, blockIdx, gridDim);
@@ -509,7 +509,7 @@ __device__ __forceinline__ void k_halo_prim_body(double* __restrict__ W, float* 
 }
 
 template <bool MIXED>
-__global__ void k_halo_prim(double* __restrict__ W, float* __restrict__ W32, Geo g, Phys ph, BC bc,
+__global__ void k_halo_prim(double* W, float* W32, Geo g, Phys ph, BC bc,
                             Ctl* ctl, long long total) {
   step_wait();
   k_halo_prim_body<MIXED>(W, W32, g, ph, bc, ctl, total, blockIdx, gridDim);
@@ -609,7 +609,7 @@ __device__ __forceinline__ void k_dt_body(const double* __restrict__ W, const Ge
   if (threadIdx.x == 0) dt_store(best, ph, ctl, dt_out, clip, t_end);
 }
 
-__global__ void __launch_bounds__(kDtBlock) k_dt(const double* __restrict__ W, const __grid_constant__ Geo g,
+__global__ void __launch_bounds__(kDtBlock) k_dt(const double* W, const __grid_constant__ Geo g,
                                                  const __grid_constant__ Phys ph, double* partial, int nparts,
                                                  Ctl* ctl, double* dt_out, int clip, double t_end) {
   step_wait();

@@ -224,7 +224,7 @@ __device__ __forceinline__ void hllc_delta(const float b[5], const float dL[5], 
 }
 
 __device__ __forceinline__ float interp32(const float* __restrict__ f, int s) {
-  return s_mul(s_fma(9.0f, s_add(__ldg(f), __ldg(f + s)), -s_add(__ldg(f - s), __ldg(f + 2 * s))), 0.0625f);
+  return s_mul(s_fma(9.0f, s_add(ld(f), ld(f + s)), -s_add(ld(f - s), ld(f + 2 * s))), 0.0625f);
 }
 
 // The Euler flux of a cell's pairs along D plus the increment X, as FP64
@@ -244,12 +244,12 @@ __device__ __forceinline__ void assemble_flux(const ff q[5], const Phys& ph, con
 
 // The face flux at i+1/2 (cell i: `cell`) from its cell's pairs q, the corrections cL, cR, D = q_{i+1} -
 // q_i, and for the dissipative flux Ts = T_i + T_{i+1}, Td = T_{i+1} - T_i of the velocities and, last, the
-// temperature, whose D is Dt
+// temperature, whose D is Dt and cell value Tc
 template <int D, bool VISC>
 __device__ __forceinline__ void mixed_face(const float* __restrict__ W32, const float* __restrict__ G32, int cell,
                                            int s, int i, const Geo& g, const Phys& ph, const PhysF& pf, const ff q[5],
                                            const float cL[5], const float cR[5], const float Dv[5], const float Ts[4],
-                                           const float Td[4], float Dt, double F[5]) {
+                                           const float Td[4], float Dt, float Tc, double F[5]) {
   const int nc = g.ncell;
   float b[5], dL[5], J[5], X[5];
 #pragma unroll
@@ -268,7 +268,7 @@ __device__ __forceinline__ void mixed_face(const float* __restrict__ W32, const 
       vf[c] = s_add(b[1 + c], s_fma(-0.0625f, Ts[c], s_mul(0.5f, Dv[1 + c])));
       dn[c] = s_mul(s_fma(-1.0f / 24.0f, Td[c], Dv[1 + c]), mfa);
     }
-    const float Tf = s_add(__ldg(W32 + 5 * nc + cell), s_fma(-0.0625f, Ts[3], s_mul(0.5f, Dt)));
+    const float Tf = s_add(Tc, s_fma(-0.0625f, Ts[3], s_mul(0.5f, Dt)));
     const float dT = s_mul(s_fma(-1.0f / 24.0f, Td[3], Dt), mfa);
     float tr = 0.0f;
 #pragma unroll
@@ -402,15 +402,16 @@ __device__ __forceinline__ void k_face_mixed_body(const float* __restrict__ W32,
         }
     }
   }
-  float D0[NVW];
+  float D0[NVW], Tc = 0.0f;
   ff q[5];
 #pragma unroll
   for (int v = 0; v < NVW; ++v) {
     const float* hp = W32 + v * nc + cell;
     const float* lp = W32 + (NW + v) * nc + cell;
-    const ff q0{__ldg(hp), __ldg(lp)};
-    D0[v] = tc.pair ? s_add(s_sub(__ldg(hp + s), q0.h), s_sub(__ldg(lp + s), q0.l)) : 0.0f;
+    const ff q0{ld(hp), ld(lp)};
+    D0[v] = tc.pair ? s_add(s_sub(ld(hp + s), q0.h), s_sub(ld(lp + s), q0.l)) : 0.0f;
     if (v < 5) q[v] = q0;
+    else Tc = q0.h;
     sh.D[v][t] = D0[v];
   }
   __syncthreads();
@@ -456,7 +457,7 @@ __device__ __forceinline__ void k_face_mixed_body(const float* __restrict__ W32,
       Ts[3] = s_add(Ta, Tj);
       Td[3] = s_sub(Tj, Ta);
     }
-    mixed_face<D, VISC>(W32, G32, cell, s, i, g, ph, pf, q, cL, cR, D0, Ts, Td, D0[NVW - 1], F);
+    mixed_face<D, VISC>(W32, G32, cell, s, i, g, ph, pf, q, cL, cR, D0, Ts, Td, D0[NVW - 1], Tc, F);
 #pragma unroll
     for (int v = 0; v < 5; ++v) sh.F[v][t] = F[v];
   }
@@ -478,7 +479,7 @@ __device__ __forceinline__ void k_face_mixed_body(const float* __restrict__ W32,
 
 template <int SCHEME, bool VISC>
 __global__ void __launch_bounds__(MixedShape<0>::threads, MixedShape<0>::blocks) k_face_mixed_x(
-    const float* __restrict__ W32, const float* __restrict__ G32, double* __restrict__ R,
+    const float* W32, const float* G32, double* R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf) {
   step_wait();
   extern __shared__ __align__(16) unsigned char raw[];
@@ -491,7 +492,7 @@ __global__ void __launch_bounds__(MixedShape<0>::threads, MixedShape<0>::blocks)
 // the tangential axes
 template <int D, int SCHEME, bool VISC>
 __global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed_t(
-    const float* __restrict__ W32, const float* __restrict__ G32, double* __restrict__ R,
+    const float* W32, const float* G32, double* R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf) {
   step_wait();
   extern __shared__ __align__(16) unsigned char raw[];
@@ -504,7 +505,7 @@ __global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks)
 // the last axis's kernel with the stage fused (StageOut): R is read, not written
 template <int D, int SCHEME, bool VISC>
 __global__ void __launch_bounds__(MixedShape<D>::threads, MixedShape<D>::blocks) k_face_mixed_ts(
-    const float* __restrict__ W32, const float* __restrict__ G32, const double* __restrict__ R,
+    const float* W32, const float* G32, const double* R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph, PhysF pf, const __grid_constant__ StageOut so) {
   step_wait();
   extern __shared__ __align__(16) unsigned char raw[];
@@ -531,23 +532,28 @@ __device__ __forceinline__ void k_grad32_body(const float* __restrict__ W32, flo
     c[1] = lo[1] + r % ext[1];
     c[2] = lo[2] + r / ext[1];
     const int cell = c[0] + c[1] * g.sy + c[2] * g.sz;
+    // all loads before the first store: TGV 128^3 37 us a launch, 45 with the stores between them
+    float d[9];
+#pragma unroll
     for (int b = 0; b < 3; ++b) {
       const bool inb = b < g.ndim && c[b] >= g.h[b] && c[b] < g.h[b] + g.n[b];
       const int s = b == 0 ? 1 : (b == 1 ? g.sy : g.sz);
       const float m = inb ? g.mc32[b][c[b]] : 0.0f;
+#pragma unroll
       for (int comp = 0; comp < 3; ++comp) {
-        float d = 0.0f;
+        d[comp * 3 + b] = 0.0f;
         if (inb) {
           const float* f = W32 + (1 + comp) * g.ncell + cell;
-          d = ((f[-2 * s] - f[2 * s]) + 8.0f * (f[s] - f[-s])) * (1.0f / 12.0f) * m;
+          d[comp * 3 + b] = ((f[-2 * s] - f[2 * s]) + 8.0f * (f[s] - f[-s])) * (1.0f / 12.0f) * m;
         }
-        G32[(comp * 3 + b) * g.ncell + cell] = d;
       }
     }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) G32[k * g.ncell + cell] = d[k];
   }
 }
 
-__global__ void k_grad32(const float* __restrict__ W32, float* __restrict__ G32, Geo g) {
+__global__ void k_grad32(const float* W32, float* G32, Geo g) {
   step_wait();
   k_grad32_body(W32, G32, g, blockIdx, gridDim);
 }
@@ -601,7 +607,7 @@ __device__ __forceinline__ void k_dt32_body(const float* __restrict__ W32, const
   if (threadIdx.x == 0) dt_store(top, ph, ctl, dt_out, clip, t_end);
 }
 
-__global__ void __launch_bounds__(kDtBlock) k_dt32(const float* __restrict__ W32, const __grid_constant__ Geo g,
+__global__ void __launch_bounds__(kDtBlock) k_dt32(const float* W32, const __grid_constant__ Geo g,
                                                    const __grid_constant__ Phys ph, const __grid_constant__ PhysF pf,
                                                    double* partial, int nparts, Ctl* ctl, double* dt_out, int clip,
                                                    double t_end) {

@@ -32,7 +32,7 @@ __device__ __noinline__ TwoValues face_values_fp64(const double* __restrict__ f,
                                                    const double (*omega)[16]) {
   double q[6], d[5];
 #pragma unroll
-  for (int o = 0; o < 6; ++o) q[o] = __ldg(f + (o - 2) * s);
+  for (int o = 0; o < 6; ++o) q[o] = ld(f + (o - 2) * s);
 #pragma unroll
   for (int o = 0; o < 5; ++o) d[o] = q[o + 1] - q[o];
   double b3[3] = {weno_B(q[1], q[2], q[3]), weno_C(q[2], q[3], q[4]), weno_A(q[0], q[1], q[2])};
@@ -52,13 +52,14 @@ struct TenoShared {
   double T[NVW][N];           // second differences
   double d[NVW][N];           // q_{j+1} - q_j
   double F[5][N];
+  double q[5][N];             // primitives, for the reads after the calls (from global memory: x, y, z launches 3, 2, 2.5 % longer)
   unsigned char lev[5][N];    // cut-off levels of the cells
   double alpha[4][16], omega[4][16];
 };
 
 template <int D, int NP>
 __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>::threads) k_face_teno(
-    const double* __restrict__ W, const double* __restrict__ G, double* __restrict__ R,
+    const double* W, const double* G, double* R,
     const __grid_constant__ Geo g, const __grid_constant__ Phys ph) {
   step_wait();
   constexpr int TX = TileShape<D>::TX, TD = TileShape<D>::TD, N = TileShape<D>::threads;
@@ -77,7 +78,9 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
 #pragma unroll
   for (int v = 0; v < NVW; ++v) {
     const double* f = W + v * nc + cell;
-    sh.d[v][t] = c.pair ? __ldg(f + s) - __ldg(f) : 0.0;
+    const double q = ld(f);
+    if (v < 5) sh.q[v][t] = q;
+    sh.d[v][t] = c.pair ? ld(f + s) - q : 0.0;
   }
   __syncthreads();
 #pragma unroll 1
@@ -96,7 +99,7 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
   const bool face = row >= 2 && row < TD - 2 && c.live && i >= g.h[D] - 1 && i < g.h[D] + g.n[D];
   double F[5];
   if (face) {
-    const Scale sc = scale_of(__ldg(W + cell + s), __ldg(W + 4 * nc + cell + s), ph);
+    const Scale sc = scale_of(sh.q[0][t + TX], sh.q[4][t + TX], ph);
     double cL[5], cR[5], d[5];
     bool small = sc.ok;
 #pragma unroll
@@ -117,7 +120,7 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
         cR[v] = fma(sh.alpha[0][mR], Tp, fma(sh.alpha[1][mR], T1, fma(sh.alpha[2][mR], T0, sh.alpha[3][mR] * Tm)));
       } else {
         const TwoValues w = face_values_fp64(W + v * nc + cell, s, teno::cutoff_of_level(lev), sh.omega);
-        const double q0 = __ldg(W + v * nc + cell), q1 = __ldg(W + v * nc + cell + s);
+        const double q0 = sh.q[v][t], q1 = sh.q[v][t + TX];
         cL[v] = fma(6.0, w.l - q0, -3.0 * d[v]);
         cR[v] = fma(6.0, w.r - q1, 3.0 * d[v]);
       }
@@ -128,7 +131,7 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
       ff wl[5], J[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const ff m = ff_of(__ldg(W + v * nc + cell)) + ff_scale(ff_of(d[v]), 0.5f);
+        const ff m = ff_of(sh.q[v][t]) + ff_scale(ff_of(d[v]), 0.5f);
         if (NP && v >= 1 && v <= 3) m3[v - 1] = m;
         J[v] = ff_of(cR[v] - cL[v]) * sixth();
         wl[v] = ff_fma(ff_of(cL[v]), sixth(), m);
@@ -139,35 +142,34 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
         bool left;
         hllc_ff<D>(wl, J, ph.k, left, X);
         double w[5];
-        const int o = left ? 0 : s;
+        const int o = left ? 0 : TX;
         const double three = left ? 3.0 : -3.0;
 #pragma unroll
         for (int v = 0; v < 5; ++v)
-          w[v] = fma(kSixth, fma(three, d[v], left ? cL[v] : cR[v]), __ldg(W + v * nc + cell + o));
+          w[v] = fma(kSixth, fma(three, d[v], left ? cL[v] : cR[v]), sh.q[v][t + o]);
         euler_flux<D>(w, ph, F);
       }
     } else if (NP) {
 #pragma unroll
       for (int v = 1; v <= 3; ++v)
-        m3[v - 1] = ff_of(__ldg(W + v * nc + cell)) + ff_scale(ff_of(d[v]), 0.5f);
+        m3[v - 1] = ff_of(sh.q[v][t]) + ff_scale(ff_of(d[v]), 0.5f);
     }
     if (!small) {
       Flux5 l, r;
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double* f = W + v * nc + cell;
-        l.f[v] = fma(kSixth, fma(3.0, d[v], cL[v]), __ldg(f));
-        r.f[v] = fma(kSixth, fma(-3.0, d[v], cR[v]), __ldg(f + s));
+        l.f[v] = fma(kSixth, fma(3.0, d[v], cL[v]), sh.q[v][t]);
+        r.f[v] = fma(kSixth, fma(-3.0, d[v], cR[v]), sh.q[v][t + TX]);
         X[v] = ff{0.0f, 0.0f};
       }
       // interpolation limiter
       if (l.f[0] <= 0.0 || l.f[4] <= 0.0) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) l.f[v] = __ldg(W + v * nc + cell);
+        for (int v = 0; v < 5; ++v) l.f[v] = sh.q[v][t];
       }
       if (r.f[0] <= 0.0 || r.f[4] <= 0.0) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) r.f[v] = __ldg(W + v * nc + cell + s);
+        for (int v = 0; v < 5; ++v) r.f[v] = sh.q[v][t + TX];
       }
       const Flux5 e = hllc_fp64<D>(l, r, &ph);
 #pragma unroll
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(TileShape<D>::threads, 16 * 32 / TileShape<D>:
       for (int c4 = 0; c4 < 4; ++c4) {
         const int v = c4 < 3 ? 1 + c4 : NVW - 1;
         const ff Dv = ff_of(sh.d[v][t]);
-        const ff m = c4 < 3 ? m3[c4] : ff_of(__ldg(W + 5 * nc + cell)) + ff_scale(Dv, 0.5f);
+        const ff m = c4 < 3 ? m3[c4] : ff_of(ld(W + 5 * nc + cell)) + ff_scale(Dv, 0.5f);
         const ff f0 = ff_of(sh.T[v][t]), f1 = ff_of(sh.T[v][t + TX]);
         if (NP == 4) {
           dv[c4] = Dv - add_weak(f1, -f0) * ff{k24H, k24L};
