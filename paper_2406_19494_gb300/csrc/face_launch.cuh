@@ -54,8 +54,8 @@ cudaError_t launch_scheme(int D, const double* W, const double* G, double* R, co
     if (D == 1) return launch_tile<1, SCHEME, VISC>(W, G, R, g, ph, st);
     return launch_tile<2, SCHEME, VISC>(W, G, R, g, ph, st);
   }
-  int grid;
-  face_shape(D, g, block, seg, grid);
+  if (block <= 0) block = 128;
+  const int grid = face_grid(D, g, block, seg);
   double* FB = seam_buffer(D, g, seg, fb);
   if (D == 0) launch_step(k_face<0, SCHEME, VISC>, grid, block, 0, st, W, G, R, FB, g, ph, seg);
   else if (D == 1) launch_step(k_face<1, SCHEME, VISC>, grid, block, 0, st, W, G, R, FB, g, ph, seg);

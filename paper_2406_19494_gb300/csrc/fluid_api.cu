@@ -442,15 +442,6 @@ bool batch_slot_of(fluid_solver* s, double* U, double t_end, BatchSlot& out) {
   out.nparts = s->ph.dt_fixed > 0.0 ? 0 : s->nparts;
   out.ctl = s->ctl;
   out.t_end = t_end;
-  for (int D = 0; D < 3; ++D) {
-    out.seg[D] = 1;
-    out.FB[D] = nullptr;
-    if (D == 0 || D >= s->geo.ndim || s->mixed) continue;
-    int block = 128, seg = s->face_seg_d[D], grid = 0;
-    face_shape(D, s->geo, block, seg, grid);
-    out.seg[D] = seg;
-    out.FB[D] = seam_buffer(D, s->geo, seg, SeamBuf{s->FB, s->fb_cap});
-  }
   return true;
 }
 }  // namespace fl

@@ -253,8 +253,8 @@ __device__ __forceinline__ void step_wait() {
 cudaError_t launch_prim_bc(const double* U, double* W, float* W32, const Geo& g, const Phys& ph,
                            const BC& bc, Ctl* ctl, cudaStream_t st);
 cudaError_t launch_grad(const double* W, double* G, const Geo& g, const Phys& ph, cudaStream_t st);
-// launch shape of the marching FP64 face kernels: block/seg 0 pick the defaults; grid out
-void face_shape(int D, const Geo& g, int& block, int& seg, int& grid);
+// blocks of the marching FP64 face kernels: one thread per segment of `seg` cells along D
+int face_grid(int D, const Geo& g, int block, int seg);
 // Seam buffer of the FP64 face kernels: 10 doubles per segment item (lines x segments of a launch),
 // cap items; a launch whose segments are shorter than kSeamMinSeg or that does not fit runs without
 // it (same result).  {nullptr, 0} turns it off.
@@ -372,7 +372,7 @@ cudaError_t launch_wall_velocity(const double* phi, double* vw, const double* xc
 // between chunks as solves are admitted and retire.
 constexpr int kBatchMax = 64;   // solves per bucket
 enum BatchKernel {
-  BK_PRIM = 0, BK_DT, BK_GRAD, BK_FACE0, BK_FACE1, BK_FACE2, BK_SEAM0, BK_SEAM1, BK_SEAM2,
+  BK_PRIM = 0, BK_DT, BK_GRAD, BK_FACE0, BK_FACE1, BK_FACE2,
   BK_STAGEP, BK_HALO, BK_STAGE, BK_COUNT
 };
 struct BatchSlot {
@@ -386,12 +386,10 @@ struct BatchSlot {
   double* G;          // FP64 gradients (FP64 viscous)
   float* W32;         // primitives (mixed)
   float* G32;         // FP32 gradients (mixed viscous)
-  double* FB[3];      // seam buffer per axis (null: none)
   double* partial;    // CFL partial maxima
   int nparts;         // their count (0 with a fixed dt)
   Ctl* ctl;
   double t_end;
-  int seg[3];         // FP64 face segment length per axis
   int steps;          // steps of the current chunk; the solve idles at later steps
   int vgrid[BK_COUNT][3];
 };
@@ -447,8 +445,8 @@ int solver_create_async(const fluid_config* cfg, cudaStream_t st, fluid_solver**
 // a solver's part of a batch (its geometry, physics, boundaries and scratch, state U, t_end); false
 // when its configuration has no batched kernels (TENO6-A, sixth-order stencils, exchange faces)
 bool batch_slot_of(fluid_solver* s, double* U, double t_end, BatchSlot& out);
-// fill slot.vgrid and the prefixes for the solves of t (their Geo, Phys, seg and FB set)
-void batch_plan(BatchTable& t, bool mixed);
+// fill slot.vgrid and the prefixes for the solves of t (their Geo and Phys set)
+void batch_plan(BatchTable& t);
 // enqueue the batched kernels of `chunk` RK3 steps (what fluid_step(U, chunk) does for every solve)
 cudaError_t launch_batch_chunk(const BatchTable* dev, int chunk, bool mixed, int weno, bool visc,
                                cudaStream_t st);

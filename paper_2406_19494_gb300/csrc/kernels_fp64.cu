@@ -691,13 +691,6 @@ __global__ void __launch_bounds__(256) kb_grad(const BatchTable* __restrict__ t,
   FL_BATCH_END
 }
 
-template <int D>
-__global__ void __launch_bounds__(256) kb_seam(const BatchTable* __restrict__ t, int step) {
-  FL_BATCH_LOOP(BK_SEAM0 + D)
-  if (step < S.steps) k_face_seam_body<D>(S.FB[D], S.R, S.g, S.seg[D], bid, gdim);
-  FL_BATCH_END
-}
-
 template <bool MIXED>
 __global__ void __launch_bounds__(128) kb_stage_prim(const BatchTable* __restrict__ t, int stage, int step) {
   FL_BATCH_LOOP(BK_STAGEP)
@@ -726,20 +719,17 @@ __global__ void __launch_bounds__(256) kb_stage(const BatchTable* __restrict__ t
 
 cudaError_t launch_batch_faces(const BatchTable* dev, int step, int weno, bool visc,
                                cudaStream_t st) {
-  static const int gs = batch_grid(kb_seam<1>, 256);
   for (int D = 0; D < 3; ++D) {
     const cudaError_t e = weno == FLUID_WENO_JS ? launch_batch_face_js(dev, D, step, visc, st)
                                                 : launch_batch_face_z(dev, D, step, visc, st);
     if (e != cudaSuccess) return e;
-    if (D == 1) (kb_seam<1><<<gs, 256, 0, st>>>(dev, step), ++t_launches);
-    if (D == 2) (kb_seam<2><<<gs, 256, 0, st>>>(dev, step), ++t_launches);
   }
   return cudaGetLastError();
 }
 
 }  // namespace
 
-void batch_plan(BatchTable& t, bool mixed) {
+void batch_plan(BatchTable& t) {
   auto ceil_div = [](long long a, long long b) { return (a + b - 1) / b; };
   for (int k = 0; k < BK_COUNT; ++k) t.prefix[k][0] = 0;
   for (int i = 0; i < t.nslots; ++i) {
@@ -760,16 +750,10 @@ void batch_plan(BatchTable& t, bool mixed) {
     for (int a = 0; a < 3; ++a) gt *= g.n[a] + (a < g.ndim ? 4 : 0);   // order-4 stencils, both paths
     set(BK_GRAD, visc ? ceil_div(gt, 256) : 0);
     for (int D = 0; D < 3; ++D) {
-      const long long lines = (long long)g.n[D == 0 ? 1 : 0] * g.n[D == 2 ? 1 : 2];
-      if (D >= g.ndim) {
-        set(BK_FACE0 + D, 0);
-        set(BK_SEAM0 + D, 0);
-        continue;
-      }
-      if (D == 0) set(BK_FACE0, tile_cols<0>(g), tile_rows<0>(g));
+      if (D >= g.ndim) set(BK_FACE0 + D, 0);
+      else if (D == 0) set(BK_FACE0, tile_cols<0>(g), tile_rows<0>(g));
       else if (D == 1) set(BK_FACE1, tile_cols<1>(g), tile_rows<1>(g));
       else set(BK_FACE2, tile_cols<2>(g), tile_rows<2>(g));
-      set(BK_SEAM0 + D, 0);
     }
     set(BK_STAGEP, ceil_div(g.n[0], 128), std::min((g.n[1] + 1) / 2, 65535), std::min(g.n[2], 65535));
     set(BK_HALO, ceil_div(npad - nint, 256));
@@ -837,23 +821,9 @@ cudaError_t launch_face_seam(int D, const double* FB, double* R, const Geo& g, i
   return cudaGetLastError();
 }
 
-void face_shape(int D, const Geo& g, int& block, int& seg, int& grid) {
-  const int A1 = (D == 0) ? 1 : 0;
-  const int A2 = (D == 2) ? 1 : 2;
-  const long long lines = (long long)g.n[A1] * g.n[A2];
-  if (block <= 0) block = 128;
-  if (seg <= 0) {
-    // longest segment (fewest redundant faces) that still gives >= 4 blocks of 128 per SM, down
-    // to 8 cells; 4 cells only where segments of 8 would leave SMs without a block (small 2-D
-    // grids such as the 512 x 128 boundary layer: there segments of 4 take 40 % less time than 8,
-    // while on TGV 64^3, which 8 already spreads over every SM, they take 14 % more).  The result
-    // does not depend on the choice.
-    seg = 64;
-    auto threads = [&](int sg) { return lines * ((g.n[D] + sg - 1) / sg); };
-    while (seg > 8 && threads(seg) < 152LL * 4 * 128) seg >>= 1;
-    if (seg == 8 && threads(8) < 152LL * 128) seg = 4;
-  }
-  grid = grid_for(lines * ((g.n[D] + seg - 1) / seg), block);
+int face_grid(int D, const Geo& g, int block, int seg) {
+  const long long lines = (long long)g.n[D == 0 ? 1 : 0] * g.n[D == 2 ? 1 : 2];
+  return grid_for(lines * ((g.n[D] + seg - 1) / seg), block);
 }
 
 cudaError_t launch_prim_bc(const double* U, double* W, float* W32, const Geo& g, const Phys& ph,

@@ -315,7 +315,7 @@ struct fluid_server {
       ++t.nslots;
     }
     if (t.nslots == 0) return busy;
-    fl::batch_plan(t, b.mixed);
+    fl::batch_plan(t);
     cudaMemcpyAsync(b.dev, b.host, sizeof(fl::BatchTable), cudaMemcpyHostToDevice, b.stream);
     if (cfg.use_graphs && !b.graph) {
       cudaGraph_t gr = nullptr;
