@@ -291,11 +291,11 @@ int fluid_check(fluid_solver* s, void* stream);
 int fluid_tune_faces(fluid_solver* s, int block, int seg);
 
 /* Time the FP64 face kernels (the automatic choice and segments of 8 to 32 cells with blocks of 128
- * threads, then blocks of 64 and 32 threads with the fastest segment length) on the
+ * threads, then, if a segment length was fastest, blocks of 64 and 32 threads with it) on the
  * primitives of U_dev (device, the solver's padded layout; not modified) and keep the fastest shape
  * per axis; the launch shape never changes a result, so this only changes speed.
  * Enqueued on `stream` and synchronised; uses the solver's scratch, so no other call on the solver
- * may run meanwhile.  No-op (FLUID_OK) for FLUID_PREC_MIXED.  FLUID_EINVAL for a NULL solver or a
+ * may run meanwhile.  No-op (FLUID_OK) for FLUID_PREC_MIXED and the channel scheme.  FLUID_EINVAL for a NULL solver or a
  * foreign pointer, FLUID_ECUDA on a launch error. */
 int fluid_autotune_faces(fluid_solver* s, const double* U_dev, void* stream);
 

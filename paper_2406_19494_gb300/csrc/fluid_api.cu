@@ -1038,7 +1038,7 @@ int fluid_tune_faces(fluid_solver* s, int block, int seg) {
 int fluid_autotune_faces(fluid_solver* s, const double* U_dev, void* stream) {
   if (!s) return FLUID_EINVAL;
   if (int r = check_ptr(s, U_dev, "U_dev")) return r;
-  if (s->mixed) return FLUID_OK;
+  if (s->mixed || s->ph.weno == FLUID_TENO6A) return FLUID_OK;   // one shape
   cudaStream_t st = as_stream(stream);
   const Geo& g = s->geo;
   FL_CUDA(s, fl::launch_prim_bc(U_dev, s->W, s->W32, g, s->ph, s->bc, s->ctl, st));
@@ -1081,7 +1081,7 @@ int fluid_autotune_faces(fluid_solver* s, const double* U_dev, void* stream) {
       if (e != cudaSuccess) break;
     }
     for (int b : {64, 32}) {
-      if (e != cudaSuccess) break;
+      if (e != cudaSuccess || best_seg == 0) break;      // the tiles have one block size
       trial(b, best_seg);
     }
     if (e == cudaSuccess) {

@@ -352,14 +352,15 @@ struct fluid_server {
     auto it = tuned.find(key);
     if (it == tuned.end()) {
       std::vector<std::pair<int, int>> cand = {{0, 0}, {32, 64}, {64, 16}, {128, 32}};
-      // every FP64 segment length gives bitwise the default shape's results; the mixed path has
-      // one shape
-      if (c.precision == FLUID_PREC_MIXED) cand = {{0, 0}};
+      // every FP64 segment length gives bitwise the default shape's results; the mixed path and the
+      // channel scheme have one shape, with nothing to time
+      if (c.precision == FLUID_PREC_MIXED || c.weno == FLUID_TENO6A) cand.clear();
       double* tmp = nullptr;
       float best = 1e30f;
       std::pair<int, int> pick{0, 0};
       cudaEvent_t a, b;
-      if (cudaMallocAsync((void**)&tmp, s.job->nstate * sizeof(double), s.stream) == cudaSuccess &&
+      if (!cand.empty() &&
+          cudaMallocAsync((void**)&tmp, s.job->nstate * sizeof(double), s.stream) == cudaSuccess &&
           cudaEventCreate(&a) == cudaSuccess && cudaEventCreate(&b) == cudaSuccess) {
         for (auto& cs : cand) {
           if (fluid_tune_faces(s.solver, cs.first, cs.second) != FLUID_OK) continue;
