@@ -348,9 +348,10 @@ def run_decomposed(args, ws, rank, local):
         "e2e": {"value": ncell * ws / (e2e_ms * 1e-3), "unit": UNIT, "h2d_bytes_per_step": nbytes,
                 "d2h_bytes_per_step": nbytes},
         "gpu_launches": launches,
-        "roofline": {"bound": "alu", "kernel": "k_face_tile (x, y, z), FP64 with two-float terms", "achieved": achieved,
-                     "peak": peak64, "unit": "TFLOP/s", "frac": achieved / peak64 if achieved else None,
-                     "flops_basis": "executed FP64 (ncu: 2 DFMA + DADD + DMUL per cell and axis)", "traffic": None},
+        "roofline": dict(face_roofline(ncell, t_face), traffic=None,
+                         fp64={"achieved": achieved, "peak": peak64, "unit": "TFLOP/s",
+                               "frac": achieved / peak64 if achieved else None,
+                               "flops_basis": "executed FP64 (ncu: 2 DFMA + DADD + DMUL per cell and axis)"}),
         "kernels_ms_per_step": {k: v[0] / args.steps for k, v in prof.items() if v[1]},
         "clocks": clk.summary(),
     }
@@ -454,7 +455,7 @@ def run_fluid(args):
 
     # ---- rooflines of the dominant kernel class (the face kernels) ----------------------------
     def face_time(p, calls):
-        """seconds per face-kernel call (one axis of one stage: the face kernel with its seam kernel)"""
+        """seconds per face-kernel call (one axis of one stage: the face kernel, with its seam kernel where a segment length is set)"""
         ms = sum(v[0] for k, v in p.items() if k.startswith("face_"))
         return (ms / calls * 1e-3) if calls and ms > 0 else None
 
@@ -486,19 +487,19 @@ def run_fluid(args):
         "e2e": {"value": ncell * ws / (e2e_ms * 1e-3), "unit": UNIT, "h2d_bytes_per_step": nbytes,
                 "d2h_bytes_per_step": nbytes},
         "gpu_launches": launches,
-        "roofline": {"bound": "alu", "kernel": "k_face_tile (x, y, z), FP64 with two-float terms", "achieved": achieved, "peak": peak64,
-                     "unit": "TFLOP/s", "frac": achieved / peak64 if achieved else None,
-                     "traffic": face_traffic(ncell),
-                     "traffic_note": "bytes per launch: ncu dram__bytes_read.sum + dram__bytes_write.sum of the x, y and z face launches of this workload (mean), null when the kernel sources changed since that capture",
-                     "peak_source": "FP64 units x max SM clock (152 SMs x 2 FMA/clk x 2 flops x 2.07 GHz); "
-                                    "measured by the FMA probe as fp64_fma_probe_tflops",
-                     "fp64_fma_probe_tflops": fp64_probe / 1e3 if fp64_probe else None,
-                     "flops_per_cell_axis": accounting.EXECUTED["k_face"],
-                     "flops_basis": "executed FP64 (ncu: 2 DFMA + DADD + DMUL per cell and axis); the definition's "
-                                    "other flops run as two-float FP32 arithmetic, which shares the issue slots",
-                     "flops_algorithmic_per_cell_axis": accounting.cell_axis_flops(3, case["weno"], case["visc"]),
-                     "achieved_algorithmic": algorithmic,
-                     "flops_per_cell_update": accounting.cell_update_flops(3, case["weno"], case["visc"])},
+        "roofline": dict(
+            face_roofline(ncell, t_face), traffic=face_traffic(ncell),
+            traffic_note="bytes per launch: ncu dram__bytes_read.sum + dram__bytes_write.sum of the x, y and z face launches of this workload (mean), null when the kernel sources changed since that capture",
+            fp64={"achieved": achieved, "peak": peak64, "unit": "TFLOP/s", "frac": achieved / peak64 if achieved else None,
+                  "peak_source": "FP64 units x max SM clock (152 SMs x 2 FMA/clk x 2 flops x 2.07 GHz); "
+                                 "measured by the FMA probe as fp64_fma_probe_tflops",
+                  "fp64_fma_probe_tflops": fp64_probe / 1e3 if fp64_probe else None,
+                  "flops_per_cell_axis": accounting.EXECUTED["k_face"],
+                  "flops_basis": "executed FP64 (ncu: 2 DFMA + DADD + DMUL per cell and axis); the definition's "
+                                 "other flops run as two-float FP32 arithmetic, which shares the issue slots"},
+            flops_algorithmic_per_cell_axis=accounting.cell_axis_flops(3, case["weno"], case["visc"]),
+            achieved_algorithmic_tflops=algorithmic,
+            flops_per_cell_update=accounting.cell_update_flops(3, case["weno"], case["visc"])),
         "kernels_ms_per_step": {k: v[0] / args.steps for k, v in prof.items() if v[1]},
         "mixed": {
             "value": whole_job_rate(ncell, args.steps, ws, mixed_ms), "unit": UNIT,
@@ -945,9 +946,9 @@ MIXED_SOURCES = ("kernels_mixed.cu", "kernels_fp64.cu", "face_kernels.cuh", "fac
                  "fluid_internal.cuh", "flux_math.cuh", "fast_math.cuh")
 
 
-def face_traffic(ncell):
-    """DRAM bytes per face-kernel launch from the committed ncu summary, scaled by cells; None if the
-    kernel sources changed since the counters were taken."""
+def face_capture():
+    """The committed ncu counters of the FP64 face kernels (profiles/k_face_traffic.json); None if the
+    kernel sources changed since they were taken."""
     import hashlib
     try:
         info = json.load(open(os.path.join(ROOT, "profiles", "k_face_traffic.json")))
@@ -956,10 +957,33 @@ def face_traffic(ncell):
     csrc = os.path.join(ROOT, "paper_2406_19494_gb300", "csrc")
     src = b"".join(open(os.path.join(csrc, f), "rb").read()
                    for f in FACE_SOURCES)
-    if hashlib.sha256(src).hexdigest()[:16] != info.get("source_sha256_16"):
+    return info if hashlib.sha256(src).hexdigest()[:16] == info.get("source_sha256_16") else None
+
+
+def face_traffic(ncell):
+    """DRAM bytes per face-kernel launch from that capture, scaled by cells."""
+    info = face_capture()
+    if info is None:
         return None
     per = sum(info["dram_bytes_per_launch"]) / len(info["dram_bytes_per_launch"])
     return per * ncell / info["cells"]
+
+
+def face_roofline(ncell, t_face):
+    """What bounds the FP64 face kernels: instruction issue.  Warp instructions per launch from the committed
+    capture, scaled by cells, over the time per launch, against one warp instruction per clock and
+    scheduler (152 SMs x 4 at the maximum SM clock); None fields where the capture is stale."""
+    peak = 152 * 4 * 2.07
+    info = face_capture()
+    done = None
+    if info is not None and t_face:
+        per = sum(info["warp_inst_per_launch"]) / len(info["warp_inst_per_launch"])
+        done = per * ncell / info["cells"] / t_face / 1e9
+    return {"bound": "issue", "kernel": "k_face_tile (x, y, z), FP64 with two-float terms", "achieved": done, "peak": peak,
+            "unit": "Gwarp-inst/s", "frac": done / peak if done else None,
+            "inst_basis": "ncu smsp__inst_executed.sum of the x, y and z launches (mean), null when the kernel sources "
+                          "changed since that capture",
+            "peak_source": "152 SMs x 4 schedulers x 1 warp instruction per clock x 2.07 GHz"}
 
 
 def mixed_step_roofline(ms_per_step, ncell):

@@ -346,8 +346,7 @@ int fluid_check_pow(const double* x_dev, double* fast_dev, double* lib_dev, int 
                     void* stream);
 
 
-/* Check of the FP32 -> FP64 widening the mixed face kernels build from the bit fields with integer
- * operations: bits[i] = that widening of x[i], cvt[i] = the conversion instruction's result, for n
+/* Check of the FP32 -> FP64 widening built from the bit fields with integer operations (fl_widen): bits[i] = that widening of x[i], cvt[i] = the conversion instruction's result, for n
  * device values.  For tests. */
 int fluid_check_widen(const float* x_dev, double* bits_dev, double* cvt_dev, int n, void* stream);
 
@@ -355,7 +354,7 @@ int fluid_check_widen(const float* x_dev, double* bits_dev, double* cvt_dev, int
 /* Check of the bulk-copy helpers (cp.async.bulk on an mbarrier with a bounded wait): one warp
  * stages nrows (1..8) rows of 36 floats from src_dev (16-byte aligned, device) into shared memory
  * with cp.async.bulk on an mbarrier expecting the rows' bytes plus extra_bytes, waits with the
- * tiles' bounded wait and writes the rows to dst_dev.  extra_bytes > 0 makes the wait run out
+ * a bounded wait and writes the rows to dst_dev.  extra_bytes > 0 makes the wait run out
  * (every copy lands, the expected count is never reached): FLAG_STAGING (4) is then ORed into
  * *flags_dev (device) and dst_dev is not written.  Enqueued on `stream`.  For tests. */
 int fluid_check_bulk_staging(const float* src_dev, float* dst_dev, int nrows, int extra_bytes,

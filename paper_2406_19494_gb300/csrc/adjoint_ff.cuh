@@ -1,10 +1,12 @@
 // Adjoint of a face in two-float arithmetic (ff_math.cuh): the reconstruction's gradients, the reverse
 // HLLC flux and the reverse dissipative flux of adjoint_math.cuh.  The FP64 forms take about 1,400
 // FP64-pipe instructions per face.  Their terms are formed from cell differences, which are taken in FP64
-// first, and a gradient inherits the rounding of the primitives relative to those differences, which is
-// larger than the error of the two floats: over porous layers of 96 x 48 to 700 x 256 cells the step
-// adjoint's error against 80-bit arithmetic is 3.5e-13 to 2.9e-12 of its norm with either, and the
-// two differ by 0.6e-14 to 1.1e-14.  Cells and faces whose terms leave the FP32 range, and faces whose
+// first, and a gradient inherits the rounding of the primitives relative to those differences, which on
+// smooth fields is larger than the error of the two floats: over porous layers of 96 x 48 to 700 x 256 cells
+// the step adjoint's error against 80-bit arithmetic is 3.5e-13 to 2.9e-12 of its norm with either, and the
+// two differ by 0.6e-14 to 1.1e-14; at Mach 0.1 to 1e-5 both lose the same digits.  Where the weights are
+// well conditioned (WENO5-JS, noise at the grid scale, jumps) the two floats show: 1e-15 to 7e-15 of the
+// summed terms, 1e-17 to 1e-15 in FP64.  Cells and faces whose terms leave the FP32 range, and faces whose
 // upwind side rounding may have decided, take the FP64 forms.
 #pragma once
 

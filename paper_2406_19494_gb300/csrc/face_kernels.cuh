@@ -434,9 +434,11 @@ struct TileShape {
 };
 
 // Tiles of a quarter of the threads along y and z, for grids that leave SMs without a tile of the shape above
-// (a tile's FP64 instructions pass through one SM's pipe): vortex 64 x 64, three steps 1.02 -> 0.96 ms;
-// right-hand side of a box of 24 x 30 x 20 cells in FP64 throughout 0.31 -> 0.28 ms.  Along x, 32
-// threads took longer than 128 (shock tube 1.35 -> 1.59 ms: fewer threads share the FP64 faces).
+// (a tile's instructions pass through one SM).  Against that shape on the same grids: vortex of 32^2 to 80^2,
+// ten steps, 4 to 5 % shorter (64^2: 1.03 -> 0.98 ms), 90^2 to 128^2 0 to 2 %; right-hand sides of boxes in
+// FP64 throughout, 12^3 to 18^3 16 to 21 %, 20^3 to 26^3 7 to 12 %; TGV 12^3 to 20^3 4 to 8 %.  TGV 22^3 to
+// 26^3 took 6 to 11 % longer, boundary layers of 64 x 64 to 140 x 100 1 to 4 %.  Along x, 32 threads took
+// longer than 128 (shock tube 1.35 -> 1.59 ms: fewer threads share the FP64 faces).
 struct SmallTile {
   static constexpr int TX = 2, TD = 32, threads = TX * TD, step = TD - 5, blocks = 24 * 32 / threads;
 };

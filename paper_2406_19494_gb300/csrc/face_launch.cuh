@@ -8,7 +8,8 @@ namespace fl {
 
 namespace {
 
-// grids of at most this many tiles (one per SM) take the small ones along y and z
+// launches of at most this many tiles (one per SM of this GPU) take the small ones along y and z (SmallTile has
+// both sides measured)
 constexpr long long kSmallTiles = 152;
 
 template <int D, int SCHEME, bool VISC>

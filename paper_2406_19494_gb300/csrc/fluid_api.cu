@@ -1014,8 +1014,6 @@ int fluid_check(fluid_solver* s, void* stream) {
   if (flags) {
     const unsigned zero = 0;
     FL_CUDA(s, cudaMemcpy(&s->ctl->flags, &zero, sizeof(unsigned), cudaMemcpyHostToDevice));
-    if (flags & fl::FLAG_STAGING)
-      return fail(s, FLUID_ECUDA, "a bulk copy into shared memory did not complete within its wait limit");
     return fail(s, FLUID_ENONFINITE,
                 (flags & fl::FLAG_GHOST_T) ? "non-positive ghost temperature at an isothermal wall"
                                            : "non-finite value in the state");

@@ -18,7 +18,7 @@ constexpr int NG = 9;   // velocity-gradient scratch, component c * 3 + b = d u_
 // flag bits of Ctl::flags
 constexpr unsigned FLAG_NONFINITE = 1u;
 constexpr unsigned FLAG_GHOST_T = 2u;
-constexpr unsigned FLAG_STAGING = 4u;   // a shared-memory staging copy did not complete in time
+constexpr unsigned FLAG_STAGING = 4u;   // the bulk-copy check's wait ran out (k_bulk_probe; never in Ctl::flags)
 
 // Grid geometry: padded sizes, strides and per-axis 1-D metric arrays (device, length p[a]).
 struct Geo {
@@ -219,7 +219,7 @@ inline thread_local long long t_launches = 0;
 // next kernel is set up while the last blocks of this one run, and waits (step_wait, the first
 // statement of every kernel launched this way) until this one has finished and its writes are
 // visible.  A launch that follows or precedes anything else on the stream is ordered as usual.  Shock
-// tube of 200 cells, 20 steps of 13 launches: 2.28 -> 1.91 ms (with the CFL reduction as one kernel);
+// tube of 200 cells, 20 steps of 10 launches: 2.28 -> 1.91 ms (with the CFL reduction as one kernel);
 // step adjoint of 96 x 48 and 512 x 128 cells: 427 -> 374 and 600 -> 533 us.
 // Such a kernel begins before the kernel that writes its input has ended.  The read-only load path (__ldg, or
 // what the compiler makes of a const __restrict__ kernel parameter) is defined only for data that no one

@@ -7,15 +7,14 @@
 //               order (Section 3.2: halo cells take values assigned by the boundary conditions)
 //   k_grad      fourth- or sixth-order central velocity gradients at cell centres (tangential
 //               derivatives of the dissipative fluxes)
-//   k_face_x, k_face<D>   per axis (face_kernels.cuh): WENO5 reconstruction of the primitives, HLLC
-//               convective flux, the dissipative flux at the same face, and the flux difference
-//               -(F+ - F-)/dx into R.  Along y and z one thread marches along a segment of a grid
-//               line so each face is computed once and reused by the two cells that share it; a
-//               segment starts with the carried terms formed by the march's own operations
-//               (march_start), so the result is the same for every segment length.
-//   k_face_seam<D>   the first cell of every segment after a line's first, from the two fluxes
-//               the neighbouring segments hand over in the seam buffer (with the buffer no face
-//               is formed twice)
+//   k_face_tile<D>   per axis (face_kernels.cuh, launched from kernels_face_js.cu and kernels_face_z.cu):
+//               WENO5 reconstruction of the primitives, HLLC convective flux, the dissipative flux at the
+//               same face, and the flux difference -(F+ - F-)/dx into R; one thread per cell of a tile.
+//               TENO6-A has its own (k_face_teno, kernels_teno.cu)
+//   k_face<D>, k_face_seam<D>   where a caller sets a segment length (fluid_tune_faces): one thread
+//               marches along a segment of a grid line, and the first cell of every segment after a
+//               line's first gets its update from the two fluxes that the neighbouring segments hand over
+//               in the seam buffer.  Same bits as the tiles
 //   k_source / k_stage   body-force source, RK3 stage combination, non-finite check
 //   k_stage_prim / k_halo_prim   the stage combination fused with the primitives of its result
 //               (interior cells), then the halo cells from those; fluid_step uses this pair in
@@ -571,8 +570,8 @@ __device__ __forceinline__ float cell_rate32(const double* __restrict__ W, const
 }
 
 // Per-block maxima of the rate go to `partial`; the last block to finish reduces them and stores dt (no
-// second launch).  nparts 0: a fixed dt, one block.  Block 0 counts nothing it did not write: the
-// ticket wraps to 0 for the next call.
+// second launch).  nparts 0: a fixed dt, one block.  The ticket wraps to 0 at the last block, so nothing has
+// to reset it for the next call.
 // The FP64 rates bind (about 60 FP64-pipe instructions per cell), so a block first finds its largest
 // FP32 rate and forms in FP64 only the cells within 1e-3 of it: the maximum is among them, bit
 // for bit (TGV 128^3: 228 us with every cell in FP64 and the second launch).

@@ -47,7 +47,9 @@ __device__ __forceinline__ float rsqrtf_a(float y) {
   float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y)); return r;
 }
 
-// ---- bulk-copy staging: cp.async.bulk (the TMA unit's untiled copy) completing on an mbarrier ----
+// ---- bulk copies into shared memory: cp.async.bulk (the TMA unit's untiled copy) completing on an mbarrier,
+// with a bounded wait.  The face kernels load plainly (bulk-staged tiles were slower); what is here serves
+// fluid_check_bulk_staging (k_bulk_probe) ----
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
 }
@@ -722,7 +724,7 @@ constexpr int kBulkRow = 36;    // floats per row of the probe
 namespace {
 // Check of the bulk-staging helpers: one warp stages nrows rows of 36 floats (16-byte aligned) from
 // src into shared memory on one mbarrier whose expected transaction count is the rows' bytes plus
-// extra_tx, waits with the tiles' bounded wait and copies the rows to dst.  With extra_tx > 0 the
+// extra_tx, waits with the bounded wait and copies the rows to dst.  With extra_tx > 0 the
 // phase cannot complete (every copy lands, the count stays short), so the wait runs out: the block
 // sets FLAG_STAGING in *flags, waits once more and returns without writing dst.
 constexpr int kProbeRows = 8;

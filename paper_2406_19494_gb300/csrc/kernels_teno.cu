@@ -12,7 +12,7 @@
 // not decide (about 2 windows in 1e5).  The face values are FP64 combinations of the second differences
 // with tabulated factors; HLLC's star correction and the dissipative flux are two-float terms where
 // they are small against the state, else FP64.  On the channel 192 x 128 x 128 with 5 % noise (where
-// HLLC stays FP64 on most faces) a launch takes 1.8 to 2.2 ms; with everything in FP64 (1,149 FP64-pipe
+// HLLC stays FP64 on most faces) a launch takes 1.7 to 2.1 ms; with everything in FP64 (1,149 FP64-pipe
 // instructions per face) it took 7.8 ms.
 #include <cuda_runtime.h>
 
@@ -52,7 +52,8 @@ struct TenoShared {
   double T[NVW][N];           // second differences
   double d[NVW][N];           // q_{j+1} - q_j
   double F[5][N];
-  double q[5][N];             // primitives, for the reads after the calls (from global memory: x, y, z launches 3, 2, 2.5 % longer)
+  // primitives, for the reads after the calls (from global memory the x, y, z launches took 3, 2, 2.5 % longer)
+  double q[5][N];
   unsigned char lev[5][N];    // cut-off levels of the cells
   double alpha[4][16], omega[4][16];
 };
